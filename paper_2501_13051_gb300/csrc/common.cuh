@@ -158,13 +158,105 @@ __device__ __forceinline__ uint32_t block_exclusive_max(uint32_t v, uint32_t* sm
 // is bit sum_k v_k << shift_k, with shift_k the bits of the columns after k.
 // Increasing bit order is then the tuples' lexicographic order, and setting
 // a bit twice is a no-op, so the bitmap is a sorted set.
+//
+// Two uses: the new tuples of one round (append == 0: join outputs only set
+// bits, which are read back in order), and Full itself (append == 1: a join
+// output whose bit was not set yet is new, and is appended to the round's
+// delta rows by whoever set it).
 struct DenseSet {
   uint32_t* words;  // nbits / 32 words (at least one)
   uint64_t nbits;   // 2^T
   uint32_t k;
+  uint32_t append;
   uint32_t shift[kMaxK];
   uint32_t mask[kMaxK];  // 2^bits_k - 1
 };
+
+// Position of tuple v in the packed tuple space of d; kNoTuple when v lies
+// outside it.
+constexpr uint64_t kNoTuple = ~0ull;
+__device__ __forceinline__ uint64_t set_pack(const DenseSet& d, const uint32_t (&v)[kMaxK]) {
+  uint64_t idx = 0;
+  bool out = false;
+#pragma unroll
+  for (int k = 0; k < kMaxK; ++k)
+    if (k < (int)d.k) {
+      idx |= (uint64_t)v[k] << d.shift[k];
+      out |= v[k] > d.mask[k];
+    }
+  return out || idx >= d.nbits ? kNoTuple : idx;
+}
+__device__ __forceinline__ uint32_t set_column(const DenseSet& d, uint64_t idx, int k) {
+  return (uint32_t)(idx >> d.shift[k]) & d.mask[k];
+}
+
+// Adds the tuples idx[0..N) (kNoTuple: none) to Full's bitmap; bit q of the
+// result tells that this call set tuple q's bit, i.e. the tuple is new.  A
+// set bit never goes back, so one seen set by a plain read (of any age, from
+// L1 or L2) needs no atomic; the N reads, then the N atomics, are in flight
+// together.
+template <int N>
+__device__ __forceinline__ uint32_t set_add(const DenseSet& d, const uint64_t (&idx)[N]) {
+  uint32_t seen[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    seen[q] = idx[q] != kNoTuple ? d.words[idx[q] >> 5] >> (idx[q] & 31) & 1u : 1u;
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if (!seen[q]) seen[q] = atomicOr(d.words + (idx[q] >> 5), 1u << (idx[q] & 31)) >> (idx[q] & 31) & 1u;
+  uint32_t fresh = 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q) fresh |= (seen[q] ^ 1u) << q;
+  return fresh;
+}
+
+// Writes a block's new tuples (bit q of fresh: tuple idx[q] is new) packed at
+// *cursor: one claim per block, each warp's tuples of one q side by side.
+// wsum: THREADS / 32 + 2 words of shared memory (the last two hold the
+// claimed position).  Rows past cap are dropped; false tells the caller.
+template <int THREADS, int N>
+__device__ __forceinline__ bool set_emit(const DenseSet& d, const uint64_t (&idx)[N],
+                                         uint32_t fresh, ColsOut out, uint64_t base,
+                                         unsigned long long* cursor, uint64_t cap,
+                                         uint32_t* wsum) {
+  constexpr int W = THREADS / 32;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint32_t n = 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q) n += __popc(__ballot_sync(0xffffffffu, (fresh >> q) & 1u));
+  if (lane == 0) wsum[warp] = n;
+  __syncthreads();
+  unsigned long long* at = reinterpret_cast<unsigned long long*>(wsum + W);
+  uint32_t before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    const uint32_t c = wsum[w];
+    before += w < (int)warp ? c : 0u;
+    total += c;
+  }
+  if (total == 0) return true;  // uniform
+  if (threadIdx.x == 0) *at = atomicAdd(cursor, (unsigned long long)total);
+  __syncthreads();
+  uint64_t pos = base + *at + before;
+  bool ok = true;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const uint32_t bal = __ballot_sync(0xffffffffu, (fresh >> q) & 1u);
+    if ((fresh >> q) & 1u) {
+      const uint64_t p = pos + __popc(bal & lt);
+      if (p < cap) {
+#pragma unroll
+        for (int k = 0; k < kMaxK; ++k)
+          if (k < (int)d.k) out.c[k][p] = set_column(d, idx[q], k);
+      } else {
+        ok = false;
+      }
+    }
+    pos += __popc(bal);
+  }
+  return ok;
+}
 
 // The word and bit of tuple v in d; false when v lies outside d.
 __device__ __forceinline__ bool dense_locate(const DenseSet& d, const uint32_t (&v)[kMaxK],

@@ -36,6 +36,37 @@ __global__ void __launch_bounds__(256) k_dense_insert(DenseSet d, ColsIn rows, u
   }
 }
 
+// Rows appended to Full's bitmap: the new ones (their bit was clear) go out
+// packed at *cursor.
+constexpr int kAT = 256, kAItems = 4;
+__global__ void __launch_bounds__(kAT) k_set_insert(DenseSet d, ColsIn rows, uint64_t n,
+                                                    ColsOut out, unsigned long long* cursor,
+                                                    uint64_t cap, uint32_t* err) {
+  __shared__ __align__(8) uint32_t red[kAT / 32 + 2];
+  constexpr uint64_t kTile = (uint64_t)kAT * kAItems;
+  for (uint64_t b = blockIdx.x * kTile; b < n; b += gridDim.x * kTile) {
+    uint64_t idx[kAItems];
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < kAItems; ++q) {
+      const uint64_t i = b + (uint64_t)q * kAT + threadIdx.x;
+      uint32_t v[kMaxK] = {0, 0, 0, 0};
+      idx[q] = kNoTuple;
+      if (i < n) {
+#pragma unroll
+        for (int k = 0; k < kMaxK; ++k)
+          if (k < (int)d.k) v[k] = __ldg(rows.c[k] + i);
+        idx[q] = set_pack(d, v);
+        bad |= idx[q] == kNoTuple;
+      }
+    }
+    const uint32_t fresh = set_add<kAItems>(d, idx);
+    bad |= !set_emit<kAT, kAItems>(d, idx, fresh, out, 0, cursor, cap, red);
+    if (bad && err) atomicOr(err, kErrCapacity);
+    __syncthreads();  // the next tile reuses red
+  }
+}
+
 // The words a thread owns: [w0, w0 + kXWords) clipped to nw.
 __device__ __forceinline__ void load_words(const uint32_t* words, uint64_t w0, uint64_t nw,
                                            uint32_t (&w)[kXWords]) {
@@ -64,12 +95,18 @@ __global__ void __launch_bounds__(kXT) k_dense_count(const uint32_t* __restrict_
   if (threadIdx.x == 0) counts[blockIdx.x] = total;
 }
 
-// Rows of the set bits at their ranks, in bit order; the words are cleared
-// behind the read so that the bitmap starts the next round empty.
+// Rows of the set bits at their ranks, in bit order; a round's bitmap is
+// cleared behind the read so that it starts the next round empty.  The set
+// bits' positions in the block's words (16 bits each) are staged in shared
+// memory, kXStage at a time, so that a column's rows leave as contiguous
+// stores whatever the density.
+constexpr uint32_t kXStage = 4096;
 __global__ void __launch_bounds__(kXT) k_dense_write(DenseSet d, uint64_t nw,
                                                      const uint64_t* __restrict__ offs,
                                                      ColsOut out, uint64_t cap, uint32_t* err) {
+  static_assert(kXTile * 32 <= 65536, "a staged position has 16 bits");
   __shared__ uint32_t red[kXT / 32 + 1];
+  __shared__ uint16_t stage[kXStage];
   const uint64_t w0 = (uint64_t)blockIdx.x * kXTile + (uint64_t)threadIdx.x * kXWords;
   uint32_t w[kXWords];
   load_words(d.words, w0, nw, w);
@@ -77,23 +114,39 @@ __global__ void __launch_bounds__(kXT) k_dense_write(DenseSet d, uint64_t nw,
 #pragma unroll
   for (int i = 0; i < kXWords; ++i) c += __popc(w[i]);
   uint32_t total;
-  uint64_t pos = offs[blockIdx.x] + block_exclusive_sum<kXT, uint32_t>(c, red, &total);
+  uint32_t pos = block_exclusive_sum<kXT, uint32_t>(c, red, &total);
+  if (!d.append) {
 #pragma unroll
-  for (int i = 0; i < kXWords; ++i) {
-    uint32_t x = w[i];
-    if (x) d.words[w0 + i] = 0u;
-    while (x) {
-      const uint64_t idx = ((w0 + i) << 5) | (uint64_t)(__ffs(x) - 1);
-      x &= x - 1;
-      if (pos < cap) {
+    for (int i = 0; i < kXWords; ++i)
+      if (w[i]) d.words[w0 + i] = 0u;
+  }
+  const uint64_t first = offs[blockIdx.x];
+  const uint64_t bit0 = (uint64_t)blockIdx.x * kXTile * 32;
+  for (uint32_t s0 = 0; s0 < total; s0 += kXStage) {
+    if (pos < s0 + kXStage) {  // the thread's next positions, up to the stage's end
+#pragma unroll
+      for (int i = 0; i < kXWords; ++i) {
+        while (w[i] && pos < s0 + kXStage) {
+          stage[pos - s0] = (uint16_t)(((threadIdx.x * kXWords + i) << 5) | (__ffs(w[i]) - 1));
+          w[i] &= w[i] - 1;
+          ++pos;
+        }
+      }
+    }
+    __syncthreads();
+    const uint32_t m = total - s0 < kXStage ? total - s0 : kXStage;
+    for (uint32_t i = threadIdx.x; i < m; i += kXT) {
+      const uint64_t idx = bit0 + stage[i];
+      const uint64_t at = first + s0 + i;
+      if (at < cap) {
 #pragma unroll
         for (int k = 0; k < kMaxK; ++k)
-          if (k < (int)d.k) out.c[k][pos] = (uint32_t)(idx >> d.shift[k]) & d.mask[k];
+          if (k < (int)d.k) out.c[k][at] = set_column(d, idx, k);
       } else {
         atomicOr(err, kErrCapacity);
       }
-      ++pos;
     }
+    __syncthreads();
   }
 }
 
@@ -105,6 +158,17 @@ cudaError_t dense_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n) {
   uint64_t blocks = (n + 255) / 256;
   if (blocks > 152 * 16) blocks = 152 * 16;
   k_dense_insert<<<(unsigned)blocks, 256, 0, c.st>>>(d, rows, n, c.d_err);
+  return cudaGetLastError();
+}
+
+cudaError_t set_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n, ColsOut out,
+                       uint64_t* d_cursor, uint64_t out_cap) {
+  if (n == 0) return cudaSuccess;
+  ProfScope p(c, kDense, 4.0 * d.k * n);
+  uint64_t blocks = (n + kAT * kAItems - 1) / (kAT * kAItems);
+  if (blocks > 152 * 16) blocks = 152 * 16;
+  k_set_insert<<<(unsigned)blocks, kAT, 0, c.st>>>(
+      d, rows, n, out, reinterpret_cast<unsigned long long*>(d_cursor), out_cap, c.d_err);
   return cudaGetLastError();
 }
 

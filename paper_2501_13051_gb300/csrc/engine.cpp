@@ -313,6 +313,19 @@ struct Relation {
   uint64_t dense_ub = 0;  // tuples sent to dset this round: a bound on its bits
   DCols dense_rows;
   Dsm dsm;
+  // Full as a set (step (d) of relations whose Full no rule variant reads
+  // after round 1): one bit per tuple of the tuple space.  A join output
+  // whose bit was clear is new and goes straight to the round's delta rows;
+  // nothing is sorted or merged, and Full's rows are taken out of the bitmap
+  // in order when the run ends.  full.n is then |Full|, its columns unused.
+  bool set_ok = false;   // no rule variant reads Full after round 1
+  bool set_on = false;   // Full is fset now
+  bool set_free = false; // within dense_bits: a round's join outputs are not limited to 2^32
+  DenseSet fset{};
+  DBuf fset_buf;
+  DCols sdelta;          // the round's new tuples so far (dslot(kSlotDelta + i) of them)
+  uint64_t sdelta_ub = 0;
+  double merged_bytes = 0;  // row form: bytes its sorts and merges have moved
 };
 
 struct Term {
@@ -429,6 +442,25 @@ struct cdl_engine {
   static constexpr uint64_t kPredictMinRows = 1 << 15;  // smaller probes keep the count pass
   static constexpr int kDenseBits = 28;  // default bound of a dense relation's tuple space (32 MB)
   static constexpr int kDenseBitsMax = 34;  // largest bitmap form accepted (2 GB per relation)
+  // Full as a bitmap that the row form goes over to (set_switch): at most
+  // 2^37 bits (16 GB, and 32-bit word numbers), once its sorts and merges
+  // have moved kSetSwitch times the bitmap's bytes.  Same generation on
+  // 200,000 nodes (2^36 bits), ms per fixpoint: 267 in the row form
+  // throughout, 129 with a factor of 3, 112 with 1, 109 with 0.2, 107 with
+  // 0.05; a fixpoint that ends soon after pays the bitmap's passes for
+  // nothing, so not lower.
+  static constexpr uint32_t kSetBits = 37;
+  static constexpr double kSetSwitch = 0.2;
+  // hub joins (hub_join): outputs in all, and per row of both sides, from
+  // which they are tried (below, the second count and the other index are
+  // not small beside the write); build rows that make a hub, where OR-ing
+  // its words beats setting its bits.  The share of words per row hardly
+  // matters between 1 and 64 (points-to at 2^-7: 15.7 to 15.3 ms); 16 bounds
+  // the hubs' bitmaps to 64 bytes per build row.
+  static constexpr uint64_t kHubOutputs = 1 << 22;
+  static constexpr uint64_t kHubOutputsPerRow = 8;
+  static constexpr uint32_t kHubMinRows = 32;
+  static constexpr uint32_t kHubWordsPerRow = 16;
   static constexpr uint64_t kGroupRows = 1 << 21;  // larger new-tuple sets sort on their own
   static constexpr size_t kGroupMin = 4;           // fewer relations sort one by one
   struct Deferred {
@@ -726,7 +758,157 @@ struct cdl_engine {
       R.dsm.on = opt.dedup > 0 && R.idb && !full_read[i] && !opt.n_instances;
       // out of core: Full that only step (d) reads lives in pinned host memory
       R.host_full = opt.host_full > 0 && R.idb && !full_read[i] && !opt.n_instances && !R.dsm.on;
+      // Full as a set leaves deltas in no order; the estimator's features are
+      // stride samples of sorted ones
+      R.set_ok = opt.dense_bits >= 0 && !opt.graph && !opt.estimator && R.idb && !full_read[i] &&
+                 !opt.n_instances && !R.dsm.on && !R.host_full;
     }
+  }
+
+  // ------------------------------------------------------ Full as a set
+  // The packed tuple space of R's column bounds; false past 2^max_bits.
+  bool tuple_space(const Relation& R, uint32_t max_bits, DenseSet& d) const {
+    uint32_t bits[kMaxK], T = 0;
+    for (uint32_t k = 0; k < R.arity; ++k) T += bits[k] = bits_of(R.bound[k]);
+    if (R.arity == 0 || T > max_bits) return false;
+    d = DenseSet{};
+    d.nbits = 1ull << T;
+    d.k = R.arity;
+    uint32_t sh = 0;
+    for (int k = (int)R.arity - 1; k >= 0; --k) {
+      d.shift[k] = sh;
+      d.mask[k] = (uint32_t)((1ull << bits[k]) - 1);
+      sh += bits[k];
+    }
+    return true;
+  }
+
+  // Full's rows move into a bitmap of the tuple space (rows stay while
+  // round 1 reads them).  false without an error when memory is short.
+  cdl_status set_start(Relation& R, const DenseSet& space, bool keep_rows) {
+    const uint64_t bytes = 4 * (space.nbits >= 32 ? space.nbits >> 5 : 1);
+    R.fset_buf = alloc(bytes);
+    if (!R.fset_buf.p) return CDL_OK;
+    R.fset = space;
+    R.fset.words = static_cast<uint32_t*>(R.fset_buf.p);
+    R.fset.append = 1;
+    cudaError_t e = cudaMemsetAsync(R.fset_buf.p, 0, bytes, st);
+    DenseSet plain = R.fset;  // the rows only set bits here
+    plain.append = 0;
+    if (e == cudaSuccess) e = dense_insert(ctx, plain, R.full.in(), R.full.n);
+    if (e != cudaSuccess) return cuda_fail(e, "full set");
+    R.set_on = true;
+    if (!keep_rows) set_drop_rows(R);
+    return CDL_OK;
+  }
+
+  void set_drop_rows(Relation& R) {
+    const uint64_t n = R.full.n;
+    R.full.clear();
+    R.full.k = R.arity;
+    R.full.n = n;
+  }
+
+  // A relation in the row form whose sorts and merges have cost about what
+  // its bitmap costs (cleared once, read twice at the end) goes over to it:
+  // whatever the number of rounds to come, the two forms' costs together
+  // stay within a small factor of the better one's.  The bitmap must fit
+  // beside the rows: a quarter of the free device memory, or, under a memory
+  // limit, no more than Full's rows take (the row form holds Full twice).
+  cdl_status set_switch(Relation& R) {
+    DenseSet space;
+    if (!R.set_ok || R.set_on || R.dset.words || !tuple_space(R, kSetBits, space)) return CDL_OK;
+    const uint64_t bytes = space.nbits >> 3;
+    if (R.merged_bytes < kSetSwitch * (double)bytes) return CDL_OK;
+    if (opt.mem_limit) {
+      if (bytes > 4ull * R.arity * R.full.n) return CDL_OK;
+    } else {
+      size_t free_b = 0, total_b = 0;
+      if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return CDL_OK;
+      if (bytes > free_b / 4) return CDL_OK;
+    }
+    return set_start(R, space, false);
+  }
+
+  // Room for the round's new tuples of a join with `extra` outputs.
+  cdl_status ensure_sdelta(Relation& R, uint64_t extra) {
+    if (!R.set_free && R.sdelta_ub + extra > 0xFFFFFFFFull)
+      return fail(CDL_E_CAPACITY, "relation " + R.name + " would receive more than 2^32 new "
+                                  "tuples in one round");
+    const uint64_t old_ub = R.sdelta_ub;
+    R.sdelta_ub += extra;
+    const uint64_t need = std::min(R.sdelta_ub, R.fset.nbits - std::min(R.fset.nbits, R.full.n));
+    if (R.sdelta.buf.p && need <= R.sdelta.cap) return CDL_OK;
+    DCols nb;
+    uint64_t cap = std::max<uint64_t>(need, 1024);
+    if (R.sdelta.buf.p) cap = std::max(cap, std::min(R.sdelta.cap + R.sdelta.cap / 2, R.fset.nbits));
+    if (!alloc_cols(nb, R.arity, cap)) return fail(CDL_E_NOMEM, "new-tuple buffer");
+    const uint64_t rows = std::min(old_ub, R.sdelta.cap);
+    for (uint32_t k = 0; k < R.arity && R.sdelta.buf.p && rows; ++k) {
+      cudaError_t e = cudaMemcpyAsync(nb.c[k], R.sdelta.c[k], rows * 4, cudaMemcpyDeviceToDevice, st);
+      if (e != cudaSuccess) return cuda_fail(e, "grow new-tuple buffer");
+    }
+    R.sdelta = std::move(nb);
+    return CDL_OK;
+  }
+
+  // The rows written to fresh this round (copies, single-pass joins) join
+  // the set as well.
+  cdl_status set_fresh_rows() {
+    for (uint32_t i = 0; i < rels.size(); ++i) {
+      Relation& R = *rels[i];
+      if (!R.set_on) continue;
+      const uint64_t nf = std::min<uint64_t>(h_ctl[kSlotCursor + i], R.fresh.cap);
+      if (nf == 0) continue;
+      cdl_status r = ensure_sdelta(R, nf);
+      if (r != CDL_OK) return r;
+      cudaError_t e = set_insert(ctx, R.fset, R.fresh.in(), nf, R.sdelta.out(), dslot(kSlotDelta + i),
+                                 R.sdelta.cap);
+      if (e != cudaSuccess) return cuda_fail(e, "full set");
+    }
+    return CDL_OK;
+  }
+
+  // At the end of the run Full's rows come out of the set in order; a delta
+  // that a checkpoint may save is put in order too.  After a failed run the
+  // set also holds the stopped round's tuples so far.
+  cdl_status set_finish(bool failed) {
+    for (auto& rp : rels) {
+      Relation& R = *rp;
+      if (!R.set_on) continue;
+      uint64_t n = R.full.n;
+      if (failed) n = std::min(R.fset.nbits, n + std::min(R.sdelta_ub, R.sdelta.cap));
+      R.sdelta.clear();
+      DCols rows;
+      DBuf ws = alloc(dense_extract_workspace(R.fset.nbits));
+      if (!alloc_cols(rows, R.arity, n) || !ws.p) {
+        R.set_on = false;  // (no rows to export)
+        R.full.n = 0;
+        return fail(CDL_E_NOMEM, "sorted rows");
+      }
+      if (n) {
+        cudaError_t e = dense_extract(ctx, R.fset, rows.out(), n, dslot(kSlotScratch), ws.p);
+        if (e == cudaSuccess && failed) {
+          e = cudaMemcpyAsync(h_ctl + kSlotScratch, dslot(kSlotScratch), 8, cudaMemcpyDeviceToHost, st);
+          if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+          n = std::min(n, h_ctl[kSlotScratch]);
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "sorted rows");
+      }
+      rows.n = n;
+      R.full = std::move(rows);
+      R.version[kFull]++;
+      R.fset_buf.reset();
+      R.fset = DenseSet{};
+      R.set_on = false;
+      if (R.delta.n) {
+        uint32_t bits[kMaxK];
+        for (uint32_t k = 0; k < R.arity; ++k) bits[k] = bits_of(R.bound[k]);
+        cdl_status r = sort_cols(R.delta, bits);
+        if (r != CDL_OK) return r;
+      }
+    }
+    return CDL_OK;
   }
 
   DsmView dsm_view(const Relation& R) const {
@@ -940,6 +1122,8 @@ struct cdl_engine {
     ix->n = s.n;
     bool prefix = true;
     for (size_t i = 0; i < key.size(); ++i) prefix &= key[i] == i;
+    // (a delta of a relation kept as a set is in no order)
+    if (s.rel >= 0 && s.ver == kDelta && rels[s.rel]->set_on) prefix = false;
     if (prefix) {
       for (uint32_t c = 0; c < s.k; ++c) ix->cols[c] = s.c[c];
     } else {
@@ -1493,7 +1677,8 @@ struct cdl_engine {
       // a prediction pays off where the count pass it saves is not trivial
       // (a dense head needs no buffer sized: its tuples become bits)
       const bool predict = ix != nullptr && !js.star && est_ready() && !force_exact &&
-                           !(last && rels[rule.head.rel]->dset.words) &&
+                           !(last && (rels[rule.head.rel]->dset.words ||
+                                      rels[rule.head.rel]->set_on)) &&
                            P.n >= (opt.est_min_rows ? opt.est_min_rows : kPredictMinRows);
       const bool feats = ix != nullptr && !js.star && (predict || opt.estimator >= 2);
       auto features = [&]() {
@@ -1675,9 +1860,24 @@ struct cdl_engine {
       }
       if (total == 0) return CDL_OK;
       ws.reset();
+      if (last && !C && !filter && !js.cross && opt.estimator < 2) {
+        bool done = false;
+        r = hub_join(rule, P, B, js, ix, hkey, bkey.size(), total, done);
+        if (r != CDL_OK || done) return r;
+      }
       const size_t wws = join_write_workspace(P.n, total);
       DBuf wsp = alloc(wws);
       if (!wsp.p) return fail(CDL_E_NOMEM, "join splits");
+      if (last && rels[rule.head.rel]->set_on) {  // Full is a set: new tuples go to delta
+        Relation& H = *rels[rule.head.rel];
+        r = ensure_sdelta(H, total);
+        if (r != CDL_OK) return r;
+        e = join_write(ctx, js, static_cast<const uint64_t*>(off.p), total, H.sdelta.out(), 0,
+                       dslot(kSlotDelta + rule.head.rel), H.sdelta.cap, wsp.p, wws, nullptr, nullptr,
+                       nullptr, &H.fset);
+        if (e != cudaSuccess) return cuda_fail(e, "join write");
+        return CDL_OK;
+      }
       if (last && rels[rule.head.rel]->dset.words) {  // a dense head: bits, not rows
         Relation& H = *rels[rule.head.rel];
         H.dense_ub += total;
@@ -1719,6 +1919,96 @@ struct cdl_engine {
     return CDL_OK;
   }
 
+  // A join with many outputs per input row whose head is a bitmap, where one
+  // side gives the last head column and the other (or constants) the rest:
+  // hub keys OR their bitmap row into their probe rows' head rows
+  // (kernels.h, HubPlan); the side of the last column is the build side,
+  // whichever the plan chose.  Taken when the counted outputs are far more
+  // than the rows on both sides, so that the other side's index and the
+  // second count cost little beside the write; done = false leaves the join
+  // to the plain write.
+  cdl_status hub_join(const RuleR& rule, Src& P, Src& B, JoinSpec js, Index* ix,
+                      const std::vector<uint32_t>& hkey, size_t nkeys, uint64_t total, bool& done) {
+    Relation& H = *rels[rule.head.rel];
+    const DenseSet* d = H.set_on ? &H.fset : H.dset.words ? &H.dset : nullptr;
+    const uint32_t lastc = H.arity - 1;
+    if (!d || nkeys > 2 || total < kHubOutputs || total / kHubOutputsPerRow < P.n + B.n)
+      return CDL_OK;
+    const uint32_t bits = bits_of(d->mask[lastc]);
+    if (bits < 8 || d->k != js.out_k) return CDL_OK;
+    // the last head column's side builds; every other one comes from the other
+    const uint32_t side = js.out[lastc].side;
+    if (side > 1) return CDL_OK;
+    for (uint32_t k = 0; k < lastc; ++k)
+      if (js.out[k].side == side) return CDL_OK;
+    // (a key column holds one value for all of a key's build rows)
+    const uint32_t lv = js.out[lastc].v;
+    if (side == 1 && std::find(hkey.begin(), hkey.end(), lv) != hkey.end()) return CDL_OK;
+    if (side == 0 && (lv == js.pk0 || lv == js.pk1)) return CDL_OK;
+    // both sides indexed on the key: the build side's index lists the hubs,
+    // the other's gives each hub's probe rows (its columns are the probe's)
+    std::unique_ptr<Index> temp;
+    Index* pix = nullptr;
+    std::vector<uint32_t> pkey{js.pk0};
+    if (js.pk1 != 0xFFu) pkey.push_back(js.pk1);
+    cdl_status r = get_index(P, pkey, &pix, temp);
+    if (r != CDL_OK) return r;
+    if (side == 0) std::swap(ix, pix);  // (ix: the build side)
+    const std::vector<uint32_t>& key = side == 0 ? hkey : pkey;
+    JoinSpec f{};
+    f.n_probe = pix->n;
+    f.pk0 = key[0];
+    f.pk1 = key.size() > 1 ? key[1] : 0xFFu;
+    const uint32_t pk = side == 0 ? B.k : P.k, bk = side == 0 ? P.k : B.k;
+    for (uint32_t c = 0; c < pk; ++c) f.probe.c[c] = pix->cols[c];
+    for (uint32_t c = 0; c < bk; ++c) f.build.c[c] = ix->cols[c];
+    f.table = static_cast<const Slot*>(ix->table.p);
+    f.slots = ix->slots;
+    f.out_k = js.out_k;
+    for (uint32_t k = 0; k < js.out_k; ++k)
+      f.out[k] = js.out[k].side > 1 ? js.out[k]
+                                    : Ref{(uint8_t)(js.out[k].side == side ? 1 : 0), js.out[k].v};
+    HubPlan hp{};
+    hp.words = 1u << (bits - 5);
+    hp.col = f.build.c[f.out[lastc].v];
+    hp.probe_table = static_cast<const Slot*>(pix->table.p);
+    hp.probe_slots = pix->slots;
+    f.hub_min = std::max<uint32_t>(kHubMinRows, hp.words / kHubWordsPerRow);
+    hp.cap = std::min<uint64_t>(ix->n / f.hub_min, ix->distinct);
+    if (hp.cap == 0) return CDL_OK;  // no key can be a hub
+    DBuf off = alloc(std::max<uint64_t>(f.n_probe, 1) * 8), ws = alloc(join_count_workspace(f.n_probe)),
+         hws = alloc(hub_workspace(f, hp));
+    if (!off.p || !ws.p || !hws.p) return CDL_OK;
+    // the keys that are no hubs: counted again, written pair by pair
+    cudaError_t e = join_count_scan(ctx, f, static_cast<uint64_t*>(off.p), dslot(kSlotScratch), ws.p);
+    if (e != cudaSuccess) return cuda_fail(e, "hub join");
+    r = fetch(kSlotScratch, 1);
+    if (r != CDL_OK) return r;
+    const uint64_t light = h_ctl[kSlotScratch];
+    if (light == total) return CDL_OK;  // no hubs after all
+    const size_t wws = join_write_workspace(f.n_probe, light);
+    DBuf wsp = alloc(wws);
+    if (!wsp.p) return fail(CDL_E_NOMEM, "join splits");
+    ColsOut out{};
+    uint64_t* cursor = nullptr;
+    uint64_t cap = 0;
+    if (H.set_on) {
+      r = ensure_sdelta(H, total);
+      if (r != CDL_OK) return r;
+      out = H.sdelta.out();
+      cursor = dslot(kSlotDelta + rule.head.rel);
+      cap = H.sdelta.cap;
+    } else {
+      H.dense_ub += total;
+    }
+    e = join_write(ctx, f, static_cast<const uint64_t*>(off.p), light, out, 0, cursor, cap, wsp.p, wws,
+                   nullptr, nullptr, nullptr, d);
+    if (e == cudaSuccess) e = hub_or(ctx, f, hp, *d, out, cursor, cap, hws.p);
+    if (e != cudaSuccess) return cuda_fail(e, "join write");
+    done = true;
+    return CDL_OK;
+  }
+
   // A body atom that reads its relation's columns as they are (distinct
   // variables only): its source needs no selection kernel.
   static bool plain_atom(const AtomR& a) {
@@ -1755,7 +2045,8 @@ struct cdl_engine {
   }
 
   // Derived relations whose tuple space has at most 2^dense_bits tuples (not
-  // batched) get a bitmap of that space, empty between rounds.
+  // batched) get a bitmap of that space: of a round's new tuples, empty
+  // between rounds, or, where no rule variant reads Full, of Full itself.
   cdl_status setup_dense() {
     const int dmax = opt.dense_bits == 0 ? kDenseBits : opt.dense_bits;
     for (auto& rp : rels) {
@@ -1763,24 +2054,26 @@ struct cdl_engine {
       R.dset = DenseSet{};
       R.dset_buf.reset();
       R.dense_rows.clear();
-      if (!R.idb || opt.n_instances || dmax <= 0 || R.arity == 0) continue;
-      uint32_t bits[kMaxK], T = 0;
-      for (uint32_t k = 0; k < R.arity; ++k) T += bits[k] = bits_of(R.bound[k]);
-      if (T > (uint32_t)std::min(dmax, kDenseBitsMax)) continue;
-      const uint64_t nw = T >= 5 ? (1ull << (T - 5)) : 1;
+      R.set_on = R.set_free = false;
+      R.fset_buf.reset();
+      R.merged_bytes = 0;
+      if (!R.idb || opt.n_instances || dmax <= 0) continue;
+      DenseSet space;
+      if (!tuple_space(R, (uint32_t)std::min(dmax, kDenseBitsMax), space)) continue;
+      if (R.set_ok) {  // Full itself as a bitmap
+        cdl_status r = set_start(R, space, true);
+        if (r != CDL_OK) return r;
+        if (!R.set_on) return fail(CDL_E_NOMEM, "dense set");
+        R.set_free = true;
+        continue;
+      }
+      const uint64_t nw = space.nbits >= 32 ? space.nbits >> 5 : 1;
       R.dset_buf = alloc(4 * nw);
       if (!R.dset_buf.p) return fail(CDL_E_NOMEM, "dense set");
       cudaError_t e = cudaMemsetAsync(R.dset_buf.p, 0, 4 * nw, st);
       if (e != cudaSuccess) return cuda_fail(e, "dense set");
+      R.dset = space;
       R.dset.words = static_cast<uint32_t*>(R.dset_buf.p);
-      R.dset.nbits = 1ull << T;
-      R.dset.k = R.arity;
-      uint32_t sh = 0;
-      for (int k = (int)R.arity - 1; k >= 0; --k) {
-        R.dset.shift[k] = sh;
-        R.dset.mask[k] = (uint32_t)((1ull << bits[k]) - 1);
-        sh += bits[k];
-      }
     }
     return CDL_OK;
   }
@@ -2017,7 +2310,7 @@ struct cdl_engine {
       for (uint32_t i = 0; i < rels.size(); ++i) {
         const Relation& R = *rels[i];
         const uint64_t n = h_ctl[kSlotCursor + i];
-        if (R.idb && !R.dset.words && R.arity == k && n > 0 && n <= kGroupRows &&
+        if (R.idb && !R.dset.words && !R.set_on && R.arity == k && n > 0 && n <= kGroupRows &&
             n <= R.fresh.cap && R.full.n + n <= 0xFFFFFFFFull)
           grp.push_back(i);
       }
@@ -2103,6 +2396,7 @@ struct cdl_engine {
     est_slot.clear();
     est_nb = 0;
     cudaError_t e = cudaMemsetAsync(dslot(kSlotCursor), 0, 8 * nr, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(dslot(kSlotDelta), 0, 8 * nr, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(dslot(kSlotRoundOverflow), 0, 8, st);
     if (e == cudaSuccess && est_ready()) e = cudaMemsetAsync(join_sizes.p, 0, 8 * kMaxDeferred, st);
     if (e != cudaSuccess) return cuda_fail(e, "round reset");
@@ -2110,6 +2404,7 @@ struct cdl_engine {
       r->fresh_ub = 0;
       r->fresh_overflow = false;
       r->dense_ub = 0;
+      r->sdelta_ub = 0;
     }
     if (est_ready() && est_bio.p) {  // the round's predictions, with one wait
       est_plan = true;
@@ -2614,9 +2909,9 @@ struct cdl_engine {
     for (auto& r : rels) r->idb = false;
     for (const RuleR& rule : rules) rels[rule.head.rel]->idb = true;
     propagate_bounds();
+    dsm_select();
     cdl_status ds = setup_dense();
     if (ds != CDL_OK) return ds;
-    dsm_select();
     prof.reset();
     joins = 0;
     index_merges = 0;
@@ -2670,6 +2965,7 @@ struct cdl_engine {
       status = eval_round(round);
       recording = false;
       if (status == CDL_OK) status = extract_dense();
+      if (status == CDL_OK) status = set_fresh_rows();
       if (status != CDL_OK) break;
       // relations of one arity with few new tuples each are sorted as one
       std::vector<DCols> group_bufs, sorted_rows(nr);
@@ -2684,6 +2980,14 @@ struct cdl_engine {
         R.delta.clear();
         R.delta.k = R.arity;
         R.version[kDelta]++;
+        if (R.set_on) {  // the new tuples are delta already
+          if (R.full.buf.p) set_drop_rows(R);
+          R.delta = std::move(R.sdelta);
+          R.sdelta = DCols{};
+          merged[i] = R.sdelta_ub > 0;
+          R.version[kFull]++;
+          continue;
+        }
         e = cudaMemsetAsync(dslot(kSlotDelta + i), 0, 8, st);
         if (e != cudaSuccess) {
           status = cuda_fail(e, "delta reset");
@@ -2730,7 +3034,15 @@ struct cdl_engine {
         const uint64_t nd = merged[i] ? h_ctl[kSlotDelta + i] : 0;
         R.delta.n = nd;
         R.full.n += nd;
-        if (merged[i] && R.dsm.on) {
+        if (R.set_on && R.full.n > 0xFFFFFFFFull) {
+          status = fail(CDL_E_CAPACITY, "relation " + R.name + " would exceed 2^32 tuples");
+          break;
+        }
+        if (merged[i] && !R.set_on)  // the sort's passes and the merge, about
+          R.merged_bytes += 8.0 * R.arity * (double)R.full.n + 64.0 * (double)R.fresh.n;
+        if (R.set_on) {
+          prof.add_bytes(kJoinWrite, 4.0 * R.arity * nd);
+        } else if (merged[i] && R.dsm.on) {
           prof.add_bytes(kDedup, 4.0 * R.arity * nd);  // delta written by the compaction
           status = dsm_append(R);
           if (status != CDL_OK) break;
@@ -2762,6 +3074,9 @@ struct cdl_engine {
         status = fail(CDL_E_MAXITER, "the fixpoint needs more rounds than max_iters");
         break;
       }
+      for (uint32_t i = 0; i < nr && status == CDL_OK; ++i)
+        if (rels[i]->idb) status = set_switch(*rels[i]);
+      if (status != CDL_OK) break;
       if (opt.graph && round == first_semi) {
         graph_ready = graph_plan();
         if (graph_ready) graph_caps();
@@ -2776,8 +3091,13 @@ struct cdl_engine {
     graph_release();
     prev_full.clear();
     if (status == CDL_OK || status == CDL_E_MAXITER) {
-      const cdl_status fs = dsm_finish();
+      cdl_status fs = dsm_finish();
+      if (fs == CDL_OK) fs = set_finish(false);
       if (status == CDL_OK) status = fs;
+    } else {
+      const std::string why = err;
+      set_finish(true);
+      err = why;
     }
     if (opt.n_instances && status == CDL_OK) status = assemble();
     last_rounds = rounds;

@@ -73,6 +73,7 @@ __device__ __forceinline__ uint32_t row_count(const JoinSpec& j, const ColsIn& p
                                              uint64_t mask, uint64_t row, uint32_t* err) {
   uint32_t st;
   const uint32_t c1 = lookup(j, probe, mask, row, &st);
+  if (j.hub_min && c1 >= j.hub_min) return 0;  // hub_or's
   if (!j.star || c1 == 0) return c1;
   const uint64_t prod = (uint64_t)c1 * lookup2(j, probe, row, &st);
   if (prod > 0xFFFFFFFFull) {
@@ -180,16 +181,23 @@ __device__ __forceinline__ uint32_t ref_value(const JoinSpec& j, const ColsIn& p
 // bounded by shared memory); the bit-setting loop is latency-bound, and on
 // points-to at 2^-5 this cap took the write from 6.6 s to 5.6 s per
 // fixpoint against four or five blocks.
-// DENSE: each output tuple sets its bit in dset instead of being written.
-// STAR: output n of probe row j (local index l = n - pos_buf[j]) pairs the
-// first range's row l / c2 with the second range's row l % c2.
-template <bool FILTER, bool DENSE, bool STAR>
-__global__ void __launch_bounds__(kJT, DENSE ? 8 : 5) k_join_write(const JoinSpec j, const uint64_t* __restrict__ off,
+// FORM kBits: each output tuple sets its bit in dset instead of being written.
+// FORM kSet: dset is Full itself; an output whose bit was clear is new and is
+// appended to the delta rows (out, packed at *cursor, one claim per block),
+// so the round needs no sort and no merge.  Bound by the random accesses to
+// the bitmap: a block's outputs are taken in one sweep, eight per thread,
+// all reads and then all atomics in flight.  Same generation on 200,000
+// nodes, where the bitmap is 8 GB: 1.6e9 outputs in 62 ms (2.6e10 per
+// second; the sorts, merges and writes it replaces took 231 ms of 267).
+enum Form : int { kRows = 0, kBits = 1, kSet = 2 };
+template <bool FILTER, int FORM, bool STAR>
+__global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5) k_join_write(const JoinSpec j, const uint64_t* __restrict__ off,
                                                     uint64_t total, ColsOut out, uint64_t base,
                                                     unsigned long long* cursor, uint64_t out_cap,
                                                     const uint64_t* __restrict__ splits,
                                                     uint32_t* err, const uint64_t* dtotal,
                                                     const uint64_t* dbase, const DenseSet dset) {
+  constexpr bool DENSE = FORM == kBits;
   // row r's first output: the carried-in row 0 keeps its global start,
   // every later row starts inside the block's window of at most kJTile
   // outputs and keeps its start relative to the window
@@ -200,7 +208,7 @@ __global__ void __launch_bounds__(kJT, DENSE ? 8 : 5) k_join_write(const JoinSpe
   __shared__ uint32_t s_cnt2[STAR ? kJTile + 1 : 1];
   __shared__ uint16_t s_row[DENSE ? 1 : kJTile];  // staged row of each of the block's outputs
   __shared__ uint64_t s_split[2];
-  __shared__ uint32_t red[kJT / 32 + 1];
+  __shared__ __align__(8) uint32_t red[kJT / 32 + 2];
   __shared__ unsigned long long s_base;
   const uint64_t n_probe = dev_size(j.dn, j.n_probe);
   const ColsIn probe = probe_cols(j);
@@ -225,7 +233,7 @@ __global__ void __launch_bounds__(kJT, DENSE ? 8 : 5) k_join_write(const JoinSpe
     if (threadIdx.x == 32) s_split[1] = merge_split(off, n_probe, total, d1);
   }
   // (a device-sized launch had its range claimed by the split kernel)
-  if (!FILTER && !DENSE && !dbase && tile == 0 && threadIdx.x == 0)
+  if (!FILTER && FORM == kRows && !dbase && tile == 0 && threadIdx.x == 0)
     atomicAdd(cursor, (unsigned long long)total);
   __syncthreads();
   const uint64_t j0 = s_split[0], j1 = s_split[1];
@@ -383,7 +391,24 @@ __global__ void __launch_bounds__(kJT, DENSE ? 8 : 5) k_join_write(const JoinSpe
     if (bad && err) atomicOr(err, kErrCapacity);
    }
   }
-  if constexpr (!DENSE)
+  if constexpr (FORM == kSet) {
+    uint64_t idx[kJItems];
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < kJItems; ++q) {
+      const uint64_t o = o0 + (uint64_t)q * kJT + threadIdx.x;
+      uint32_t vals[kMaxK] = {0, 0, 0, 0};
+      idx[q] = kNoTuple;
+      if (o < o1 && tuple_at(o, vals)) {
+        idx[q] = set_pack(dset, vals);
+        bad |= idx[q] == kNoTuple;
+      }
+    }
+    const uint32_t fresh = set_add<kJItems>(dset, idx);
+    bad |= !set_emit<kJT, kJItems>(dset, idx, fresh, out, wbase, cursor, out_cap, red);
+    if (bad && err) atomicOr(err, kErrCapacity);
+  }
+  if constexpr (FORM == kRows)
   for (uint64_t ob = o0; ob < o1; ob += kJT) {
     const uint64_t o = ob + threadIdx.x;
     const bool valid = o < o1;
@@ -446,6 +471,207 @@ cudaError_t join_count_scan(Ctx& c, const JoinSpec& j, uint64_t* d_off, uint64_t
                                                            static_cast<uint64_t*>(scan_ws), c.d_err);
   }
   return scan_finish(c, counts, j.n_probe, d_off, d_total, scan_ws, j.dn);
+}
+
+// ------------------------------------------------------------- hub keys
+// Numbers the build index's keys with at least hub_min rows and cuts each
+// one's probe rows into tasks of kHubRows.
+constexpr uint32_t kHubRows = 64;
+struct HubTask {
+  uint32_t hub, row, rows;
+};
+
+__global__ void __launch_bounds__(kCT) k_hub_list(const JoinSpec j, const Slot* __restrict__ ptable,
+                                                  uint64_t pslots, uint2* __restrict__ hubs,
+                                                  uint64_t cap, HubTask* __restrict__ tasks,
+                                                  uint64_t task_cap, unsigned long long* n) {
+  for (uint64_t i = (uint64_t)blockIdx.x * kCT + threadIdx.x; i < j.slots;
+       i += (uint64_t)gridDim.x * kCT) {
+    const Slot s = load_slot(j.table, i);
+    if ((s.k0 == kEmpty && s.k1 == kEmpty) || s.count < j.hub_min) continue;
+    uint32_t prow;
+    const uint32_t pn = probe_table(ptable, pslots - 1, s.k0, s.k1, &prow);
+    if (pn == 0) continue;
+    const uint64_t h = atomicAdd(n, 1ull);
+    if (h >= cap) continue;  // (cannot happen: cap counts every such key)
+    hubs[h] = make_uint2(s.start, s.count);
+    const uint32_t nt = (pn + kHubRows - 1) / kHubRows;
+    const uint64_t t0 = atomicAdd(n + 1, (unsigned long long)nt);
+    for (uint32_t t = 0; t < nt && t0 + t < task_cap; ++t)
+      tasks[t0 + t] = HubTask{(uint32_t)h, prow + t * kHubRows,
+                              pn - t * kHubRows < kHubRows ? pn - t * kHubRows : kHubRows};
+  }
+}
+
+// A hub's values as bits; gridDim.y blocks share a hub's rows.
+__global__ void __launch_bounds__(kCT) k_hub_render(const uint2* __restrict__ hubs,
+                                                    const unsigned long long* n_hubs, uint64_t cap,
+                                                    const uint32_t* __restrict__ col,
+                                                    uint32_t* __restrict__ bits, uint32_t words) {
+  const uint64_t n = *n_hubs < cap ? *n_hubs : cap;
+  for (uint64_t h = blockIdx.x; h < n; h += gridDim.x) {
+    const uint2 u = hubs[h];
+    for (uint32_t i = blockIdx.y * kCT + threadIdx.x; i < u.y; i += gridDim.y * kCT) {
+      const uint32_t v = __ldg(col + u.x + i);
+      if ((v >> 5) < words) atomicOr(bits + h * words + (v >> 5), 1u << (v & 31));
+    }
+  }
+}
+
+// One task per block: a thread holds four words of the hub's bitmap row and
+// walks the task's head rows (kHubU of them in flight), reading the four
+// words there and setting only what is missing.  A hub of d build rows costs
+// a probe row 2^b / 128 coalesced 16-byte reads (b the bits of the last head
+// column) instead of d scattered bit reads; bound by the reads of the head's
+// bitmap from L2.  Points-to at scale 2^-7: the joins on hubs took 137 ms
+// pair by pair, 6.8 ms here (the fixpoint 143 -> 15.4 ms); one word per
+// output inside the write kernel took 92 ms (row searches per word).
+constexpr int kHubU = 4;
+template <bool APPEND>
+__global__ void __launch_bounds__(kCT) k_hub_or(const JoinSpec j, const DenseSet d,
+                                                const HubTask* __restrict__ tasks,
+                                                uint64_t task_cap, const unsigned long long* n_tasks,
+                                                const uint32_t* __restrict__ bits, uint32_t words,
+                                                ColsOut out, unsigned long long* cursor,
+                                                uint64_t out_cap, uint32_t* err) {
+  __shared__ uint32_t s_word[kHubRows];  // first word of each head row
+  const uint64_t n = *n_tasks < task_cap ? *n_tasks : task_cap;
+  const uint32_t quads = words / 4, lane = lane_id();
+  // threads side by side on a row's quads; with few quads, several rows at once
+  const uint32_t across = quads < kCT ? quads : kCT;
+  const uint32_t q0 = threadIdx.x % across, r0 = threadIdx.x / across, rstep = kCT / across;
+  for (uint64_t t = blockIdx.x; t < n; t += gridDim.x) {
+    const HubTask k = tasks[t];
+    __syncthreads();  // the last task's rows are done
+    if (threadIdx.x < k.rows) {
+      uint32_t v[kMaxK] = {0, 0, 0, 0};
+#pragma unroll
+      for (int c = 0; c < kMaxK; ++c)
+        if (c + 1 < (int)j.out_k)
+          v[c] = ref_value(j, j.probe, j.out[c], (uint64_t)k.row + threadIdx.x, 0);
+      const uint64_t idx = set_pack(d, v);  // (last column 0: the row's first bit)
+      if (idx == kNoTuple) atomicOr(err, kErrCapacity);
+      s_word[threadIdx.x] = idx == kNoTuple ? 0xFFFFFFFFu : (uint32_t)(idx >> 5);
+    }
+    __syncthreads();
+    // the loops' bounds are the same for a warp's threads (rounded up), so
+    // that the warp packs its new tuples together
+    for (uint32_t qb = 0; qb < quads; qb += across) {
+      const uint32_t q = qb + q0;
+      uint4 h = make_uint4(0u, 0u, 0u, 0u);
+      if (q < quads && r0 < rstep)
+        h = __ldg(reinterpret_cast<const uint4*>(bits + (uint64_t)k.hub * words) + q);
+      const bool any_h = (h.x | h.y | h.z | h.w) != 0u;
+      if (!__any_sync(0xffffffffu, any_h)) continue;
+      for (uint32_t rb = 0; rb < k.rows; rb += rstep * kHubU) {
+        uint4 m[kHubU];
+        uint32_t w[kHubU];
+#pragma unroll
+        for (int u = 0; u < kHubU; ++u) {
+          const uint32_t r = rb + u * rstep + r0;
+          m[u] = make_uint4(0u, 0u, 0u, 0u);
+          w[u] = any_h && r < k.rows ? s_word[r] : 0xFFFFFFFFu;
+          if (w[u] != 0xFFFFFFFFu) {
+            w[u] += 4 * q;
+            const uint4 cur = *reinterpret_cast<const uint4*>(d.words + w[u]);
+            m[u] = make_uint4(h.x & ~cur.x, h.y & ~cur.y, h.z & ~cur.z, h.w & ~cur.w);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kHubU; ++u) {
+          if (m[u].x) m[u].x &= ~atomicOr(d.words + w[u], m[u].x);
+          if (m[u].y) m[u].y &= ~atomicOr(d.words + w[u] + 1, m[u].y);
+          if (m[u].z) m[u].z &= ~atomicOr(d.words + w[u] + 2, m[u].z);
+          if (m[u].w) m[u].w &= ~atomicOr(d.words + w[u] + 3, m[u].w);
+        }
+        if constexpr (APPEND) {
+          uint32_t c = 0;
+#pragma unroll
+          for (int u = 0; u < kHubU; ++u)
+            c += __popc(m[u].x) + __popc(m[u].y) + __popc(m[u].z) + __popc(m[u].w);
+          if (!__any_sync(0xffffffffu, c)) continue;
+          uint32_t inc = c;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= (uint32_t)o) inc += x;
+          }
+          unsigned long long at = 0;
+          if (lane == 31) at = atomicAdd(cursor, (unsigned long long)inc);
+          uint64_t pos = __shfl_sync(0xffffffffu, at, 31) + inc - c;
+          auto emit = [&](uint32_t word, uint32_t x) {
+            while (x) {
+              const uint64_t idx = ((uint64_t)word << 5) | (uint64_t)(__ffs(x) - 1);
+              x &= x - 1;
+              if (pos < out_cap) {
+#pragma unroll
+                for (int c2 = 0; c2 < kMaxK; ++c2)
+                  if (c2 < (int)d.k) out.c[c2][pos] = set_column(d, idx, c2);
+              } else {
+                atomicOr(err, kErrCapacity);
+              }
+              ++pos;
+            }
+          };
+#pragma unroll
+          for (int u = 0; u < kHubU; ++u) {
+            emit(w[u], m[u].x);
+            emit(w[u] + 1, m[u].y);
+            emit(w[u] + 2, m[u].z);
+            emit(w[u] + 3, m[u].w);
+          }
+        }
+      }
+    }
+  }
+}
+
+static uint64_t hub_tasks_cap(const JoinSpec& j, const HubPlan& h) {
+  return j.n_probe / kHubRows + h.cap;
+}
+
+size_t hub_workspace(const JoinSpec& j, const HubPlan& h) {
+  auto up = [](uint64_t b) { return (b + 255) & ~uint64_t(255); };
+  return 256 + up(8 * h.cap) + up(4ull * h.cap * h.words) + up(sizeof(HubTask) * hub_tasks_cap(j, h));
+}
+
+cudaError_t hub_or(Ctx& c, const JoinSpec& j, const HubPlan& h, const DenseSet& d, ColsOut out,
+                   uint64_t* d_cursor, uint64_t out_cap, void* ws) {
+  auto up = [](uint64_t b) { return (b + 255) & ~uint64_t(255); };
+  char* p = static_cast<char*>(ws);
+  auto* n = reinterpret_cast<unsigned long long*>(p);  // hubs, tasks
+  p += 256;
+  uint2* hubs = reinterpret_cast<uint2*>(p);
+  p += up(8 * h.cap);
+  uint32_t* bits = reinterpret_cast<uint32_t*>(p);
+  p += up(4ull * h.cap * h.words);
+  HubTask* tasks = reinterpret_cast<HubTask*>(p);
+  const uint64_t task_cap = hub_tasks_cap(j, h);
+  cudaError_t e = cudaMemsetAsync(n, 0, 256, c.st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(bits, 0, 4ull * h.cap * h.words, c.st);
+  if (e != cudaSuccess) return e;
+  {
+    ProfScope ps(c, kDense, 16.0 * j.slots);
+    uint64_t blocks = (j.slots + kCT - 1) / kCT;
+    if (blocks > 152 * 8) blocks = 152 * 8;
+    k_hub_list<<<(unsigned)blocks, kCT, 0, c.st>>>(j, h.probe_table, h.probe_slots, hubs, h.cap, tasks,
+                                                   task_cap, n);
+  }
+  {
+    ProfScope ps(c, kDense, 4.0 * h.cap * h.words);
+    k_hub_render<<<dim3((unsigned)(h.cap < 1024 ? h.cap : 1024), 4), kCT, 0, c.st>>>(
+        hubs, n, h.cap, h.col, bits, h.words);
+  }
+  ProfScope ps(c, kJoinWrite, 0.0);  // (its reads are of L2-resident words)
+  const unsigned grid = (unsigned)(task_cap < 152 * 8 ? task_cap : 152 * 8);
+  auto* cur = reinterpret_cast<unsigned long long*>(d_cursor);
+  if (d.append)
+    k_hub_or<true><<<grid, kCT, 0, c.st>>>(j, d, tasks, task_cap, n + 1, bits, h.words, out, cur,
+                                           out_cap, c.d_err);
+  else
+    k_hub_or<false><<<grid, kCT, 0, c.st>>>(j, d, tasks, task_cap, n + 1, bits, h.words, out, cur,
+                                            out_cap, c.d_err);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ single pass
@@ -686,19 +912,21 @@ cudaError_t join_write(Ctx& c, const JoinSpec& j, const uint64_t* d_off, uint64_
   uint32_t* err = d_soft_err ? d_soft_err : c.d_err;
   const DenseSet ds = dense ? *dense : DenseSet{};
   const unsigned grid = dev_grid(blocks, d_total);
-#define CDL_JOIN_WRITE(F, D, S)                                                          \
-  k_join_write<F, D, S><<<grid, kJT, 0, c.st>>>(j, d_off, total, out, base, cur, out_cap, \
-                                                splits, err, d_total, d_base, ds)
-  if (j.star) {
-    if (dense && filter) CDL_JOIN_WRITE(true, true, true);
-    else if (dense) CDL_JOIN_WRITE(false, true, true);
-    else if (filter) CDL_JOIN_WRITE(true, false, true);
-    else CDL_JOIN_WRITE(false, false, true);
+  auto launch = [&](auto kernel) {
+    kernel<<<grid, kJT, 0, c.st>>>(j, d_off, total, out, base, cur, out_cap, splits, err, d_total,
+                                   d_base, ds);
+  };
+#define CDL_JOIN_WRITE(FORM)                                                                 \
+  if (j.star)                                                                                \
+    filter ? launch(k_join_write<true, FORM, true>) : launch(k_join_write<false, FORM, true>); \
+  else                                                                                       \
+    filter ? launch(k_join_write<true, FORM, false>) : launch(k_join_write<false, FORM, false>)
+  if (!dense) {
+    CDL_JOIN_WRITE(kRows);
+  } else if (!dense->append) {
+    CDL_JOIN_WRITE(kBits);
   } else {
-    if (dense && filter) CDL_JOIN_WRITE(true, true, false);
-    else if (dense) CDL_JOIN_WRITE(false, true, false);
-    else if (filter) CDL_JOIN_WRITE(true, false, false);
-    else CDL_JOIN_WRITE(false, false, false);
+    CDL_JOIN_WRITE(kSet);
   }
 #undef CDL_JOIN_WRITE
   return cudaGetLastError();

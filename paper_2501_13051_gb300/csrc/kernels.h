@@ -133,7 +133,28 @@ struct JoinSpec {
   ColsIn build2;
   const Slot* table2;
   uint64_t slots2;
+  // rows matching a key of at least hub_min build rows count 0 outputs: they
+  // are left to hub_or (0: no such keys)
+  uint32_t hub_min;
 };
+// Hub keys of an unfiltered join into a bitmap, where the build side gives
+// the last head column (the lowest bits of a tuple's position, hub_words
+// words of bits) and the probe side or constants the others: every key with
+// at least j.hub_min build rows has its rows' values of column `col` rendered
+// once as a bitmap row, which is OR-ed into the head row of each of the
+// key's probe rows.  probe_table: the probe side's own index on the key; the
+// probe columns are in its order.  The plain write covers the other keys.
+struct HubPlan {
+  const uint32_t* col;      // build column of the last head column
+  uint32_t words;           // words of a head row (a multiple of 8)
+  const Slot* probe_table;  // probe side's index on the join key
+  uint64_t probe_slots;
+  uint64_t cap;             // hubs at most
+};
+size_t hub_workspace(const JoinSpec& j, const HubPlan& h);
+// New tuples (d.append) go to out at *d_cursor, as join_write's.
+cudaError_t hub_or(Ctx& c, const JoinSpec& j, const HubPlan& h, const DenseSet& d, ColsOut out,
+                   uint64_t* d_cursor, uint64_t out_cap, void* ws);
 size_t join_count_workspace(uint64_t n_probe);
 // Pass 1 alone: counts[i] for every probe row.
 cudaError_t join_count_only(Ctx& c, const JoinSpec& j, uint32_t* counts);
@@ -157,15 +178,21 @@ cudaError_t join_write(Ctx& c, const JoinSpec& j, const uint64_t* d_off, uint64_
                        uint64_t* d_base = nullptr, uint32_t* d_soft_err = nullptr,
                        const DenseSet* dense = nullptr);
 // (dense != null: each output tuple sets its bit in *dense instead of being
-// written; out, base, d_cursor and out_cap are then unused.)
+// written; out, base, d_cursor and out_cap are then unused.  With
+// dense->append the outputs whose bits were clear are also written, packed
+// at *d_cursor in no order, at most out_cap rows.)
 
 // -------------------------------------------------------------- dense sets
 // Bits of n rows set in d (a row outside d raises kErrCapacity).
 cudaError_t dense_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n);
+// The same for Full's bitmap: rows whose bits were clear are appended to out
+// (packed at *d_cursor, at most out_cap rows; more raise kErrCapacity).
+cudaError_t set_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n, ColsOut out,
+                       uint64_t* d_cursor, uint64_t out_cap);
 size_t dense_extract_workspace(uint64_t nbits);
 // The set bits of d as rows in increasing bit order (lexicographic, no
 // repeats) into out (cap rows; more raise kErrCapacity); their number in
-// *d_count.  Clears d.
+// *d_count.  Clears d (unless d.append: Full's bitmap keeps its bits).
 cudaError_t dense_extract(Ctx& c, const DenseSet& d, ColsOut out, uint64_t cap,
                           uint64_t* d_count, void* ws);
 
