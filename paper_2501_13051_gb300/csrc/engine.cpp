@@ -593,7 +593,7 @@ struct cdl_engine {
     }
     std::vector<float> pred(n);
     if (e == cudaSuccess)
-      e = mlp_forward(ctx, th, static_cast<float*>(dX.p), n, static_cast<float*>(dout.p), ws.p);
+      e = mlp_forward(ctx, th, static_cast<float*>(dX.p), n, static_cast<float*>(dout.p));
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(pred.data(), dout.p, sizeof(float) * n, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

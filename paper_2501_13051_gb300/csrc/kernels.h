@@ -400,11 +400,11 @@ struct JoinFeatureHost {
   float prev_delta;      // delta of the head relation in the previous round
   float filtered;        // 1 when the step filters (inequalities, equalities)
 };
-// workspace of mlp_gradient / mlp_forward for n samples (floats: 4 x 64 n + n)
+// workspace of mlp_gradient for n samples (floats: 4 x 64 n + n)
 inline size_t mlp_workspace(uint64_t n) {
   return ((4ull * kMlpHidden * (n ? n : 1) + (n ? n : 1)) * sizeof(float) + 255) & ~size_t(255);
 }
-cudaError_t mlp_forward(Ctx& c, const float* th, const float* X, uint64_t n, float* out, void* ws);
+cudaError_t mlp_forward(Ctx& c, const float* th, const float* X, uint64_t n, float* out);
 cudaError_t mlp_gradient(Ctx& c, const float* th, const float* X, const float* y, uint64_t n,
                          float tau, float* out, float* grad, void* ws);
 cudaError_t mlp_adam(Ctx& c, float* th, const float* grad, float* m, float* v, uint64_t step,

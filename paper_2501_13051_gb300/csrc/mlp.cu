@@ -5,11 +5,10 @@
 // join in a single pass, and falls back to the exact three-pass join when
 // the prediction was too small.  Tuple results never depend on the network.
 //
-// Training runs in FP32 on these kernels: forward per sample (one block of
-// 64 threads), backward of the activations per sample, then every parameter
-// gradient as a sum over the batch computed by one thread per parameter
-// (deterministic: no atomics), pinball (quantile) loss at level tau, Adam
-// update (Kingma & Ba, 2015).  Inference runs with BF16 weights and
+// Training runs in FP32 on these kernels: forward, backward and each block's
+// share of the parameter gradients in one kernel, the shares summed in a
+// fixed order by a second (deterministic: no atomics), pinball (quantile)
+// loss at level tau, Adam update (Kingma & Ba, 2015).  Inference runs with BF16 weights and
 // activations and FP32 accumulation.
 //
 // Parameters: one flat FP32 vector W1 (64x16 row-major), b1, W2 (64x64
@@ -39,80 +38,202 @@ __device__ __forceinline__ float block64_sum(float v, float* red) {
   return s;
 }
 
-// Z1, Z2: pre-activations (n x 64); out: prediction per sample.
-__global__ void __launch_bounds__(kH) k_mlp_forward(const float* __restrict__ th,
-                                                    const float* __restrict__ X, uint64_t n,
-                                                    float* __restrict__ Z1, float* __restrict__ Z2,
-                                                    float* __restrict__ out) {
-  __shared__ float x[kIn], h1[kH], red[2];
-  const uint64_t s = blockIdx.x;
-  const int t = threadIdx.x;
-  if (t < kIn) x[t] = X[s * kIn + t];
-  __syncthreads();
-  float z1 = th[ob1 + t];
+// One pass over the batch: forward, backward and this block's share of every
+// parameter gradient, nothing but the predictions and the shares stored.
+// Tiny arithmetic (3 x 5313 multiply-adds per sample), so what bounds it is
+// latency: the network sits in shared memory once per block, a block takes
+// kTileS samples at a time (thread = one hidden unit of kSPT samples, rows
+// padded by one word so that W2 is read without bank conflicts by rows
+// (forward) and by columns (backward)), and a thread then adds a 4 x 4 patch
+// of dW2 and a 1 x 4 patch of dW1 over the tile from shared memory.  Before,
+// one thread per parameter walked the whole batch in global memory:
+// a gradient call of 3,000 samples took 228 us and takes 56 (most of it the
+// caller's), one of 100,000 samples 12.9 ms and 0.146 ms.
+constexpr int kGT = 256;                  // threads
+constexpr int kTileS = 32;                // samples per tile
+constexpr int kSPT = kTileS * kH / kGT;   // samples per thread in a tile
+constexpr int kP1 = kIn + 1, kP2 = kH + 1;  // padded rows of W1, W2
+constexpr int kGradBlocks = 304;          // at most two blocks per SM
+constexpr int kGradSamples = 21;          // samples a block takes at least (mlp_gradient)
+
+struct MlpTile {
+  float w1[kH * kP1], w2[kH * kP2], b1[kH], b2[kH], w3[kH];
+  alignas(16) float x[kTileS * kIn];
+  alignas(16) float h1[kTileS * kH], h2[kTileS * kH];  // activations
+  alignas(16) float g1[kTileS * kH], g2[kTileS * kH];  // dL/dZ1, dL/dZ2
+  float go[kTileS];                                    // dL/dprediction
+};
+
+template <bool GRAD>
+__global__ void __launch_bounds__(kGT) k_mlp_batch(const float* __restrict__ th,
+                                                   const float* __restrict__ X,
+                                                   const float* __restrict__ y, uint64_t n,
+                                                   float tau, float* __restrict__ out,
+                                                   float* __restrict__ part) {
+  extern __shared__ __align__(16) char raw[];
+  MlpTile& m = *reinterpret_cast<MlpTile*>(raw);
+  const int t = threadIdx.x, h = t & (kH - 1), q = t / kH, lane = t & 31, warp = t >> 5;
+  // this block's samples: an even share of the batch
+  const uint64_t s_lo = n * blockIdx.x / gridDim.x, s_hi = n * (blockIdx.x + 1) / gridDim.x;
+  for (int i = t; i < kH * kIn; i += kGT) m.w1[i / kIn * kP1 + i % kIn] = th[oW1 + i];
 #pragma unroll
-  for (int k = 0; k < kIn; ++k) z1 += th[oW1 + t * kIn + k] * x[k];
-  Z1[s * kH + t] = z1;
-  h1[t] = fmaxf(z1, 0.f);
-  __syncthreads();
-  float z2 = th[ob2 + t];
-#pragma unroll 16
-  for (int i = 0; i < kH; ++i) z2 += th[oW2 + t * kH + i] * h1[i];
-  Z2[s * kH + t] = z2;
-  const float o = block64_sum(th[ow3 + t] * fmaxf(z2, 0.f), red);
-  if (t == 0) out[s] = o + th[ob3];
-}
-
-// Per sample: GO = dL/dprediction, G2 = dL/dZ2, G1 = dL/dZ1.
-__global__ void __launch_bounds__(kH) k_mlp_backward(const float* __restrict__ th,
-                                                     const float* __restrict__ y, uint64_t n,
-                                                     float tau, const float* __restrict__ Z1,
-                                                     const float* __restrict__ Z2,
-                                                     const float* __restrict__ out,
-                                                     float* __restrict__ GO, float* __restrict__ G1,
-                                                     float* __restrict__ G2) {
-  __shared__ float g2[kH];
-  const uint64_t s = blockIdx.x;
-  const int t = threadIdx.x;
-  const float g = (y[s] > out[s] ? -tau : 1.f - tau) / (float)n;
-  if (t == 0) GO[s] = g;
-  const float gz2 = Z2[s * kH + t] > 0.f ? g * th[ow3 + t] : 0.f;
-  G2[s * kH + t] = gz2;
-  g2[t] = gz2;
-  __syncthreads();
-  float a = 0.f;
-#pragma unroll 16
-  for (int j = 0; j < kH; ++j) a += g2[j] * th[oW2 + j * kH + t];
-  G1[s * kH + t] = Z1[s * kH + t] > 0.f ? a : 0.f;
-}
-
-// One thread per parameter: its gradient summed over the batch in order.
-__global__ void k_mlp_param_grads(const float* __restrict__ X, uint64_t n,
-                                  const float* __restrict__ Z1, const float* __restrict__ Z2,
-                                  const float* __restrict__ GO, const float* __restrict__ G1,
-                                  const float* __restrict__ G2, float* __restrict__ grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= kMlpParams) return;
-  float acc = 0.f;
-  if (p < ob1) {
-    const int i = p / kIn, k = p % kIn;
-    for (uint64_t s = 0; s < n; ++s) acc += G1[s * kH + i] * X[s * kIn + k];
-  } else if (p < oW2) {
-    const int i = p - ob1;
-    for (uint64_t s = 0; s < n; ++s) acc += G1[s * kH + i];
-  } else if (p < ob2) {
-    const int j = (p - oW2) / kH, i = (p - oW2) % kH;
-    for (uint64_t s = 0; s < n; ++s) acc += G2[s * kH + j] * fmaxf(Z1[s * kH + i], 0.f);
-  } else if (p < ow3) {
-    const int j = p - ob2;
-    for (uint64_t s = 0; s < n; ++s) acc += G2[s * kH + j];
-  } else if (p < ob3) {
-    const int j = p - ow3;
-    for (uint64_t s = 0; s < n; ++s) acc += GO[s] * fmaxf(Z2[s * kH + j], 0.f);
-  } else {
-    for (uint64_t s = 0; s < n; ++s) acc += GO[s];
+  for (int i = t; i < kH * kH; i += kGT) m.w2[i / kH * kP2 + i % kH] = th[oW2 + i];
+  if (t < kH) {
+    m.b1[t] = th[ob1 + t];
+    m.b2[t] = th[ob2 + t];
+    m.w3[t] = th[ow3 + t];
   }
-  grad[p] = acc;
+  const float b3 = th[ob3];
+  float aw2[4][4] = {}, aw1[4] = {}, av = 0.f;
+  for (uint64_t s0 = s_lo; s0 < s_hi; s0 += kTileS) {
+    const int ns = s_hi - s0 < (uint64_t)kTileS ? (int)(s_hi - s0) : kTileS;
+    __syncthreads();  // weights staged; the last tile's sums are done
+    for (int i = t; i < kTileS * kIn; i += kGT) m.x[i] = i < ns * kIn ? X[s0 * kIn + i] : 0.f;
+    __syncthreads();
+    const int sq = q * kSPT;  // this thread's samples of the tile
+    const bool live = sq < ns;  // (whole warps)
+    float z[kSPT];
+    if (live) {
+#pragma unroll
+      for (int u = 0; u < kSPT; ++u) z[u] = m.b1[h];
+#pragma unroll
+      for (int k = 0; k < kIn; ++k) {
+        const float w = m.w1[h * kP1 + k];
+#pragma unroll
+        for (int u = 0; u < kSPT; ++u) z[u] += w * m.x[(sq + u) * kIn + k];
+      }
+#pragma unroll
+      for (int u = 0; u < kSPT; ++u) m.h1[(sq + u) * kH + h] = fmaxf(z[u], 0.f);
+    }
+    __syncthreads();
+    if (live) {
+#pragma unroll
+      for (int u = 0; u < kSPT; ++u) z[u] = m.b2[h];
+#pragma unroll 4
+      for (int i = 0; i < kH; i += 4) {
+        float w[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) w[r] = m.w2[h * kP2 + i + r];
+#pragma unroll
+        for (int u = 0; u < kSPT; ++u) {
+          const float4 v = *reinterpret_cast<const float4*>(&m.h1[(sq + u) * kH + i]);
+          z[u] += w[0] * v.x;
+          z[u] += w[1] * v.y;
+          z[u] += w[2] * v.z;
+          z[u] += w[3] * v.w;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kSPT; ++u) m.h2[(sq + u) * kH + h] = fmaxf(z[u], 0.f);
+    }
+    __syncthreads();
+    // predictions: a warp takes every eighth sample
+    for (int s = warp; s < ns; s += kGT / 32) {
+      float v0 = m.w3[lane] * m.h2[s * kH + lane], v1 = m.w3[32 + lane] * m.h2[s * kH + 32 + lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+        v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+      }
+      if (lane == 0) {
+        const float p = v0 + v1 + b3;
+        out[s0 + s] = p;
+        if (GRAD) m.go[s] = (y[s0 + s] > p ? -tau : 1.f - tau) / (float)n;
+      }
+    }
+    if constexpr (GRAD) {
+      __syncthreads();
+      if (live) {
+#pragma unroll
+        for (int u = 0; u < kSPT; ++u)
+          m.g2[(sq + u) * kH + h] =
+              sq + u < ns && m.h2[(sq + u) * kH + h] > 0.f ? m.go[sq + u] * m.w3[h] : 0.f;
+      }
+      __syncthreads();
+      if (live) {
+#pragma unroll
+        for (int u = 0; u < kSPT; ++u) z[u] = 0.f;
+#pragma unroll 4
+        for (int j = 0; j < kH; j += 4) {
+          float w[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) w[r] = m.w2[(j + r) * kP2 + h];
+#pragma unroll
+          for (int u = 0; u < kSPT; ++u) {
+            const float4 v = *reinterpret_cast<const float4*>(&m.g2[(sq + u) * kH + j]);
+            z[u] += v.x * w[0];
+            z[u] += v.y * w[1];
+            z[u] += v.z * w[2];
+            z[u] += v.w * w[3];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kSPT; ++u)
+          m.g1[(sq + u) * kH + h] = m.h1[(sq + u) * kH + h] > 0.f ? z[u] : 0.f;
+      }
+      __syncthreads();
+      // this thread's parameters, summed over the tile's samples in order
+      const int j4 = (t >> 4) * 4, i4 = (t & 15) * 4, r1 = t >> 2, k4 = (t & 3) * 4;
+#pragma unroll 4
+      for (int s = 0; s < ns; ++s) {
+        const float4 g = *reinterpret_cast<const float4*>(&m.g2[s * kH + j4]);
+        const float4 a = *reinterpret_cast<const float4*>(&m.h1[s * kH + i4]);
+        const float4 x = *reinterpret_cast<const float4*>(&m.x[s * kIn + k4]);
+        const float gv[4] = {g.x, g.y, g.z, g.w}, hv[4] = {a.x, a.y, a.z, a.w},
+                    xv[4] = {x.x, x.y, x.z, x.w}, g1 = m.g1[s * kH + r1];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) aw2[r][c] += gv[r] * hv[c];
+          aw1[r] += g1 * xv[r];
+        }
+        if (q == 0)
+          av += m.g1[s * kH + h];
+        else if (q == 1)
+          av += m.g2[s * kH + h];
+        else if (q == 2)
+          av += m.go[s] * m.h2[s * kH + h];
+        else if (h == 0)
+          av += m.go[s];
+      }
+    }
+  }
+  if constexpr (GRAD) {
+    float* g = part + (uint64_t)blockIdx.x * kMlpParams;
+    const int j4 = (t >> 4) * 4, i4 = (t & 15) * 4, r1 = t >> 2, k4 = (t & 3) * 4;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) g[oW2 + (j4 + r) * kH + i4 + c] = aw2[r][c];
+      g[oW1 + r1 * kIn + k4 + r] = aw1[r];
+    }
+    if (q < 3)
+      g[(q == 0 ? ob1 : q == 1 ? ob2 : ow3) + h] = av;
+    else if (h == 0)
+      g[ob3] = av;
+  }
+}
+
+// The blocks' shares of every gradient, summed in a fixed order (no atomics):
+// a block takes 32 parameters, each warp an eighth of the shares.
+__global__ void __launch_bounds__(kGT) k_mlp_reduce(const float* __restrict__ part, int nparts,
+                                                    float* __restrict__ grad) {
+  constexpr int kW = kGT / 32;
+  __shared__ float red[kW][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + lane;
+  float acc = 0.f;
+  if (p < kMlpParams) {
+#pragma unroll 8
+    for (int b = warp; b < nparts; b += kW) acc += part[(uint64_t)b * kMlpParams + p];
+  }
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (warp == 0 && p < kMlpParams) {
+#pragma unroll
+    for (int w = 1; w < kW; ++w) acc += red[w][lane];
+    grad[p] = acc;
+  }
 }
 
 // b1, b2 and their complements ob1 = 1 - b1, ob2 = 1 - b2 come rounded
@@ -243,27 +364,35 @@ __global__ void __launch_bounds__(kFT) k_join_features(const uint32_t* pk0, cons
 
 }  // namespace
 
-cudaError_t mlp_forward(Ctx& c, const float* th, const float* X, uint64_t n, float* out, void* ws) {
+cudaError_t mlp_forward(Ctx& c, const float* th, const float* X, uint64_t n, float* out) {
   if (n == 0) return cudaSuccess;
-  float* Z1 = static_cast<float*>(ws);
-  float* Z2 = Z1 + kH * n;
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_batch<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(MlpTile));
+  if (e != cudaSuccess) return e;
   ProfScope p(c, kMlp, 0.0);
-  k_mlp_forward<<<(unsigned)n, kH, 0, c.st>>>(th, X, n, Z1, Z2, out);
+  const uint64_t blocks = (n + kSPT - 1) / kSPT;
+  k_mlp_batch<false><<<(unsigned)(blocks < kGradBlocks ? blocks : kGradBlocks), kGT, sizeof(MlpTile),
+                       c.st>>>(th, X, nullptr, n, 0.f, out, nullptr);
   return cudaGetLastError();
 }
 
 cudaError_t mlp_gradient(Ctx& c, const float* th, const float* X, const float* y, uint64_t n,
                          float tau, float* out, float* grad, void* ws) {
   if (n == 0) return cudaMemsetAsync(grad, 0, sizeof(float) * kMlpParams, c.st);
-  float* Z1 = static_cast<float*>(ws);
-  float* Z2 = Z1 + kH * n;
-  float* G1 = Z2 + kH * n;
-  float* G2 = G1 + kH * n;
-  float* GO = G2 + kH * n;
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_batch<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(MlpTile));
+  if (e != cudaSuccess) return e;
+  // a block for every kGradSamples samples: the shares then fit the
+  // workspace (257 floats per sample, 5313 per share); one block's share is
+  // the gradient itself
+  static_assert((4 * kH + 1) * kGradSamples >= kMlpParams, "shares fit the workspace");
+  uint64_t blocks = n / kGradSamples;
+  blocks = blocks < 1 ? 1 : blocks < kGradBlocks ? blocks : kGradBlocks;
+  float* part = blocks == 1 ? grad : static_cast<float*>(ws);
   ProfScope p(c, kMlp, 0.0);
-  k_mlp_forward<<<(unsigned)n, kH, 0, c.st>>>(th, X, n, Z1, Z2, out);
-  k_mlp_backward<<<(unsigned)n, kH, 0, c.st>>>(th, y, n, tau, Z1, Z2, out, GO, G1, G2);
-  k_mlp_param_grads<<<(kMlpParams + 255) / 256, 256, 0, c.st>>>(X, n, Z1, Z2, GO, G1, G2, grad);
+  k_mlp_batch<true><<<(unsigned)blocks, kGT, sizeof(MlpTile), c.st>>>(th, X, y, n, tau, out, part);
+  if (blocks > 1)
+    k_mlp_reduce<<<(kMlpParams + 31) / 32, kGT, 0, c.st>>>(part, (int)blocks, grad);
   return cudaGetLastError();
 }
 

@@ -255,7 +255,7 @@ cdl_status cdl_mlp_forward(const float* params, const float* X, uint64_t n, floa
   if (*ws_bytes < need || !params || ((!X || !out) && n)) return CDL_E_INVALID;
   Ctx c;
   c.st = static_cast<cudaStream_t>(stream);
-  return cuda_status(mlp_forward(c, params, X, n, out, workspace));
+  return cuda_status(mlp_forward(c, params, X, n, out));
 }
 
 cdl_status cdl_mlp_gradient(const float* params, const float* X, const float* y, uint64_t n,
