@@ -450,6 +450,17 @@ cdl_status cdl_join(const uint32_t* const* probe_cols, uint32_t probe_arity, uin
                     uint64_t out_cap, uint64_t* n_out, void* workspace, size_t* ws_bytes,
                     void* stream);
 
+/* The write of cdl_join alone, for a caller that sizes its output first: to
+ * be called after a cdl_join with the same arguments and workspace that
+ * returned CDL_E_CAPACITY, the workspace untouched since, with *n_out as
+ * that call left it.  Nothing is indexed or counted again. */
+cdl_status cdl_join_write(const uint32_t* const* probe_cols, uint32_t probe_arity,
+                          uint64_t n_probe, uint32_t probe_key, const uint32_t* const* build_cols,
+                          uint32_t build_arity, uint64_t n_build, uint32_t build_key,
+                          const cdl_colref* spec, uint32_t out_arity, const cdl_colref* neq,
+                          uint32_t nneq, uint32_t* const* out_cols, uint64_t out_cap,
+                          uint64_t* n_out, void* workspace, const size_t* ws_bytes, void* stream);
+
 /* Step (c): sorts n tuples of arity columns lexicographically (LSD radix
  * sort, stable), drops repeats, writes the unique tuples to out_cols and
  * their number to *n_out.  cols are left unchanged. */

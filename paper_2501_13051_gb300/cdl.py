@@ -131,6 +131,8 @@ def lib():
         "cdl_exclusive_scan_noalloc": (ctypes.c_int, [VP, U64, VP, P(U64), VP]),
         "cdl_join": (ctypes.c_int, [PP, U32, U64, U32, PP, U32, U64, U32, P(ColRef), U32,
                                     P(ColRef), U32, PP, U64, P(U64), VP, P(ctypes.c_size_t), VP]),
+        "cdl_join_write": (ctypes.c_int, [PP, U32, U64, U32, PP, U32, U64, U32, P(ColRef), U32,
+                                    P(ColRef), U32, PP, U64, P(U64), VP, P(ctypes.c_size_t), VP]),
         "cdl_sort_unique": (ctypes.c_int, [PP, U32, U64, PP, P(U64), VP, P(ctypes.c_size_t), VP]),
         "cdl_diff_merge": (ctypes.c_int, [PP, U64, PP, U64, U32, PP, P(U64), PP, VP,
                                           P(ctypes.c_size_t), VP]),
@@ -616,10 +618,11 @@ def join(probe_cols, probe_key, build_cols, build_key, spec, neq=(), out_cap=Non
     total = int(n_out.value)
     cap = total if out_cap is None else out_cap
     outs = [torch.empty(max(1, cap), dtype=torch.int32, device="cuda") for _ in spec]
-    st = L.cdl_join(*args_head, _ptrs(outs), cap, ctypes.byref(n_out), ws.data_ptr(),
-                    ctypes.byref(need), s)
-    if st != 0:
-        raise CdlError(st)
+    if total:  # the size query left the index and the offsets in the workspace
+        st = L.cdl_join_write(*args_head, _ptrs(outs), cap, ctypes.byref(n_out), ws.data_ptr(),
+                              ctypes.byref(need), s)
+        if st != 0:
+            raise CdlError(st)
     return [o[:n_out.value] for o in outs]
 
 

@@ -352,8 +352,12 @@ struct Index {
   const uint32_t* cols[kMaxK] = {nullptr, nullptr, nullptr, nullptr};  // original numbering
   uint64_t n = 0;
   DBuf table;
-  uint64_t slots = 0;
-  uint64_t distinct = 0;  // distinct keys
+  uint64_t slots = 0;     // hash form
+  uint32_t range = 0;     // direct form: keys below it (KeyIndex)
+  uint64_t distinct = 0;  // distinct keys, or a bound on them
+  KeyIndex key_index() const {
+    return KeyIndex{static_cast<const Slot*>(table.p), slots, range, nullptr};
+  }
   std::string tkey;       // tuner decision of the load factor, if any
   int tcand = 0;
 };
@@ -460,6 +464,11 @@ struct cdl_engine {
   static constexpr uint64_t kHubOutputs = 1 << 22;
   static constexpr uint64_t kHubOutputsPerRow = 8;
   static constexpr uint32_t kHubMinRows = 32;
+  // an index up to this size stays in L2 between a join's count and write
+  static constexpr size_t kCachedIndex = 32 << 20;
+  // a hash index over at most so many rows has slots for all of them: their
+  // keys are not counted first (a launch and a wait; 2 MB of slots at most)
+  static constexpr uint64_t kUncountedRows = 1 << 16;
   static constexpr uint32_t kHubWordsPerRow = 16;
   static constexpr uint64_t kGroupRows = 1 << 21;  // larger new-tuple sets sort on their own
   static constexpr size_t kGroupMin = 4;           // fewer relations sort one by one
@@ -1181,11 +1190,29 @@ struct cdl_engine {
     }
     const uint32_t* k0 = ix->cols[key[0]];
     const uint32_t* k1 = key.size() > 1 ? ix->cols[key[1]] : nullptr;
-    cudaError_t e = count_heads(ctx, k0, k1, s.n, dslot(kSlotScratch));
-    if (e != cudaSuccess) return cuda_fail(e, "count_heads");
-    cdl_status r = fetch(kSlotScratch, 1);
-    if (r != CDL_OK) return r;
-    ix->distinct = h_ctl[kSlotScratch];
+    // One-word keys below a bound not far above the rows: the direct form,
+    // with no count of the keys and no wait for it.  (The estimator's
+    // features read the exact count, the tuner times hash tables, and under
+    // a memory limit the direct form, up to 32 bytes a row where the hash
+    // form may need few slots, stays small.)
+    const uint64_t bound = 1ull << s.bits[key[0]];
+    const bool counted = opt.estimator || tuner.mode;
+    if (!k1 && !counted && bound <= direct_keys(opt.mem_limit ? 0 : s.n)) {
+      ix->table = alloc(8 * bound);
+      if (ix->table.p) ix->range = (uint32_t)bound;
+    }
+    cudaError_t e = cudaSuccess;
+    if (ix->range) {
+      ix->distinct = std::min(bound, s.n);
+    } else if (!counted && s.n <= kUncountedRows) {
+      ix->distinct = s.n;
+    } else {
+      e = count_heads(ctx, k0, k1, s.n, dslot(kSlotScratch));
+      if (e != cudaSuccess) return cuda_fail(e, "count_heads");
+      cdl_status r = fetch(kSlotScratch, 1);
+      if (r != CDL_OK) return r;
+      ix->distinct = h_ctl[kSlotScratch];
+    }
     double load = hash_load;
     if (tuner.mode && ix->distinct >= 4096) {  // candidates: the configured load, 0.6, 0.7, 0.8
       static const double kLoads[4] = {0.0, 0.6, 0.7, 0.8};
@@ -1194,11 +1221,15 @@ struct cdl_engine {
       ix->tcand = tuner.choose(ix->tkey, 4, &unused);
       if (ix->tcand) load = kLoads[ix->tcand];
     }
-    ix->slots = table_slots(ix->distinct, load);
-    ix->table = alloc(ix->slots * sizeof(Slot));
-    if (!ix->table.p) return fail(CDL_E_NOMEM, "hash table");
-    e = hash_build(ctx, k0, k1, s.n, static_cast<Slot*>(ix->table.p), ix->slots);
-    if (e != cudaSuccess) return cuda_fail(e, "hash_build");
+    if (ix->range) {
+      e = index_build(ctx, k0, s.n, ix->key_index());
+    } else {
+      ix->slots = table_slots(ix->distinct, load);
+      ix->table = alloc(ix->slots * sizeof(Slot));
+      if (!ix->table.p) return fail(CDL_E_NOMEM, "hash table");
+      e = hash_build(ctx, k0, k1, s.n, static_cast<Slot*>(ix->table.p), ix->slots);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "index build");
     *out = ix.get();
     if (cacheable)
       cache.push_back(std::move(ix));
@@ -1605,15 +1636,14 @@ struct cdl_engine {
         js.pk0 = 0;
         js.pk1 = 0xFFu;
         for (uint32_t c = 0; c < B.k; ++c) js.build.c[c] = B.c[c];
-        js.slots = 1;
+        js.ix.slots = 1;
       } else {
         r = get_index(B, hkey, &ix, temp_ix);
         if (r != CDL_OK) return r;
         js.pk0 = pkey[0];
         js.pk1 = pkey.size() > 1 ? pkey[1] : 0xFFu;
         for (uint32_t c = 0; c < B.k; ++c) js.build.c[c] = ix->cols[c];
-        js.table = static_cast<const Slot*>(ix->table.p);
-        js.slots = ix->slots;
+        js.ix = ix->key_index();
       }
       std::unique_ptr<Index> temp_ix2;
       Index* ix2 = nullptr;
@@ -1624,8 +1654,7 @@ struct cdl_engine {
         js.qk0 = cpkey[0];
         js.qk1 = cpkey.size() > 1 ? cpkey[1] : 0xFFu;
         for (uint32_t c = 0; c < C->k; ++c) js.build2.c[c] = ix2->cols[c];
-        js.table2 = static_cast<const Slot*>(ix2->table.p);
-        js.slots2 = ix2->slots;
+        js.ix2 = ix2->key_index();
         ++star_joins;
       }
       for (size_t q = 2; q < bkey.size(); ++q) {
@@ -1821,6 +1850,13 @@ struct cdl_engine {
       DBuf off = alloc(std::max<uint64_t>(P.n, 1) * 8);
       DBuf ws = alloc(join_count_workspace(P.n));
       if (!off.p || !ws.p) return fail(CDL_E_NOMEM, "join offsets");
+      // an index past the caches is looked up once: the count stores each
+      // row's first build row for the write
+      DBuf starts;
+      if (ix && !C && !recording && !opt.mem_limit && ix->table.bytes > kCachedIndex) {
+        starts = alloc(4 * std::max<uint64_t>(P.n, 1));
+        js.starts = static_cast<uint32_t*>(starts.p);
+      }
       // the probe cost per row measures the index's load factor for the tuner
       Tuner::Probe tp;
       // (a star join's count measures it where one index serves both sides)
@@ -1962,8 +1998,7 @@ struct cdl_engine {
     const uint32_t pk = side == 0 ? B.k : P.k, bk = side == 0 ? P.k : B.k;
     for (uint32_t c = 0; c < pk; ++c) f.probe.c[c] = pix->cols[c];
     for (uint32_t c = 0; c < bk; ++c) f.build.c[c] = ix->cols[c];
-    f.table = static_cast<const Slot*>(ix->table.p);
-    f.slots = ix->slots;
+    f.ix = ix->key_index();
     f.out_k = js.out_k;
     for (uint32_t k = 0; k < js.out_k; ++k)
       f.out[k] = js.out[k].side > 1 ? js.out[k]
@@ -1971,8 +2006,7 @@ struct cdl_engine {
     HubPlan hp{};
     hp.words = 1u << (bits - 5);
     hp.col = f.build.c[f.out[lastc].v];
-    hp.probe_table = static_cast<const Slot*>(pix->table.p);
-    hp.probe_slots = pix->slots;
+    hp.probe = pix->key_index();
     f.hub_min = std::max<uint32_t>(kHubMinRows, hp.words / kHubWordsPerRow);
     hp.cap = std::min<uint64_t>(ix->n / f.hub_min, ix->distinct);
     if (hp.cap == 0) return CDL_OK;  // no key can be a hub

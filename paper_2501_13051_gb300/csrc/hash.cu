@@ -26,13 +26,11 @@ __device__ __forceinline__ bool key_ne(const uint32_t* k0, const uint32_t* k1, u
   return __ldg(k0 + i) != a0;
 }
 
+// Row i's part of the hash form.
 template <bool TWO>
-__global__ void __launch_bounds__(kThreads) k_hash_build(const uint32_t* __restrict__ k0,
-                                                         const uint32_t* __restrict__ k1,
-                                                         uint64_t n, Slot* __restrict__ t,
-                                                         uint64_t mask, uint32_t* err) {
-  const uint64_t i = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (i >= n) return;
+__device__ __forceinline__ void hash_row(const uint32_t* __restrict__ k0,
+                                         const uint32_t* __restrict__ k1, uint64_t i, uint64_t n,
+                                         Slot* __restrict__ t, uint64_t mask, uint32_t* err) {
   const uint32_t a0 = __ldg(k0 + i);
   const uint32_t a1 = TWO ? __ldg(k1 + i) : 0u;
   if (i > 0 && !key_ne<TWO>(k0, k1, i - 1, a0, a1)) return;  // not a run head
@@ -72,6 +70,45 @@ __global__ void __launch_bounds__(kThreads) k_hash_build(const uint32_t* __restr
 }
 
 template <bool TWO>
+__global__ void __launch_bounds__(kThreads) k_hash_build(const uint32_t* __restrict__ k0,
+                                                         const uint32_t* __restrict__ k1,
+                                                         uint64_t n, Slot* __restrict__ t,
+                                                         uint64_t mask, uint32_t* err) {
+  const uint64_t i = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
+  if (i < n) hash_row<TWO>(k0, k1, i, n, t, mask, err);
+}
+
+// Direct form: the row that starts a key's run stores the run's start, the
+// row that ends it the end, so nothing is searched and, the keys being
+// sorted, the writes go up the array.  Bound by memory: keys read, 8 bytes
+// per entry cleared and 8 per distinct key written.  (A key at or past the
+// range -- of a build side that is not sorted -- is left out.)
+__global__ void __launch_bounds__(kThreads) k_index_build(const uint32_t* __restrict__ k0,
+                                                          uint64_t n, KeyIndex x, uint32_t* err) {
+  const uint64_t i = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
+  if (i >= n) return;
+  const uint32_t range = direct_range(x);
+  Slot* t = const_cast<Slot*>(x.table);
+  if (!range) return hash_row<false>(k0, nullptr, i, n, t, x.slots - 1, err);
+  const uint32_t a = __ldg(k0 + i);
+  if (a >= range) return;
+  uint32_t* e = reinterpret_cast<uint32_t*>(t) + 2ull * a;
+  if (i == 0 || __ldg(k0 + i - 1) != a) e[0] = (uint32_t)i;
+  if (i + 1 == n || __ldg(k0 + i + 1) != a) e[1] = (uint32_t)(i + 1);
+}
+
+// Clears the form that *x.last gives.
+__global__ void __launch_bounds__(kThreads) k_index_clear(KeyIndex x) {
+  const uint32_t range = direct_range(x);
+  const uint64_t words = range ? ((uint64_t)range + 1) / 2 : x.slots;  // 16 bytes each
+  const uint32_t v = range ? 0u : 0xFFFFFFFFu;
+  uint4* t = reinterpret_cast<uint4*>(const_cast<Slot*>(x.table));
+  for (uint64_t i = (uint64_t)blockIdx.x * kThreads + threadIdx.x; i < words;
+       i += (uint64_t)gridDim.x * kThreads)
+    t[i] = make_uint4(v, v, v, v);
+}
+
+template <bool TWO>
 __global__ void __launch_bounds__(kThreads) k_count_heads(const uint32_t* __restrict__ k0,
                                                           const uint32_t* __restrict__ k1,
                                                           uint64_t n, unsigned long long* out) {
@@ -106,6 +143,25 @@ cudaError_t hash_build(Ctx& c, const uint32_t* k0, const uint32_t* k1, uint64_t 
     k_hash_build<true><<<grid, kThreads, 0, c.st>>>(k0, k1, n, table, slots - 1, c.d_err);
   else
     k_hash_build<false><<<grid, kThreads, 0, c.st>>>(k0, k1, n, table, slots - 1, c.d_err);
+  return cudaGetLastError();
+}
+
+uint64_t direct_keys(uint64_t n) { return 4 * n > 65536 ? 4 * n : 65536; }
+
+cudaError_t index_build(Ctx& c, const uint32_t* k0, uint64_t n, const KeyIndex& x) {
+  if (!x.range) return hash_build(c, k0, nullptr, n, const_cast<Slot*>(x.table), x.slots);
+  const unsigned grid = (unsigned)((n + kThreads - 1) / kThreads);
+  if (x.last) {
+    uint64_t blocks = (x.slots + kThreads * 4 - 1) / (kThreads * 4);
+    if (blocks > 152 * 16) blocks = 152 * 16;
+    k_index_clear<<<(unsigned)blocks, kThreads, 0, c.st>>>(x);
+  } else {
+    cudaError_t e = cudaMemsetAsync(const_cast<Slot*>(x.table), 0, 8ull * x.range, c.st);
+    if (e != cudaSuccess) return e;
+  }
+  if (n == 0) return cudaGetLastError();
+  ProfScope p(c, kHashBuild, 4.0 * n);
+  k_index_build<<<grid, kThreads, 0, c.st>>>(k0, n, x, c.d_err);
   return cudaGetLastError();
 }
 

@@ -49,30 +49,31 @@ __device__ __forceinline__ uint32_t probe_key1(const JoinSpec& j, const ColsIn& 
 
 // Range of build rows matching probe row `row`: the hybrid index lookup, or
 // every build row for a join without shared variables.
-__device__ __forceinline__ uint32_t lookup(const JoinSpec& j, const ColsIn& probe, uint64_t mask,
+// (range: direct_range of the index)
+__device__ __forceinline__ uint32_t lookup(const JoinSpec& j, const ColsIn& probe, uint32_t range,
                                           uint64_t row, uint32_t* start) {
   if (j.cross) {
     *start = 0;
     return j.n_build;
   }
-  return probe_table(j.table, mask, __ldg(col_of(probe, j.pk0) + row), probe_key1(j, probe, row),
-                     start);
+  return find_key(j.ix, range, __ldg(col_of(probe, j.pk0) + row), probe_key1(j, probe, row), start);
 }
 
 // Range of second-build-side rows matching probe row `row` (star joins).
 __device__ __forceinline__ uint32_t lookup2(const JoinSpec& j, const ColsIn& probe, uint64_t row,
                                            uint32_t* start) {
   const uint32_t k1 = j.qk1 == 0xFFu ? 0u : __ldg(col_of(probe, j.qk1) + row);
-  return probe_table(j.table2, j.slots2 - 1, __ldg(col_of(probe, j.qk0) + row), k1, start);
+  return find_key(j.ix2, direct_range(j.ix2), __ldg(col_of(probe, j.qk0) + row), k1, start);
 }
 
 // Output count of probe row `row`: its range length, or for a star join the
 // product of its two range lengths (a product past 2^32 - 1 raises
 // kErrCapacity and counts 0: no relation holds that many rows).
 __device__ __forceinline__ uint32_t row_count(const JoinSpec& j, const ColsIn& probe,
-                                             uint64_t mask, uint64_t row, uint32_t* err) {
+                                             uint32_t range, uint64_t row, uint32_t* err) {
   uint32_t st;
-  const uint32_t c1 = lookup(j, probe, mask, row, &st);
+  const uint32_t c1 = lookup(j, probe, range, row, &st);
+  if (j.starts) j.starts[row] = st;
   if (j.hub_min && c1 >= j.hub_min) return 0;  // hub_or's
   if (!j.star || c1 == 0) return c1;
   const uint64_t prod = (uint64_t)c1 * lookup2(j, probe, row, &st);
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(kCT) k_join_count(const JoinSpec j, uint32_t* 
   __shared__ uint64_t red[kCT / 32 + 1];
   const uint64_t n = dev_size(j.dn, j.n_probe);
   const ColsIn probe = probe_cols(j);
-  const uint64_t mask = j.slots - 1;
+  const uint32_t range = direct_range(j.ix);
   // tile 0 is written even for n == 0; blocks loop over the tiles
   const uint64_t ntiles = n ? (n + kScanTile - 1) / kScanTile : 1;
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -106,7 +107,7 @@ __global__ void __launch_bounds__(kCT) k_join_count(const JoinSpec j, uint32_t* 
     for (int i = 0; i < kCItems; ++i) {
       const uint64_t row = base + (uint64_t)i * kCT + threadIdx.x;
       if (row < n) {
-        const uint32_t cnt = row_count(j, probe, mask, row, err);
+        const uint32_t cnt = row_count(j, probe, range, row, err);
         counts[row] = cnt;
         s += cnt;
       }
@@ -122,7 +123,7 @@ __global__ void __launch_bounds__(kCT) k_join_count_only(const JoinSpec j,
                                                          uint32_t* err) {
   const uint64_t row = (uint64_t)blockIdx.x * kCT + threadIdx.x;
   if (row >= j.n_probe) return;
-  counts[row] = row_count(j, j.probe, j.slots - 1, row, err);
+  counts[row] = row_count(j, j.probe, direct_range(j.ix), row, err);
 }
 
 // Number of probe rows among the first d items of the merge of the row
@@ -240,7 +241,7 @@ __global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5)
   const uint64_t o0 = d0 - j0, o1 = d1 - j1;
   const uint64_t r_lo = j0 > 0 ? j0 - 1 : 0;
   const uint32_t nrows = (uint32_t)(j1 - r_lo);
-  const uint64_t mask = j.slots - 1;
+  const uint32_t range = direct_range(j.ix);
   // the outputs' rows come from a table where the head is written as rows
   // (a bitmap head's block searches the staged starts, or walks its rows
   // one by one when it has a few: there the table's barriers cost more
@@ -256,7 +257,12 @@ __global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5)
     const uint64_t a = __ldg(off + row);
     const uint64_t b = row + 1 < n_probe ? __ldg(off + row + 1) : total;
     uint32_t st = 0;
-    if (b > a) lookup(j, probe, mask, row, &st);
+    if (b > a) {
+      if (!STAR && j.starts)
+        st = __ldg(j.starts + row);
+      else
+        lookup(j, probe, range, row, &st);
+    }
     if (r == 0)
       s_a0 = a;
     else
@@ -481,16 +487,25 @@ struct HubTask {
   uint32_t hub, row, rows;
 };
 
-__global__ void __launch_bounds__(kCT) k_hub_list(const JoinSpec j, const Slot* __restrict__ ptable,
-                                                  uint64_t pslots, uint2* __restrict__ hubs,
+__global__ void __launch_bounds__(kCT) k_hub_list(const JoinSpec j, const KeyIndex pix, uint2* __restrict__ hubs,
                                                   uint64_t cap, HubTask* __restrict__ tasks,
                                                   uint64_t task_cap, unsigned long long* n) {
-  for (uint64_t i = (uint64_t)blockIdx.x * kCT + threadIdx.x; i < j.slots;
+  const uint32_t range = direct_range(j.ix), prange = direct_range(pix);
+  const uint64_t entries = range ? range : j.ix.slots;
+  for (uint64_t i = (uint64_t)blockIdx.x * kCT + threadIdx.x; i < entries;
        i += (uint64_t)gridDim.x * kCT) {
-    const Slot s = load_slot(j.table, i);
-    if ((s.k0 == kEmpty && s.k1 == kEmpty) || s.count < j.hub_min) continue;
+    Slot s;
+    if (range) {
+      s.k0 = (uint32_t)i;
+      s.k1 = 0;
+      s.count = find_key(j.ix, range, s.k0, 0u, &s.start);
+    } else {
+      s = load_slot(j.ix.table, i);
+      if (s.k0 == kEmpty && s.k1 == kEmpty) continue;
+    }
+    if (s.count < j.hub_min) continue;
     uint32_t prow;
-    const uint32_t pn = probe_table(ptable, pslots - 1, s.k0, s.k1, &prow);
+    const uint32_t pn = find_key(pix, prange, s.k0, s.k1, &prow);
     if (pn == 0) continue;
     const uint64_t h = atomicAdd(n, 1ull);
     if (h >= cap) continue;  // (cannot happen: cap counts every such key)
@@ -651,10 +666,11 @@ cudaError_t hub_or(Ctx& c, const JoinSpec& j, const HubPlan& h, const DenseSet& 
   if (e == cudaSuccess) e = cudaMemsetAsync(bits, 0, 4ull * h.cap * h.words, c.st);
   if (e != cudaSuccess) return e;
   {
-    ProfScope ps(c, kDense, 16.0 * j.slots);
-    uint64_t blocks = (j.slots + kCT - 1) / kCT;
+    const uint64_t entries = j.ix.range ? j.ix.range : j.ix.slots;
+    ProfScope ps(c, kDense, (j.ix.range ? 8.0 : 16.0) * entries);
+    uint64_t blocks = (entries + kCT - 1) / kCT;
     if (blocks > 152 * 8) blocks = 152 * 8;
-    k_hub_list<<<(unsigned)blocks, kCT, 0, c.st>>>(j, h.probe_table, h.probe_slots, hubs, h.cap, tasks,
+    k_hub_list<<<(unsigned)blocks, kCT, 0, c.st>>>(j, h.probe, hubs, h.cap, tasks,
                                                    task_cap, n);
   }
   {
@@ -740,12 +756,12 @@ __global__ void __launch_bounds__(kDirT) k_join_direct(const JoinSpec j, ColsOut
   __shared__ uint32_t s_start[kDirT];  // first build row of each row's range
   __shared__ uint32_t red[kDirT / 32 + 1];
   __shared__ unsigned long long s_base;
-  const uint64_t mask = j.slots - 1;
+  const uint32_t range = direct_range(j.ix);
   for (uint64_t b0 = (uint64_t)blockIdx.x * kDirT; b0 < j.n_probe;
        b0 += (uint64_t)gridDim.x * kDirT) {
     const uint64_t row = b0 + threadIdx.x;
     uint32_t st = 0, cnt = 0;
-    if (row < j.n_probe) cnt = lookup(j, j.probe, mask, row, &st);
+    if (row < j.n_probe) cnt = lookup(j, j.probe, range, row, &st);
     if (cnt > kHeavyChunk) {  // a long range becomes chunks of the heavy list
       atomicAdd(total, (unsigned long long)cnt);
       uint64_t out0 = 0;

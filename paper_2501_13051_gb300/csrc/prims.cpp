@@ -3,6 +3,7 @@
 // caller-provided workspace.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
@@ -85,8 +86,8 @@ cdl_status cdl_join_count(const uint32_t* probe, uint64_t n, const void* table,
   j.n_probe = n;
   j.pk0 = 0;
   j.pk1 = 0xFFu;
-  j.table = static_cast<const Slot*>(table);
-  j.slots = slots;
+  j.ix.table = static_cast<const Slot*>(table);
+  j.ix.slots = slots;
   return cuda_status(join_count_only(c, j, counts));
 }
 
@@ -116,27 +117,27 @@ cdl_status cdl_exclusive_scan(const uint32_t* in, uint64_t n, uint64_t* out, uin
   return CDL_OK;
 }
 
-cdl_status cdl_join(const uint32_t* const* probe_cols, uint32_t probe_arity, uint64_t n_probe,
-                    uint32_t probe_key, const uint32_t* const* build_cols, uint32_t build_arity,
-                    uint64_t n_build, uint32_t build_key, const cdl_colref* spec,
-                    uint32_t out_arity, const cdl_colref* neq, uint32_t nneq,
-                    uint32_t* const* out_cols, uint64_t out_cap, uint64_t* n_out, void* workspace,
-                    size_t* ws_bytes, void* stream) {
-  if (!ws_bytes) return CDL_E_INVALID;
-  const uint64_t slots = table_slots(n_build, 0.5);
-  const size_t need = kHead + up(slots * sizeof(Slot)) + up(8 * (n_probe ? n_probe : 1)) +
-                      up(join_count_workspace(n_probe));
-  if (!workspace) {
-    *ws_bytes = need;
-    return CDL_OK;
-  }
-  if (*ws_bytes < need || !n_out) return CDL_E_INVALID;
+// cdl_join and cdl_join_write: checked arguments and the workspace's parts.
+struct JoinCall {
+  JoinSpec j{};
+  uint64_t* head;  // error word, total, output cursor
+  Slot* table;
+  uint64_t* off;
+  void* cws;
+};
+
+static cdl_status join_setup(const uint32_t* const* probe_cols, uint32_t probe_arity,
+                             uint64_t n_probe, uint32_t probe_key,
+                             const uint32_t* const* build_cols, uint32_t build_arity,
+                             uint64_t n_build, uint32_t build_key, const cdl_colref* spec,
+                             uint32_t out_arity, const cdl_colref* neq, uint32_t nneq,
+                             void* workspace, size_t ws_bytes, size_t need, JoinCall& jc) {
   if (probe_arity < 1 || probe_arity > CDL_MAX_ARITY || build_arity < 1 ||
       build_arity > CDL_MAX_ARITY || out_arity < 1 || out_arity > CDL_MAX_ARITY ||
       probe_key >= probe_arity || build_key >= build_arity || nneq > 4 || !spec)
     return CDL_E_INVALID;
   if (n_build > 0xFFFFFFFFull) return CDL_E_CAPACITY;
-  JoinSpec j{};
+  JoinSpec& j = jc.j;
   for (uint32_t k = 0; k < probe_arity; ++k) j.probe.c[k] = probe_cols[k];
   for (uint32_t k = 0; k < build_arity; ++k) j.build.c[k] = build_cols[k];
   j.n_probe = n_probe;
@@ -155,36 +156,102 @@ cdl_status cdl_join(const uint32_t* const* probe_cols, uint32_t probe_arity, uin
   j.n_neq = nneq;
   for (uint32_t q = 0; q < nneq; ++q)
     if (!conv(neq[2 * q], j.neq[q][0]) || !conv(neq[2 * q + 1], j.neq[q][1])) return CDL_E_INVALID;
+  const uint64_t slots = table_slots(n_build, 0.5);
   Carve cv(workspace);
-  uint64_t* head = static_cast<uint64_t*>(cv.take(kHead));
-  Slot* table = static_cast<Slot*>(cv.take(slots * sizeof(Slot)));
-  uint64_t* off = static_cast<uint64_t*>(cv.take(8 * (n_probe ? n_probe : 1)));
-  void* cws = cv.take(join_count_workspace(n_probe));
-  Ctx c;
-  c.st = static_cast<cudaStream_t>(stream);
-  c.d_err = reinterpret_cast<uint32_t*>(head);
-  cudaError_t e = cudaMemsetAsync(head, 0, kHead, c.st);
-  if (e == cudaSuccess) e = hash_build(c, build_cols[build_key], nullptr, n_build, table, slots);
-  j.table = table;
-  j.slots = slots;
-  if (e == cudaSuccess) e = join_count_scan(c, j, off, head + 1, cws);
+  jc.head = static_cast<uint64_t*>(cv.take(kHead));
+  jc.table = static_cast<Slot*>(cv.take(slots * sizeof(Slot)));
+  jc.off = static_cast<uint64_t*>(cv.take(8 * (n_probe ? n_probe : 1)));
+  jc.cws = cv.take(join_count_workspace(n_probe));
+  // (a workspace of the size without the rows' starts does as well: the write
+  // then looks the keys up again)
+  if (ws_bytes >= need) j.starts = static_cast<uint32_t*>(cv.take(4 * (n_probe ? n_probe : 1)));
+  // the direct form where the largest key fits the table's memory (4 to 8
+  // keys per row: it is then cleared, filled and read for less than the hash
+  // form)
+  j.ix.table = jc.table;
+  j.ix.slots = slots;
+  if (n_build) {
+    j.ix.range = (uint32_t)std::min<uint64_t>(2 * slots, 0xFFFFFFFFull);
+    j.ix.last = build_cols[build_key] + n_build - 1;
+  }
+  return CDL_OK;
+}
+
+static cdl_status join_output(const JoinCall& jc, uint32_t* const* out_cols, uint32_t out_arity,
+                              uint64_t out_cap, uint64_t total, uint64_t* n_out, Ctx& c) {
+  ColsOut out;
+  for (uint32_t k = 0; k < CDL_MAX_ARITY; ++k) out.c[k] = k < out_arity ? out_cols[k] : nullptr;
+  // the count workspace is free again: it holds the write splits if large enough
+  cudaError_t e = join_write(c, jc.j, jc.off, total, out, 0, jc.head + 2, out_cap, jc.cws,
+                             join_count_workspace(jc.j.n_probe));
   if (e != cudaSuccess) return CDL_E_CUDA;
   uint64_t h[3];
-  cdl_status s = read_flags(head, c.st, h, 2);
+  cdl_status s = read_flags(jc.head, c.st, h, 3);
+  if (s != CDL_OK) return s;
+  *n_out = h[2];
+  return CDL_OK;
+}
+
+static size_t join_need(uint64_t n_probe, uint64_t n_build, bool starts) {
+  return kHead + up(table_slots(n_build, 0.5) * sizeof(Slot)) + up(8 * (n_probe ? n_probe : 1)) +
+         up(join_count_workspace(n_probe)) + (starts ? up(4 * (n_probe ? n_probe : 1)) : 0);
+}
+
+cdl_status cdl_join(const uint32_t* const* probe_cols, uint32_t probe_arity, uint64_t n_probe,
+                    uint32_t probe_key, const uint32_t* const* build_cols, uint32_t build_arity,
+                    uint64_t n_build, uint32_t build_key, const cdl_colref* spec,
+                    uint32_t out_arity, const cdl_colref* neq, uint32_t nneq,
+                    uint32_t* const* out_cols, uint64_t out_cap, uint64_t* n_out, void* workspace,
+                    size_t* ws_bytes, void* stream) {
+  if (!ws_bytes) return CDL_E_INVALID;
+  const size_t need = join_need(n_probe, n_build, true);
+  if (!workspace) {
+    *ws_bytes = need;
+    return CDL_OK;
+  }
+  if (*ws_bytes < join_need(n_probe, n_build, false) || !n_out) return CDL_E_INVALID;
+  JoinCall jc;
+  cdl_status s = join_setup(probe_cols, probe_arity, n_probe, probe_key, build_cols, build_arity,
+                            n_build, build_key, spec, out_arity, neq, nneq, workspace, *ws_bytes,
+                            need, jc);
+  if (s != CDL_OK) return s;
+  Ctx c;
+  c.st = static_cast<cudaStream_t>(stream);
+  c.d_err = reinterpret_cast<uint32_t*>(jc.head);
+  cudaError_t e = cudaMemsetAsync(jc.head, 0, kHead, c.st);
+  if (e == cudaSuccess) e = index_build(c, build_cols[build_key], n_build, jc.j.ix);
+  if (e == cudaSuccess) e = join_count_scan(c, jc.j, jc.off, jc.head + 1, jc.cws);
+  if (e != cudaSuccess) return CDL_E_CUDA;
+  uint64_t h[2];
+  s = read_flags(jc.head, c.st, h, 2);
   if (s != CDL_OK) return s;
   const uint64_t total = h[1];
   *n_out = total;
   if (total == 0) return CDL_OK;
   if (out_cap < total) return CDL_E_CAPACITY;
-  ColsOut out;
-  for (uint32_t k = 0; k < CDL_MAX_ARITY; ++k) out.c[k] = k < out_arity ? out_cols[k] : nullptr;
-  // the count workspace is free again: it holds the write splits if large enough
-  e = join_write(c, j, off, total, out, 0, head + 2, out_cap, cws, join_count_workspace(n_probe));
-  if (e != cudaSuccess) return CDL_E_CUDA;
-  s = read_flags(head, c.st, h, 3);
+  return join_output(jc, out_cols, out_arity, out_cap, total, n_out, c);
+}
+
+cdl_status cdl_join_write(const uint32_t* const* probe_cols, uint32_t probe_arity, uint64_t n_probe,
+                          uint32_t probe_key, const uint32_t* const* build_cols,
+                          uint32_t build_arity, uint64_t n_build, uint32_t build_key,
+                          const cdl_colref* spec, uint32_t out_arity, const cdl_colref* neq,
+                          uint32_t nneq, uint32_t* const* out_cols, uint64_t out_cap,
+                          uint64_t* n_out, void* workspace, const size_t* ws_bytes, void* stream) {
+  if (!ws_bytes || !workspace || !n_out) return CDL_E_INVALID;
+  if (*ws_bytes < join_need(n_probe, n_build, false)) return CDL_E_INVALID;
+  const uint64_t total = *n_out;
+  if (total == 0) return CDL_OK;
+  if (out_cap < total) return CDL_E_CAPACITY;
+  JoinCall jc;
+  cdl_status s = join_setup(probe_cols, probe_arity, n_probe, probe_key, build_cols, build_arity,
+                            n_build, build_key, spec, out_arity, neq, nneq, workspace, *ws_bytes,
+                            join_need(n_probe, n_build, true), jc);
   if (s != CDL_OK) return s;
-  *n_out = h[2];
-  return CDL_OK;
+  Ctx c;
+  c.st = static_cast<cudaStream_t>(stream);
+  c.d_err = reinterpret_cast<uint32_t*>(jc.head);
+  return join_output(jc, out_cols, out_arity, out_cap, total, n_out, c);
 }
 
 cdl_status cdl_sort_unique(const uint32_t* const* cols, uint32_t arity, uint64_t n,
