@@ -235,6 +235,41 @@ cudaError_t radix_sort(Ctx& c, const RadixPlan& plan, ColsOut a, ColsOut b, uint
 // Column maxima into d_max[k] (for plans of unknown data).
 cudaError_t column_max(Ctx& c, ColsIn in, uint32_t k, uint64_t n, uint32_t* d_max);
 
+// Sort of at most kSmallSort tuples in one launch (out may be in); unique:
+// repeats dropped.  head, when set: head[0] = 0, head[1] = tuples written.
+constexpr uint64_t kSmallSort = 4096;
+cudaError_t sort_small(Ctx& c, uint32_t k, ColsIn in, uint64_t n, ColsOut out, bool unique,
+                       uint64_t* head);
+
+// Bucket sort (bucket_sort.cu) by a packed key of the first `keys` columns
+// (as many as 64 bits hold; the others, if any, decide between equal keys):
+// the bits above `low` choose one of `buckets` buckets of about kBucketRows /
+// 2 to kBucketRows rows, the low ones are sorted in shared memory.
+constexpr uint32_t kBucketCap = 4096;        // rows a bucket may hold
+constexpr uint64_t kBucketRows = 2304;       // aimed at: uneven data get some slack
+constexpr uint32_t kBucketMaxBits = 14;      // buckets counted in 64 KB of shared memory
+struct BucketPlan {
+  uint32_t k = 0, keys = 0, low = 0, buckets = 0;
+  uint32_t shift[kMaxK] = {}, mask[kMaxK] = {};
+};
+// false where the sort does not apply.
+// col_max: the columns' largest values, if known.
+bool bucket_plan(uint32_t k, const uint32_t* col_bits, const uint32_t* col_max, uint64_t n,
+                 BucketPlan& b);
+size_t bucket_workspace(const BucketPlan& b);
+// First part: the largest bucket's rows into *d_max.  The second may run
+// when that is at most kBucketCap.
+cudaError_t bucket_count(Ctx& c, const BucketPlan& b, ColsIn in, uint64_t n, void* ws,
+                         uint64_t* d_max);
+// Second part, with the first one's workspace: rows sorted into out; with
+// d_unique, repeats dropped and the rows' number there.  packed: 8 n bytes;
+// out may then be in (the rows are in packed before the first is written).
+// Wide tuples (keys < k): with d_unique only, packed 12 n bytes, out not in;
+// d_unique[1] (zero before) is set where the tuples came too uneven: the
+// rows are then not sorted.
+cudaError_t bucket_sort(Ctx& c, const BucketPlan& b, ColsIn in, uint64_t n, ColsOut out,
+                        uint64_t* packed, void* ws, uint64_t* d_unique);
+
 // ------------------------------------------------------- Algorithm 2 dedup
 // Full in the decomposed storage model: raw columns in insertion order (row
 // = surrogate id); per column k the ids in (value, id) order and the unique

@@ -30,6 +30,10 @@ struct Carve {
 
 constexpr size_t kHead = 256;  // error word, cursor, totals
 
+// cdl_sort_unique: bits of tuple space per row up to which the rows go
+// through a bitmap.
+constexpr uint64_t kBitmapPerRow = 64;
+
 bool pow2(uint64_t x) { return x && !(x & (x - 1)); }
 
 cdl_status cuda_status(cudaError_t e) { return e == cudaSuccess ? CDL_OK : CDL_E_CUDA; }
@@ -270,45 +274,98 @@ cdl_status cdl_sort_unique(const uint32_t* const* cols, uint32_t arity, uint64_t
   if (n > 0xFFFFFFFFull) return CDL_E_CAPACITY;
   Carve cv(workspace);
   uint64_t* head = static_cast<uint64_t*>(cv.take(kHead));
-  ColsOut a{}, b{};
-  for (uint32_t k = 0; k < arity; ++k) a.c[k] = static_cast<uint32_t*>(cv.take(rows * 4));
-  for (uint32_t k = 0; k < arity; ++k) b.c[k] = static_cast<uint32_t*>(cv.take(rows * 4));
-  void* rws = cv.take(radix_workspace(n, 9));  // room for 9-bit digits
-  void* dws = cv.take(diff_merge_workspace(0, n));
   Ctx c;
   c.st = static_cast<cudaStream_t>(stream);
   c.d_err = reinterpret_cast<uint32_t*>(head);
-  cudaError_t e = cudaMemsetAsync(head, 0, kHead, c.st);
-  for (uint32_t k = 0; k < arity && e == cudaSuccess; ++k)
-    e = cudaMemcpyAsync(a.c[k], cols[k], n * 4, cudaMemcpyDeviceToDevice, c.st);
-  ColsIn ain;
-  for (int k = 0; k < kMaxK; ++k) ain.c[k] = a.c[k];
-  uint32_t* dmax = reinterpret_cast<uint32_t*>(head + 4);
-  if (e == cudaSuccess) e = column_max(c, ain, arity, n, dmax);
-  if (e != cudaSuccess) return CDL_E_CUDA;
+  ColsIn in{};
+  ColsOut out{};
+  for (uint32_t k = 0; k < arity && n; ++k) {
+    in.c[k] = cols[k];
+    out.c[k] = out_cols[k];
+  }
   uint64_t h[8];
-  cdl_status s = read_flags(head, c.st, h, 6);
+  auto finish = [&]() {
+    cdl_status s = read_flags(head, c.st, h, 2);
+    if (s == CDL_OK) *n_out = h[1];
+    return s;
+  };
+  if (n && n <= kSmallSort) {  // one launch
+    if (sort_small(c, arity, in, n, out, true, head) != cudaSuccess) return CDL_E_CUDA;
+    return finish();
+  }
+  // room for two copies of the columns, the sort's tables and the difference's
+  char* rows_ws = static_cast<char*>(cv.take(2 * arity * col));
+  void* rws = cv.take(radix_workspace(n, 9));  // room for 9-bit digits
+  void* dws = cv.take(diff_merge_workspace(0, n));
+  cudaError_t e = cudaMemsetAsync(head, 0, kHead, c.st);
+  uint32_t* dmax = reinterpret_cast<uint32_t*>(head + 4);
+  if (e == cudaSuccess) e = column_max(c, in, arity, n, dmax);
+  if (e != cudaSuccess) return CDL_E_CUDA;
+  cdl_status s = read_flags(head, c.st, h, 8);
   if (s != CDL_OK) return s;
-  uint32_t bits[kMaxK] = {0, 0, 0, 0};
-  const uint32_t* hm = reinterpret_cast<const uint32_t*>(h + 4);
-  for (uint32_t k = 0; k < arity; ++k) bits[k] = bits_of(hm[k]);
+  uint32_t bits[kMaxK] = {0, 0, 0, 0}, max[kMaxK];
+  memcpy(max, h + 4, sizeof(max));
   uint32_t total = 0;
-  for (uint32_t k = 0; k < arity; ++k) total += bits[k];
+  for (uint32_t k = 0; k < arity; ++k) total += bits[k] = bits_of(max[k]);
+  // few possible tuples (a bitmap of them takes at most 8 bytes a row): set
+  // bits, read back in order (1M pairs of 12-bit values 359 -> 126 us, of
+  // 16.7M 14-bit pairs 1,218 -> 502 us; 1M 14-bit pairs, just past the line,
+  // take 167 us by buckets)
+  if (n && total < 40 && (1ull << total) <= kBitmapPerRow * n) {
+    DenseSet d{};
+    d.nbits = 1ull << total;
+    d.k = arity;
+    d.append = 1;  // (the bits need no clearing behind the read)
+    d.words = reinterpret_cast<uint32_t*>(rows_ws);
+    uint32_t sh = 0;
+    for (int k = (int)arity - 1; k >= 0; --k) {
+      if (bits[k]) d.shift[k] = sh;
+      d.mask[k] = (uint32_t)((1ull << bits[k]) - 1);
+      sh += bits[k];
+    }
+    const size_t bytes = d.nbits >= 32 ? d.nbits >> 3 : 4;
+    if (bytes <= 2 * arity * col && dense_extract_workspace(d.nbits) <= radix_workspace(n, 9)) {
+      e = cudaMemsetAsync(rows_ws, 0, bytes, c.st);
+      if (e == cudaSuccess) e = dense_insert(c, d, in, n);
+      if (e == cudaSuccess) e = dense_extract(c, d, out, n, head + 1, rws);
+      return e == cudaSuccess ? finish() : CDL_E_CUDA;
+    }
+  }
+  BucketPlan bp;
+  if (bucket_plan(arity, bits, max, n, bp) &&
+      bucket_workspace(bp) <= up(radix_workspace(n, 9)) + up(diff_merge_workspace(0, n)) &&
+      (bp.keys < bp.k ? 12 : 8) * n <= 2 * arity * col) {
+    e = bucket_count(c, bp, in, n, rws, head + 3);
+    if (e != cudaSuccess) return CDL_E_CUDA;
+    s = read_flags(head, c.st, h, 4);
+    if (s != CDL_OK) return s;
+    if (h[3] <= kBucketCap) {
+      e = bucket_sort(c, bp, in, n, out, reinterpret_cast<uint64_t*>(rows_ws), rws, head + 1);
+      if (e != cudaSuccess) return CDL_E_CUDA;
+      s = read_flags(head, c.st, h, 3);
+      if (s != CDL_OK) return s;
+      *n_out = h[1];
+      if (!h[2]) return CDL_OK;  // (else too uneven: the radix sort)
+    }
+  }
+  ColsOut a{}, b{};
+  for (uint32_t k = 0; k < arity; ++k) {
+    a.c[k] = reinterpret_cast<uint32_t*>(rows_ws + k * col);
+    b.c[k] = reinterpret_cast<uint32_t*>(rows_ws + (arity + k) * col);
+  }
+  for (uint32_t k = 0; k < arity && n && e == cudaSuccess; ++k)
+    e = cudaMemcpyAsync(a.c[k], cols[k], n * 4, cudaMemcpyDeviceToDevice, c.st);
+  if (e != cudaSuccess) return CDL_E_CUDA;
   RadixPlan plan = make_radix_plan(arity, bits, fit_digit_bits(total, 8));
   bool in_b = false;
   e = radix_sort(c, plan, a, b, n, rws, &in_b);
   if (e != cudaSuccess) return CDL_E_CUDA;
   ColsIn sorted;
   for (int k = 0; k < kMaxK; ++k) sorted.c[k] = in_b ? b.c[k] : a.c[k];
-  ColsOut delta{}, none{};
-  for (uint32_t k = 0; k < arity; ++k) delta.c[k] = out_cols[k];
+  ColsOut none{};
   ColsIn empty{};
-  e = diff_merge(c, arity, empty, 0, sorted, n, delta, none, head + 1, dws);
-  if (e != cudaSuccess) return CDL_E_CUDA;
-  s = read_flags(head, c.st, h, 2);
-  if (s != CDL_OK) return s;
-  *n_out = h[1];
-  return CDL_OK;
+  e = diff_merge(c, arity, empty, 0, sorted, n, out, none, head + 1, dws);
+  return e == cudaSuccess ? finish() : CDL_E_CUDA;
 }
 
 cdl_status cdl_mlp_forward(const float* params, const float* X, uint64_t n, float* out,
