@@ -250,8 +250,9 @@ __device__ __forceinline__ uint32_t set_add(const DenseSet& d, const uint64_t (&
 // Writes a block's new tuples (bit q of fresh: tuple idx[q] is new) packed at
 // *cursor: one claim per block, each warp's tuples of one q side by side.
 // wsum: THREADS / 32 + 2 words of shared memory (the last two hold the
-// claimed position).  Rows past cap are dropped; false tells the caller.
-template <int THREADS, int N>
+// claimed position).  Rows past cap are dropped; false tells the caller
+// (CLEAR: their bits are cleared again, so that a second try finds them new).
+template <int THREADS, int N, bool CLEAR = false>
 __device__ __forceinline__ bool set_emit(const DenseSet& d, const uint64_t (&idx)[N],
                                          uint32_t fresh, ColsOut out, uint64_t base,
                                          unsigned long long* cursor, uint64_t cap,
@@ -287,6 +288,7 @@ __device__ __forceinline__ bool set_emit(const DenseSet& d, const uint64_t (&idx
         for (int k = 0; k < kMaxK; ++k)
           if (k < (int)d.k) out.c[k][p] = set_column(d, idx[q], k);
       } else {
+        if (CLEAR) atomicAnd(d.words + (idx[q] >> 5), ~(1u << (idx[q] & 31)));
         ok = false;
       }
     }

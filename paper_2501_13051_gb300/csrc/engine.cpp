@@ -323,6 +323,8 @@ struct Relation {
   bool set_free = false; // within dense_bits: a round's join outputs are not limited to 2^32
   DenseSet fset{};
   DBuf fset_buf;
+  bool set_single = false;  // a single-pass join of this round wrote sdelta
+  bool set_redo = false;    // ... and ran out of room: its rules run again, exact
   DCols sdelta;          // the round's new tuples so far (dslot(kSlotDelta + i) of them)
   uint64_t sdelta_ub = 0;
   double merged_bytes = 0;  // row form: bytes its sorts and merges have moved
@@ -383,10 +385,12 @@ constexpr uint32_t kMaxRels = 1024;
 // 3 single-pass join size, 4 overflow flag, 5 overflow flag of the round's
 // deferred checks, 8 + r fresh cursor of relation r,
 // 8 + kMaxRels + r delta size of relation r
+// 8 + 2 kMaxRels + s size of the round's s-th single-pass join into a set
 constexpr uint32_t kSlotErr = 0, kSlotScratch = 1, kSlotAux = 2, kSlotDirTotal = 3,
                    kSlotOverflow = 4, kSlotRoundOverflow = 5, kSlotCursor = 8,
                    kSlotDelta = 8 + kMaxRels,
-                   kCtlSlots = 8 + 2 * kMaxRels;
+                   kSetSteps = 256, kSlotSetTotal = 8 + 2 * kMaxRels,
+                   kCtlSlots = 8 + 2 * kMaxRels + kSetSteps;
 constexpr int kEstFloats = 32;  // 16 features, the prediction, padding
 
 }  // namespace
@@ -485,6 +489,25 @@ struct cdl_engine {
   DBuf heavy_buf;  // the single-pass join's list of long-range chunks
   HeavyList heavy;
   bool force_exact = false;  // rules are being redone without predictions
+  // Joins into Full as a set run without a count (join_set) where the same
+  // step's last join had few outputs per probe row: at most kSetRatio, so
+  // that hub joins and skewed ones keep the exact form.  One-pass joins of
+  // the round (set_steps) leave their sizes in the control block.
+  struct SetSeen {
+    uint64_t probe = 0, outputs = 0;
+  };
+  static constexpr uint64_t kSetRatio = 4;
+  static constexpr uint64_t kSetHeavyCap = 1 << 16;  // chunks of long ranges
+  std::map<std::tuple<size_t, size_t, size_t>, SetSeen> set_seen;
+  struct SetStep {
+    std::tuple<size_t, size_t, size_t> key;
+    uint32_t head;
+    uint64_t probe;
+  };
+  std::vector<SetStep> set_steps;
+  bool delta_known = false;  // h_ctl holds the set relations' delta sizes
+  DBuf set_heavy_buf;
+  HeavyList set_heavy;
   // rounds captured as a CUDA graph (option graph): the join steps of the
   // first semi-naive round, recorded as they run, are the plan of every
   // later round
@@ -867,11 +890,31 @@ struct cdl_engine {
     return set_start(R, space, false);
   }
 
-  // Room for the round's new tuples of a join with `extra` outputs.
+  uint32_t rel_id(const Relation& R) const {
+    for (uint32_t i = 0; i < rels.size(); ++i)
+      if (rels[i].get() == &R) return i;
+    return 0;
+  }
+
+  // Room for the round's new tuples of a join with `extra` outputs (or
+  // set_redo where an earlier one-pass join already lacks room).
   cdl_status ensure_sdelta(Relation& R, uint64_t extra) {
     if (!R.set_free && R.sdelta_ub + extra > 0xFFFFFFFFull)
       return fail(CDL_E_CAPACITY, "relation " + R.name + " would receive more than 2^32 new "
                                   "tuples in one round");
+    if (R.set_single && R.sdelta_ub + extra > R.sdelta.cap) {
+      // the one-pass joins so far may have run out of room: their rows are
+      // all there only if not
+      cdl_status r = fetch(kSlotDelta + rel_id(R), 1);
+      if (r != CDL_OK) return r;
+      const uint64_t at = h_ctl[kSlotDelta + rel_id(R)];
+      if (at > R.sdelta.cap) {
+        R.set_redo = true;
+        return CDL_OK;
+      }
+      R.sdelta_ub = at;
+      R.set_single = false;
+    }
     const uint64_t old_ub = R.sdelta_ub;
     R.sdelta_ub += extra;
     const uint64_t need = std::min(R.sdelta_ub, R.fset.nbits - std::min(R.fset.nbits, R.full.n));
@@ -897,6 +940,10 @@ struct cdl_engine {
       if (!R.set_on) continue;
       const uint64_t nf = std::min<uint64_t>(h_ctl[kSlotCursor + i], R.fresh.cap);
       if (nf == 0) continue;
+      // (the rows so far are counted and all there)
+      R.sdelta_ub = std::max(R.sdelta_ub, h_ctl[kSlotDelta + i]);
+      R.set_single = false;
+      delta_known = false;
       cdl_status r = ensure_sdelta(R, nf);
       if (r != CDL_OK) return r;
       cudaError_t e = set_insert(ctx, R.fset, R.fresh.in(), nf, R.sdelta.out(), dslot(kSlotDelta + i),
@@ -1874,6 +1921,12 @@ struct cdl_engine {
           }
         }
       }
+      const bool into_set = last && rels[rule.head.rel]->set_on && !js.cross;
+      if (into_set && !force_exact && !recording) {
+        bool done = false;
+        r = set_join(rule, js, P.n, step_key, done);
+        if (r != CDL_OK || done) return r;
+      }
       // passes 1 and 2: counts, offsets, total
       DBuf off = alloc(std::max<uint64_t>(P.n, 1) * 8);
       DBuf ws = alloc(join_count_workspace(P.n));
@@ -1904,6 +1957,7 @@ struct cdl_engine {
       const uint64_t total = h_ctl[kSlotScratch];
       ++joins;
       log_sample(total);
+      if (into_set) set_seen[step_key] = SetSeen{P.n, total};
       if (recording) {  // a step of a capturable plan: hash join, static build side
         GStep g;
         g.rule = (size_t)(&rule - rules.data());
@@ -1935,7 +1989,7 @@ struct cdl_engine {
       if (last && rels[rule.head.rel]->set_on) {  // Full is a set: new tuples go to delta
         Relation& H = *rels[rule.head.rel];
         r = ensure_sdelta(H, total);
-        if (r != CDL_OK) return r;
+        if (r != CDL_OK || H.set_redo) return r;
         e = join_write(ctx, js, static_cast<const uint64_t*>(off.p), total, H.sdelta.out(), 0,
                        dslot(kSlotDelta + rule.head.rel), H.sdelta.cap, wsp.p, wws, nullptr, nullptr,
                        nullptr, &H.fset);
@@ -1980,6 +2034,46 @@ struct cdl_engine {
       if (next.n == 0) return CDL_OK;
       left = std::move(next);
     }
+    return CDL_OK;
+  }
+
+  // A join into Full as a set in one pass, into a buffer sized by the step's
+  // last join; done = false leaves it to the exact form.
+  cdl_status set_join(const RuleR& rule, const JoinSpec& js, uint64_t np,
+                      const std::tuple<size_t, size_t, size_t>& key, bool& done) {
+    Relation& H = *rels[rule.head.rel];
+    const auto it = set_seen.find(key);
+    if (it == set_seen.end() || opt.mem_limit || set_steps.size() >= kSetSteps) return CDL_OK;
+    const SetSeen& seen = it->second;
+    if (seen.probe == 0 || seen.outputs > kSetRatio * seen.probe) return CDL_OK;
+    const double per_row = (double)seen.outputs / (double)seen.probe;
+    const uint64_t want = (uint64_t)((2.0 * per_row + 1.0) * (double)np) + 4096;
+    if (!H.set_free && H.sdelta_ub + want > 0xFFFFFFFFull) return CDL_OK;
+    cdl_status r = ensure_sdelta(H, want);
+    if (r == CDL_E_NOMEM) {  // (nothing was changed but the bound)
+      err.clear();
+      H.sdelta_ub -= want;
+      return CDL_OK;
+    }
+    if (r != CDL_OK) return r;
+    done = true;
+    if (H.set_redo) return CDL_OK;
+    const uint32_t slot = kSlotSetTotal + (uint32_t)set_steps.size();
+    if (!set_heavy_buf.p) {
+      set_heavy_buf = alloc(256 + sizeof(HeavyChunk) * kSetHeavyCap);
+      if (!set_heavy_buf.p) return fail(CDL_E_NOMEM, "long ranges");
+      set_heavy.n = static_cast<uint64_t*>(set_heavy_buf.p);
+      set_heavy.e = reinterpret_cast<HeavyChunk*>(static_cast<char*>(set_heavy_buf.p) + 256);
+      set_heavy.cap = kSetHeavyCap;
+    }
+    cudaError_t e = cudaMemsetAsync(set_heavy.n, 0, 8, st);
+    if (e == cudaSuccess)
+      e = join_set(ctx, js, H.fset, H.sdelta.out(), dslot(kSlotDelta + rule.head.rel), H.sdelta.cap,
+                   dslot(slot), set_heavy);
+    if (e != cudaSuccess) return cuda_fail(e, "one-pass join");
+    H.set_single = true;
+    set_steps.push_back(SetStep{key, rule.head.rel, np});
+    ++joins;
     return CDL_OK;
   }
 
@@ -2057,6 +2151,10 @@ struct cdl_engine {
     if (H.set_on) {
       r = ensure_sdelta(H, total);
       if (r != CDL_OK) return r;
+      if (H.set_redo) {
+        done = true;
+        return CDL_OK;
+      }
       out = H.sdelta.out();
       cursor = dslot(kSlotDelta + rule.head.rel);
       cap = H.sdelta.cap;
@@ -2089,7 +2187,8 @@ struct cdl_engine {
                      !plain_atom(rule.body[1])))
       return CDL_OK;
     // a head relation already marked for an exact redo gains nothing more now
-    if (!force_exact && rels[rule.head.rel]->fresh_overflow) return CDL_OK;
+    if (!force_exact && (rels[rule.head.rel]->fresh_overflow || rels[rule.head.rel]->set_redo))
+      return CDL_OK;
     const size_t nb = rule.body.size();
     if (first_round) {
       if (nb == 1) return eval_copy(rule, kFull);
@@ -2447,6 +2546,40 @@ struct cdl_engine {
     return CDL_OK;
   }
 
+  // The round's words of the control block: with relations kept as sets, up
+  // to their delta sizes and their one-pass joins' sizes (a few KB).
+  cdl_status fetch_round() {
+    const uint32_t nr = (uint32_t)rels.size();
+    bool sets = false;
+    for (auto& r : rels) sets |= r->set_on;
+    const uint32_t end = sets ? kSlotSetTotal + (uint32_t)set_steps.size() : kSlotCursor + nr;
+    delta_known = sets;
+    return fetch(kSlotRoundOverflow, end - kSlotRoundOverflow);
+  }
+
+  // One-pass joins after the round's read-back: their sizes, and the
+  // relations that lacked room (to be redone).
+  cdl_status set_results(std::vector<bool>& redo, bool& any) {
+    std::map<uint32_t, uint64_t> outputs;
+    for (size_t i = 0; i < set_steps.size(); ++i) {
+      const SetStep& t = set_steps[i];
+      const uint64_t total = h_ctl[kSlotSetTotal + i];
+      if (total & kSetListFull) redo[t.head] = any = true;
+      set_seen[t.key] = SetSeen{t.probe, total & (kSetListFull - 1)};
+      prev_out[t.key] = total & (kSetListFull - 1);
+      outputs[t.head] += total & (kSetListFull - 1);
+    }
+    for (uint32_t i = 0; i < rels.size(); ++i) {
+      Relation& R = *rels[i];
+      if (!R.set_on) continue;
+      if (!R.set_free && outputs[i] > 0xFFFFFFFFull)
+        return fail(CDL_E_CAPACITY, "relation " + R.name + " would receive more than 2^32 new "
+                                    "tuples in one round");
+      if (R.set_redo || (R.set_single && h_ctl[kSlotDelta + i] > R.sdelta.cap)) redo[i] = any = true;
+    }
+    return CDL_OK;
+  }
+
   // Every rule once; then the cursors (and the deferred joins' sizes) are
   // read back.  A relation whose predicted joins claimed past its buffer has
   // only appended to that buffer: its rules run again, exact, from an empty
@@ -2457,9 +2590,10 @@ struct cdl_engine {
     force_exact = false;
     est_slot.clear();
     est_nb = 0;
-    cudaError_t e = cudaMemsetAsync(dslot(kSlotCursor), 0, 8 * nr, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dslot(kSlotDelta), 0, 8 * nr, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dslot(kSlotRoundOverflow), 0, 8, st);
+    // the round's overflow word, cursors, delta sizes and set joins' sizes
+    cudaError_t e = cudaMemsetAsync(dslot(kSlotRoundOverflow), 0, 8 * (kCtlSlots - kSlotRoundOverflow), st);
+    set_steps.clear();
+    delta_known = false;
     if (e == cudaSuccess && est_ready()) e = cudaMemsetAsync(join_sizes.p, 0, 8 * kMaxDeferred, st);
     if (e != cudaSuccess) return cuda_fail(e, "round reset");
     for (auto& r : rels) {
@@ -2467,6 +2601,7 @@ struct cdl_engine {
       r->fresh_overflow = false;
       r->dense_ub = 0;
       r->sdelta_ub = 0;
+      r->set_single = r->set_redo = false;
     }
     if (est_ready() && est_bio.p) {  // the round's predictions, with one wait
       est_plan = true;
@@ -2493,13 +2628,17 @@ struct cdl_engine {
       cdl_status s = eval_rule(rule, round == 1);
       if (s != CDL_OK) return s;
     }
-    cdl_status s = fetch(kSlotRoundOverflow, kSlotCursor + nr - kSlotRoundOverflow);
+    cdl_status s = fetch_round();
     if (s != CDL_OK) return s;
     note_cursors();
     std::vector<bool> redo(nr, false);
     bool any = false;
     for (uint32_t i = 0; i < nr; ++i)
       if (rels[i]->fresh_overflow) redo[i] = any = true;
+    if (!set_steps.empty()) {
+      s = set_results(redo, any);
+      if (s != CDL_OK) return s;
+    }
     if (!deferred.empty()) {  // exact sizes of the predicted joins
       std::vector<uint64_t> sz(deferred.size());
       e = cudaMemcpyAsync(sz.data(), join_sizes.p, 8 * sz.size(), cudaMemcpyDeviceToHost, st);
@@ -2517,12 +2656,21 @@ struct cdl_engine {
     if (!any) return CDL_OK;
     force_exact = true;
     // each overrun widens this run's later predictions by half a step (x 1.41)
-    est_boost = std::min(4.0, est_boost + 0.5);
+    if (est_ready()) est_boost = std::min(4.0, est_boost + 0.5);
     for (uint32_t i = 0; i < nr; ++i)
       if (redo[i]) {
-        ++est_over;
+        est_over += rels[i]->set_on ? 0 : 1;
         rels[i]->fresh_ub = 0;
         rels[i]->fresh_overflow = false;
+        if (rels[i]->set_on) {  // the rows that found room stay; the exact joins go on behind them
+          Relation& S = *rels[i];
+          const uint64_t at = std::min<uint64_t>(h_ctl[kSlotDelta + i], S.sdelta.cap);
+          h_ctl[kSlotDelta + i] = S.sdelta_ub = at;
+          S.set_single = S.set_redo = false;
+          e = cudaMemcpyAsync(dslot(kSlotDelta + i), h_ctl + kSlotDelta + i, 8,
+                              cudaMemcpyHostToDevice, st);
+          if (e != cudaSuccess) return cuda_fail(e, "delta reset");
+        }
         e = cudaMemsetAsync(dslot(kSlotCursor + i), 0, 8, st);
         if (e != cudaSuccess) return cuda_fail(e, "cursor reset");
       }
@@ -2532,7 +2680,7 @@ struct cdl_engine {
       if (s != CDL_OK) return s;
     }
     force_exact = false;
-    s = fetch(kSlotRoundOverflow, kSlotCursor + nr - kSlotRoundOverflow);
+    s = fetch_round();
     if (s != CDL_OK) return s;
     for (uint32_t i = 0; i < nr; ++i)
       if (redo[i] && h_ctl[kSlotCursor + i] > rels[i]->fresh.cap)
@@ -3087,7 +3235,9 @@ struct cdl_engine {
         merged[i] = 1;
       }
       if (status != CDL_OK) break;
-      status = fetch(kSlotDelta, nr);
+      for (uint32_t i = 0; i < nr; ++i)  // a merge's delta size is read now
+        if (merged[i] && !rels[i]->set_on) delta_known = false;
+      if (!delta_known) status = fetch(kSlotDelta, nr);
       if (status != CDL_OK) break;
       uint64_t new_total = 0;
       for (uint32_t i = 0; i < nr; ++i) {

@@ -890,6 +890,220 @@ cudaError_t join_direct(Ctx& c, const JoinSpec& j, ColsOut out, uint64_t* d_curs
   return cudaGetLastError();
 }
 
+// ------------------------------------------------ single pass into a set
+// Where Full is a bitmap a join needs no place computed for its outputs: the
+// new ones are packed as they come.  So no count and no scan run; a block
+// takes a tile of probe rows (eight per thread; fewer where that leaves
+// blocks idle), looks them up, scans their output counts in shared memory
+// and walks the outputs in windows of eight per thread as k_join_write does.
+// Rows with more than kHeavyChunk outputs are listed and taken in chunks by
+// a second kernel, so that one hot key does not hold one block.
+// Bound by the random accesses to the bitmap.  Same generation on 200,000
+// nodes: 25 ms of counts and scans and 66 of writes become 77 ms; a round of a
+// small closure takes one launch and one wait (4,001 nodes, 46 rounds: 4.9 ->
+// 2.9 ms).
+constexpr int kSJT = 256, kSJI = 8;
+constexpr uint32_t kSJTile = kSJT * kSJI;
+
+template <bool FILTER>
+__device__ __forceinline__ uint64_t set_tuple(const JoinSpec& j, const ColsIn& probe,
+                                              const DenseSet& d, uint64_t row, uint64_t b1,
+                                              uint64_t b2, bool& bad) {
+  uint32_t v[kMaxK] = {0, 0, 0, 0};
+#pragma unroll
+  for (int k = 0; k < kMaxK; ++k)
+    if (k < (int)j.out_k) v[k] = ref_value(j, probe, j.out[k], row, b1, b2);
+  if (FILTER) {
+    bool keep = true;
+    for (uint32_t q = 0; q < j.n_eq; ++q)
+      keep &= ref_value(j, probe, j.eq[q][0], row, b1, b2) ==
+              ref_value(j, probe, j.eq[q][1], row, b1, b2);
+    for (uint32_t q = 0; q < j.n_neq; ++q)
+      keep &= ref_value(j, probe, j.neq[q][0], row, b1, b2) !=
+              ref_value(j, probe, j.neq[q][1], row, b1, b2);
+    if (!keep) return kNoTuple;
+  }
+  const uint64_t idx = set_pack(d, v);
+  bad |= idx == kNoTuple;
+  return idx;
+}
+
+template <bool FILTER, bool STAR>
+__global__ void __launch_bounds__(kSJT, 4) k_join_set(const JoinSpec j, const DenseSet d, ColsOut out,
+                                                      unsigned long long* cursor, uint64_t cap,
+                                                      unsigned long long* total, uint32_t* err,
+                                                      uint32_t per, HeavyList heavy) {
+  // row q of thread t is slot 8 t + q; slots lie in the order of their outputs
+  __shared__ uint32_t s_off[kSJTile], s_start[kSJTile];
+  __shared__ uint32_t s_start2[STAR ? kSJTile : 1], s_cnt2[STAR ? kSJTile : 1];
+  __shared__ uint16_t s_slot[kSJTile];
+  __shared__ __align__(8) uint32_t red[kSJT / 32 + 2];
+  const uint64_t n = dev_size(j.dn, j.n_probe);
+  const ColsIn probe = probe_cols(j);
+  const uint32_t range = direct_range(j.ix), t = threadIdx.x;
+  const uint32_t rows = kSJT * per;
+  for (uint64_t base = (uint64_t)blockIdx.x * rows; base < n; base += (uint64_t)gridDim.x * rows) {
+    uint32_t cnt[kSJI], st[kSJI];
+#pragma unroll
+    for (int q = 0; q < kSJI; ++q) {
+      const uint64_t row = base + (uint64_t)q * kSJT + t;
+      cnt[q] = st[q] = 0;
+      if (q < (int)per && row < n) cnt[q] = lookup(j, probe, range, row, &st[q]);
+    }
+    uint32_t sum = 0;
+#pragma unroll
+    for (int q = 0; q < kSJI; ++q) {
+      const uint64_t row = base + (uint64_t)q * kSJT + t;
+      uint64_t c = cnt[q];
+      if constexpr (STAR) {
+        uint32_t st2 = 0, c2 = 0;
+        if (c) c2 = lookup2(j, probe, row, &st2);
+        s_start2[t * kSJI + q] = st2;
+        s_cnt2[t * kSJI + q] = c2;
+        c *= c2;
+        if (c > 0xFFFFFFFFull) {
+          if (err) atomicOr(err, kErrCapacity);
+          c = 0;
+        }
+      }
+      s_start[t * kSJI + q] = st[q];
+      if (c > kHeavyChunk) {
+        atomicAdd(total, (unsigned long long)c);
+        const uint32_t nch = (uint32_t)((c + kHeavyChunk - 1) / kHeavyChunk);
+        const uint64_t at = atomicAdd((unsigned long long*)heavy.n, (unsigned long long)nch);
+        for (uint32_t i = 0; i < nch && at + i < heavy.cap; ++i) {
+          HeavyChunk h;
+          h.prow = row;
+          h.out0 = (uint64_t)i * kHeavyChunk;  // first output of the row
+          h.brow = 0;
+          h.len = i + 1 < nch ? kHeavyChunk : (uint32_t)(c - (uint64_t)i * kHeavyChunk);
+          heavy.e[at + i] = h;
+        }
+        if (at + nch > heavy.cap) atomicOr(total, (unsigned long long)kSetListFull);
+        c = 0;
+      }
+      s_off[t * kSJI + q] = sum;
+      sum += (uint32_t)c;
+    }
+    uint32_t tot;
+    const uint32_t ex = block_exclusive_sum<kSJT, uint32_t>(sum, red, &tot);
+#pragma unroll
+    for (int q = 0; q < kSJI; ++q) s_off[t * kSJI + q] += ex;
+    if (t == 0 && tot) atomicAdd(total, (unsigned long long)tot);
+    __syncthreads();
+    for (uint32_t w = 0; w < tot; w += kSJTile) {
+      // every output takes the last slot that starts at or before it among
+      // those with outputs: marks at their first outputs, then a max-scan
+#pragma unroll
+      for (int q = 0; q < kSJI; ++q) s_slot[q * kSJT + t] = 0;
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < kSJI; ++q) {
+        const uint32_t sl = t * kSJI + q, a = s_off[sl];
+        const uint32_t b = sl + 1 < kSJTile ? s_off[sl + 1] : tot;
+        const uint32_t first = a > w ? a : w;
+        if (b > first && first - w < kSJTile) s_slot[first - w] = (uint16_t)sl;
+      }
+      __syncthreads();
+      uint32_t m = 0, loc[kSJI];
+#pragma unroll
+      for (int q = 0; q < kSJI; ++q) {
+        loc[q] = s_slot[t * kSJI + q];
+        m = loc[q] > m ? loc[q] : m;
+      }
+      uint32_t run = block_exclusive_max<kSJT>(m, red);
+#pragma unroll
+      for (int q = 0; q < kSJI; ++q) {
+        run = loc[q] > run ? loc[q] : run;
+        s_slot[t * kSJI + q] = (uint16_t)run;
+      }
+      __syncthreads();
+      uint64_t idx[kSJI];
+      bool bad = false;
+#pragma unroll
+      for (int q = 0; q < kSJI; ++q) {
+        const uint32_t o = w + q * kSJT + t;
+        idx[q] = kNoTuple;
+        if (o < tot) {
+          const uint32_t sl = s_slot[q * kSJT + t], l = o - s_off[sl];
+          const uint64_t row = base + (uint64_t)(sl % kSJI) * kSJT + sl / kSJI;
+          if constexpr (STAR) {
+            const uint32_t c2 = s_cnt2[sl], l1 = l / c2;
+            idx[q] = set_tuple<FILTER>(j, probe, d, row, (uint64_t)s_start[sl] + l1,
+                                       (uint64_t)s_start2[sl] + (l - l1 * c2), bad);
+          } else {
+            idx[q] = set_tuple<FILTER>(j, probe, d, row, (uint64_t)s_start[sl] + l, 0, bad);
+          }
+        }
+      }
+      if (bad && err) atomicOr(err, kErrCapacity);
+      const uint32_t fresh = set_add<kSJI>(d, idx);
+      set_emit<kSJT, kSJI, true>(d, idx, fresh, out, 0, cursor, cap, red);
+      __syncthreads();  // the next window rewrites s_slot and red
+    }
+    __syncthreads();  // the next tile rewrites the slots
+  }
+}
+
+// The listed chunks, one block at a time (their number from device memory).
+template <bool FILTER, bool STAR>
+__global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, const DenseSet d,
+                                                            ColsOut out, unsigned long long* cursor,
+                                                            uint64_t cap, uint32_t* err,
+                                                            HeavyList heavy) {
+  static_assert(kHeavyChunk <= kSJTile, "a chunk is one window");
+  __shared__ __align__(8) uint32_t red[kSJT / 32 + 2];
+  const ColsIn probe = probe_cols(j);
+  const uint32_t range = direct_range(j.ix);
+  const uint64_t n = *heavy.n < heavy.cap ? *heavy.n : heavy.cap;
+  for (uint64_t b = blockIdx.x; b < n; b += gridDim.x) {
+    const HeavyChunk h = heavy.e[b];
+    uint32_t st = 0, st2 = 0, c2 = 1;
+    lookup(j, probe, range, h.prow, &st);
+    if constexpr (STAR) c2 = lookup2(j, probe, h.prow, &st2);
+    uint64_t idx[kSJI];
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < kSJI; ++q) {
+      const uint32_t o = q * kSJT + threadIdx.x;
+      idx[q] = kNoTuple;
+      if (o < h.len && c2) {
+        const uint32_t l = (uint32_t)h.out0 + o, l1 = STAR ? l / c2 : l;
+        idx[q] = set_tuple<FILTER>(j, probe, d, h.prow, (uint64_t)st + l1,
+                                   (uint64_t)st2 + (l - l1 * c2), bad);
+      }
+    }
+    if (bad && err) atomicOr(err, kErrCapacity);
+    const uint32_t fresh = set_add<kSJI>(d, idx);
+    set_emit<kSJT, kSJI, true>(d, idx, fresh, out, 0, cursor, cap, red);
+    __syncthreads();  // the next chunk reuses red
+  }
+}
+
+cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, uint64_t* d_cursor,
+                     uint64_t out_cap, uint64_t* d_total, const HeavyList& heavy) {
+  if (j.n_probe == 0) return cudaSuccess;
+  const bool filter = j.n_neq > 0 || j.n_eq > 0;
+  // rows per thread: eight once four blocks per SM are busy, else fewer
+  uint64_t per = j.n_probe / ((uint64_t)kSJT * 152 * 4);
+  per = per < 1 ? 1 : per > (uint64_t)kSJI ? (uint64_t)kSJI : per;
+  const unsigned grid = dev_grid((j.n_probe + kSJT * per - 1) / (kSJT * per), j.dn);
+  ProfScope p(c, kJoinWrite, ((j.star ? 48.0 : 24.0) + 4.0 * j.out_k) * j.n_probe);
+  auto* cur = reinterpret_cast<unsigned long long*>(d_cursor);
+  auto* tot = reinterpret_cast<unsigned long long*>(d_total);
+  auto launch = [&](auto rows, auto chunks) {
+    rows<<<grid, kSJT, 0, c.st>>>(j, d, out, cur, out_cap, tot, c.d_err, (uint32_t)per, heavy);
+    chunks<<<152, kSJT, 0, c.st>>>(j, d, out, cur, out_cap, c.d_err, heavy);
+  };
+  if (j.star)
+    filter ? launch(k_join_set<true, true>, k_join_set_heavy<true, true>)
+           : launch(k_join_set<false, true>, k_join_set_heavy<false, true>);
+  else
+    filter ? launch(k_join_set<true, false>, k_join_set_heavy<true, false>)
+           : launch(k_join_set<false, false>, k_join_set_heavy<false, false>);
+  return cudaGetLastError();
+}
+
 size_t join_write_workspace(uint64_t n_probe, uint64_t total) {
   const uint64_t blocks = (n_probe + total + kJTile - 1) / kJTile;
   return ((blocks + 1) * 8 + 255) & ~uint64_t(255);

@@ -192,6 +192,18 @@ cudaError_t join_write(Ctx& c, const JoinSpec& j, const uint64_t* d_off, uint64_
 // dense->append the outputs whose bits were clear are also written, packed
 // at *d_cursor in no order, at most out_cap rows.)
 
+// Single-pass join into Full's bitmap (d.append; no count, no scan): the new
+// tuples go to out, packed at *d_cursor.  A tuple that finds no room below
+// out_cap has its bit cleared again and *d_cursor left past out_cap: the
+// caller makes room, sets the cursor to out_cap (that many rows are there)
+// and joins again.  *d_total grows by the join's size, with kSetListFull set in
+// it when the list of long ranges (heavy, as join_direct's, its counter
+// zeroed by the caller) was too short: then too the join runs again.
+struct HeavyList;
+constexpr uint64_t kSetListFull = 1ull << 62;
+cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, uint64_t* d_cursor,
+                     uint64_t out_cap, uint64_t* d_total, const HeavyList& heavy);
+
 // -------------------------------------------------------------- dense sets
 // Bits of n rows set in d (a row outside d raises kErrCapacity).
 cudaError_t dense_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n);
