@@ -36,6 +36,18 @@ __global__ void __launch_bounds__(256) k_dense_insert(DenseSet d, ColsIn rows, u
   }
 }
 
+__global__ void __launch_bounds__(256) k_dense_remove(DenseSet d, ColsIn rows, uint64_t n) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    uint32_t v[kMaxK] = {0, 0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < kMaxK; ++k)
+      if (k < (int)d.k) v[k] = __ldg(rows.c[k] + i);
+    const uint64_t idx = set_pack(d, v);
+    if (idx != kNoTuple) atomicAnd(d.words + (idx >> 5), ~(1u << (idx & 31)));
+  }
+}
+
 // Rows appended to Full's bitmap: the new ones (their bit was clear) go out
 // packed at *cursor.
 constexpr int kAT = 256, kAItems = 4;
@@ -158,6 +170,15 @@ cudaError_t dense_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n) {
   uint64_t blocks = (n + 255) / 256;
   if (blocks > 152 * 16) blocks = 152 * 16;
   k_dense_insert<<<(unsigned)blocks, 256, 0, c.st>>>(d, rows, n, c.d_err);
+  return cudaGetLastError();
+}
+
+cudaError_t dense_remove(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n) {
+  if (n == 0) return cudaSuccess;
+  ProfScope p(c, kDense, 4.0 * d.k * n);
+  uint64_t blocks = (n + 255) / 256;
+  if (blocks > 152 * 16) blocks = 152 * 16;
+  k_dense_remove<<<(unsigned)blocks, 256, 0, c.st>>>(d, rows, n);
   return cudaGetLastError();
 }
 

@@ -529,6 +529,7 @@ struct cdl_engine {
     DBuf sort_ws, merge_ws;
     RadixPlan plan;
     bool sorted_in_alt = false;
+    bool set = false;  // Full is the relation's bitmap
     uint64_t Fcap = 0, Ucap = 0;
   };
   struct GStepRes {
@@ -820,7 +821,7 @@ struct cdl_engine {
       R.host_full = opt.host_full > 0 && R.idb && !full_read[i] && !opt.n_instances && !R.dsm.on;
       // Full as a set leaves deltas in no order; the estimator's features are
       // stride samples of sorted ones
-      R.set_ok = opt.dense_bits >= 0 && !opt.graph && !opt.estimator && R.idb && !full_read[i] &&
+      R.set_ok = opt.dense_bits >= 0 && !opt.estimator && R.idb && !full_read[i] &&
                  !opt.n_instances && !R.dsm.on && !R.host_full;
     }
   }
@@ -877,7 +878,8 @@ struct cdl_engine {
   // limit, no more than Full's rows take (the row form holds Full twice).
   cdl_status set_switch(Relation& R) {
     DenseSet space;
-    if (!R.set_ok || R.set_on || R.dset.words || !tuple_space(R, kSetBits, space)) return CDL_OK;
+    if (!R.set_ok || R.set_on || R.dset.words || opt.graph || !tuple_space(R, kSetBits, space))
+      return CDL_OK;
     const uint64_t bytes = space.nbits >> 3;
     if (R.merged_bytes < kSetSwitch * (double)bytes) return CDL_OK;
     if (opt.mem_limit) {
@@ -2037,6 +2039,16 @@ struct cdl_engine {
     return CDL_OK;
   }
 
+  bool set_heavy_list() {
+    if (set_heavy_buf.p) return true;
+    set_heavy_buf = alloc(256 + sizeof(HeavyChunk) * kSetHeavyCap);
+    if (!set_heavy_buf.p) return false;
+    set_heavy.n = static_cast<uint64_t*>(set_heavy_buf.p);
+    set_heavy.e = reinterpret_cast<HeavyChunk*>(static_cast<char*>(set_heavy_buf.p) + 256);
+    set_heavy.cap = kSetHeavyCap;
+    return true;
+  }
+
   // A join into Full as a set in one pass, into a buffer sized by the step's
   // last join; done = false leaves it to the exact form.
   cdl_status set_join(const RuleR& rule, const JoinSpec& js, uint64_t np,
@@ -2059,13 +2071,7 @@ struct cdl_engine {
     done = true;
     if (H.set_redo) return CDL_OK;
     const uint32_t slot = kSlotSetTotal + (uint32_t)set_steps.size();
-    if (!set_heavy_buf.p) {
-      set_heavy_buf = alloc(256 + sizeof(HeavyChunk) * kSetHeavyCap);
-      if (!set_heavy_buf.p) return fail(CDL_E_NOMEM, "long ranges");
-      set_heavy.n = static_cast<uint64_t*>(set_heavy_buf.p);
-      set_heavy.e = reinterpret_cast<HeavyChunk*>(static_cast<char*>(set_heavy_buf.p) + 256);
-      set_heavy.cap = kSetHeavyCap;
-    }
+    if (!set_heavy_list()) return fail(CDL_E_NOMEM, "long ranges");
     cudaError_t e = cudaMemsetAsync(set_heavy.n, 0, 8, st);
     if (e == cudaSuccess)
       e = join_set(ctx, js, H.fset, H.sdelta.out(), dslot(kSlotDelta + rule.head.rel), H.sdelta.cap,
@@ -2781,31 +2787,42 @@ struct cdl_engine {
       G.plan = make_radix_plan(R.arity, bits, wide ? 10 : digits_for(total_bits), 512);
       G.sorted_in_alt = G.plan.npass % 2 == 1;
       bool ok = true;
+      // (Full as a bitmap: the joins append to delta; no rows of Full, no
+      // sort, no merge)
+      G.set = R.set_on;
       for (int side = 0; side < 2; ++side) {
-        ok &= alloc_cols(G.F[side], R.arity, G.Fcap);
+        if (!G.set) ok &= alloc_cols(G.F[side], R.arity, G.Fcap);
         ok &= alloc_cols(G.D[side], R.arity, G.Ucap);
       }
-      ok &= alloc_cols(G.fresh, R.arity, G.Ucap) && alloc_cols(G.alt, R.arity, G.Ucap);
-      G.sort_ws = alloc(radix_workspace(G.Ucap, G.plan.bits, G.plan.threads));
-      G.merge_ws = alloc(diff_merge_workspace(G.Fcap, G.Ucap));
-      if (!ok || !G.sort_ws.p || !G.merge_ws.p) return fail(CDL_E_NOMEM, "graph buffers");
-      if (R.full.n > G.Fcap || R.delta.n > G.Ucap) return fail(CDL_E_CAPACITY, "graph capacities");
+      if (G.set) {
+        ok &= set_heavy_list();
+      } else {
+        ok &= alloc_cols(G.fresh, R.arity, G.Ucap) && alloc_cols(G.alt, R.arity, G.Ucap);
+        G.sort_ws = alloc(radix_workspace(G.Ucap, G.plan.bits, G.plan.threads));
+        G.merge_ws = alloc(diff_merge_workspace(G.Fcap, G.Ucap));
+        ok &= G.sort_ws.p && G.merge_ws.p;
+      }
+      if (!ok) return fail(CDL_E_NOMEM, "graph buffers");
+      if ((!G.set && R.full.n > G.Fcap) || R.delta.n > G.Ucap)
+        return fail(CDL_E_CAPACITY, "graph capacities");
       for (uint32_t k = 0; k < R.arity; ++k) {
         cudaError_t e = cudaSuccess;
-        if (R.full.n)
+        if (R.full.n && !G.set)
           e = cudaMemcpyAsync(G.F[0].c[k], R.full.c[k], 4 * R.full.n, cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess && R.delta.n)
           e = cudaMemcpyAsync(G.D[0].c[k], R.delta.c[k], 4 * R.delta.n, cudaMemcpyDeviceToDevice, st);
         if (e != cudaSuccess) return cuda_fail(e, "graph state copy");
       }
-      cur[j] = GraphRel{G.F[0].in(), G.D[0].in(), R.full.n, R.delta.n};
-      next[j] = GraphRel{G.F[1].in(), G.D[1].in(), 0, 0};
+      const uint64_t set_cap = G.set ? G.Ucap : 0;
+      cur[j] = GraphRel{G.F[0].in(), G.D[0].in(), R.full.n, R.delta.n, set_cap};
+      next[j] = GraphRel{G.F[1].in(), G.D[1].in(), 0, 0, set_cap};
     }
     for (size_t s = 0; s < grec.size(); ++s) {
       const GStep& g = grec[s];
       GStepRes& S = gstep[s];
       S.pcap = g.t == 1 ? gcap_u[g.probe_rel] : gstep[s - 1].ocap;
       S.ocap = g.last ? gcap_u[g.head] : gcap_i[s];
+      if (g.last && rels[g.head]->set_on) continue;  // one pass, no offsets
       S.off = alloc(8 * S.pcap);
       S.cws = alloc(join_count_workspace(S.pcap));
       S.wbytes = join_write_workspace(S.pcap, S.ocap);
@@ -2891,6 +2908,14 @@ struct cdl_engine {
         js.dn = g_step(s - 1, 2);
       }
       GRelRes* H = g.last ? &grel[slot[g.head]] : nullptr;
+      if (H && H->set) {
+        js.dout = reinterpret_cast<const ColsOut*>(&g_next()[slot[g.head]].D);
+        e = cudaMemsetAsync(set_heavy.n, 0, 8, st);
+        if (e == cudaSuccess)
+          e = join_set(ctx, js, rels[g.head]->fset, ColsOut{}, g_cursor(slot[g.head]), H->Ucap,
+                       g_step(s, 0), set_heavy);
+        continue;
+      }
       uint64_t* cursor = g.last ? g_cursor(slot[g.head]) : g_step(s, 2);
       const ColsOut out = g.last ? H->fresh.out() : S.inter.out();
       e = join_count_scan(ctx, js, static_cast<uint64_t*>(S.off.p), g_step(s, 0), S.cws.p);
@@ -2901,6 +2926,7 @@ struct cdl_engine {
     }
     for (size_t j = 0; j < grel.size() && e == cudaSuccess; ++j) {
       GRelRes& G = grel[j];
+      if (G.set) continue;  // the joins left its new tuples
       const Relation& R = *rels[G.rel];
       bool in_b = false;
       e = radix_sort(ctx, G.plan, G.fresh.out(), G.alt.out(), G.Ucap, G.sort_ws.p, &in_b,
@@ -3069,10 +3095,23 @@ struct cdl_engine {
     for (size_t j = 0; j < grel.size(); ++j) {
       GRelRes& G = grel[j];
       Relation& R = *rels[G.rel];
-      const int side = cur[j].F.c[0] == G.F[0].c[0] ? 0 : 1;
-      R.full = std::move(G.F[side]);
-      R.full.n = cur[j].nF;
-      R.delta = std::move(G.D[side]);
+      // (retirement moves Full between the two sides on its own)
+      const int dside = cur[j].D.c[0] == G.D[0].c[0] ? 0 : 1;
+      if (G.set) {
+        if (ctl.done == 2) {  // the unfinished round's tuples leave the bitmap again
+          uint64_t at = 0;
+          e = cudaMemcpy(&at, g_cursor(j), 8, cudaMemcpyDeviceToHost);
+          if (e == cudaSuccess)
+            e = dense_remove(ctx, R.fset, G.D[1 - dside].in(), std::min(at, G.Ucap));
+          if (e != cudaSuccess) return cuda_fail(e, "graph rounds");
+        }
+        R.full.n = cur[j].nF;
+        set_drop_rows(R);
+      } else {
+        R.full = std::move(G.F[cur[j].F.c[0] == G.F[0].c[0] ? 0 : 1]);
+        R.full.n = cur[j].nF;
+      }
+      R.delta = std::move(G.D[dside]);
       R.delta.n = cur[j].nD;
       R.version[kFull]++;
       R.version[kDelta]++;

@@ -14,13 +14,18 @@ __global__ void k_round_end(GraphRel* cur, GraphRel* next, uint32_t nrel, GraphC
                             cudaGraphConditionalHandle loop, uint64_t* cursors, uint32_t ncur,
                             uint64_t* steps, uint32_t nsteps) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  if (ctl->overflow) {  // cur holds the last complete round
+  bool overflow = ctl->overflow;
+  for (uint32_t s = 0; s < nsteps; ++s) overflow |= (steps[3 * s] & kSetListFull) != 0;
+  for (uint32_t r = 0; r < nrel; ++r)
+    overflow |= cur[r].set_cap && cursors[r] > cur[r].set_cap;
+  if (overflow) {  // cur holds the last complete round
     ctl->done = 2;
     cudaGraphSetConditional(loop, 0u);
     return;
   }
   uint64_t total = 0;
   for (uint32_t r = 0; r < nrel; ++r) {
+    if (cur[r].set_cap) next[r].nD = cursors[r];
     next[r].nF = cur[r].nF + next[r].nD;
     total += next[r].nD;
     const GraphRel t = cur[r];
@@ -35,7 +40,7 @@ __global__ void k_round_end(GraphRel* cur, GraphRel* next, uint32_t nrel, GraphC
   else if (ctl->max_iters && ctl->iterations > ctl->max_iters)
     ctl->done = 3;
   for (uint32_t i = 0; i < ncur; ++i) cursors[i] = 0;  // the next round appends from 0
-  for (uint32_t s = 0; s < nsteps; ++s) steps[3 * s + 2] = 0;
+  for (uint32_t s = 0; s < nsteps; ++s) steps[3 * s] = steps[3 * s + 2] = 0;
   cudaGraphSetConditional(loop, ctl->done ? 0u : 1u);
 }
 

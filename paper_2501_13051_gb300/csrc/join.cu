@@ -940,6 +940,7 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set(const JoinSpec j, const De
   __shared__ __align__(8) uint32_t red[kSJT / 32 + 2];
   const uint64_t n = dev_size(j.dn, j.n_probe);
   const ColsIn probe = probe_cols(j);
+  if (j.dout) out = *j.dout;  // (inside a captured round)
   const uint32_t range = direct_range(j.ix), t = threadIdx.x;
   const uint32_t rows = kSJT * per;
   for (uint64_t base = (uint64_t)blockIdx.x * rows; base < n; base += (uint64_t)gridDim.x * rows) {
@@ -1054,6 +1055,7 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, co
   static_assert(kHeavyChunk <= kSJTile, "a chunk is one window");
   __shared__ __align__(8) uint32_t red[kSJT / 32 + 2];
   const ColsIn probe = probe_cols(j);
+  if (j.dout) out = *j.dout;
   const uint32_t range = direct_range(j.ix);
   const uint64_t n = *heavy.n < heavy.cap ? *heavy.n : heavy.cap;
   for (uint64_t b = blockIdx.x; b < n; b += gridDim.x) {

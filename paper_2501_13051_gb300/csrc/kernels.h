@@ -136,6 +136,7 @@ struct JoinSpec {
   // memory (n_probe is then the capacity that sizes the grids); else null
   const ColsIn* dprobe;
   const uint64_t* dn;
+  const ColsOut* dout;  // (join_set) output columns in device memory; else null
   // star join: a second build side, also keyed on probe columns (qk0, qk1;
   // qk1 = 0xFF for one word).  A probe row then matches every pair of a row
   // of its first range and a row of its second (count c1 * c2), the join of
@@ -211,6 +212,8 @@ cudaError_t dense_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n);
 // (packed at *d_cursor, at most out_cap rows; more raise kErrCapacity).
 cudaError_t set_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n, ColsOut out,
                        uint64_t* d_cursor, uint64_t out_cap);
+// Clears the bits of n rows.
+cudaError_t dense_remove(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n);
 size_t dense_extract_workspace(uint64_t nbits);
 // The set bits of d as rows in increasing bit order (lexicographic, no
 // repeats) into out (cap rows; more raise kErrCapacity); their number in
@@ -369,6 +372,7 @@ cudaError_t mark_instances(Ctx& c, const uint32_t* inst, uint64_t n, uint32_t n_
 struct GraphRel {
   ColsIn F, D;
   uint64_t nF, nD;
+  uint64_t set_cap;  // Full is a bitmap: rows D holds (F is unused); else 0
 };
 struct GraphCtl {
   uint64_t round;       // rounds completed (all launches, numbered as the engine does)
@@ -382,8 +386,10 @@ struct GraphCtl {
 // loop stops (cur still holds the last complete round); else next.nF =
 // cur.nF + next.nD, per_round[round] = sum of next.nD, cur <-> next, and the
 // loop's condition is set to continue while the round derived something.
-// It also zeroes the next round's cursors: `ncur` words at `cursors` and
-// every third word from `steps` + 2, `nsteps` of them.
+// Where Full is a bitmap next.nD is the relation's cursor; a cursor past
+// set_cap, or kSetListFull in a step's first word, is an overflow as well.
+// It also zeroes the next round's cursors: `ncur` words at `cursors`, and of
+// the three words of each of the `nsteps` steps the first and the last.
 cudaError_t round_end(Ctx& c, GraphRel* cur, GraphRel* next, uint32_t nrel, GraphCtl* ctl,
                       uint64_t* per_round, uint64_t per_round_cap,
                       cudaGraphConditionalHandle loop, uint64_t* cursors, uint32_t ncur,
