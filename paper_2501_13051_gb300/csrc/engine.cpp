@@ -23,6 +23,7 @@
 #include <cstring>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <unordered_map>
@@ -193,6 +194,56 @@ class Pool {
         return;
       }
   }
+};
+
+// Pinned host blocks of an engine's control words, kept for the next engine:
+// pinning and unpinning take about 100 us each, as long as ten rounds of a
+// small fixpoint (create + close of an engine 430 -> 190 us).  At most
+// kKeep blocks wait; any device's engines share them (portable memory).
+class PinnedBlocks {
+ public:
+  static constexpr size_t kBytes = 32 << 10;
+  static PinnedBlocks& get() {
+    static PinnedBlocks p;
+    return p;
+  }
+  void* take() {
+    {
+      std::lock_guard<std::mutex> g(m_);
+      while (!free_.empty()) {
+        void* p = free_.back();
+        free_.pop_back();
+        cudaPointerAttributes a{};  // (gone if the program has reset the device since)
+        if (cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeHost) return p;
+        cudaGetLastError();
+      }
+    }
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, kBytes, cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return p;
+  }
+  // (no device work may still use p)
+  void give(void* p) {
+    {
+      std::lock_guard<std::mutex> g(m_);
+      if (free_.size() < kKeep) {
+        free_.push_back(p);
+        return;
+      }
+    }
+    cudaFreeHost(p);
+  }
+  ~PinnedBlocks() {
+    for (void* p : free_) cudaFreeHost(p);
+  }
+
+ private:
+  static constexpr size_t kKeep = 4;
+  std::mutex m_;
+  std::vector<void*> free_;
 };
 
 struct DBuf {
@@ -392,6 +443,8 @@ constexpr uint32_t kSlotErr = 0, kSlotScratch = 1, kSlotAux = 2, kSlotDirTotal =
                    kSetSteps = 256, kSlotSetTotal = 8 + 2 * kMaxRels,
                    kCtlSlots = 8 + 2 * kMaxRels + kSetSteps;
 constexpr int kEstFloats = 32;  // 16 features, the prediction, padding
+static_assert(kCtlSlots * sizeof(uint64_t) + kEstFloats * sizeof(float) <= PinnedBlocks::kBytes,
+              "the host mirrors share one block");
 
 }  // namespace
 
@@ -651,8 +704,7 @@ struct cdl_engine {
     ctl.reset();
     pool.release_all();
     hpool.release_all();
-    if (h_ctl) cudaFreeHost(h_ctl);
-    if (h_est) cudaFreeHost(h_est);
+    if (h_ctl) PinnedBlocks::get().give(h_ctl);
     if (h_batch) cudaFreeHost(h_batch);
   }
 
@@ -3743,11 +3795,9 @@ cdl_status cdl_create(const cdl_options* opts, cdl_engine** out) {
   e->ctl = e->alloc(kCtlSlots * sizeof(uint64_t));
   e->est_io = e->alloc(kEstFloats * sizeof(float));
   if (!e->ctl.p || !e->est_io.p) return CDL_E_NOMEM;
-  if (cudaMallocHost(&e->h_ctl, kCtlSlots * sizeof(uint64_t)) != cudaSuccess ||
-      cudaMallocHost(&e->h_est, kEstFloats * sizeof(float)) != cudaSuccess) {
-    cudaGetLastError();
-    return CDL_E_CUDA;
-  }
+  e->h_ctl = static_cast<uint64_t*>(PinnedBlocks::get().take());
+  if (!e->h_ctl) return CDL_E_CUDA;
+  e->h_est = reinterpret_cast<float*>(e->h_ctl + kCtlSlots);
   if (cudaMemsetAsync(e->ctl.p, 0, kCtlSlots * sizeof(uint64_t), e->st) != cudaSuccess)
     return CDL_E_CUDA;
   e->ctx.st = e->st;
