@@ -207,7 +207,14 @@ struct DenseSet {
   uint32_t append;
   uint32_t shift[kMaxK];
   uint32_t mask[kMaxK];  // 2^bits_k - 1
+  // Hash form, for Full in tuple spaces too large for a bitmap (at most 2^62
+  // tuples): open addressing over the packed tuples, words unused.
+  unsigned long long* keys;  // kmask + 1 slots (a power of two), or null
+  uint64_t kmask;
 };
+constexpr unsigned long long kSetEmpty = ~0ull;     // a free slot
+constexpr unsigned long long kSetGone = ~0ull - 1;  // a tuple taken out again
+constexpr uint32_t kSetProbes = 4096;  // slots looked at before the table counts as full
 
 // Position of tuple v in the packed tuple space of d; kNoTuple when v lies
 // outside it.
@@ -245,6 +252,68 @@ __device__ __forceinline__ uint32_t set_add(const DenseSet& d, const uint64_t (&
 #pragma unroll
   for (int q = 0; q < N; ++q) fresh |= (seen[q] ^ 1u) << q;
   return fresh;
+}
+
+// 64-bit finaliser of SplitMix64 (Steele, Lea & Flood, 2014).
+__device__ __forceinline__ uint64_t mix64(uint64_t k) {
+  k = (k ^ (k >> 30)) * 0xbf58476d1ce4e5b9ull;
+  k = (k ^ (k >> 27)) * 0x94d049bb133111ebull;
+  return k ^ (k >> 31);
+}
+
+// set_add for the hash form.  A slot goes from empty to one key (to gone)
+// and never to another, so a key seen by a plain read is there.  Where no
+// free slot turns up *full is set and the tuple is left out.
+template <int N>
+__device__ __forceinline__ uint32_t set_add_hash(const DenseSet& d, const uint64_t (&key)[N],
+                                                 bool* full) {
+  unsigned long long v[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    v[q] = key[q] != kNoTuple ? d.keys[mix64(key[q]) & d.kmask] : kNoTuple;
+  uint32_t fresh = 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if (key[q] != kNoTuple && v[q] == kSetEmpty) {
+      v[q] = atomicCAS(d.keys + (mix64(key[q]) & d.kmask), kSetEmpty, key[q]);
+      if (v[q] == kSetEmpty) {
+        fresh |= 1u << q;
+        v[q] = key[q];
+      }
+    }
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if (key[q] != kNoTuple && v[q] != key[q]) {
+      uint64_t at = mix64(key[q]) & d.kmask;
+      bool done = false;
+      for (uint32_t step = 1; step < kSetProbes && !done; ++step) {
+        at = (at + 1) & d.kmask;
+        unsigned long long x = d.keys[at];
+        if (x == kSetEmpty) {
+          x = atomicCAS(d.keys + at, kSetEmpty, key[q]);
+          if (x == kSetEmpty) fresh |= 1u << q;
+        }
+        done = x == kSetEmpty || x == key[q];
+      }
+      if (!done) *full = true;
+    }
+  return fresh;
+}
+
+// Takes a tuple that is in the set out again.
+__device__ __forceinline__ void set_remove(const DenseSet& d, uint64_t idx) {
+  if (!d.keys) {
+    atomicAnd(d.words + (idx >> 5), ~(1u << (idx & 31)));
+    return;
+  }
+  uint64_t at = mix64(idx) & d.kmask;
+  for (uint32_t step = 0; step < kSetProbes; ++step) {
+    if (d.keys[at] == idx) {
+      d.keys[at] = kSetGone;
+      return;
+    }
+    at = (at + 1) & d.kmask;
+  }
 }
 
 // Writes a block's new tuples (bit q of fresh: tuple idx[q] is new) packed at
@@ -288,7 +357,7 @@ __device__ __forceinline__ bool set_emit(const DenseSet& d, const uint64_t (&idx
         for (int k = 0; k < kMaxK; ++k)
           if (k < (int)d.k) out.c[k][p] = set_column(d, idx[q], k);
       } else {
-        if (CLEAR) atomicAnd(d.words + (idx[q] >> 5), ~(1u << (idx[q] & 31)));
+        if (CLEAR) set_remove(d, idx[q]);
         ok = false;
       }
     }

@@ -44,13 +44,15 @@ __global__ void __launch_bounds__(256) k_dense_remove(DenseSet d, ColsIn rows, u
     for (int k = 0; k < kMaxK; ++k)
       if (k < (int)d.k) v[k] = __ldg(rows.c[k] + i);
     const uint64_t idx = set_pack(d, v);
-    if (idx != kNoTuple) atomicAnd(d.words + (idx >> 5), ~(1u << (idx & 31)));
+    if (idx != kNoTuple) set_remove(d, idx);
   }
 }
 
 // Rows appended to Full's bitmap: the new ones (their bit was clear) go out
 // packed at *cursor.
+// (HASH: Full's hash form; EMIT false: the rows only join the set.)
 constexpr int kAT = 256, kAItems = 4;
+template <bool HASH, bool EMIT>
 __global__ void __launch_bounds__(kAT) k_set_insert(DenseSet d, ColsIn rows, uint64_t n,
                                                     ColsOut out, unsigned long long* cursor,
                                                     uint64_t cap, uint32_t* err) {
@@ -72,10 +74,82 @@ __global__ void __launch_bounds__(kAT) k_set_insert(DenseSet d, ColsIn rows, uin
         bad |= idx[q] == kNoTuple;
       }
     }
-    const uint32_t fresh = set_add<kAItems>(d, idx);
-    bad |= !set_emit<kAT, kAItems>(d, idx, fresh, out, 0, cursor, cap, red);
+    uint32_t fresh;
+    if constexpr (HASH)
+      fresh = set_add_hash<kAItems>(d, idx, &bad);
+    else
+      fresh = set_add<kAItems>(d, idx);
+    if constexpr (EMIT) {
+      bad |= !set_emit<kAT, kAItems>(d, idx, fresh, out, 0, cursor, cap, red);
+      __syncthreads();  // the next tile reuses red
+    }
     if (bad && err) atomicOr(err, kErrCapacity);
-    __syncthreads();  // the next tile reuses red
+  }
+}
+
+// The keys of another table into d (a larger table takes over).
+__global__ void __launch_bounds__(kAT) k_hash_move(DenseSet d, const unsigned long long* old,
+                                                   uint64_t slots, uint32_t* err) {
+  constexpr uint64_t kTile = (uint64_t)kAT * kAItems;
+  for (uint64_t b = blockIdx.x * kTile; b < slots; b += gridDim.x * kTile) {
+    uint64_t idx[kAItems];
+#pragma unroll
+    for (int q = 0; q < kAItems; ++q) {
+      const uint64_t i = b + (uint64_t)q * kAT + threadIdx.x;
+      const unsigned long long v = i < slots ? old[i] : kSetEmpty;
+      idx[q] = v < kSetGone ? v : kNoTuple;
+    }
+    bool full = false;
+    set_add_hash<kAItems>(d, idx, &full);
+    if (full && err) atomicOr(err, kErrTable);
+  }
+}
+
+// The table's keys, packed in no order, as their high and low words.
+__global__ void __launch_bounds__(kAT) k_hash_keys(DenseSet d, uint32_t* __restrict__ hi,
+                                                   uint32_t* __restrict__ lo, uint64_t cap,
+                                                   unsigned long long* cursor, uint32_t* err) {
+  constexpr int kI = 8;
+  __shared__ uint32_t red[kAT / 32 + 1];
+  __shared__ unsigned long long s_at;
+  const uint64_t slots = d.kmask + 1;
+  for (uint64_t b = blockIdx.x * (uint64_t)kAT * kI; b < slots; b += gridDim.x * (uint64_t)kAT * kI) {
+    unsigned long long v[kI];
+    uint32_t n = 0;
+#pragma unroll
+    for (int q = 0; q < kI; ++q) {
+      const uint64_t i = b + (uint64_t)q * kAT + threadIdx.x;
+      v[q] = i < slots ? d.keys[i] : kSetEmpty;
+      n += v[q] < kSetGone ? 1u : 0u;
+    }
+    uint32_t tot;
+    const uint32_t ex = block_exclusive_sum<kAT, uint32_t>(n, red, &tot);
+    if (threadIdx.x == 0) s_at = tot ? atomicAdd(cursor, (unsigned long long)tot) : 0ull;
+    __syncthreads();
+    uint64_t at = s_at + ex;
+#pragma unroll
+    for (int q = 0; q < kI; ++q)
+      if (v[q] < kSetGone) {
+        if (at < cap) {
+          hi[at] = (uint32_t)(v[q] >> 32);
+          lo[at] = (uint32_t)v[q];
+        } else if (err) {
+          atomicOr(err, kErrCapacity);
+        }
+        ++at;
+      }
+    __syncthreads();  // the next tile rewrites s_at
+  }
+}
+
+__global__ void __launch_bounds__(256) k_hash_unpack(DenseSet d, const uint32_t* __restrict__ hi,
+                                                     const uint32_t* __restrict__ lo, uint64_t n,
+                                                     ColsOut out) {
+  for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) {
+    const uint64_t idx = ((uint64_t)__ldg(hi + i) << 32) | __ldg(lo + i);
+#pragma unroll
+    for (int k = 0; k < kMaxK; ++k)
+      if (k < (int)d.k) out.c[k][i] = set_column(d, idx, k);
   }
 }
 
@@ -167,6 +241,13 @@ __global__ void __launch_bounds__(kXT) k_dense_write(DenseSet d, uint64_t nw,
 cudaError_t dense_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n) {
   if (n == 0) return cudaSuccess;
   ProfScope p(c, kDense, 4.0 * d.k * n);
+  if (d.keys) {
+    uint64_t tiles = (n + kAT * kAItems - 1) / (kAT * kAItems);
+    if (tiles > 152 * 16) tiles = 152 * 16;
+    k_set_insert<true, false><<<(unsigned)tiles, kAT, 0, c.st>>>(d, rows, n, ColsOut{}, nullptr, 0,
+                                                                 c.d_err);
+    return cudaGetLastError();
+  }
   uint64_t blocks = (n + 255) / 256;
   if (blocks > 152 * 16) blocks = 152 * 16;
   k_dense_insert<<<(unsigned)blocks, 256, 0, c.st>>>(d, rows, n, c.d_err);
@@ -188,8 +269,41 @@ cudaError_t set_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n, ColsO
   ProfScope p(c, kDense, 4.0 * d.k * n);
   uint64_t blocks = (n + kAT * kAItems - 1) / (kAT * kAItems);
   if (blocks > 152 * 16) blocks = 152 * 16;
-  k_set_insert<<<(unsigned)blocks, kAT, 0, c.st>>>(
-      d, rows, n, out, reinterpret_cast<unsigned long long*>(d_cursor), out_cap, c.d_err);
+  auto* cur = reinterpret_cast<unsigned long long*>(d_cursor);
+  if (d.keys)
+    k_set_insert<true, true><<<(unsigned)blocks, kAT, 0, c.st>>>(d, rows, n, out, cur, out_cap, c.d_err);
+  else
+    k_set_insert<false, true><<<(unsigned)blocks, kAT, 0, c.st>>>(d, rows, n, out, cur, out_cap, c.d_err);
+  return cudaGetLastError();
+}
+
+cudaError_t hash_move(Ctx& c, const DenseSet& d, const unsigned long long* old, uint64_t slots) {
+  ProfScope p(c, kDense, 8.0 * slots);
+  uint64_t blocks = (slots + kAT * kAItems - 1) / (kAT * kAItems);
+  if (blocks > 152 * 16) blocks = 152 * 16;
+  k_hash_move<<<(unsigned)blocks, kAT, 0, c.st>>>(d, old, slots, c.d_err);
+  return cudaGetLastError();
+}
+
+cudaError_t hash_keys(Ctx& c, const DenseSet& d, uint32_t* hi, uint32_t* lo, uint64_t cap,
+                      uint64_t* d_count) {
+  ProfScope p(c, kDense, 8.0 * (d.kmask + 1));
+  cudaError_t e = cudaMemsetAsync(d_count, 0, 8, c.st);
+  if (e != cudaSuccess) return e;
+  uint64_t blocks = (d.kmask + 1 + 2047) / 2048;
+  if (blocks > 152 * 16) blocks = 152 * 16;
+  k_hash_keys<<<(unsigned)blocks, kAT, 0, c.st>>>(
+      d, hi, lo, cap, reinterpret_cast<unsigned long long*>(d_count), c.d_err);
+  return cudaGetLastError();
+}
+
+cudaError_t hash_unpack(Ctx& c, const DenseSet& d, const uint32_t* hi, const uint32_t* lo,
+                        uint64_t n, ColsOut out) {
+  if (n == 0) return cudaSuccess;
+  ProfScope p(c, kDense, (8.0 + 4.0 * d.k) * n);
+  uint64_t blocks = (n + 1023) / 1024;
+  if (blocks > 152 * 64) blocks = 152 * 64;
+  k_hash_unpack<<<(unsigned)blocks, 256, 0, c.st>>>(d, hi, lo, n, out);
   return cudaGetLastError();
 }
 

@@ -370,6 +370,7 @@ struct Relation {
   // nothing is sorted or merged, and Full's rows are taken out of the bitmap
   // in order when the run ends.  full.n is then |Full|, its columns unused.
   bool set_ok = false;   // no rule variant reads Full after round 1
+  bool hash_ok = false;  // the same in a batched run: Full may become a hash set
   bool set_on = false;   // Full is fset now
   bool set_free = false; // within dense_bits: a round's join outputs are not limited to 2^32
   DenseSet fset{};
@@ -514,6 +515,9 @@ struct cdl_engine {
   // 0.05; a fixpoint that ends soon after pays the bitmap's passes for
   // nothing, so not lower.
   static constexpr uint32_t kSetBits = 37;
+  static constexpr uint32_t kHashBits = 62;        // a packed tuple beside the two marks
+  static constexpr uint64_t kHashRows = 4 << 20;   // 48 MB of triples and their merged copy
+  bool hashed = false;  // batched run: the derived relations' Fulls are hash sets
   static constexpr double kSetSwitch = 0.2;
   // hub joins (hub_join): outputs in all, and per row of both sides, from
   // which they are tried (below, the second count and the other index are
@@ -600,7 +604,8 @@ struct cdl_engine {
   DBuf gret;
   uint64_t gret_room = 1;  // retired buffers start at this many times Full's capacity
   uint64_t g_retirements = 0;  // rounds whose converged rows the graph moved out of Full
-  bool graph_retires() const { return opt.n_instances && opt.retire >= 0; }
+  bool graph_retires() const { return opt.n_instances && opt.retire >= 0 && !hashed; }
+  uint64_t hash_room = 8;  // a hash set's table in the graph: so many times the rows there are
   RetireCtl* g_rctl() const { return static_cast<RetireCtl*>(gret.p); }
   RetireRel* g_rrel() const {
     return reinterpret_cast<RetireRel*>(static_cast<char*>(gret.p) + 256);
@@ -875,6 +880,8 @@ struct cdl_engine {
       // stride samples of sorted ones
       R.set_ok = opt.dense_bits >= 0 && !opt.estimator && R.idb && !full_read[i] &&
                  !opt.n_instances && !R.dsm.on && !R.host_full;
+      R.hash_ok = opt.dense_bits >= 0 && !opt.estimator && R.idb && !full_read[i] &&
+                  opt.n_instances && !opt.mem_limit && !tuner.mode;  // (a tuned run tunes its sorts)
     }
   }
 
@@ -913,6 +920,71 @@ struct cdl_engine {
     R.set_on = true;
     if (!keep_rows) set_drop_rows(R);
     return CDL_OK;
+  }
+
+  // Batched runs (tuple spaces far past any bitmap): Full of every derived
+  // relation as a hash set, once a first semi-naive round has left more rows
+  // than the caches hold.  The row form then sorts and merges all rows of all
+  // running instances every round (and moves converged instances' rows out of
+  // its way); the set takes every new tuple once, at random, and sorts all of
+  // them once at the end.  512 instances, 279M tuples, 233 captured rounds:
+  // 222 ms with rows, 97 with sets.
+  cdl_status hash_switch() {
+    uint64_t rows = 0, steps = 0;
+    for (const RuleR& rule : rules)
+      for (const AtomR& a : rule.body) steps += rels[a.rel]->idb;
+    if (2 * steps > kSetSteps) return CDL_OK;  // (a round run again doubles its joins)
+    for (auto& r : rels) {
+      DenseSet space;
+      if (!r->idb) continue;
+      if (!r->hash_ok || r->set_on || !tuple_space(*r, kHashBits, space)) return CDL_OK;
+      rows += r->full.n;
+    }
+    size_t free_b = 0, total_b = 0;
+    if (rows < kHashRows || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return CDL_OK;
+    if (hash_slots(8 * rows) * 8 > free_b / 4) return CDL_OK;
+    for (auto& r : rels) {
+      if (!r->idb) continue;
+      tuple_space(*r, kHashBits, r->fset);
+      r->fset.append = 1;
+      bool ok = false;
+      cdl_status s = hash_reserve(*r, 4 * r->full.n + 1024, false, ok);
+      if (s == CDL_OK && !ok) s = fail(CDL_E_NOMEM, "full set");
+      if (s != CDL_OK) return s;
+      cudaError_t e = dense_insert(ctx, r->fset, r->full.in(), r->full.n);
+      if (e != cudaSuccess) return cuda_fail(e, "full set");
+      r->set_on = true;
+      set_drop_rows(*r);
+    }
+    hashed = true;
+    return CDL_OK;
+  }
+
+  static uint64_t hash_slots(uint64_t rows) {
+    uint64_t s = 1 << 16;
+    while (s < 2 * rows) s <<= 1;
+    return s;
+  }
+
+  // A table for `rows` rows at a load of at most a half, the present one's
+  // keys moved over (fresh: into a new table even if this one is large
+  // enough, which drops the slots of tuples taken out).  ok = false, with
+  // nothing changed, when memory is short.
+  cdl_status hash_reserve(Relation& R, uint64_t rows, bool fresh, bool& ok) {
+    const uint64_t had = R.fset.keys ? R.fset.kmask + 1 : 0;
+    ok = true;
+    if (had >= 2 * rows && !fresh) return CDL_OK;
+    const uint64_t slots = std::max(had, hash_slots(rows));
+    DBuf nb = alloc(8 * slots);
+    ok = nb.p != nullptr;
+    if (!ok) return CDL_OK;
+    const unsigned long long* old = R.fset.keys;
+    R.fset.keys = static_cast<unsigned long long*>(nb.p);
+    R.fset.kmask = slots - 1;
+    cudaError_t e = cudaMemsetAsync(nb.p, 0xFF, 8 * slots, st);
+    if (e == cudaSuccess && old) e = hash_move(ctx, R.fset, old, had);
+    R.fset_buf = std::move(nb);
+    return e == cudaSuccess ? CDL_OK : cuda_fail(e, "full set");
   }
 
   void set_drop_rows(Relation& R) {
@@ -998,6 +1070,12 @@ struct cdl_engine {
       R.sdelta_ub = std::max(R.sdelta_ub, h_ctl[kSlotDelta + i]);
       R.set_single = false;
       delta_known = false;
+      if (R.fset.keys) {
+        bool ok = false;
+        cdl_status s = hash_reserve(R, R.full.n + R.sdelta_ub + nf, false, ok);
+        if (s == CDL_OK && !ok) s = fail(CDL_E_NOMEM, "full set");
+        if (s != CDL_OK) return s;
+      }
       cdl_status r = ensure_sdelta(R, nf);
       if (r != CDL_OK) return r;
       cudaError_t e = set_insert(ctx, R.fset, R.fresh.in(), nf, R.sdelta.out(), dslot(kSlotDelta + i),
@@ -1018,6 +1096,19 @@ struct cdl_engine {
       if (failed) n = std::min(R.fset.nbits, n + std::min(R.sdelta_ub, R.sdelta.cap));
       R.sdelta.clear();
       DCols rows;
+      if (R.fset.keys) {
+        cdl_status r = hash_rows(R, n, rows);
+        R.set_on = false;
+        if (r != CDL_OK) {
+          R.full.n = 0;
+          return r;
+        }
+        R.full = std::move(rows);
+        R.version[kFull]++;
+        r = set_sorted_delta(R);
+        if (r != CDL_OK) return r;
+        continue;
+      }
       DBuf ws = alloc(dense_extract_workspace(R.fset.nbits));
       if (!alloc_cols(rows, R.arity, n) || !ws.p) {
         R.set_on = false;  // (no rows to export)
@@ -1036,17 +1127,41 @@ struct cdl_engine {
       rows.n = n;
       R.full = std::move(rows);
       R.version[kFull]++;
-      R.fset_buf.reset();
-      R.fset = DenseSet{};
       R.set_on = false;
-      if (R.delta.n) {
-        uint32_t bits[kMaxK];
-        for (uint32_t k = 0; k < R.arity; ++k) bits[k] = bits_of(R.bound[k]);
-        cdl_status r = sort_cols(R.delta, bits);
-        if (r != CDL_OK) return r;
-      }
+      cdl_status r = set_sorted_delta(R);
+      if (r != CDL_OK) return r;
     }
     return CDL_OK;
+  }
+
+  cdl_status set_sorted_delta(Relation& R) {
+    R.fset_buf.reset();
+    R.fset = DenseSet{};
+    if (!R.delta.n) return CDL_OK;
+    uint32_t bits[kMaxK];
+    for (uint32_t k = 0; k < R.arity; ++k) bits[k] = bits_of(R.bound[k]);
+    return sort_cols(R.delta, bits);
+  }
+
+  // The keys of a hash set (at most n) as sorted rows.
+  cdl_status hash_rows(Relation& R, uint64_t n, DCols& rows) {
+    DCols keys;
+    if (!alloc_cols(keys, 2, n)) return fail(CDL_E_NOMEM, "sorted rows");
+    cudaError_t e = hash_keys(ctx, R.fset, keys.c[0], keys.c[1], n, dslot(kSlotScratch));
+    if (e != cudaSuccess) return cuda_fail(e, "sorted rows");
+    cdl_status r = fetch(kSlotScratch, 1);
+    if (r != CDL_OK) return r;
+    keys.n = h_ctl[kSlotScratch];
+    const DenseSet d = R.fset;
+    R.fset_buf.reset();
+    const uint32_t t = bits_of(d.nbits - 1);
+    const uint32_t bits[2] = {t > 32 ? t - 32 : 0, std::min<uint32_t>(t, 32)};
+    r = sort_cols(keys, bits);
+    if (r != CDL_OK) return r;
+    if (!alloc_cols(rows, R.arity, keys.n)) return fail(CDL_E_NOMEM, "sorted rows");
+    rows.n = keys.n;
+    e = hash_unpack(ctx, d, keys.c[0], keys.c[1], keys.n, rows.out());
+    return e == cudaSuccess ? CDL_OK : cuda_fail(e, "sorted rows");
   }
 
   DsmView dsm_view(const Relation& R) const {
@@ -2040,6 +2155,10 @@ struct cdl_engine {
       const size_t wws = join_write_workspace(P.n, total);
       DBuf wsp = alloc(wws);
       if (!wsp.p) return fail(CDL_E_NOMEM, "join splits");
+      if (last && rels[rule.head.rel]->set_on && rels[rule.head.rel]->fset.keys) {
+        bool done = false;
+        return set_join(rule, js, P.n, step_key, done, total);
+      }
       if (last && rels[rule.head.rel]->set_on) {  // Full is a set: new tuples go to delta
         Relation& H = *rels[rule.head.rel];
         r = ensure_sdelta(H, total);
@@ -2091,30 +2210,40 @@ struct cdl_engine {
     return CDL_OK;
   }
 
-  bool set_heavy_list() {
-    if (set_heavy_buf.p) return true;
-    set_heavy_buf = alloc(256 + sizeof(HeavyChunk) * kSetHeavyCap);
-    if (!set_heavy_buf.p) return false;
+  bool set_heavy_list(uint64_t cap) {
+    if (set_heavy_buf.p && set_heavy.cap >= cap) return true;
+    DBuf b = alloc(256 + sizeof(HeavyChunk) * cap);
+    if (!b.p) return false;
+    set_heavy_buf = std::move(b);
     set_heavy.n = static_cast<uint64_t*>(set_heavy_buf.p);
     set_heavy.e = reinterpret_cast<HeavyChunk*>(static_cast<char*>(set_heavy_buf.p) + 256);
-    set_heavy.cap = kSetHeavyCap;
+    set_heavy.cap = cap;
     return true;
   }
 
   // A join into Full as a set in one pass, into a buffer sized by the step's
-  // last join; done = false leaves it to the exact form.
+  // last join (done = false leaves it to the exact form) or, with a hash set,
+  // by its exact size.
   cdl_status set_join(const RuleR& rule, const JoinSpec& js, uint64_t np,
-                      const std::tuple<size_t, size_t, size_t>& key, bool& done) {
+                      const std::tuple<size_t, size_t, size_t>& key, bool& done,
+                      uint64_t exact = 0) {
     Relation& H = *rels[rule.head.rel];
-    const auto it = set_seen.find(key);
-    if (it == set_seen.end() || opt.mem_limit || set_steps.size() >= kSetSteps) return CDL_OK;
-    const SetSeen& seen = it->second;
-    if (seen.probe == 0 || seen.outputs > kSetRatio * seen.probe) return CDL_OK;
-    const double per_row = (double)seen.outputs / (double)seen.probe;
-    const uint64_t want = (uint64_t)((2.0 * per_row + 1.0) * (double)np) + 4096;
-    if (!H.set_free && H.sdelta_ub + want > 0xFFFFFFFFull) return CDL_OK;
+    uint64_t want = exact;
+    if (!exact) {
+      const auto it = set_seen.find(key);
+      if (it == set_seen.end() || opt.mem_limit) return CDL_OK;
+      const SetSeen& seen = it->second;
+      if (seen.probe == 0 || seen.outputs > kSetRatio * seen.probe) return CDL_OK;
+      const double per_row = (double)seen.outputs / (double)seen.probe;
+      want = (uint64_t)((2.0 * per_row + 1.0) * (double)np) + 4096;
+      if (!H.set_free && H.sdelta_ub + want > 0xFFFFFFFFull) return CDL_OK;
+    }
+    if (set_steps.size() >= kSetSteps) {
+      if (!exact) return CDL_OK;
+      return fail(CDL_E_CAPACITY, "too many joins into hash sets in one round");
+    }
     cdl_status r = ensure_sdelta(H, want);
-    if (r == CDL_E_NOMEM) {  // (nothing was changed but the bound)
+    if (r == CDL_E_NOMEM && !exact) {  // (nothing was changed but the bound)
       err.clear();
       H.sdelta_ub -= want;
       return CDL_OK;
@@ -2122,8 +2251,16 @@ struct cdl_engine {
     if (r != CDL_OK) return r;
     done = true;
     if (H.set_redo) return CDL_OK;
+    if (H.fset.keys) {
+      bool ok = false;
+      r = hash_reserve(H, H.full.n + std::min(H.sdelta_ub, H.sdelta.cap), false, ok);
+      if (r == CDL_OK && !ok) r = fail(CDL_E_NOMEM, "full set");
+      if (r != CDL_OK) return r;
+    }
     const uint32_t slot = kSlotSetTotal + (uint32_t)set_steps.size();
-    if (!set_heavy_list()) return fail(CDL_E_NOMEM, "long ranges");
+    // (an exact size also bounds the chunks: at most two per kHeavyChunk outputs)
+    if (!set_heavy_list(std::max(kSetHeavyCap, 2 * exact / kHeavyChunk + 2)))
+      return fail(CDL_E_NOMEM, "long ranges");
     cudaError_t e = cudaMemsetAsync(set_heavy.n, 0, 8, st);
     if (e == cudaSuccess)
       e = join_set(ctx, js, H.fset, H.sdelta.out(), dslot(kSlotDelta + rule.head.rel), H.sdelta.cap,
@@ -2148,7 +2285,7 @@ struct cdl_engine {
     Relation& H = *rels[rule.head.rel];
     const DenseSet* d = H.set_on ? &H.fset : H.dset.words ? &H.dset : nullptr;
     const uint32_t lastc = H.arity - 1;
-    if (!d || nkeys > 2 || total < kHubOutputs || total / kHubOutputsPerRow < P.n + B.n)
+    if (!d || d->keys || nkeys > 2 || total < kHubOutputs || total / kHubOutputsPerRow < P.n + B.n)
       return CDL_OK;
     const uint32_t bits = bits_of(d->mask[lastc]);
     if (bits < 8 || d->k != js.out_k) return CDL_OK;
@@ -2713,6 +2850,7 @@ struct cdl_engine {
     }
     if (!any) return CDL_OK;
     force_exact = true;
+    const size_t steps_before = set_steps.size();
     // each overrun widens this run's later predictions by half a step (x 1.41)
     if (est_ready()) est_boost = std::min(4.0, est_boost + 0.5);
     for (uint32_t i = 0; i < nr; ++i)
@@ -2725,6 +2863,12 @@ struct cdl_engine {
           const uint64_t at = std::min<uint64_t>(h_ctl[kSlotDelta + i], S.sdelta.cap);
           h_ctl[kSlotDelta + i] = S.sdelta_ub = at;
           S.set_single = S.set_redo = false;
+          if (S.fset.keys) {  // without the slots of the tuples that found no room
+            bool ok = false;
+            s = hash_reserve(S, S.full.n + at, true, ok);
+            if (s == CDL_OK && !ok) s = fail(CDL_E_NOMEM, "full set");
+            if (s != CDL_OK) return s;
+          }
           e = cudaMemcpyAsync(dslot(kSlotDelta + i), h_ctl + kSlotDelta + i, 8,
                               cudaMemcpyHostToDevice, st);
           if (e != cudaSuccess) return cuda_fail(e, "delta reset");
@@ -2740,6 +2884,9 @@ struct cdl_engine {
     force_exact = false;
     s = fetch_round();
     if (s != CDL_OK) return s;
+    for (size_t i = steps_before; i < set_steps.size(); ++i)
+      if (h_ctl[kSlotSetTotal + i] & kSetListFull)
+        return fail(CDL_E_CAPACITY, "a hash set ran out of slots");
     for (uint32_t i = 0; i < nr; ++i)
       if (redo[i] && h_ctl[kSlotCursor + i] > rels[i]->fresh.cap)
         return fail(CDL_E_CAPACITY, "an exact join overflowed its buffer");
@@ -2842,12 +2989,20 @@ struct cdl_engine {
       // (Full as a bitmap: the joins append to delta; no rows of Full, no
       // sort, no merge)
       G.set = R.set_on;
+      uint64_t set_full = ~0ull;
+      if (R.fset.keys && G.set) {  // room for the rows of many rounds, and what one may add
+        set_full = std::max<uint64_t>(hash_room * R.full.n, 1 << 16);
+        bool fits = false;
+        cdl_status hs = hash_reserve(R, set_full + G.Ucap / 8, false, fits);
+        if (hs != CDL_OK) return hs;
+        ok &= fits;
+      }
       for (int side = 0; side < 2; ++side) {
         if (!G.set) ok &= alloc_cols(G.F[side], R.arity, G.Fcap);
         ok &= alloc_cols(G.D[side], R.arity, G.Ucap);
       }
       if (G.set) {
-        ok &= set_heavy_list();
+        ok &= set_heavy_list(kSetHeavyCap);
       } else {
         ok &= alloc_cols(G.fresh, R.arity, G.Ucap) && alloc_cols(G.alt, R.arity, G.Ucap);
         G.sort_ws = alloc(radix_workspace(G.Ucap, G.plan.bits, G.plan.threads));
@@ -2866,8 +3021,8 @@ struct cdl_engine {
         if (e != cudaSuccess) return cuda_fail(e, "graph state copy");
       }
       const uint64_t set_cap = G.set ? G.Ucap : 0;
-      cur[j] = GraphRel{G.F[0].in(), G.D[0].in(), R.full.n, R.delta.n, set_cap};
-      next[j] = GraphRel{G.F[1].in(), G.D[1].in(), 0, 0, set_cap};
+      cur[j] = GraphRel{G.F[0].in(), G.D[0].in(), R.full.n, R.delta.n, set_cap, set_full};
+      next[j] = GraphRel{G.F[1].in(), G.D[1].in(), 0, 0, set_cap, set_full};
     }
     for (size_t s = 0; s < grec.size(); ++s) {
       const GStep& g = grec[s];
@@ -2978,7 +3133,13 @@ struct cdl_engine {
     }
     for (size_t j = 0; j < grel.size() && e == cudaSuccess; ++j) {
       GRelRes& G = grel[j];
-      if (G.set) continue;  // the joins left its new tuples
+      if (G.set) {  // the joins left its new tuples
+        if (opt.n_instances)
+          e = mark_instances(ctx, nullptr, G.Ucap, opt.n_instances,
+                             static_cast<uint64_t*>(inst_last.p), 1, &g_next()[j].D, g_cursor(j),
+                             &g_ctl()->round);
+        continue;
+      }
       const Relation& R = *rels[G.rel];
       bool in_b = false;
       e = radix_sort(ctx, G.plan, G.fresh.out(), G.alt.out(), G.Ucap, G.sort_ws.p, &in_b,
@@ -3174,6 +3335,13 @@ struct cdl_engine {
     finished = ctl.done == 1;
     if (ctl.done == 2)  // a buffer was too small: the next round runs on the host, then larger
       for (auto& c : gcap_u) c *= 2;
+    for (size_t i = 0; i < rels.size() && ctl.done == 2; ++i)  // (without the undone tuples' slots)
+      if (rels[i]->set_on && rels[i]->fset.keys) {
+        bool ok = false;
+        r = hash_reserve(*rels[i], rels[i]->full.n, true, ok);
+        if (r == CDL_OK && !ok) r = fail(CDL_E_NOMEM, "full set");
+        if (r != CDL_OK) return r;
+      }
     if (ctl.done == 2) {
       for (auto& c : gcap_i) c *= 2;
       for (size_t i = 0; i < rels.size(); ++i)
@@ -3257,7 +3425,7 @@ struct cdl_engine {
       }
     }
     grec.clear();
-    grec_bad = graph_ready = false;
+    grec_bad = graph_ready = hashed = false;
     g_rounds = g_builds = g_retirements = 0;
     for (uint64_t round = resume_rounds + 1; status == CDL_OK; ++round) {
       cur_round = round;
@@ -3363,7 +3531,7 @@ struct cdl_engine {
         }
       }
       if (status != CDL_OK) break;
-      if (opt.n_instances && new_total && opt.retire >= 0) {
+      if (opt.n_instances && new_total && opt.retire >= 0 && !hashed) {
         status = retire(round);
         if (status != CDL_OK) break;
       }
@@ -3379,6 +3547,7 @@ struct cdl_engine {
       }
       for (uint32_t i = 0; i < nr && status == CDL_OK; ++i)
         if (rels[i]->idb) status = set_switch(*rels[i]);
+      if (status == CDL_OK && opt.n_instances && !hashed && round >= first_semi) status = hash_switch();
       if (status != CDL_OK) break;
       if (opt.graph && round == first_semi) {
         graph_ready = graph_plan();

@@ -17,7 +17,8 @@ __global__ void k_round_end(GraphRel* cur, GraphRel* next, uint32_t nrel, GraphC
   bool overflow = ctl->overflow;
   for (uint32_t s = 0; s < nsteps; ++s) overflow |= (steps[3 * s] & kSetListFull) != 0;
   for (uint32_t r = 0; r < nrel; ++r)
-    overflow |= cur[r].set_cap && cursors[r] > cur[r].set_cap;
+    overflow |= cur[r].set_cap &&
+                (cursors[r] > cur[r].set_cap || cur[r].nF + cursors[r] > cur[r].set_full);
   if (overflow) {  // cur holds the last complete round
     ctl->done = 2;
     cudaGraphSetConditional(loop, 0u);

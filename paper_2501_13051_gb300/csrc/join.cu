@@ -905,6 +905,17 @@ cudaError_t join_direct(Ctx& c, const JoinSpec& j, ColsOut out, uint64_t* d_curs
 constexpr int kSJT = 256, kSJI = 8;
 constexpr uint32_t kSJTile = kSJT * kSJI;
 
+// Both forms of the set; a full table is noted in *total.
+template <bool HASH, int N>
+__device__ __forceinline__ uint32_t set_add_any(const DenseSet& d, const uint64_t (&idx)[N],
+                                                unsigned long long* total) {
+  if constexpr (!HASH) return set_add<N>(d, idx);
+  bool full = false;
+  const uint32_t fresh = set_add_hash<N>(d, idx, &full);
+  if (full) atomicOr(total, (unsigned long long)kSetListFull);
+  return fresh;
+}
+
 template <bool FILTER>
 __device__ __forceinline__ uint64_t set_tuple(const JoinSpec& j, const ColsIn& probe,
                                               const DenseSet& d, uint64_t row, uint64_t b1,
@@ -928,7 +939,7 @@ __device__ __forceinline__ uint64_t set_tuple(const JoinSpec& j, const ColsIn& p
   return idx;
 }
 
-template <bool FILTER, bool STAR>
+template <bool FILTER, bool STAR, bool HASH>
 __global__ void __launch_bounds__(kSJT, 4) k_join_set(const JoinSpec j, const DenseSet d, ColsOut out,
                                                       unsigned long long* cursor, uint64_t cap,
                                                       unsigned long long* total, uint32_t* err,
@@ -1038,7 +1049,7 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set(const JoinSpec j, const De
         }
       }
       if (bad && err) atomicOr(err, kErrCapacity);
-      const uint32_t fresh = set_add<kSJI>(d, idx);
+      const uint32_t fresh = set_add_any<HASH, kSJI>(d, idx, total);
       set_emit<kSJT, kSJI, true>(d, idx, fresh, out, 0, cursor, cap, red);
       __syncthreads();  // the next window rewrites s_slot and red
     }
@@ -1047,11 +1058,12 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set(const JoinSpec j, const De
 }
 
 // The listed chunks, one block at a time (their number from device memory).
-template <bool FILTER, bool STAR>
+template <bool FILTER, bool STAR, bool HASH>
 __global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, const DenseSet d,
                                                             ColsOut out, unsigned long long* cursor,
-                                                            uint64_t cap, uint32_t* err,
-                                                            HeavyList heavy) {
+                                                            uint64_t cap,
+                                                            unsigned long long* total,
+                                                            uint32_t* err, HeavyList heavy) {
   static_assert(kHeavyChunk <= kSJTile, "a chunk is one window");
   __shared__ __align__(8) uint32_t red[kSJT / 32 + 2];
   const ColsIn probe = probe_cols(j);
@@ -1076,7 +1088,7 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, co
       }
     }
     if (bad && err) atomicOr(err, kErrCapacity);
-    const uint32_t fresh = set_add<kSJI>(d, idx);
+    const uint32_t fresh = set_add_any<HASH, kSJI>(d, idx, total);
     set_emit<kSJT, kSJI, true>(d, idx, fresh, out, 0, cursor, cap, red);
     __syncthreads();  // the next chunk reuses red
   }
@@ -1095,14 +1107,21 @@ cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, 
   auto* tot = reinterpret_cast<unsigned long long*>(d_total);
   auto launch = [&](auto rows, auto chunks) {
     rows<<<grid, kSJT, 0, c.st>>>(j, d, out, cur, out_cap, tot, c.d_err, (uint32_t)per, heavy);
-    chunks<<<152, kSJT, 0, c.st>>>(j, d, out, cur, out_cap, c.d_err, heavy);
+    chunks<<<152, kSJT, 0, c.st>>>(j, d, out, cur, out_cap, tot, c.d_err, heavy);
   };
+#define CDL_JOIN_SET(F, S)                                                             \
+  d.keys ? launch(k_join_set<F, S, true>, k_join_set_heavy<F, S, true>)                \
+         : launch(k_join_set<F, S, false>, k_join_set_heavy<F, S, false>)
   if (j.star)
-    filter ? launch(k_join_set<true, true>, k_join_set_heavy<true, true>)
-           : launch(k_join_set<false, true>, k_join_set_heavy<false, true>);
+    if (filter)
+      CDL_JOIN_SET(true, true);
+    else
+      CDL_JOIN_SET(false, true);
+  else if (filter)
+    CDL_JOIN_SET(true, false);
   else
-    filter ? launch(k_join_set<true, false>, k_join_set_heavy<true, false>)
-           : launch(k_join_set<false, false>, k_join_set_heavy<false, false>);
+    CDL_JOIN_SET(false, false);
+#undef CDL_JOIN_SET
   return cudaGetLastError();
 }
 

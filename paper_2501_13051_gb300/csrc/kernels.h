@@ -199,7 +199,8 @@ cudaError_t join_write(Ctx& c, const JoinSpec& j, const uint64_t* d_off, uint64_
 // caller makes room, sets the cursor to out_cap (that many rows are there)
 // and joins again.  *d_total grows by the join's size, with kSetListFull set in
 // it when the list of long ranges (heavy, as join_direct's, its counter
-// zeroed by the caller) was too short: then too the join runs again.
+// zeroed by the caller) was too short or a hash set full: then too the join
+// runs again.
 struct HeavyList;
 constexpr uint64_t kSetListFull = 1ull << 62;
 cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, uint64_t* d_cursor,
@@ -212,7 +213,15 @@ cudaError_t dense_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n);
 // (packed at *d_cursor, at most out_cap rows; more raise kErrCapacity).
 cudaError_t set_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n, ColsOut out,
                        uint64_t* d_cursor, uint64_t out_cap);
-// Clears the bits of n rows.
+// The hash form (d.keys; the three above and below take it as well): the keys
+// of another table of `slots` slots inserted; all keys as two columns, their
+// number (at most cap) in *d_count; such columns as rows.
+cudaError_t hash_move(Ctx& c, const DenseSet& d, const unsigned long long* old, uint64_t slots);
+cudaError_t hash_keys(Ctx& c, const DenseSet& d, uint32_t* hi, uint32_t* lo, uint64_t cap,
+                      uint64_t* d_count);
+cudaError_t hash_unpack(Ctx& c, const DenseSet& d, const uint32_t* hi, const uint32_t* lo,
+                        uint64_t n, ColsOut out);
+// Takes n rows out of the set.
 cudaError_t dense_remove(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n);
 size_t dense_extract_workspace(uint64_t nbits);
 // The set bits of d as rows in increasing bit order (lexicographic, no
@@ -372,7 +381,8 @@ cudaError_t mark_instances(Ctx& c, const uint32_t* inst, uint64_t n, uint32_t n_
 struct GraphRel {
   ColsIn F, D;
   uint64_t nF, nD;
-  uint64_t set_cap;  // Full is a bitmap: rows D holds (F is unused); else 0
+  uint64_t set_cap;   // Full is a set: rows D holds (F is unused); else 0
+  uint64_t set_full;  // ... and the rows its table is sized for
 };
 struct GraphCtl {
   uint64_t round;       // rounds completed (all launches, numbered as the engine does)
@@ -386,8 +396,9 @@ struct GraphCtl {
 // loop stops (cur still holds the last complete round); else next.nF =
 // cur.nF + next.nD, per_round[round] = sum of next.nD, cur <-> next, and the
 // loop's condition is set to continue while the round derived something.
-// Where Full is a bitmap next.nD is the relation's cursor; a cursor past
-// set_cap, or kSetListFull in a step's first word, is an overflow as well.
+// Where Full is a set next.nD is the relation's cursor; a cursor past
+// set_cap, more rows than set_full or kSetListFull in a step's first word is
+// an overflow as well.
 // It also zeroes the next round's cursors: `ncur` words at `cursors`, and of
 // the three words of each of the `nsteps` steps the first and the last.
 cudaError_t round_end(Ctx& c, GraphRel* cur, GraphRel* next, uint32_t nrel, GraphCtl* ctl,
