@@ -281,22 +281,29 @@ __device__ __forceinline__ uint32_t set_add_hash(const DenseSet& d, const uint64
         v[q] = key[q];
       }
     }
+  // the others look on, one after another (code for one, not for N)
+  uint32_t left = 0;
 #pragma unroll
-  for (int q = 0; q < N; ++q)
-    if (key[q] != kNoTuple && v[q] != key[q]) {
-      uint64_t at = mix64(key[q]) & d.kmask;
-      bool done = false;
-      for (uint32_t step = 1; step < kSetProbes && !done; ++step) {
-        at = (at + 1) & d.kmask;
-        unsigned long long x = d.keys[at];
-        if (x == kSetEmpty) {
-          x = atomicCAS(d.keys + at, kSetEmpty, key[q]);
-          if (x == kSetEmpty) fresh |= 1u << q;
-        }
-        done = x == kSetEmpty || x == key[q];
+  for (int q = 0; q < N; ++q) left |= (key[q] != kNoTuple && v[q] != key[q] ? 1u : 0u) << q;
+  while (left) {
+    const uint32_t b = left & (0u - left);
+    left ^= b;
+    uint64_t k = key[0];
+#pragma unroll
+    for (int q = 1; q < N; ++q) k = (b >> q) & 1u ? key[q] : k;
+    uint64_t at = mix64(k) & d.kmask;
+    bool done = false;
+    for (uint32_t step = 1; step < kSetProbes && !done; ++step) {
+      at = (at + 1) & d.kmask;
+      unsigned long long x = d.keys[at];
+      if (x == kSetEmpty) {
+        x = atomicCAS(d.keys + at, kSetEmpty, k);
+        if (x == kSetEmpty) fresh |= b;
       }
-      if (!done) *full = true;
+      done = x == kSetEmpty || x == k;
     }
+    if (!done) *full = true;
+  }
   return fresh;
 }
 
@@ -319,9 +326,8 @@ __device__ __forceinline__ void set_remove(const DenseSet& d, uint64_t idx) {
 // Writes a block's new tuples (bit q of fresh: tuple idx[q] is new) packed at
 // *cursor: one claim per block, each warp's tuples of one q side by side.
 // wsum: THREADS / 32 + 2 words of shared memory (the last two hold the
-// claimed position).  Rows past cap are dropped; false tells the caller
-// (CLEAR: their bits are cleared again, so that a second try finds them new).
-template <int THREADS, int N, bool CLEAR = false>
+// claimed position).  Rows past cap are dropped; false tells the caller.
+template <int THREADS, int N>
 __device__ __forceinline__ bool set_emit(const DenseSet& d, const uint64_t (&idx)[N],
                                          uint32_t fresh, ColsOut out, uint64_t base,
                                          unsigned long long* cursor, uint64_t cap,
@@ -357,7 +363,6 @@ __device__ __forceinline__ bool set_emit(const DenseSet& d, const uint64_t (&idx
         for (int k = 0; k < kMaxK; ++k)
           if (k < (int)d.k) out.c[k][p] = set_column(d, idx[q], k);
       } else {
-        if (CLEAR) set_remove(d, idx[q]);
         ok = false;
       }
     }

@@ -928,7 +928,7 @@ struct cdl_engine {
   // running instances every round (and moves converged instances' rows out of
   // its way); the set takes every new tuple once, at random, and sorts all of
   // them once at the end.  512 instances, 279M tuples, 233 captured rounds:
-  // 222 ms with rows, 97 with sets.
+  // 222 ms with rows, 90 with sets.
   cdl_status hash_switch() {
     uint64_t rows = 0, steps = 0;
     for (const RuleR& rule : rules)
@@ -942,13 +942,16 @@ struct cdl_engine {
     }
     size_t free_b = 0, total_b = 0;
     if (rows < kHashRows || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return CDL_OK;
-    if (hash_slots(8 * rows) * 8 > free_b / 4) return CDL_OK;
+    if (hash_slots((hash_room + 1) * rows) * 8 > free_b / 4) return CDL_OK;
     for (auto& r : rels) {
       if (!r->idb) continue;
       tuple_space(*r, kHashBits, r->fset);
       r->fset.append = 1;
       bool ok = false;
-      cdl_status s = hash_reserve(*r, 4 * r->full.n + 1024, false, ok);
+      // (a graph wants its room at once: moving the keys later costs as much
+      // as inserting them)
+      const uint64_t room = opt.graph ? hash_room + 1 : 4;
+      cdl_status s = hash_reserve(*r, room * r->full.n + (1 << 16), false, ok);
       if (s == CDL_OK && !ok) s = fail(CDL_E_NOMEM, "full set");
       if (s != CDL_OK) return s;
       cudaError_t e = dense_insert(ctx, r->fset, r->full.in(), r->full.n);

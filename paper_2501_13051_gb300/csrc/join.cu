@@ -899,9 +899,9 @@ cudaError_t join_direct(Ctx& c, const JoinSpec& j, ColsOut out, uint64_t* d_curs
 // Rows with more than kHeavyChunk outputs are listed and taken in chunks by
 // a second kernel, so that one hot key does not hold one block.
 // Bound by the random accesses to the bitmap.  Same generation on 200,000
-// nodes: 25 ms of counts and scans and 66 of writes become 77 ms; a round of a
+// nodes: 25 ms of counts and scans and 66 of writes become 47 ms; a round of a
 // small closure takes one launch and one wait (4,001 nodes, 46 rounds: 4.9 ->
-// 2.9 ms).
+// 2.6 ms).
 constexpr int kSJT = 256, kSJI = 8;
 constexpr uint32_t kSJTile = kSJT * kSJI;
 
@@ -916,27 +916,174 @@ __device__ __forceinline__ uint32_t set_add_any(const DenseSet& d, const uint64_
   return fresh;
 }
 
-template <bool FILTER>
-__device__ __forceinline__ uint64_t set_tuple(const JoinSpec& j, const ColsIn& probe,
-                                              const DenseSet& d, uint64_t row, uint64_t b1,
-                                              uint64_t b2, bool& bad) {
-  uint32_t v[kMaxK] = {0, 0, 0, 0};
-#pragma unroll
-  for (int k = 0; k < kMaxK; ++k)
-    if (k < (int)j.out_k) v[k] = ref_value(j, probe, j.out[k], row, b1, b2);
-  if (FILTER) {
-    bool keep = true;
-    for (uint32_t q = 0; q < j.n_eq; ++q)
-      keep &= ref_value(j, probe, j.eq[q][0], row, b1, b2) ==
-              ref_value(j, probe, j.eq[q][1], row, b1, b2);
-    for (uint32_t q = 0; q < j.n_neq; ++q)
-      keep &= ref_value(j, probe, j.neq[q][0], row, b1, b2) !=
-              ref_value(j, probe, j.neq[q][1], row, b1, b2);
-    if (!keep) return kNoTuple;
+// Where a launch's values come from, staged once per block: the head
+// columns, then the pairs of the equalities and of the inequalities.  The
+// loops over columns read this table and are not unrolled; only the loop over
+// a thread's outputs is, so that its loads are in flight together.  (With the
+// columns unrolled as well -- eight outputs times eight columns times the
+// sides a value may come from -- half of all warp cycles waited for
+// instructions: 77 ms of same generation on 200,000 nodes; 47 so.)
+struct SetRefs {
+  const uint32_t* p[kMaxK + 16];
+  uint32_t side[kMaxK + 16], v[kMaxK + 16];
+  uint32_t* out[kMaxK];
+  uint32_t shift[kMaxK], mask[kMaxK];
+};
+
+__device__ __forceinline__ void stage_refs(const JoinSpec& j, const DenseSet& d, const ColsOut& out,
+                                           SetRefs& s) {
+  const uint32_t t = threadIdx.x;
+  if (t < kMaxK + 16) {
+    Ref f{2, 0};
+    if (t < kMaxK) {
+      if (t < j.out_k) f = j.out[t];
+      s.out[t] = j.dout ? j.dout->c[t] : out.c[t];
+      s.shift[t] = d.shift[t];
+      s.mask[t] = d.mask[t];
+    } else {
+      const uint32_t i = t - kMaxK;
+      if (i < 2 * j.n_eq)
+        f = j.eq[i >> 1][i & 1];
+      else if (i < 2 * (j.n_eq + j.n_neq))
+        f = j.neq[(i >> 1) - j.n_eq][i & 1];
+    }
+    s.side[t] = f.side;
+    s.v[t] = f.v;
+    s.p[t] = f.side == 0 ? (j.dprobe ? j.dprobe->c[f.v] : j.probe.c[f.v])
+             : f.side == 1 ? j.build.c[f.v]
+             : f.side == 3 ? j.build2.c[f.v]
+                           : nullptr;
   }
-  const uint64_t idx = set_pack(d, v);
-  bad |= idx == kNoTuple;
-  return idx;
+  __syncthreads();
+}
+
+// Value i of the table for the N outputs in `live`: probe row base + row[q],
+// build rows b1[q] and b2[q].
+template <int N>
+__device__ __forceinline__ void set_values(const SetRefs& s, uint32_t i, uint32_t live,
+                                           uint64_t base, const uint32_t (&row)[N],
+                                           const uint32_t (&b1)[N], const uint32_t (&b2)[N],
+                                           uint32_t (&v)[N]) {
+  const uint32_t side = s.side[i];
+  const uint32_t* p = s.p[i] + (side == 0 ? base : 0ull);
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    v[q] = s.v[i];
+    if (side != 2 && ((live >> q) & 1u)) v[q] = __ldg(p + (side == 0 ? row[q] : side == 1 ? b1[q] : b2[q]));
+  }
+}
+
+// Packed tuples of the outputs in `live` (kNoTuple: none, dropped by a filter
+// or outside the set's space, which sets bad).
+template <bool FILTER, int N>
+__device__ __forceinline__ void set_tuples(const JoinSpec& j, const SetRefs& s, uint32_t live,
+                                           uint64_t base, const uint32_t (&row)[N],
+                                           const uint32_t (&b1)[N], const uint32_t (&b2)[N],
+                                           uint64_t (&idx)[N], bool& bad) {
+  if (FILTER) {
+#pragma unroll 1
+    for (uint32_t f = 0; f < j.n_eq + j.n_neq; ++f) {
+      uint32_t x[N], y[N];
+      set_values<N>(s, kMaxK + 2 * f, live, base, row, b1, b2, x);
+      set_values<N>(s, kMaxK + 2 * f + 1, live, base, row, b1, b2, y);
+#pragma unroll
+      for (int q = 0; q < N; ++q)
+        if ((x[q] == y[q]) != (f < j.n_eq)) live &= ~(1u << q);
+    }
+  }
+  uint32_t out = 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q) idx[q] = 0;
+#pragma unroll 1
+  for (uint32_t k = 0; k < j.out_k; ++k) {
+    uint32_t v[N];
+    set_values<N>(s, k, live, base, row, b1, b2, v);
+    const uint32_t sh = s.shift[k], mask = s.mask[k];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      idx[q] |= (uint64_t)v[q] << sh;
+      out |= (v[q] > mask ? 1u : 0u) << q;
+    }
+  }
+  bad |= (out & live) != 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if (!((live & ~out) >> q & 1u)) idx[q] = kNoTuple;
+}
+
+// As set_emit with CLEAR, the columns from the staged table.
+template <int THREADS, int N>
+__device__ __forceinline__ void set_store(const JoinSpec& j, const DenseSet& d, const SetRefs& s,
+                                          const uint64_t (&idx)[N], uint32_t fresh,
+                                          unsigned long long* cursor, uint64_t cap, uint32_t* wsum) {
+  constexpr int W = THREADS / 32;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, lt = (1u << lane) - 1u;
+  uint32_t at[N], n = 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const uint32_t bal = __ballot_sync(0xffffffffu, (fresh >> q) & 1u);
+    at[q] = n + __popc(bal & lt);
+    n += __popc(bal);
+  }
+  if (lane == 0) wsum[warp] = n;
+  __syncthreads();
+  unsigned long long* claim = reinterpret_cast<unsigned long long*>(wsum + W);
+  uint32_t before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    const uint32_t c = wsum[w];
+    before += w < (int)warp ? c : 0u;
+    total += c;
+  }
+  if (total == 0) return;  // uniform
+  if (threadIdx.x == 0) *claim = atomicAdd(cursor, (unsigned long long)total);
+  __syncthreads();
+  const uint64_t pos = *claim + before;
+  const uint64_t room = cap > pos ? cap - pos : 0;
+#pragma unroll 1
+  for (uint32_t k = 0; k < j.out_k; ++k) {
+    uint32_t* o = s.out[k] + pos;
+    const uint32_t sh = s.shift[k], mask = s.mask[k];
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (((fresh >> q) & 1u) && at[q] < room) o[at[q]] = (uint32_t)(idx[q] >> sh) & mask;
+  }
+  if (n > room) {  // (rare: past the buffer)
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (((fresh >> q) & 1u) && at[q] >= room) set_remove(d, idx[q]);
+  }
+}
+
+// Ranges of a thread's eight probe rows.  The direct form's reads go out
+// together; the hash form's probes are a loop each.
+template <int N>
+__device__ __forceinline__ void set_lookup(const JoinSpec& j, const KeyIndex& x, uint32_t range,
+                                           const uint32_t* c0, const uint32_t* c1, uint64_t base,
+                                           uint32_t live, uint32_t (&st)[N], uint32_t (&cnt)[N]) {
+  uint32_t k0[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    k0[q] = 0;
+    st[q] = cnt[q] = 0;
+    if ((live >> q) & 1u) k0[q] = __ldg(c0 + base + (uint64_t)q * kSJT + threadIdx.x);
+  }
+  if (range) {
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (((live >> q) & 1u) && k0[q] < range) {
+        const uint2 e = __ldg(reinterpret_cast<const uint2*>(x.table) + k0[q]);
+        st[q] = e.x;
+        cnt[q] = e.y > e.x ? e.y - e.x : 0u;
+      }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if ((live >> q) & 1u) {
+      const uint32_t k1 = c1 ? __ldg(c1 + base + (uint64_t)q * kSJT + threadIdx.x) : 0u;
+      cnt[q] = probe_table(x.table, x.slots - 1, k0[q], k1, &st[q]);
+    }
 }
 
 template <bool FILTER, bool STAR, bool HASH>
@@ -949,18 +1096,41 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set(const JoinSpec j, const De
   __shared__ uint32_t s_start2[STAR ? kSJTile : 1], s_cnt2[STAR ? kSJTile : 1];
   __shared__ uint16_t s_slot[kSJTile];
   __shared__ __align__(8) uint32_t red[kSJT / 32 + 2];
+  __shared__ SetRefs refs;
+  stage_refs(j, d, out, refs);
   const uint64_t n = dev_size(j.dn, j.n_probe);
-  const ColsIn probe = probe_cols(j);
-  if (j.dout) out = *j.dout;  // (inside a captured round)
-  const uint32_t range = direct_range(j.ix), t = threadIdx.x;
+  const ColsIn* probe = j.dprobe ? j.dprobe : &j.probe;
+  const uint32_t* pk0 = j.cross ? nullptr : probe->c[j.pk0];
+  const uint32_t* pk1 = j.cross || j.pk1 == 0xFFu ? nullptr : probe->c[j.pk1];
+  const uint32_t *qk0 = nullptr, *qk1 = nullptr;
+  if constexpr (STAR) {
+    qk0 = probe->c[j.qk0];
+    qk1 = j.qk1 == 0xFFu ? nullptr : probe->c[j.qk1];
+  }
+  const uint32_t range = direct_range(j.ix), range2 = STAR ? direct_range(j.ix2) : 0u;
+  const uint32_t t = threadIdx.x;
   const uint32_t rows = kSJT * per;
   for (uint64_t base = (uint64_t)blockIdx.x * rows; base < n; base += (uint64_t)gridDim.x * rows) {
     uint32_t cnt[kSJI], st[kSJI];
+    uint32_t live = 0;
 #pragma unroll
-    for (int q = 0; q < kSJI; ++q) {
-      const uint64_t row = base + (uint64_t)q * kSJT + t;
-      cnt[q] = st[q] = 0;
-      if (q < (int)per && row < n) cnt[q] = lookup(j, probe, range, row, &st[q]);
+    for (int q = 0; q < kSJI; ++q)
+      live |= (q < (int)per && base + (uint64_t)q * kSJT + t < n ? 1u : 0u) << q;
+    if (j.cross) {
+#pragma unroll
+      for (int q = 0; q < kSJI; ++q) {
+        st[q] = 0;
+        cnt[q] = (live >> q) & 1u ? j.n_build : 0u;
+      }
+    } else {
+      set_lookup<kSJI>(j, j.ix, range, pk0, pk1, base, live, st, cnt);
+    }
+    uint32_t st2[kSJI], cnt2[kSJI];
+    if constexpr (STAR) {
+      uint32_t found = 0;
+#pragma unroll
+      for (int q = 0; q < kSJI; ++q) found |= (cnt[q] ? 1u : 0u) << q;
+      set_lookup<kSJI>(j, j.ix2, range2, qk0, qk1, base, found, st2, cnt2);
     }
     uint32_t sum = 0;
 #pragma unroll
@@ -968,11 +1138,9 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set(const JoinSpec j, const De
       const uint64_t row = base + (uint64_t)q * kSJT + t;
       uint64_t c = cnt[q];
       if constexpr (STAR) {
-        uint32_t st2 = 0, c2 = 0;
-        if (c) c2 = lookup2(j, probe, row, &st2);
-        s_start2[t * kSJI + q] = st2;
-        s_cnt2[t * kSJI + q] = c2;
-        c *= c2;
+        s_start2[t * kSJI + q] = st2[q];
+        s_cnt2[t * kSJI + q] = cnt2[q];
+        c *= cnt2[q];
         if (c > 0xFFFFFFFFull) {
           if (err) atomicOr(err, kErrCapacity);
           c = 0;
@@ -1031,26 +1199,29 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set(const JoinSpec j, const De
       }
       __syncthreads();
       uint64_t idx[kSJI];
+      uint32_t row[kSJI], b1[kSJI], b2[kSJI], have = 0;
       bool bad = false;
 #pragma unroll
       for (int q = 0; q < kSJI; ++q) {
         const uint32_t o = w + q * kSJT + t;
-        idx[q] = kNoTuple;
+        row[q] = b1[q] = b2[q] = 0;
         if (o < tot) {
+          have |= 1u << q;
           const uint32_t sl = s_slot[q * kSJT + t], l = o - s_off[sl];
-          const uint64_t row = base + (uint64_t)(sl % kSJI) * kSJT + sl / kSJI;
+          row[q] = sl % kSJI * kSJT + sl / kSJI;
           if constexpr (STAR) {
             const uint32_t c2 = s_cnt2[sl], l1 = l / c2;
-            idx[q] = set_tuple<FILTER>(j, probe, d, row, (uint64_t)s_start[sl] + l1,
-                                       (uint64_t)s_start2[sl] + (l - l1 * c2), bad);
+            b1[q] = s_start[sl] + l1;
+            b2[q] = s_start2[sl] + (l - l1 * c2);
           } else {
-            idx[q] = set_tuple<FILTER>(j, probe, d, row, (uint64_t)s_start[sl] + l, 0, bad);
+            b1[q] = s_start[sl] + l;
           }
         }
       }
+      set_tuples<FILTER, kSJI>(j, refs, have, base, row, b1, b2, idx, bad);
       if (bad && err) atomicOr(err, kErrCapacity);
       const uint32_t fresh = set_add_any<HASH, kSJI>(d, idx, total);
-      set_emit<kSJT, kSJI, true>(d, idx, fresh, out, 0, cursor, cap, red);
+      set_store<kSJT, kSJI>(j, d, refs, idx, fresh, cursor, cap, red);
       __syncthreads();  // the next window rewrites s_slot and red
     }
     __syncthreads();  // the next tile rewrites the slots
@@ -1066,8 +1237,9 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, co
                                                             uint32_t* err, HeavyList heavy) {
   static_assert(kHeavyChunk <= kSJTile, "a chunk is one window");
   __shared__ __align__(8) uint32_t red[kSJT / 32 + 2];
+  __shared__ SetRefs refs;
+  stage_refs(j, d, out, refs);
   const ColsIn probe = probe_cols(j);
-  if (j.dout) out = *j.dout;
   const uint32_t range = direct_range(j.ix);
   const uint64_t n = *heavy.n < heavy.cap ? *heavy.n : heavy.cap;
   for (uint64_t b = blockIdx.x; b < n; b += gridDim.x) {
@@ -1076,20 +1248,23 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, co
     lookup(j, probe, range, h.prow, &st);
     if constexpr (STAR) c2 = lookup2(j, probe, h.prow, &st2);
     uint64_t idx[kSJI];
+    uint32_t row[kSJI], b1[kSJI], b2[kSJI], have = 0;
     bool bad = false;
 #pragma unroll
     for (int q = 0; q < kSJI; ++q) {
       const uint32_t o = q * kSJT + threadIdx.x;
-      idx[q] = kNoTuple;
+      row[q] = b1[q] = b2[q] = 0;
       if (o < h.len && c2) {
+        have |= 1u << q;
         const uint32_t l = (uint32_t)h.out0 + o, l1 = STAR ? l / c2 : l;
-        idx[q] = set_tuple<FILTER>(j, probe, d, h.prow, (uint64_t)st + l1,
-                                   (uint64_t)st2 + (l - l1 * c2), bad);
+        b1[q] = st + l1;
+        b2[q] = st2 + (l - l1 * c2);
       }
     }
+    set_tuples<FILTER, kSJI>(j, refs, have, h.prow, row, b1, b2, idx, bad);
     if (bad && err) atomicOr(err, kErrCapacity);
     const uint32_t fresh = set_add_any<HASH, kSJI>(d, idx, total);
-    set_emit<kSJT, kSJI, true>(d, idx, fresh, out, 0, cursor, cap, red);
+    set_store<kSJT, kSJI>(j, d, refs, idx, fresh, cursor, cap, red);
     __syncthreads();  // the next chunk reuses red
   }
 }
