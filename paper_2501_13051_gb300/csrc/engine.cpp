@@ -437,12 +437,13 @@ constexpr uint32_t kMaxRels = 1024;
 // 3 single-pass join size, 4 overflow flag, 5 overflow flag of the round's
 // deferred checks, 8 + r fresh cursor of relation r,
 // 8 + kMaxRels + r delta size of relation r
-// 8 + 2 kMaxRels + s size of the round's s-th single-pass join into a set
+// 8 + 2 kMaxRels + 2 s size of the round's s-th single-pass join into a set,
+// then the number of its listed chunks
 constexpr uint32_t kSlotErr = 0, kSlotScratch = 1, kSlotAux = 2, kSlotDirTotal = 3,
                    kSlotOverflow = 4, kSlotRoundOverflow = 5, kSlotCursor = 8,
                    kSlotDelta = 8 + kMaxRels,
                    kSetSteps = 256, kSlotSetTotal = 8 + 2 * kMaxRels,
-                   kCtlSlots = 8 + 2 * kMaxRels + kSetSteps;
+                   kCtlSlots = 8 + 2 * kMaxRels + 2 * kSetSteps;
 constexpr int kEstFloats = 32;  // 16 features, the prediction, padding
 static_assert(kCtlSlots * sizeof(uint64_t) + kEstFloats * sizeof(float) <= PinnedBlocks::kBytes,
               "the host mirrors share one block");
@@ -552,6 +553,7 @@ struct cdl_engine {
   // the round (set_steps) leave their sizes in the control block.
   struct SetSeen {
     uint64_t probe = 0, outputs = 0;
+    bool chunks = true;  // it had rows with long ranges (or may have)
   };
   static constexpr uint64_t kSetRatio = 4;
   static constexpr uint64_t kSetHeavyCap = 1 << 16;  // chunks of long ranges
@@ -560,6 +562,7 @@ struct cdl_engine {
     std::tuple<size_t, size_t, size_t> key;
     uint32_t head;
     uint64_t probe;
+    bool chunks;  // the kernel for long ranges was launched
   };
   std::vector<SetStep> set_steps;
   bool delta_known = false;  // h_ctl holds the set relations' delta sizes
@@ -2129,7 +2132,7 @@ struct cdl_engine {
       const uint64_t total = h_ctl[kSlotScratch];
       ++joins;
       log_sample(total);
-      if (into_set) set_seen[step_key] = SetSeen{P.n, total};
+      if (into_set) set_seen[step_key] = SetSeen{P.n, total, true};
       if (recording) {  // a step of a capturable plan: hash join, static build side
         GStep g;
         g.rule = (size_t)(&rule - rules.data());
@@ -2215,11 +2218,10 @@ struct cdl_engine {
 
   bool set_heavy_list(uint64_t cap) {
     if (set_heavy_buf.p && set_heavy.cap >= cap) return true;
-    DBuf b = alloc(256 + sizeof(HeavyChunk) * cap);
+    DBuf b = alloc(sizeof(HeavyChunk) * cap);
     if (!b.p) return false;
     set_heavy_buf = std::move(b);
-    set_heavy.n = static_cast<uint64_t*>(set_heavy_buf.p);
-    set_heavy.e = reinterpret_cast<HeavyChunk*>(static_cast<char*>(set_heavy_buf.p) + 256);
+    set_heavy.e = static_cast<HeavyChunk*>(set_heavy_buf.p);
     set_heavy.cap = cap;
     return true;
   }
@@ -2260,17 +2262,21 @@ struct cdl_engine {
       if (r == CDL_OK && !ok) r = fail(CDL_E_NOMEM, "full set");
       if (r != CDL_OK) return r;
     }
-    const uint32_t slot = kSlotSetTotal + (uint32_t)set_steps.size();
+    const uint32_t slot = kSlotSetTotal + 2 * (uint32_t)set_steps.size();
+    // a step without long ranges last time goes without the launch for them
+    const auto last = set_seen.find(key);
+    const bool chunks = exact || last == set_seen.end() || last->second.chunks;
+    HeavyList list;
     // (an exact size also bounds the chunks: at most two per kHeavyChunk outputs)
     if (!set_heavy_list(std::max(kSetHeavyCap, 2 * exact / kHeavyChunk + 2)))
       return fail(CDL_E_NOMEM, "long ranges");
-    cudaError_t e = cudaMemsetAsync(set_heavy.n, 0, 8, st);
-    if (e == cudaSuccess)
-      e = join_set(ctx, js, H.fset, H.sdelta.out(), dslot(kSlotDelta + rule.head.rel), H.sdelta.cap,
-                   dslot(slot), set_heavy);
+    list = set_heavy;
+    list.n = dslot(slot + 1);  // (zeroed with the round's words)
+    cudaError_t e = join_set(ctx, js, H.fset, H.sdelta.out(), dslot(kSlotDelta + rule.head.rel),
+                             H.sdelta.cap, dslot(slot), list, chunks);
     if (e != cudaSuccess) return cuda_fail(e, "one-pass join");
     H.set_single = true;
-    set_steps.push_back(SetStep{key, rule.head.rel, np});
+    set_steps.push_back(SetStep{key, rule.head.rel, np, chunks});
     ++joins;
     return CDL_OK;
   }
@@ -2750,7 +2756,7 @@ struct cdl_engine {
     const uint32_t nr = (uint32_t)rels.size();
     bool sets = false;
     for (auto& r : rels) sets |= r->set_on;
-    const uint32_t end = sets ? kSlotSetTotal + (uint32_t)set_steps.size() : kSlotCursor + nr;
+    const uint32_t end = sets ? kSlotSetTotal + 2 * (uint32_t)set_steps.size() : kSlotCursor + nr;
     delta_known = sets;
     return fetch(kSlotRoundOverflow, end - kSlotRoundOverflow);
   }
@@ -2761,9 +2767,9 @@ struct cdl_engine {
     std::map<uint32_t, uint64_t> outputs;
     for (size_t i = 0; i < set_steps.size(); ++i) {
       const SetStep& t = set_steps[i];
-      const uint64_t total = h_ctl[kSlotSetTotal + i];
-      if (total & kSetListFull) redo[t.head] = any = true;
-      set_seen[t.key] = SetSeen{t.probe, total & (kSetListFull - 1)};
+      const uint64_t total = h_ctl[kSlotSetTotal + 2 * i], listed = h_ctl[kSlotSetTotal + 2 * i + 1];
+      if ((total & kSetListFull) || (listed && !t.chunks)) redo[t.head] = any = true;
+      set_seen[t.key] = SetSeen{t.probe, total & (kSetListFull - 1), listed != 0};
       prev_out[t.key] = total & (kSetListFull - 1);
       outputs[t.head] += total & (kSetListFull - 1);
     }
@@ -2888,7 +2894,7 @@ struct cdl_engine {
     s = fetch_round();
     if (s != CDL_OK) return s;
     for (size_t i = steps_before; i < set_steps.size(); ++i)
-      if (h_ctl[kSlotSetTotal + i] & kSetListFull)
+      if (h_ctl[kSlotSetTotal + 2 * i] & kSetListFull)
         return fail(CDL_E_CAPACITY, "a hash set ran out of slots");
     for (uint32_t i = 0; i < nr; ++i)
       if (redo[i] && h_ctl[kSlotCursor + i] > rels[i]->fresh.cap)
@@ -3120,10 +3126,10 @@ struct cdl_engine {
       GRelRes* H = g.last ? &grel[slot[g.head]] : nullptr;
       if (H && H->set) {
         js.dout = reinterpret_cast<const ColsOut*>(&g_next()[slot[g.head]].D);
-        e = cudaMemsetAsync(set_heavy.n, 0, 8, st);
-        if (e == cudaSuccess)
-          e = join_set(ctx, js, rels[g.head]->fset, ColsOut{}, g_cursor(slot[g.head]), H->Ucap,
-                       g_step(s, 0), set_heavy);
+        HeavyList list = set_heavy;
+        list.n = g_step(s, 1);  // (zero, as the round's end leaves it)
+        e = join_set(ctx, js, rels[g.head]->fset, ColsOut{}, g_cursor(slot[g.head]), H->Ucap,
+                     g_step(s, 0), list);
         continue;
       }
       uint64_t* cursor = g.last ? g_cursor(slot[g.head]) : g_step(s, 2);

@@ -41,7 +41,7 @@ __global__ void k_round_end(GraphRel* cur, GraphRel* next, uint32_t nrel, GraphC
   else if (ctl->max_iters && ctl->iterations > ctl->max_iters)
     ctl->done = 3;
   for (uint32_t i = 0; i < ncur; ++i) cursors[i] = 0;  // the next round appends from 0
-  for (uint32_t s = 0; s < nsteps; ++s) steps[3 * s] = steps[3 * s + 2] = 0;
+  for (uint32_t s = 0; s < nsteps; ++s) steps[3 * s] = steps[3 * s + 1] = steps[3 * s + 2] = 0;
   cudaGraphSetConditional(loop, ctl->done ? 0u : 1u);
 }
 

@@ -93,8 +93,13 @@ __global__ void __launch_bounds__(kThreads) k_index_build(const uint32_t* __rest
   const uint32_t a = __ldg(k0 + i);
   if (a >= range) return;
   uint32_t* e = reinterpret_cast<uint32_t*>(t) + 2ull * a;
-  if (i == 0 || __ldg(k0 + i - 1) != a) e[0] = (uint32_t)i;
-  if (i + 1 == n || __ldg(k0 + i + 1) != a) e[1] = (uint32_t)(i + 1);
+  const bool first = i == 0 || __ldg(k0 + i - 1) != a, last = i + 1 == n || __ldg(k0 + i + 1) != a;
+  if (first && last) {
+    *reinterpret_cast<uint2*>(e) = make_uint2((uint32_t)i, (uint32_t)(i + 1));
+  } else {
+    if (first) e[0] = (uint32_t)i;
+    if (last) e[1] = (uint32_t)(i + 1);
+  }
 }
 
 // Clears the form that *x.last gives.

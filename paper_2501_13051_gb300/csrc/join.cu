@@ -91,27 +91,105 @@ __device__ __forceinline__ ColsIn probe_cols(const JoinSpec& j) {
   return j.dprobe ? *j.dprobe : j.probe;
 }
 
+// Ranges of a thread's eight probe rows.  The direct form's reads go out
+// together; the hash form's probes are a loop each.
+template <int N>
+__device__ __forceinline__ void set_lookup(const JoinSpec& j, const KeyIndex& x, uint32_t range,
+                                           const uint32_t* c0, const uint32_t* c1, uint64_t base,
+                                           uint32_t live, uint32_t (&st)[N], uint32_t (&cnt)[N]) {
+  uint32_t k0[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    k0[q] = 0;
+    st[q] = cnt[q] = 0;
+    if ((live >> q) & 1u) k0[q] = __ldg(c0 + base + (uint64_t)q * kCT + threadIdx.x);
+  }
+  if (range) {
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (((live >> q) & 1u) && k0[q] < range) {
+        const uint2 e = __ldg(reinterpret_cast<const uint2*>(x.table) + k0[q]);
+        st[q] = e.x;
+        cnt[q] = e.y > e.x ? e.y - e.x : 0u;
+      }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if ((live >> q) & 1u) {
+      const uint32_t k1 = c1 ? __ldg(c1 + base + (uint64_t)q * kCT + threadIdx.x) : 0u;
+      cnt[q] = probe_table(x.table, x.slots - 1, k0[q], k1, &st[q]);
+    }
+}
+
+// Key columns of the probe side, for set_lookup.
+__device__ __forceinline__ const uint32_t* key_col(const ColsIn& probe, uint32_t v) {
+  return v == 0xFFu ? nullptr : col_of(probe, v);
+}
+
+// A thread's eight rows of a tile are looked up together: their keys, then
+// their entries, are in flight at once.  Points-to's 17 counts 421 -> 270 us;
+// 16M rows over 2^25 entries by key stay at 252 us, bound by the 256 MB
+// array's sectors (a read of one in 64 bytes of HBM for each row).
 __global__ void __launch_bounds__(kCT) k_join_count(const JoinSpec j, uint32_t* __restrict__ counts,
                                                     uint64_t* __restrict__ tile_sums,
                                                     uint32_t* err) {
   __shared__ uint64_t red[kCT / 32 + 1];
   const uint64_t n = dev_size(j.dn, j.n_probe);
   const ColsIn probe = probe_cols(j);
-  const uint32_t range = direct_range(j.ix);
+  const uint32_t *pk0 = key_col(probe, j.pk0), *pk1 = key_col(probe, j.pk1);
+  const uint32_t *qk0 = nullptr, *qk1 = nullptr;
+  if (j.star) {
+    qk0 = key_col(probe, j.qk0);
+    qk1 = key_col(probe, j.qk1);
+  }
+  const uint32_t range = direct_range(j.ix), range2 = j.star ? direct_range(j.ix2) : 0u;
   // tile 0 is written even for n == 0; blocks loop over the tiles
   const uint64_t ntiles = n ? (n + kScanTile - 1) / kScanTile : 1;
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const uint64_t base = tile * kScanTile;
-    uint64_t s = 0;
-#pragma unroll 4
-    for (int i = 0; i < kCItems; ++i) {
-      const uint64_t row = base + (uint64_t)i * kCT + threadIdx.x;
-      if (row < n) {
-        const uint32_t cnt = row_count(j, probe, range, row, err);
-        counts[row] = cnt;
-        s += cnt;
+    uint32_t live = 0, st[kCItems], cnt[kCItems];
+#pragma unroll
+    for (int i = 0; i < kCItems; ++i)
+      live |= (base + (uint64_t)i * kCT + threadIdx.x < n ? 1u : 0u) << i;
+    if (j.cross) {
+#pragma unroll
+      for (int i = 0; i < kCItems; ++i) {
+        st[i] = 0;
+        cnt[i] = (live >> i) & 1u ? j.n_build : 0u;
+      }
+    } else {
+      set_lookup<kCItems>(j, j.ix, range, pk0, pk1, base, live, st, cnt);
+    }
+    if (j.starts) {
+#pragma unroll
+      for (int i = 0; i < kCItems; ++i)
+        if ((live >> i) & 1u) j.starts[base + (uint64_t)i * kCT + threadIdx.x] = st[i];
+    }
+    if (j.hub_min) {  // hub_or's
+#pragma unroll
+      for (int i = 0; i < kCItems; ++i)
+        if (cnt[i] >= j.hub_min) cnt[i] = 0;
+    }
+    if (j.star) {
+      uint32_t found = 0, cnt2[kCItems];
+#pragma unroll
+      for (int i = 0; i < kCItems; ++i) found |= (cnt[i] ? 1u : 0u) << i;
+      set_lookup<kCItems>(j, j.ix2, range2, qk0, qk1, base, found, st, cnt2);
+#pragma unroll
+      for (int i = 0; i < kCItems; ++i) {
+        const uint64_t prod = (uint64_t)cnt[i] * cnt2[i];
+        if (prod > 0xFFFFFFFFull && err) atomicOr(err, kErrCapacity);
+        cnt[i] = prod > 0xFFFFFFFFull ? 0u : (uint32_t)prod;
       }
     }
+    uint64_t s = 0;
+#pragma unroll
+    for (int i = 0; i < kCItems; ++i)
+      if ((live >> i) & 1u) {
+        counts[base + (uint64_t)i * kCT + threadIdx.x] = cnt[i];
+        s += cnt[i];
+      }
     uint64_t total;
     block_exclusive_sum<kCT, uint64_t>(s, red, &total);  // ends with a barrier
     if (threadIdx.x == 0) tile_sums[tile] = total;
@@ -177,6 +255,172 @@ __device__ __forceinline__ uint32_t ref_value(const JoinSpec& j, const ColsIn& p
   return r.v;
 }
 
+// Where a launch's values come from, staged once per block: the head
+// columns, then the pairs of the equalities and of the inequalities.  The
+// loops over columns read this table and are not unrolled; only the loop over
+// a thread's outputs is, so that its loads are in flight together.  (With the
+// columns unrolled as well -- eight outputs times eight columns times the
+// sides a value may come from -- half of all warp cycles waited for
+// instructions: 77 ms of same generation on 200,000 nodes; 47 so.)
+struct SetRefs {
+  const uint32_t* p[kMaxK + 16];
+  uint32_t side[kMaxK + 16], v[kMaxK + 16];
+  uint32_t* out[kMaxK];
+  uint32_t shift[kMaxK], mask[kMaxK];
+};
+
+__device__ __forceinline__ void stage_refs(const JoinSpec& j, const DenseSet& d, const ColsOut& out,
+                                           SetRefs& s) {
+  const uint32_t t = threadIdx.x;
+  if (t < kMaxK + 16) {
+    Ref f{2, 0};
+    if (t < kMaxK) {
+      if (t < j.out_k) f = j.out[t];
+      s.out[t] = j.dout ? j.dout->c[t] : out.c[t];
+      s.shift[t] = d.shift[t];
+      s.mask[t] = d.mask[t];
+    } else {
+      const uint32_t i = t - kMaxK;
+      if (i < 2 * j.n_eq)
+        f = j.eq[i >> 1][i & 1];
+      else if (i < 2 * (j.n_eq + j.n_neq))
+        f = j.neq[(i >> 1) - j.n_eq][i & 1];
+    }
+    s.side[t] = f.side;
+    s.v[t] = f.v;
+    s.p[t] = f.side == 0 ? (j.dprobe ? j.dprobe->c[f.v] : j.probe.c[f.v])
+             : f.side == 1 ? j.build.c[f.v]
+             : f.side == 3 ? j.build2.c[f.v]
+                           : nullptr;
+  }
+  __syncthreads();
+}
+
+// Value i of the table for the N outputs in `live`: probe row base + row[q],
+// build rows b1[q] and b2[q].
+template <int N>
+__device__ __forceinline__ void set_values(const SetRefs& s, uint32_t i, uint32_t live,
+                                           uint64_t base, const uint32_t (&row)[N],
+                                           const uint32_t (&b1)[N], const uint32_t (&b2)[N],
+                                           uint32_t (&v)[N]) {
+  const uint32_t side = s.side[i];
+  const uint32_t* p = s.p[i] + (side == 0 ? base : 0ull);
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    v[q] = s.v[i];
+    if (side != 2 && ((live >> q) & 1u)) v[q] = __ldg(p + (side == 0 ? row[q] : side == 1 ? b1[q] : b2[q]));
+  }
+}
+
+// The outputs in `live` that pass the equalities and inequalities.
+template <int N>
+__device__ __forceinline__ uint32_t filter_outputs(const JoinSpec& j, const SetRefs& s,
+                                                   uint32_t live, uint64_t base,
+                                                   const uint32_t (&row)[N],
+                                                   const uint32_t (&b1)[N],
+                                                   const uint32_t (&b2)[N]) {
+#pragma unroll 1
+  for (uint32_t f = 0; f < j.n_eq + j.n_neq; ++f) {
+    uint32_t x[N], y[N];
+    set_values<N>(s, kMaxK + 2 * f, live, base, row, b1, b2, x);
+    set_values<N>(s, kMaxK + 2 * f + 1, live, base, row, b1, b2, y);
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if ((x[q] == y[q]) != (f < j.n_eq)) live &= ~(1u << q);
+  }
+  return live;
+}
+
+// Packed tuples of the outputs in `live` (kNoTuple: none, dropped by a filter
+// or outside the set's space, which sets bad).
+template <bool FILTER, int N>
+__device__ __forceinline__ void set_tuples(const JoinSpec& j, const SetRefs& s, uint32_t live,
+                                           uint64_t base, const uint32_t (&row)[N],
+                                           const uint32_t (&b1)[N], const uint32_t (&b2)[N],
+                                           uint64_t (&idx)[N], bool& bad) {
+  if (FILTER) live = filter_outputs<N>(j, s, live, base, row, b1, b2);
+  uint32_t out = 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q) idx[q] = 0;
+#pragma unroll 1
+  for (uint32_t k = 0; k < j.out_k; ++k) {
+    uint32_t v[N];
+    set_values<N>(s, k, live, base, row, b1, b2, v);
+    const uint32_t sh = s.shift[k], mask = s.mask[k];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      idx[q] |= (uint64_t)v[q] << sh;
+      out |= (v[q] > mask ? 1u : 0u) << q;
+    }
+  }
+  bad |= (out & live) != 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if (!((live & ~out) >> q & 1u)) idx[q] = kNoTuple;
+}
+
+// Places for a block's outputs in `mask`, packed at *cursor with one claim:
+// output q goes to *pos + at[q].  wsum: THREADS / 32 + 2 words.  false (for
+// the whole block) where there are none.
+template <int THREADS, int N>
+__device__ __forceinline__ bool claim_places(uint32_t mask, unsigned long long* cursor,
+                                             uint32_t* wsum, uint32_t (&at)[N], uint64_t* pos) {
+  constexpr int W = THREADS / 32;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, lt = (1u << lane) - 1u;
+  uint32_t n = 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const uint32_t bal = __ballot_sync(0xffffffffu, (mask >> q) & 1u);
+    at[q] = n + __popc(bal & lt);
+    n += __popc(bal);
+  }
+  if (lane == 0) wsum[warp] = n;
+  __syncthreads();
+  unsigned long long* claim = reinterpret_cast<unsigned long long*>(wsum + W);
+  uint32_t before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    const uint32_t c = wsum[w];
+    before += w < (int)warp ? c : 0u;
+    total += c;
+  }
+  if (total == 0) return false;
+  if (threadIdx.x == 0) *claim = atomicAdd(cursor, (unsigned long long)total);
+  __syncthreads();
+  *pos = *claim + before;
+  return true;
+}
+
+// New tuples (bit q of fresh) to the head's columns; those past cap are taken
+// out of the set again and true is returned to their threads.
+template <int THREADS, int N>
+__device__ __forceinline__ bool set_store(const JoinSpec& j, const DenseSet& d, const SetRefs& s,
+                                          const uint64_t (&idx)[N], uint32_t fresh,
+                                          unsigned long long* cursor, uint64_t cap, uint32_t* wsum) {
+  uint32_t at[N];
+  uint64_t pos;
+  if (!claim_places<THREADS, N>(fresh, cursor, wsum, at, &pos)) return false;
+  const uint64_t room = cap > pos ? cap - pos : 0;
+#pragma unroll 1
+  for (uint32_t k = 0; k < j.out_k; ++k) {
+    uint32_t* o = s.out[k] + pos;
+    const uint32_t sh = s.shift[k], mask = s.mask[k];
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (((fresh >> q) & 1u) && at[q] < room) o[at[q]] = (uint32_t)(idx[q] >> sh) & mask;
+  }
+  bool over = false;
+  if (room < (uint64_t)N * 32) {  // (rare: near or past the buffer's end)
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (((fresh >> q) & 1u) && at[q] >= room) {
+        set_remove(d, idx[q]);
+        over = true;
+      }
+  }
+  return over;
+}
+
 // Row heads: five resident blocks per SM (registers capped at 51).  Bitmap
 // heads: registers capped at 32, eight blocks per SM (seven for star joins,
 // bounded by shared memory); the bit-setting loop is latency-bound, and on
@@ -211,6 +455,8 @@ __global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5)
   __shared__ uint64_t s_split[2];
   __shared__ __align__(8) uint32_t red[kJT / 32 + 2];
   __shared__ unsigned long long s_base;
+  __shared__ SetRefs refs;
+  if constexpr (FORM == kSet) stage_refs(j, dset, out, refs);
   const uint64_t n_probe = dev_size(j.dn, j.n_probe);
   const ColsIn probe = probe_cols(j);
   // a device-given join size past the capacity the launch was sized for:
@@ -398,20 +644,30 @@ __global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5)
    }
   }
   if constexpr (FORM == kSet) {
-    uint64_t idx[kJItems];
-    bool bad = false;
+    // the block's outputs in one sweep, eight per thread side by side
+    uint32_t row[kJItems], b1[kJItems], b2[kJItems], live = 0;
 #pragma unroll
     for (int q = 0; q < kJItems; ++q) {
       const uint64_t o = o0 + (uint64_t)q * kJT + threadIdx.x;
-      uint32_t vals[kMaxK] = {0, 0, 0, 0};
-      idx[q] = kNoTuple;
-      if (o < o1 && tuple_at(o, vals)) {
-        idx[q] = set_pack(dset, vals);
-        bad |= idx[q] == kNoTuple;
+      row[q] = b1[q] = b2[q] = 0;
+      if (o < o1) {
+        live |= 1u << q;
+        const uint32_t r = s_row[o - o0], l = (uint32_t)(o - off_of(r));
+        row[q] = r;
+        if constexpr (STAR) {
+          const uint32_t c2 = s_cnt2[r], l1 = l / c2;
+          b1[q] = s_start[r] + l1;
+          b2[q] = s_start2[r] + (l - l1 * c2);
+        } else {
+          b1[q] = s_start[r] + l;
+        }
       }
     }
+    uint64_t idx[kJItems];
+    bool bad = false;
+    set_tuples<FILTER, kJItems>(j, refs, live, r_lo, row, b1, b2, idx, bad);
     const uint32_t fresh = set_add<kJItems>(dset, idx);
-    bad |= !set_emit<kJT, kJItems>(dset, idx, fresh, out, wbase, cursor, out_cap, red);
+    bad |= set_store<kJT, kJItems>(j, dset, refs, idx, fresh, cursor, out_cap, red);
     if (bad && err) atomicOr(err, kErrCapacity);
   }
   if constexpr (FORM == kRows)
@@ -903,6 +1159,7 @@ cudaError_t join_direct(Ctx& c, const JoinSpec& j, ColsOut out, uint64_t* d_curs
 // small closure takes one launch and one wait (4,001 nodes, 46 rounds: 4.9 ->
 // 2.6 ms).
 constexpr int kSJT = 256, kSJI = 8;
+static_assert(kSJT == kCT, "set_lookup's rows lie kCT apart");
 constexpr uint32_t kSJTile = kSJT * kSJI;
 
 // Both forms of the set; a full table is noted in *total.
@@ -914,176 +1171,6 @@ __device__ __forceinline__ uint32_t set_add_any(const DenseSet& d, const uint64_
   const uint32_t fresh = set_add_hash<N>(d, idx, &full);
   if (full) atomicOr(total, (unsigned long long)kSetListFull);
   return fresh;
-}
-
-// Where a launch's values come from, staged once per block: the head
-// columns, then the pairs of the equalities and of the inequalities.  The
-// loops over columns read this table and are not unrolled; only the loop over
-// a thread's outputs is, so that its loads are in flight together.  (With the
-// columns unrolled as well -- eight outputs times eight columns times the
-// sides a value may come from -- half of all warp cycles waited for
-// instructions: 77 ms of same generation on 200,000 nodes; 47 so.)
-struct SetRefs {
-  const uint32_t* p[kMaxK + 16];
-  uint32_t side[kMaxK + 16], v[kMaxK + 16];
-  uint32_t* out[kMaxK];
-  uint32_t shift[kMaxK], mask[kMaxK];
-};
-
-__device__ __forceinline__ void stage_refs(const JoinSpec& j, const DenseSet& d, const ColsOut& out,
-                                           SetRefs& s) {
-  const uint32_t t = threadIdx.x;
-  if (t < kMaxK + 16) {
-    Ref f{2, 0};
-    if (t < kMaxK) {
-      if (t < j.out_k) f = j.out[t];
-      s.out[t] = j.dout ? j.dout->c[t] : out.c[t];
-      s.shift[t] = d.shift[t];
-      s.mask[t] = d.mask[t];
-    } else {
-      const uint32_t i = t - kMaxK;
-      if (i < 2 * j.n_eq)
-        f = j.eq[i >> 1][i & 1];
-      else if (i < 2 * (j.n_eq + j.n_neq))
-        f = j.neq[(i >> 1) - j.n_eq][i & 1];
-    }
-    s.side[t] = f.side;
-    s.v[t] = f.v;
-    s.p[t] = f.side == 0 ? (j.dprobe ? j.dprobe->c[f.v] : j.probe.c[f.v])
-             : f.side == 1 ? j.build.c[f.v]
-             : f.side == 3 ? j.build2.c[f.v]
-                           : nullptr;
-  }
-  __syncthreads();
-}
-
-// Value i of the table for the N outputs in `live`: probe row base + row[q],
-// build rows b1[q] and b2[q].
-template <int N>
-__device__ __forceinline__ void set_values(const SetRefs& s, uint32_t i, uint32_t live,
-                                           uint64_t base, const uint32_t (&row)[N],
-                                           const uint32_t (&b1)[N], const uint32_t (&b2)[N],
-                                           uint32_t (&v)[N]) {
-  const uint32_t side = s.side[i];
-  const uint32_t* p = s.p[i] + (side == 0 ? base : 0ull);
-#pragma unroll
-  for (int q = 0; q < N; ++q) {
-    v[q] = s.v[i];
-    if (side != 2 && ((live >> q) & 1u)) v[q] = __ldg(p + (side == 0 ? row[q] : side == 1 ? b1[q] : b2[q]));
-  }
-}
-
-// Packed tuples of the outputs in `live` (kNoTuple: none, dropped by a filter
-// or outside the set's space, which sets bad).
-template <bool FILTER, int N>
-__device__ __forceinline__ void set_tuples(const JoinSpec& j, const SetRefs& s, uint32_t live,
-                                           uint64_t base, const uint32_t (&row)[N],
-                                           const uint32_t (&b1)[N], const uint32_t (&b2)[N],
-                                           uint64_t (&idx)[N], bool& bad) {
-  if (FILTER) {
-#pragma unroll 1
-    for (uint32_t f = 0; f < j.n_eq + j.n_neq; ++f) {
-      uint32_t x[N], y[N];
-      set_values<N>(s, kMaxK + 2 * f, live, base, row, b1, b2, x);
-      set_values<N>(s, kMaxK + 2 * f + 1, live, base, row, b1, b2, y);
-#pragma unroll
-      for (int q = 0; q < N; ++q)
-        if ((x[q] == y[q]) != (f < j.n_eq)) live &= ~(1u << q);
-    }
-  }
-  uint32_t out = 0;
-#pragma unroll
-  for (int q = 0; q < N; ++q) idx[q] = 0;
-#pragma unroll 1
-  for (uint32_t k = 0; k < j.out_k; ++k) {
-    uint32_t v[N];
-    set_values<N>(s, k, live, base, row, b1, b2, v);
-    const uint32_t sh = s.shift[k], mask = s.mask[k];
-#pragma unroll
-    for (int q = 0; q < N; ++q) {
-      idx[q] |= (uint64_t)v[q] << sh;
-      out |= (v[q] > mask ? 1u : 0u) << q;
-    }
-  }
-  bad |= (out & live) != 0;
-#pragma unroll
-  for (int q = 0; q < N; ++q)
-    if (!((live & ~out) >> q & 1u)) idx[q] = kNoTuple;
-}
-
-// As set_emit with CLEAR, the columns from the staged table.
-template <int THREADS, int N>
-__device__ __forceinline__ void set_store(const JoinSpec& j, const DenseSet& d, const SetRefs& s,
-                                          const uint64_t (&idx)[N], uint32_t fresh,
-                                          unsigned long long* cursor, uint64_t cap, uint32_t* wsum) {
-  constexpr int W = THREADS / 32;
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, lt = (1u << lane) - 1u;
-  uint32_t at[N], n = 0;
-#pragma unroll
-  for (int q = 0; q < N; ++q) {
-    const uint32_t bal = __ballot_sync(0xffffffffu, (fresh >> q) & 1u);
-    at[q] = n + __popc(bal & lt);
-    n += __popc(bal);
-  }
-  if (lane == 0) wsum[warp] = n;
-  __syncthreads();
-  unsigned long long* claim = reinterpret_cast<unsigned long long*>(wsum + W);
-  uint32_t before = 0, total = 0;
-#pragma unroll
-  for (int w = 0; w < W; ++w) {
-    const uint32_t c = wsum[w];
-    before += w < (int)warp ? c : 0u;
-    total += c;
-  }
-  if (total == 0) return;  // uniform
-  if (threadIdx.x == 0) *claim = atomicAdd(cursor, (unsigned long long)total);
-  __syncthreads();
-  const uint64_t pos = *claim + before;
-  const uint64_t room = cap > pos ? cap - pos : 0;
-#pragma unroll 1
-  for (uint32_t k = 0; k < j.out_k; ++k) {
-    uint32_t* o = s.out[k] + pos;
-    const uint32_t sh = s.shift[k], mask = s.mask[k];
-#pragma unroll
-    for (int q = 0; q < N; ++q)
-      if (((fresh >> q) & 1u) && at[q] < room) o[at[q]] = (uint32_t)(idx[q] >> sh) & mask;
-  }
-  if (n > room) {  // (rare: past the buffer)
-#pragma unroll
-    for (int q = 0; q < N; ++q)
-      if (((fresh >> q) & 1u) && at[q] >= room) set_remove(d, idx[q]);
-  }
-}
-
-// Ranges of a thread's eight probe rows.  The direct form's reads go out
-// together; the hash form's probes are a loop each.
-template <int N>
-__device__ __forceinline__ void set_lookup(const JoinSpec& j, const KeyIndex& x, uint32_t range,
-                                           const uint32_t* c0, const uint32_t* c1, uint64_t base,
-                                           uint32_t live, uint32_t (&st)[N], uint32_t (&cnt)[N]) {
-  uint32_t k0[N];
-#pragma unroll
-  for (int q = 0; q < N; ++q) {
-    k0[q] = 0;
-    st[q] = cnt[q] = 0;
-    if ((live >> q) & 1u) k0[q] = __ldg(c0 + base + (uint64_t)q * kSJT + threadIdx.x);
-  }
-  if (range) {
-#pragma unroll
-    for (int q = 0; q < N; ++q)
-      if (((live >> q) & 1u) && k0[q] < range) {
-        const uint2 e = __ldg(reinterpret_cast<const uint2*>(x.table) + k0[q]);
-        st[q] = e.x;
-        cnt[q] = e.y > e.x ? e.y - e.x : 0u;
-      }
-    return;
-  }
-#pragma unroll
-  for (int q = 0; q < N; ++q)
-    if ((live >> q) & 1u) {
-      const uint32_t k1 = c1 ? __ldg(c1 + base + (uint64_t)q * kSJT + threadIdx.x) : 0u;
-      cnt[q] = probe_table(x.table, x.slots - 1, k0[q], k1, &st[q]);
-    }
 }
 
 template <bool FILTER, bool STAR, bool HASH>
@@ -1270,7 +1357,7 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, co
 }
 
 cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, uint64_t* d_cursor,
-                     uint64_t out_cap, uint64_t* d_total, const HeavyList& heavy) {
+                     uint64_t out_cap, uint64_t* d_total, const HeavyList& heavy, bool run_chunks) {
   if (j.n_probe == 0) return cudaSuccess;
   const bool filter = j.n_neq > 0 || j.n_eq > 0;
   // rows per thread: eight once four blocks per SM are busy, else fewer
@@ -1282,7 +1369,7 @@ cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, 
   auto* tot = reinterpret_cast<unsigned long long*>(d_total);
   auto launch = [&](auto rows, auto chunks) {
     rows<<<grid, kSJT, 0, c.st>>>(j, d, out, cur, out_cap, tot, c.d_err, (uint32_t)per, heavy);
-    chunks<<<152, kSJT, 0, c.st>>>(j, d, out, cur, out_cap, tot, c.d_err, heavy);
+    if (run_chunks) chunks<<<152, kSJT, 0, c.st>>>(j, d, out, cur, out_cap, tot, c.d_err, heavy);
   };
 #define CDL_JOIN_SET(F, S)                                                             \
   d.keys ? launch(k_join_set<F, S, true>, k_join_set_heavy<F, S, true>)                \

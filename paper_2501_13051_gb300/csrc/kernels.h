@@ -200,11 +200,13 @@ cudaError_t join_write(Ctx& c, const JoinSpec& j, const uint64_t* d_off, uint64_
 // and joins again.  *d_total grows by the join's size, with kSetListFull set in
 // it when the list of long ranges (heavy, as join_direct's, its counter
 // zeroed by the caller) was too short or a hash set full: then too the join
-// runs again.
+// runs again.  chunks false: the listed chunks are left alone (the caller
+// expects none, and runs the join again should *heavy.n tell otherwise).
 struct HeavyList;
 constexpr uint64_t kSetListFull = 1ull << 62;
 cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, uint64_t* d_cursor,
-                     uint64_t out_cap, uint64_t* d_total, const HeavyList& heavy);
+                     uint64_t out_cap, uint64_t* d_total, const HeavyList& heavy,
+                     bool chunks = true);
 
 // -------------------------------------------------------------- dense sets
 // Bits of n rows set in d (a row outside d raises kErrCapacity).
@@ -399,8 +401,8 @@ struct GraphCtl {
 // Where Full is a set next.nD is the relation's cursor; a cursor past
 // set_cap, more rows than set_full or kSetListFull in a step's first word is
 // an overflow as well.
-// It also zeroes the next round's cursors: `ncur` words at `cursors`, and of
-// the three words of each of the `nsteps` steps the first and the last.
+// It also zeroes the next round's cursors, `ncur` words at `cursors`, and the
+// three words of each of the `nsteps` steps.
 cudaError_t round_end(Ctx& c, GraphRel* cur, GraphRel* next, uint32_t nrel, GraphCtl* ctl,
                       uint64_t* per_round, uint64_t per_round_cap,
                       cudaGraphConditionalHandle loop, uint64_t* cursors, uint32_t ncur,
