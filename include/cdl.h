@@ -461,9 +461,11 @@ cdl_status cdl_join_write(const uint32_t* const* probe_cols, uint32_t probe_arit
                           uint32_t nneq, uint32_t* const* out_cols, uint64_t out_cap,
                           uint64_t* n_out, void* workspace, const size_t* ws_bytes, void* stream);
 
-/* Step (c): sorts n tuples of arity columns lexicographically (LSD radix
- * sort, stable), drops repeats, writes the unique tuples to out_cols and
- * their number to *n_out.  cols are left unchanged. */
+/* Step (c): sorts n tuples of arity columns lexicographically, drops
+ * repeats, writes the unique tuples to out_cols and their number to *n_out.
+ * cols are left unchanged (unless out_cols lie over them).  By size and
+ * shape the sort is one block's (up to 4,096 tuples), a bitmap of the tuple
+ * space, buckets sorted in shared memory, or LSD radix passes. */
 cdl_status cdl_sort_unique(const uint32_t* const* cols, uint32_t arity, uint64_t n,
                            uint32_t* const* out_cols, uint64_t* n_out, void* workspace,
                            size_t* ws_bytes, void* stream);

@@ -9,7 +9,7 @@
 //
 // The combined sequence is cut into tiles of 4096 items by merge-path splits
 // (Green, McColl & Bader, "GPU merge path", ICS 2012), computed for all
-// tiles at once by a small kernel with one thread per split.  Then:
+// tiles at once by a small kernel with one warp or thread per split.  Then:
 //   count  -- per tile, every New tuple finds its co-rank in the tile's Full
 //             slice (how many of its Full tuples are <= it) and whether it
 //             repeats a Full tuple.  A tile whose New tuples are at least a
@@ -54,17 +54,36 @@ __device__ __forceinline__ bool g_le(const ColsIn& a, uint64_t i, const ColsIn& 
   return true;
 }
 
-// Number of Full tuples among the first d of the merged order.
-template <int K>
+// Number of Full tuples among the first d of the merged order.  WARP: by a
+// whole warp, which tests 32 places a step, so that a split among 50M tuples
+// is five dependent reads away instead of 26.  That is the faster form while
+// there are few splits (an OWL-RL fixpoint of 135 merges of 0.1M to 5M rows,
+// 14.6 us of splits each by single threads: 46.9 -> 42.2 ms together with the
+// grouped loads' copies); with many, single threads hide their latency behind
+// one another and read less (a merge of 50M and 6M pairs: 504 us by threads,
+// 514 by warps).
+constexpr uint64_t kWarpSplits = 4096;
+template <int K, bool WARP>
 __device__ __forceinline__ uint64_t merge_split(const ColsIn& F, uint64_t nF, const ColsIn& U,
                                                 uint64_t nU, uint64_t d) {
   uint64_t lo = d > nU ? d - nU : 0, hi = d < nF ? d : nF;
+  const uint32_t lane = lane_id();
   while (lo < hi) {
-    const uint64_t mid = lo + ((hi - lo) >> 1);
-    if (g_le<K>(F, mid, U, d - mid - 1))
-      lo = mid + 1;
-    else
-      hi = mid;
+    if constexpr (WARP) {
+      const uint64_t step = (hi - lo + 32) / 33;
+      const uint64_t mid = lo + (lane + 1) * step - 1;
+      const bool le = mid < hi && g_le<K>(F, mid, U, d - mid - 1);
+      const uint32_t c = __popc(__ballot_sync(0xffffffffu, le));  // (the first c places)
+      const uint64_t next = lo + (c + 1) * step - 1;  // the first place tested false, if any was
+      lo += c * step;
+      if (c < 32 && next < hi) hi = next;
+    } else {
+      const uint64_t mid = lo + ((hi - lo) >> 1);
+      if (g_le<K>(F, mid, U, d - mid - 1))
+        lo = mid + 1;
+      else
+        hi = mid;
+    }
   }
   return lo;
 }
@@ -81,20 +100,23 @@ __device__ __forceinline__ bool resolve(const DevMerge& dm, ColsIn& F, uint64_t&
   return nF + nU <= dm.cap_merged;
 }
 
-template <int K>
+template <int K, bool WARP>
 __global__ void k_merge_splits(ColsIn F, uint64_t nF, ColsIn U, uint64_t nU,
                                uint64_t* __restrict__ splits, uint64_t ntiles, DevMerge dm,
                                uint64_t* d_tiles) {
-  const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t t = WARP ? i >> 5 : i;
+  const bool first = i == 0;
   const bool fits = resolve(dm, F, nF, nU, ntiles);
-  if (d_tiles && t == 0) *d_tiles = fits ? ntiles : 0;  // the scan's length (0: nothing fits)
+  if (d_tiles && first) *d_tiles = fits ? ntiles : 0;  // the scan's length (0: nothing fits)
   if (!fits) {
-    if (t == 0) atomicOr(dm.overflow, 1u);
+    if (first) atomicOr(dm.overflow, 1u);
     return;
   }
   if (t > ntiles) return;
   const uint64_t d = t * kDTile < nF + nU ? t * kDTile : nF + nU;
-  splits[t] = merge_split<K>(F, nF, U, nU, d);
+  const uint64_t at = merge_split<K, WARP>(F, nF, U, nU, d);
+  if (!WARP || lane_id() == 0) splits[t] = at;
 }
 
 // Co-ranks (or kRepeat) of the New tuples j + 32 q, q < Q (those below b1),
@@ -526,8 +548,12 @@ cudaError_t run_diff_merge(Ctx& c, ColsIn full, uint64_t n_full, ColsIn fresh, u
   {
     // New read, co-ranks written; Full sectors are read only where touched
     ProfScope p(c, kDiffCount, (4.0 * K + 4.0) * n_fresh);
-    k_merge_splits<K><<<(unsigned)((tiles + 1 + 255) / 256), 256, 0, c.st>>>(
-        full, n_full, fresh, n_fresh, splits, tiles, dm, d_tiles);
+    if (tiles < kWarpSplits)
+      k_merge_splits<K, true><<<(unsigned)((tiles + 1 + 7) / 8), 256, 0, c.st>>>(
+          full, n_full, fresh, n_fresh, splits, tiles, dm, d_tiles);
+    else
+      k_merge_splits<K, false><<<(unsigned)((tiles + 1 + 255) / 256), 256, 0, c.st>>>(
+          full, n_full, fresh, n_fresh, splits, tiles, dm, d_tiles);
     k_count_new<K><<<(unsigned)count_grid, kDT, smem_count, c.st>>>(
         full, fresh, n_full, n_fresh, splits, corank, cnt, tiles, dm, (uint32_t)group);
   }

@@ -1454,7 +1454,7 @@ struct cdl_engine {
     cudaError_t e = cudaSuccess;
     if (ix->range) {
       ix->distinct = std::min(bound, s.n);
-    } else if (!counted && s.n <= kUncountedRows) {
+    } else if (!counted && !opt.mem_limit && s.n <= kUncountedRows) {
       ix->distinct = s.n;
     } else {
       e = count_heads(ctx, k0, k1, s.n, dslot(kSlotScratch));
@@ -3466,11 +3466,6 @@ struct cdl_engine {
           R.version[kFull]++;
           continue;
         }
-        e = cudaMemsetAsync(dslot(kSlotDelta + i), 0, 8, st);
-        if (e != cudaSuccess) {
-          status = cuda_fail(e, "delta reset");
-          break;
-        }
         if (R.dset.words) {  // the dense form: the round's rows come out sorted and unique
           DCols rows = std::move(R.dense_rows);
           if (rows.n == 0) continue;
@@ -3722,7 +3717,7 @@ struct cdl_engine {
           std::fclose(f);
           return cuda_fail(e, "checkpoint check");
         }
-        cdl_status r = fetch(kSlotScratch + 1, 2);
+        cdl_status r = fetch(kSlotScratch + 1, 4);
         if (r != CDL_OK) {
           std::fclose(f);
           return r;
@@ -3756,10 +3751,10 @@ struct cdl_engine {
                                       st);
       if (e != cudaSuccess) return cuda_fail(e, "load copy");
     }
-    uint32_t* dmax = reinterpret_cast<uint32_t*>(dslot(kSlotScratch + 1));  // slots 2..3
+    uint32_t* dmax = reinterpret_cast<uint32_t*>(dslot(kSlotScratch + 1));  // slots 2..5
     cudaError_t e = check_values(ctx, in.in(), R.arity, n, dmax);
     if (e != cudaSuccess) return cuda_fail(e, "load check");
-    cdl_status r = fetch(kSlotScratch + 1, 2);
+    cdl_status r = fetch(kSlotScratch + 1, 4);
     if (r != CDL_OK) {
       cudaMemsetAsync(dslot(kSlotErr), 0, 8, st);
       return r;
@@ -3839,16 +3834,32 @@ struct cdl_engine {
     if (!alloc_cols(comb, k + 1, N) || !doff.p) return fail(CDL_E_NOMEM, "grouped load");
     comb.n = N;
     cudaError_t e = cudaMemcpyAsync(doff.p, off.data(), 8 * off.size(), cudaMemcpyHostToDevice, st);
-    for (uint32_t g = 0; g < ng && e == cudaSuccess; ++g) {
-      uint64_t at = off[g];
-      for (const DCols& p : rels[grp[g]]->pending) {
-        for (uint32_t c = 0; c < k && e == cudaSuccess; ++c)
-          e = cudaMemcpyAsync(comb.c[c + 1] + at, p.c[c], 4 * p.n, cudaMemcpyDeviceToDevice, st);
-        at += p.n;
+    // one load each, as a rule: all put together by one kernel (for 202
+    // relations that and the split below take the place of 808 copies)
+    bool single = true;
+    for (uint32_t i : grp) single &= rels[i]->pending.size() == 1;
+    DBuf dsrc;
+    if (single && e == cudaSuccess) {
+      std::vector<ColsIn> src;
+      for (uint32_t i : grp) src.push_back(rels[i]->pending[0].in());
+      dsrc = alloc(sizeof(ColsIn) * ng);
+      if (!dsrc.p) return fail(CDL_E_NOMEM, "grouped load");
+      e = cudaMemcpyAsync(dsrc.p, src.data(), sizeof(ColsIn) * ng, cudaMemcpyHostToDevice, st);
+      if (e == cudaSuccess)
+        e = concat_segments(ctx, comb.out(), static_cast<const ColsIn*>(dsrc.p), k,
+                            static_cast<const uint64_t*>(doff.p), ng, N);
+    } else {
+      for (uint32_t g = 0; g < ng && e == cudaSuccess; ++g) {
+        uint64_t at = off[g];
+        for (const DCols& p : rels[grp[g]]->pending) {
+          for (uint32_t c = 0; c < k && e == cudaSuccess; ++c)
+            e = cudaMemcpyAsync(comb.c[c + 1] + at, p.c[c], 4 * p.n, cudaMemcpyDeviceToDevice, st);
+          at += p.n;
+        }
       }
+      if (e == cudaSuccess)
+        e = fill_segments(ctx, comb.c[0], static_cast<const uint64_t*>(doff.p), ng, N);
     }
-    if (e == cudaSuccess)
-      e = fill_segments(ctx, comb.c[0], static_cast<const uint64_t*>(doff.p), ng, N);
     if (e != cudaSuccess) return cuda_fail(e, "grouped load");
     for (uint32_t i : grp) rels[i]->pending.clear();
     uint32_t bits[kMaxK] = {bits_of(ng - 1), 0, 0, 0};
@@ -3873,17 +3884,24 @@ struct cdl_engine {
     if (e == cudaSuccess) e = cudaMemcpyAsync(b.data(), db.p, 8 * b.size(), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "grouped load");
+    std::vector<ColsOut> dst;
     for (uint32_t g = 0; g < ng; ++g) {
       Relation& R = *rels[grp[g]];
       const uint64_t cnt = b[g + 1] - b[g];
       if (!alloc_cols(R.full, k, std::max<uint64_t>(cnt, 1))) return fail(CDL_E_NOMEM, "grouped load");
-      for (uint32_t c = 0; c < k && cnt; ++c) {
-        e = cudaMemcpyAsync(R.full.c[c], uniq.c[c + 1] + b[g], 4 * cnt, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return cuda_fail(e, "grouped load");
-      }
+      dst.push_back(R.full.out());
       R.full.n = cnt;
       R.version[kFull]++;
     }
+    DBuf ddst = alloc(sizeof(ColsOut) * ng);
+    if (!ddst.p) return fail(CDL_E_NOMEM, "grouped load");
+    ColsIn rows{};
+    for (uint32_t c = 0; c < k; ++c) rows.c[c] = uniq.c[c + 1];
+    e = cudaMemcpyAsync(ddst.p, dst.data(), sizeof(ColsOut) * ng, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+      e = split_segments(ctx, rows, static_cast<const ColsOut*>(ddst.p), k,
+                         static_cast<const uint64_t*>(db.p), ng, nu);
+    if (e != cudaSuccess) return cuda_fail(e, "grouped load");
     evict_stale();
     return CDL_OK;
   }

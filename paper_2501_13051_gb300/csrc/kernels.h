@@ -449,6 +449,10 @@ cudaError_t fill_segments(Ctx& c, uint32_t* col, const uint64_t* off, uint32_t n
 // c < k <= 3.
 cudaError_t concat_segments(Ctx& c, ColsOut out, const ColsIn* src, uint32_t k,
                             const uint64_t* off, uint32_t nseg, uint64_t total);
+// The reverse: row j of in, in segment s, goes to row j - off[s] of dst[s]
+// (k columns; dst and off in device memory).
+cudaError_t split_segments(Ctx& c, ColsIn in, const ColsOut* dst, uint32_t k, const uint64_t* off,
+                           uint32_t nseg, uint64_t total);
 // bounds[i] (i = 0..n_instances) = first row of the sorted column inst whose
 // value is >= i: instance i occupies rows [bounds[i], bounds[i + 1]).
 cudaError_t instance_bounds(Ctx& c, const uint32_t* inst, uint64_t n, uint32_t n_instances,

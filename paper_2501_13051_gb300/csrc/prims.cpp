@@ -331,8 +331,13 @@ cdl_status cdl_sort_unique(const uint32_t* const* cols, uint32_t arity, uint64_t
       return e == cudaSuccess ? finish() : CDL_E_CUDA;
     }
   }
+  // (wide tuples are read again while the output is written: not over the input)
+  bool overlap = false;
+  for (uint32_t i = 0; i < arity; ++i)
+    for (uint32_t j = 0; j < arity; ++j)
+      overlap |= out_cols[i] < cols[j] + n && cols[j] < out_cols[i] + n;
   BucketPlan bp;
-  if (bucket_plan(arity, bits, max, n, bp) &&
+  if (bucket_plan(arity, bits, max, n, bp) && (bp.keys == bp.k || !overlap) &&
       bucket_workspace(bp) <= up(radix_workspace(n, 9)) + up(diff_merge_workspace(0, n)) &&
       (bp.keys < bp.k ? 12 : 8) * n <= 2 * arity * col) {
     e = bucket_count(c, bp, in, n, rws, head + 3);

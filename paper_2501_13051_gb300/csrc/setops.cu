@@ -203,6 +203,36 @@ __global__ void k_concat_segments(ColsOut out, const ColsIn* __restrict__ src, u
   }
 }
 
+// The reverse: row j of segment s goes to row j - off[s] of dst[s].
+__global__ void k_split_segments(ColsIn in, const ColsOut* __restrict__ dst, uint32_t k,
+                                 const uint64_t* __restrict__ off, uint32_t nseg, uint64_t total) {
+  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < total;
+       j += (uint64_t)gridDim.x * blockDim.x) {
+    uint32_t lo = 0, hi = nseg;  // the last segment starting at or before j
+    while (hi - lo > 1) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (__ldg(off + mid) <= j)
+        lo = mid;
+      else
+        hi = mid;
+    }
+    const uint64_t r = j - __ldg(off + lo);
+#pragma unroll
+    for (uint32_t c = 0; c < (uint32_t)kMaxK; ++c)
+      if (c < k) dst[lo].c[c][r] = __ldg(in.c[c] + j);
+  }
+}
+
+cudaError_t split_segments(Ctx& c, ColsIn in, const ColsOut* dst, uint32_t k, const uint64_t* off,
+                           uint32_t nseg, uint64_t total) {
+  if (total == 0 || nseg == 0) return cudaSuccess;
+  ProfScope p(c, kMisc, 8.0 * k * total);
+  uint64_t blocks = (total + 255) / 256;
+  if (blocks > 152 * 16) blocks = 152 * 16;
+  k_split_segments<<<(unsigned)blocks, 256, 0, c.st>>>(in, dst, k, off, nseg, total);
+  return cudaGetLastError();
+}
+
 cudaError_t concat_segments(Ctx& c, ColsOut out, const ColsIn* src, uint32_t k,
                             const uint64_t* off, uint32_t nseg, uint64_t total) {
   if (total == 0 || nseg == 0) return cudaSuccess;
