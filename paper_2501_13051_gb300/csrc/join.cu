@@ -91,7 +91,7 @@ __device__ __forceinline__ ColsIn probe_cols(const JoinSpec& j) {
   return j.dprobe ? *j.dprobe : j.probe;
 }
 
-// Ranges of a thread's eight probe rows.  The direct form's reads go out
+// Ranges of a thread's N probe rows.  The direct form's reads go out
 // together; the hash form's probes are a loop each.
 template <int N>
 __device__ __forceinline__ void set_lookup(const JoinSpec& j, const KeyIndex& x, uint32_t range,
@@ -1149,16 +1149,18 @@ cudaError_t join_direct(Ctx& c, const JoinSpec& j, ColsOut out, uint64_t* d_curs
 // ------------------------------------------------ single pass into a set
 // Where Full is a bitmap a join needs no place computed for its outputs: the
 // new ones are packed as they come.  So no count and no scan run; a block
-// takes a tile of probe rows (eight per thread; fewer where that leaves
+// takes a tile of probe rows (four per thread; fewer where that leaves
 // blocks idle), looks them up, scans their output counts in shared memory
-// and walks the outputs in windows of eight per thread as k_join_write does.
+// and walks the outputs in windows of four per thread as k_join_write does.
 // Rows with more than kHeavyChunk outputs are listed and taken in chunks by
 // a second kernel, so that one hot key does not hold one block.
 // Bound by the random accesses to the bitmap.  Same generation on 200,000
 // nodes: 25 ms of counts and scans and 66 of writes become 47 ms; a round of a
 // small closure takes one launch and one wait (4,001 nodes, 46 rounds: 4.9 ->
-// 2.6 ms).
-constexpr int kSJT = 256, kSJI = 8;
+// 2.3 ms).  Four rows and outputs a thread in 48 registers and five blocks per
+// SM: 57.1 ms for the run on 200,000 nodes (six blocks, 40 registers, 57.4;
+// eight rows in four blocks 62.7, in five blocks, spilling, 77.8).
+constexpr int kSJT = 256, kSJI = 4, kSJH = 8;
 static_assert(kSJT == kCT, "set_lookup's rows lie kCT apart");
 constexpr uint32_t kSJTile = kSJT * kSJI;
 
@@ -1174,11 +1176,11 @@ __device__ __forceinline__ uint32_t set_add_any(const DenseSet& d, const uint64_
 }
 
 template <bool FILTER, bool STAR, bool HASH>
-__global__ void __launch_bounds__(kSJT, 4) k_join_set(const JoinSpec j, const DenseSet d, ColsOut out,
+__global__ void __launch_bounds__(kSJT, 5) k_join_set(const JoinSpec j, const DenseSet d, ColsOut out,
                                                       unsigned long long* cursor, uint64_t cap,
                                                       unsigned long long* total, uint32_t* err,
                                                       uint32_t per, HeavyList heavy) {
-  // row q of thread t is slot 8 t + q; slots lie in the order of their outputs
+  // row q of thread t is slot kSJI t + q; slots lie in the order of their outputs
   __shared__ uint32_t s_off[kSJTile], s_start[kSJTile];
   __shared__ uint32_t s_start2[STAR ? kSJTile : 1], s_cnt2[STAR ? kSJTile : 1];
   __shared__ uint16_t s_slot[kSJTile];
@@ -1322,7 +1324,7 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, co
                                                             uint64_t cap,
                                                             unsigned long long* total,
                                                             uint32_t* err, HeavyList heavy) {
-  static_assert(kHeavyChunk <= kSJTile, "a chunk is one window");
+  static_assert(kHeavyChunk <= kSJT * kSJH, "a chunk is one window");
   __shared__ __align__(8) uint32_t red[kSJT / 32 + 2];
   __shared__ SetRefs refs;
   stage_refs(j, d, out, refs);
@@ -1334,11 +1336,11 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, co
     uint32_t st = 0, st2 = 0, c2 = 1;
     lookup(j, probe, range, h.prow, &st);
     if constexpr (STAR) c2 = lookup2(j, probe, h.prow, &st2);
-    uint64_t idx[kSJI];
-    uint32_t row[kSJI], b1[kSJI], b2[kSJI], have = 0;
+    uint64_t idx[kSJH];
+    uint32_t row[kSJH], b1[kSJH], b2[kSJH], have = 0;
     bool bad = false;
 #pragma unroll
-    for (int q = 0; q < kSJI; ++q) {
+    for (int q = 0; q < kSJH; ++q) {
       const uint32_t o = q * kSJT + threadIdx.x;
       row[q] = b1[q] = b2[q] = 0;
       if (o < h.len && c2) {
@@ -1348,10 +1350,10 @@ __global__ void __launch_bounds__(kSJT, 4) k_join_set_heavy(const JoinSpec j, co
         b2[q] = st2 + (l - l1 * c2);
       }
     }
-    set_tuples<FILTER, kSJI>(j, refs, have, h.prow, row, b1, b2, idx, bad);
+    set_tuples<FILTER, kSJH>(j, refs, have, h.prow, row, b1, b2, idx, bad);
     if (bad && err) atomicOr(err, kErrCapacity);
-    const uint32_t fresh = set_add_any<HASH, kSJI>(d, idx, total);
-    set_store<kSJT, kSJI>(j, d, refs, idx, fresh, cursor, cap, red);
+    const uint32_t fresh = set_add_any<HASH, kSJH>(d, idx, total);
+    set_store<kSJT, kSJH>(j, d, refs, idx, fresh, cursor, cap, red);
     __syncthreads();  // the next chunk reuses red
   }
 }
@@ -1360,8 +1362,8 @@ cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, 
                      uint64_t out_cap, uint64_t* d_total, const HeavyList& heavy, bool run_chunks) {
   if (j.n_probe == 0) return cudaSuccess;
   const bool filter = j.n_neq > 0 || j.n_eq > 0;
-  // rows per thread: eight once four blocks per SM are busy, else fewer
-  uint64_t per = j.n_probe / ((uint64_t)kSJT * 152 * 4);
+  // rows per thread: all once five blocks per SM are busy, else fewer
+  uint64_t per = j.n_probe / ((uint64_t)kSJT * 152 * 5);
   per = per < 1 ? 1 : per > (uint64_t)kSJI ? (uint64_t)kSJI : per;
   const unsigned grid = dev_grid((j.n_probe + kSJT * per - 1) / (kSJT * per), j.dn);
   ProfScope p(c, kJoinWrite, ((j.star ? 48.0 : 24.0) + 4.0 * j.out_k) * j.n_probe);
