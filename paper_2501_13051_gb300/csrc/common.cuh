@@ -70,7 +70,7 @@ __device__ __forceinline__ uint32_t probe_table(const Slot* t, uint64_t mask, ui
   return 0;
 }
 
-// An index over build rows sorted by key, in one of two forms.  Hash form
+// An index over build rows sorted by key, in one of three forms.  Hash form
 // (range 0): the hybrid index's slots.  Direct form, for one-word keys whose
 // values lie below a range not much larger than the rows: entry k of an
 // array of `range` (start, end) pairs, both 0 for an absent key, so that a
@@ -81,28 +81,47 @@ __device__ __forceinline__ uint32_t probe_table(const Slot* t, uint64_t mask, ui
 // of 16M rows with an index of 16M rows over 2^25 keys: 2.73 ms with hash
 // slots built and looked up in its size query and again in its write, 0.86 ms
 // with entries built once and the rows' starts kept from the count.)
+// Offset form (rows > 0, with last): entry k is the number of keys below k,
+// *last + 2 of them, so that key k's rows are [entry k, entry k + 1): half the
+// bytes of the direct form and nothing to clear first, but two reads a lookup
+// and a split search before it is filled.  It pays once the direct form's
+// array is larger than L2 (the join above: 838 us with entries, 735 with
+// offsets).
 struct KeyIndex {
   const Slot* table;
   uint64_t slots;  // hash form: slots, a power of two
   uint32_t range;
   const uint32_t* last;
+  uint32_t rows;   // offset form: the build rows
 };
+
+// Rows [*start, *start + count) of key k < range in the direct or offset
+// form.  (An entry of a build side that is not sorted may be anything: it is
+// held within the rows.)
+__device__ __forceinline__ uint32_t find_entry(const KeyIndex& x, uint32_t k, uint32_t* start) {
+  uint2 e;
+  if (x.rows) {
+    const uint32_t* t = reinterpret_cast<const uint32_t*>(x.table) + k;
+    e.x = min(__ldg(t), x.rows);
+    e.y = min(__ldg(t + 1), x.rows);
+  } else {
+    e = __ldg(reinterpret_cast<const uint2*>(x.table) + k);
+  }
+  *start = e.x;
+  return e.y > e.x ? e.y - e.x : 0u;
+}
 
 // The direct form's range as it applies: 0 for the hash form.
 __device__ __forceinline__ uint32_t direct_range(const KeyIndex& x) {
   return x.last ? (__ldg(x.last) < x.range ? __ldg(x.last) + 1u : 0u) : x.range;
 }
 
-// Build rows of key (k0, k1); range as direct_range gives it.  (An entry of
-// a build side that is not sorted may have its end before its start: such a
-// key counts no rows.)
+// Build rows of key (k0, k1); range as direct_range gives it.
 __device__ __forceinline__ uint32_t find_key(const KeyIndex& x, uint32_t range, uint32_t k0,
                                              uint32_t k1, uint32_t* start) {
   if (range) {
-    const uint2 e = k0 < range ? __ldg(reinterpret_cast<const uint2*>(x.table) + k0)
-                               : make_uint2(0u, 0u);
-    *start = e.x;
-    return e.y > e.x ? e.y - e.x : 0u;
+    *start = 0;
+    return k0 < range ? find_entry(x, k0, start) : 0u;
   }
   return probe_table(x.table, x.slots - 1, k0, k1, start);
 }

@@ -410,7 +410,7 @@ struct Index {
   uint32_t range = 0;     // direct form: keys below it (KeyIndex)
   uint64_t distinct = 0;  // distinct keys, or a bound on them
   KeyIndex key_index() const {
-    return KeyIndex{static_cast<const Slot*>(table.p), slots, range, nullptr};
+    return KeyIndex{static_cast<const Slot*>(table.p), slots, range, nullptr, 0};
   }
   std::string tkey;       // tuner decision of the load factor, if any
   int tcand = 0;

@@ -102,9 +102,65 @@ __global__ void __launch_bounds__(kThreads) k_index_build(const uint32_t* __rest
   }
 }
 
-// Clears the form that *x.last gives.
+// Offset form.  The keys and the entries 0 .. range are merged (an entry
+// after the keys below it) and cut into equal shares by merge-path splits, so
+// that a run of one key or a gap between two costs a block no more than its
+// share; a row then writes the entries from the key before it up to its own.
+// Bound by memory: keys read, 4 bytes per entry written.
+constexpr int kOffTile = 4096;
+__global__ void __launch_bounds__(kThreads) k_offset_splits(const uint32_t* __restrict__ k0,
+                                                            uint64_t n, KeyIndex x,
+                                                            uint64_t* __restrict__ splits) {
+  const uint32_t range = direct_range(x);
+  if (!range) return;
+  const uint64_t b = (uint64_t)blockIdx.x * kThreads + threadIdx.x, total = n + range + 1ull;
+  if (b > (total + kOffTile - 1) / kOffTile) return;
+  const uint64_t d = b * kOffTile < total ? b * kOffTile : total;
+  uint64_t lo = d > range + 1ull ? d - (range + 1ull) : 0, hi = d < n ? d : n;
+  while (lo < hi) {
+    const uint64_t mid = lo + ((hi - lo) >> 1);
+    if (__ldg(k0 + mid) < d - mid - 1)  // key mid comes before entry d - mid - 1
+      lo = mid + 1;
+    else
+      hi = mid;
+  }
+  splits[b] = lo;
+}
+
+__global__ void __launch_bounds__(kThreads) k_offset_fill(const uint32_t* __restrict__ k0,
+                                                          uint64_t n, KeyIndex x,
+                                                          const uint64_t* __restrict__ splits,
+                                                          uint32_t* err) {
+  const uint32_t range = direct_range(x);
+  Slot* table = const_cast<Slot*>(x.table);
+  if (!range) {  // the hash form
+    for (uint64_t i = (uint64_t)blockIdx.x * kThreads + threadIdx.x; i < n;
+         i += (uint64_t)gridDim.x * kThreads)
+      hash_row<false>(k0, nullptr, i, n, table, x.slots - 1, err);
+    return;
+  }
+  uint32_t* t = reinterpret_cast<uint32_t*>(table);
+  const uint64_t total = n + range + 1ull, tiles = (total + kOffTile - 1) / kOffTile;
+  for (uint64_t b = blockIdx.x; b < tiles; b += gridDim.x) {
+    const uint64_t d1 = (b + 1) * kOffTile < total ? (b + 1) * kOffTile : total;
+    const uint64_t a0 = splits[b], a1 = splits[b + 1];
+    const uint64_t e0 = b * kOffTile - a0, e1 = d1 - a1;  // the tile's entries
+    // row i writes the tile's entries in (key i - 1, key i]; row a1 (of the
+    // next tile, or past the end) those behind the tile's last key
+    for (uint64_t i = a0 + threadIdx.x; i <= a1; i += kThreads) {
+      uint64_t lo = i > 0 ? (uint64_t)__ldg(k0 + i - 1) + 1 : 0;
+      uint64_t hi = i < a1 ? (uint64_t)__ldg(k0 + i) + 1 : e1;
+      lo = lo > e0 ? lo : e0;
+      hi = hi < e1 ? hi : e1;
+      for (uint64_t e = lo; e < hi; ++e) t[e] = (uint32_t)i;
+    }
+  }
+}
+
+// Clears the form that *x.last gives (the offset form needs none).
 __global__ void __launch_bounds__(kThreads) k_index_clear(KeyIndex x) {
   const uint32_t range = direct_range(x);
+  if (range && x.rows) return;
   const uint64_t words = range ? ((uint64_t)range + 1) / 2 : x.slots;  // 16 bytes each
   const uint32_t v = range ? 0u : 0xFFFFFFFFu;
   uint4* t = reinterpret_cast<uint4*>(const_cast<Slot*>(x.table));
@@ -166,6 +222,16 @@ cudaError_t index_build(Ctx& c, const uint32_t* k0, uint64_t n, const KeyIndex& 
   }
   if (n == 0) return cudaGetLastError();
   ProfScope p(c, kHashBuild, 4.0 * n);
+  if (x.rows) {
+    auto* splits = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(const_cast<Slot*>(x.table)) +
+                                               8 * x.slots + 256);
+    const uint64_t tiles = (n + x.range + 1ull + kOffTile - 1) / kOffTile;  // at most
+    k_offset_splits<<<(unsigned)((tiles + 1 + kThreads - 1) / kThreads), kThreads, 0, c.st>>>(k0, n, x,
+                                                                                              splits);
+    k_offset_fill<<<(unsigned)(tiles < 152 * 64 ? tiles : 152 * 64), kThreads, 0, c.st>>>(
+        k0, n, x, splits, c.d_err);
+    return cudaGetLastError();
+  }
   k_index_build<<<grid, kThreads, 0, c.st>>>(k0, n, x, c.d_err);
   return cudaGetLastError();
 }

@@ -107,11 +107,7 @@ __device__ __forceinline__ void set_lookup(const JoinSpec& j, const KeyIndex& x,
   if (range) {
 #pragma unroll
     for (int q = 0; q < N; ++q)
-      if (((live >> q) & 1u) && k0[q] < range) {
-        const uint2 e = __ldg(reinterpret_cast<const uint2*>(x.table) + k0[q]);
-        st[q] = e.x;
-        cnt[q] = e.y > e.x ? e.y - e.x : 0u;
-      }
+      if (((live >> q) & 1u) && k0[q] < range) cnt[q] = find_entry(x, k0[q], &st[q]);
     return;
   }
 #pragma unroll

@@ -93,7 +93,8 @@ cudaError_t hash_build(Ctx& c, const uint32_t* k0, const uint32_t* k1, uint64_t 
 uint64_t direct_keys(uint64_t n);
 // Fills x.table (8 * range bytes, or 16 * slots) from n sorted one-word
 // keys: the form x describes (a hash form through hash_build).  With x.last
-// the table holds the larger of the two.
+// the table has room for 16 * slots bytes whichever form the keys give; the
+// offset form leaves the half it does not need to its split search.
 cudaError_t index_build(Ctx& c, const uint32_t* k0, uint64_t n, const KeyIndex& x);
 // Number of distinct (k0, k1) keys of a sorted column pair into *d_out.
 cudaError_t count_heads(Ctx& c, const uint32_t* k0, const uint32_t* k1, uint64_t n,

@@ -177,6 +177,8 @@ static cdl_status join_setup(const uint32_t* const* probe_cols, uint32_t probe_a
   if (n_build) {
     j.ix.range = (uint32_t)std::min<uint64_t>(2 * slots, 0xFFFFFFFFull);
     j.ix.last = build_cols[build_key] + n_build - 1;
+    // (from 2^22 rows the entries by key may outgrow L2: offsets instead)
+    if (n_build >= 1ull << 22) j.ix.rows = (uint32_t)n_build;
   }
   return CDL_OK;
 }

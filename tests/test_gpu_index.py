@@ -71,3 +71,34 @@ def test_join_refuses_a_small_output(cdl):
     empty = [dev(np.zeros(0)), dev(np.zeros(0))]
     assert len(cdl.join(a, 0, empty, 0, [(0, 1)])[0]) == 0
     assert len(cdl.join(empty, 0, a, 0, [(0, 1)])[0]) == 0
+
+
+@pytest.mark.parametrize("kind", ["unique", "runs", "one-key", "gap", "sparse", "dense-then-far"])
+def test_join_over_offsets(cdl, kind):
+    """From 2^22 build rows the entries by key become offsets: gaps and runs
+    longer than a tile of the fill, and keys that leave them to the hash form."""
+    n = (1 << 22) + 5
+    rng = np.random.default_rng(7)
+    if kind == "unique":
+        key = np.unique(rng.integers(0, 3 * n, 2 * n))[:n]
+    elif kind == "runs":
+        key = np.sort(rng.integers(0, 900, n))
+    elif kind == "one-key":
+        key = np.full(n, 123_457)
+    elif kind == "gap":
+        key = np.concatenate([np.arange(n // 2), np.arange(n - n // 2) + 3 * n])
+    elif kind == "sparse":
+        key = np.sort(rng.integers(0, 1 << 32, n) & 0xFFFFFFFE)
+    else:
+        key = np.arange(n)
+        key[-1] = 0xFFFFFFFE
+    m = 100_003
+    build = [key.astype(np.uint32), rng.integers(0, 1 << 30, len(key)).astype(np.uint32)]
+    probe = [np.where(rng.random(m) < 0.5, key[rng.integers(0, len(key), m)],
+                      rng.integers(0, int(key[-1]) + 1000, m)).clip(0, 0xFFFFFFFE).astype(np.uint32),
+             rng.integers(0, 1 << 30, m).astype(np.uint32)]
+    if kind in ("runs", "one-key"):  # few probe rows meet long runs
+        probe = [c[:4 if kind == "one-key" else 50] for c in probe]
+    got = cdl.join([dev(c) for c in probe], 0, [dev(c) for c in build], 0, [(0, 1), (1, 1)])
+    for g, w in zip(got, reference(probe, build)):
+        assert np.array_equal(g.cpu().numpy().view(np.uint32), w)
