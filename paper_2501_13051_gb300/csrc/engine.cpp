@@ -517,7 +517,11 @@ struct cdl_engine {
   // nothing, so not lower.
   static constexpr uint32_t kSetBits = 37;
   static constexpr uint32_t kHashBits = 62;        // a packed tuple beside the two marks
-  static constexpr uint64_t kHashRows = 4 << 20;   // 48 MB of triples and their merged copy
+  // rows from which it pays to have no sort, merge and retirement in a round
+  // (266 instances of at most 7,282 edges, 6.0M tuples in 114 captured rounds:
+  // 34.3 ms with rows, 10.1 with sets; 40 of at most 60,000, 65 rounds: 24.3
+  // and 7.3); fewer rows keep the form whose converged instances leave Full
+  static constexpr uint64_t kHashRows = 1 << 18;
   bool hashed = false;  // batched run: the derived relations' Fulls are hash sets
   static constexpr double kSetSwitch = 0.2;
   // hub joins (hub_join): outputs in all, and per row of both sides, from
@@ -926,8 +930,8 @@ struct cdl_engine {
   }
 
   // Batched runs (tuple spaces far past any bitmap): Full of every derived
-  // relation as a hash set, once a first semi-naive round has left more rows
-  // than the caches hold.  The row form then sorts and merges all rows of all
+  // relation as a hash set, once a first semi-naive round has left kHashRows
+  // rows.  The row form then sorts and merges all rows of all
   // running instances every round (and moves converged instances' rows out of
   // its way); the set takes every new tuple once, at random, and sorts all of
   // them once at the end.  512 instances, 279M tuples, 233 captured rounds:

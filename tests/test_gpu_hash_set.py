@@ -1,5 +1,5 @@
-"""Batched runs whose Full is kept as a hash set (more than 2^22 rows after
-the first semi-naive round): rounds that outgrow the room for their new
+"""Batched runs whose Full is kept as a hash set (from 2^18 rows after the
+first semi-naive round): rounds that outgrow the room for their new
 tuples and the table, retirement before the switch, copy rules beside the
 joins, a stop at max_iters, with the rounds driven by the host and captured
 in a graph -- each against the form with sorted rows."""
