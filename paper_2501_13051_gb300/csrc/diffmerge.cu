@@ -234,6 +234,84 @@ __device__ __forceinline__ uint32_t co_rank_smem(const ColsIn& F, const ColsIn& 
   return rep || eq ? kRepeat : lo;
 }
 
+// Merges of several relations launched as one (diff_merge_group): their tiles
+// lie side by side, and a tile finds its relation by its number.  MergeTile:
+// what a tile works on, the launch's own arguments or its relation's.
+struct MergeTile {
+  ColsIn F, U;
+  uint64_t nF, nU;
+  uint64_t tile;           // within the relation
+  const uint64_t* splits;  // the relation's
+  uint32_t* corank;        // the relation's
+};
+__device__ __forceinline__ uint32_t job_of(const MergeJob* __restrict__ jobs, uint32_t n,
+                                           uint64_t tile) {
+  uint32_t lo = 0, hi = n;  // the last job starting at or before the tile
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (jobs[mid].tile0 <= tile)
+      lo = mid;
+    else
+      hi = mid;
+  }
+  return lo;
+}
+template <int K>
+__device__ __forceinline__ MergeTile job_tile(const MergeJob& j, uint64_t tile,
+                                              const uint64_t* splits, const uint32_t* corank) {
+  MergeTile m;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    m.F.c[k] = j.F.c[k];
+    m.U.c[k] = j.U.c[k];
+  }
+  m.nF = j.nF;
+  m.nU = j.nU;
+  m.tile = tile - j.tile0;
+  m.splits = splits + j.split0;
+  m.corank = const_cast<uint32_t*>(corank) + j.u0;
+  return m;
+}
+#define CDL_MERGE_TILE(T)                                                                       \
+  const uint32_t job = GROUP ? job_of(jobs, njobs, T) : 0u;                                     \
+  const MergeTile mt = GROUP ? job_tile<K>(jobs[job], T, splits_, corank_)                      \
+                             : MergeTile{F_, U_, nF_, nU_, T, splits_,                          \
+                                         const_cast<uint32_t*>(corank_)};                       \
+  const ColsIn &F = mt.F, &U = mt.U;                                                            \
+  const uint64_t nF = mt.nF, nU = mt.nU;                                                        \
+  const uint64_t* __restrict__ splits = mt.splits;                                              \
+  uint32_t* __restrict__ corank = mt.corank;                                                    \
+  (void)job, (void)corank, (void)nF, (void)nU
+
+// Splits of grouped merges, a warp each.
+template <int K>
+__global__ void k_group_splits(const MergeJob* __restrict__ jobs, uint32_t njobs, uint64_t nsplits,
+                               uint64_t* __restrict__ splits) {
+  const uint64_t x = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (x >= nsplits) return;
+  uint32_t lo = 0, hi = njobs;
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (jobs[mid].split0 <= x)
+      lo = mid;
+    else
+      hi = mid;
+  }
+  const MergeJob& j = jobs[lo];
+  const MergeTile m = job_tile<K>(j, j.tile0, splits, nullptr);
+  const uint64_t t = x - j.split0, n = m.nF + m.nU;
+  const uint64_t at = merge_split<K, true>(m.F, m.nF, m.U, m.nU, t * kDTile < n ? t * kDTile : n);
+  if (lane_id() == 0) splits[x] = at;
+}
+
+// The relations' numbers of new tuples, from the scan over all tiles.
+__global__ void k_group_totals(const MergeJob* __restrict__ jobs, uint32_t njobs,
+                               const uint64_t* __restrict__ pre, const uint64_t* __restrict__ total) {
+  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= njobs) return;
+  *jobs[j].nd = (j + 1 < njobs ? pre[jobs[j + 1].tile0] : *total) - pre[jobs[j].tile0];
+}
+
 // Persistent over groups of `group` tiles (1..8; grid = resident blocks).
 // Warp w takes tile w of the group: a tile without New tuples costs one
 // store, a sparse one (New < Full / 16) is searched by its warp alone with
@@ -242,14 +320,16 @@ __device__ __forceinline__ uint32_t co_rank_smem(const ColsIn& F, const ColsIn& 
 // meet a large Full keeps every warp busy instead of one block per tile,
 // while a small merge (fewer tiles than eight per resident block) keeps one
 // tile per block.
-template <int K>
-__global__ void __launch_bounds__(kDT) k_count_new(ColsIn F, ColsIn U, uint64_t nF, uint64_t nU,
-                                                   const uint64_t* __restrict__ splits,
-                                                   uint32_t* __restrict__ corank,
+template <int K, bool GROUP>
+__global__ void __launch_bounds__(kDT) k_count_new(ColsIn F_, ColsIn U_, uint64_t nF_, uint64_t nU_,
+                                                   const uint64_t* __restrict__ splits_,
+                                                   uint32_t* __restrict__ corank_,
                                                    uint32_t* __restrict__ tile_cnt,
-                                                   uint64_t ntiles, DevMerge dm, uint32_t group) {
+                                                   uint64_t ntiles, DevMerge dm, uint32_t group,
+                                                   const MergeJob* __restrict__ jobs,
+                                                   uint32_t njobs) {
   extern __shared__ uint32_t s[];  // K x kSRow: the Full and New slices of a dense tile
-  if (!resolve(dm, F, nF, nU, ntiles)) return;
+  if (!resolve(dm, F_, nF_, nU_, ntiles)) return;
   __shared__ uint32_t red[kDT / 32 + 1];
   constexpr int kW = kDT / 32;
   __shared__ uint32_t dense[kW];
@@ -260,9 +340,10 @@ __global__ void __launch_bounds__(kDT) k_count_new(ColsIn F, ColsIn U, uint64_t 
     __syncthreads();
     const uint64_t tile = g * group + warp;
     if (warp < group && tile < ntiles) {
-      const uint64_t d0 = tile * kDTile;
+      CDL_MERGE_TILE(tile);
+      const uint64_t d0 = mt.tile * kDTile;
       const uint64_t d1 = d0 + kDTile < nF + nU ? d0 + kDTile : nF + nU;
-      const uint64_t a0 = splits[tile], a1 = splits[tile + 1];
+      const uint64_t a0 = splits[mt.tile], a1 = splits[mt.tile + 1];
       const uint64_t b0 = d0 - a0, b1 = d1 - a1;
       const uint64_t na = a1 - a0, nb = b1 - b0;
       if (nb * 16 < na || nb == 0) {
@@ -290,9 +371,10 @@ __global__ void __launch_bounds__(kDT) k_count_new(ColsIn F, ColsIn U, uint64_t 
     const uint32_t nd = n_dense;
     for (uint32_t q = 0; q < nd; ++q) {
       const uint64_t t = g * group + dense[q];
-      const uint64_t d0 = t * kDTile;
+      CDL_MERGE_TILE(t);
+      const uint64_t d0 = mt.tile * kDTile;
       const uint64_t d1 = d0 + kDTile < nF + nU ? d0 + kDTile : nF + nU;
-      const uint64_t a0 = splits[t], a1 = splits[t + 1];
+      const uint64_t a0 = splits[mt.tile], a1 = splits[mt.tile + 1];
       const uint64_t b0 = d0 - a0, b1 = d1 - a1;
       const uint32_t na = (uint32_t)(a1 - a0), nb = (uint32_t)(b1 - b0), nm = na + nb;
       // New at least a quarter of Full: both slices merged again; fewer New
@@ -400,27 +482,39 @@ __global__ void __launch_bounds__(kDT) k_count_new(ColsIn F, ColsIn U, uint64_t 
 __device__ __forceinline__ uint32_t pad(uint32_t i) { return i + (i >> 5); }
 constexpr int kShiftWords = kDTile + 1 + (kDTile + 1) / 32 + 1;
 
-template <int K>
-__global__ void __launch_bounds__(kDT, 5) k_merge_write(ColsIn F, uint64_t nF, ColsIn U, uint64_t nU,
-                                                     const uint64_t* __restrict__ splits,
-                                                     const uint32_t* __restrict__ corank,
+template <int K, bool GROUP>
+__global__ void __launch_bounds__(kDT, 5) k_merge_write(ColsIn F_, uint64_t nF_, ColsIn U_,
+                                                     uint64_t nU_,
+                                                     const uint64_t* __restrict__ splits_,
+                                                     const uint32_t* __restrict__ corank_,
                                                      const uint64_t* __restrict__ tile_pre,
                                                      ColsOut D, ColsOut M, DevMerge dm,
-                                                     uint64_t ntiles) {
+                                                     uint64_t ntiles,
+                                                     const MergeJob* __restrict__ jobs,
+                                                     uint32_t njobs) {
   __shared__ uint32_t shift[kShiftWords];
   __shared__ uint32_t red[kDT / 32 + 1];
-  if (!resolve(dm, F, nF, nU, ntiles)) return;  // (inside a captured round: sizes from the device)
+  if (!resolve(dm, F_, nF_, nU_, ntiles)) return;  // (inside a captured round: sizes from the device)
   if (dm.n_full) {
     D = *dm.delta;
     M = *dm.merged;
   }
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-  const uint64_t d0 = tile * kDTile;
+  CDL_MERGE_TILE(tile);
+  const uint64_t d0 = mt.tile * kDTile;
   const uint64_t d1 = d0 + kDTile < nF + nU ? d0 + kDTile : nF + nU;
-  const uint64_t a0 = splits[tile], a1 = splits[tile + 1];
+  const uint64_t a0 = splits[mt.tile], a1 = splits[mt.tile + 1];
   const uint64_t b0 = d0 - a0, b1 = d1 - a1;
   const uint32_t na = (uint32_t)(a1 - a0), nb = (uint32_t)(b1 - b0);
-  const uint64_t dpre = tile_pre[tile];
+  uint64_t dpre = tile_pre[tile];
+  if constexpr (GROUP) {
+    dpre -= tile_pre[jobs[job].tile0];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      D.c[k] = jobs[job].D.c[k];
+      M.c[k] = jobs[job].M.c[k];
+    }
+  }
   const uint64_t mbase = a0 + dpre;
   const bool merged = M.c[0] != nullptr;
   uint32_t tot_new = 0;
@@ -497,12 +591,37 @@ __global__ void __launch_bounds__(kDT, 5) k_merge_write(ColsIn F, uint64_t nF, C
   }
 }
 
+#undef CDL_MERGE_TILE
+
 uint64_t dm_tiles(uint64_t n_full, uint64_t n_fresh) {
   return (n_full + n_fresh + kDTile - 1) / kDTile;
 }
 
 
 size_t up256(size_t b) { return (b + 255) & ~size_t(255); }
+
+// Blocks of k_count_new<K, GROUP> a whole GPU holds at once, per device.
+template <int K, bool GROUP>
+cudaError_t count_resident(size_t smem_count, int* out) {
+  constexpr int kDevices = 64;
+  static int resident_of[kDevices] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int& resident = resident_of[dev < kDevices ? dev : 0];
+  if (!resident) {
+    e = cudaFuncSetAttribute(k_count_new<K, GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem_count);
+    int per_sm = 0, sms = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_count_new<K, GROUP>, kDT, smem_count);
+    if (e != cudaSuccess) return e;
+    resident = (per_sm > 0 ? per_sm : 1) * sms;
+  }
+  *out = resident;
+  return cudaSuccess;
+}
 
 template <int K>
 cudaError_t run_diff_merge(Ctx& c, ColsIn full, uint64_t n_full, ColsIn fresh, uint64_t n_fresh,
@@ -522,23 +641,9 @@ cudaError_t run_diff_merge(Ctx& c, ColsIn full, uint64_t n_full, ColsIn fresh, u
   uint64_t* d_tiles = nullptr;  // device-sized: the scan's length (the split kernel writes it)
   if (dm.n_full) d_tiles = reinterpret_cast<uint64_t*>(w + scan_workspace(tiles));
   const size_t smem_count = sizeof(uint32_t) * K * kSRow;
-  // blocks of k_count_new<K> a whole GPU holds at once, per device
-  constexpr int kDevices = 64;
-  static int resident_of[kDevices] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  int resident = 0;
+  cudaError_t e = count_resident<K, false>(smem_count, &resident);
   if (e != cudaSuccess) return e;
-  int& resident = resident_of[dev < kDevices ? dev : 0];
-  if (!resident) {
-    e = cudaFuncSetAttribute(k_count_new<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_count);
-    int per_sm = 0, sms = 0;
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_count_new<K>, kDT, smem_count);
-    if (e != cudaSuccess) return e;
-    resident = (per_sm > 0 ? per_sm : 1) * sms;
-  }
   // tiles per group: eight once there are eight per resident block, else
   // fewer, down to one per block for small merges
   uint64_t group = tiles / (uint64_t)resident;
@@ -554,8 +659,8 @@ cudaError_t run_diff_merge(Ctx& c, ColsIn full, uint64_t n_full, ColsIn fresh, u
     else
       k_merge_splits<K, false><<<(unsigned)((tiles + 1 + 255) / 256), 256, 0, c.st>>>(
           full, n_full, fresh, n_fresh, splits, tiles, dm, d_tiles);
-    k_count_new<K><<<(unsigned)count_grid, kDT, smem_count, c.st>>>(
-        full, fresh, n_full, n_fresh, splits, corank, cnt, tiles, dm, (uint32_t)group);
+    k_count_new<K, false><<<(unsigned)count_grid, kDT, smem_count, c.st>>>(
+        full, fresh, n_full, n_fresh, splits, corank, cnt, tiles, dm, (uint32_t)group, nullptr, 0);
   }
   {
     const int sc = c.scan_cls;  // the tile counts' scan is timed with the count pass
@@ -569,8 +674,48 @@ cudaError_t run_diff_merge(Ctx& c, ColsIn full, uint64_t n_full, ColsIn fresh, u
   // part of the writes (merged and delta) is added once its size is known
   const double mb = merged.c[0] ? 4.0 * K * n_full : 0.0;
   ProfScope p(c, kDiffMerge, 4.0 * K * (n_full + n_fresh) + mb);
-  k_merge_write<K><<<dev_grid(tiles, dm.n_full), kDT, 0, c.st>>>(
-      full, n_full, fresh, n_fresh, splits, corank, pre, delta, merged, dm, tiles);
+  k_merge_write<K, false><<<dev_grid(tiles, dm.n_full), kDT, 0, c.st>>>(
+      full, n_full, fresh, n_fresh, splits, corank, pre, delta, merged, dm, tiles, nullptr, 0);
+  return cudaGetLastError();
+}
+
+template <int K>
+cudaError_t run_group(Ctx& c, const MergeJob* jobs, uint32_t njobs, const MergeGroup& g, void* ws) {
+  char* w = static_cast<char*>(ws);
+  uint64_t* splits = reinterpret_cast<uint64_t*>(w);
+  w += up256(g.splits * 8);
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(w);
+  w += up256(g.tiles * 4);
+  uint64_t* pre = reinterpret_cast<uint64_t*>(w);
+  w += up256(g.tiles * 8);
+  uint32_t* corank = reinterpret_cast<uint32_t*>(w);
+  w += up256((g.fresh ? g.fresh : 1) * 4);
+  uint64_t* total = reinterpret_cast<uint64_t*>(w);
+  w += 256;
+  const size_t smem_count = sizeof(uint32_t) * K * kSRow;
+  int resident = 0;
+  cudaError_t e = count_resident<K, true>(smem_count, &resident);
+  if (e != cudaSuccess) return e;
+  uint64_t group = g.tiles / (uint64_t)resident;
+  group = group < 1 ? 1 : (group > (uint64_t)(kDT / 32) ? (uint64_t)(kDT / 32) : group);
+  const uint64_t groups = (g.tiles + group - 1) / group;
+  const uint64_t count_grid = groups < (uint64_t)resident ? groups : (uint64_t)resident;
+  const DevMerge none{};
+  {
+    ProfScope p(c, kDiffCount, (4.0 * K + 4.0) * g.fresh);
+    k_group_splits<K><<<(unsigned)((g.splits + 7) / 8), 256, 0, c.st>>>(jobs, njobs, g.splits, splits);
+    k_count_new<K, true><<<(unsigned)count_grid, kDT, smem_count, c.st>>>(
+        ColsIn{}, ColsIn{}, 0, 0, splits, corank, cnt, g.tiles, none, (uint32_t)group, jobs, njobs);
+    const int sc = c.scan_cls;
+    c.scan_cls = kDiffCount;
+    e = exclusive_scan(c, cnt, g.tiles, pre, total, w);
+    c.scan_cls = sc;
+    if (e != cudaSuccess) return e;
+    k_group_totals<<<(njobs + 255) / 256, 256, 0, c.st>>>(jobs, njobs, pre, total);
+  }
+  ProfScope p(c, kDiffMerge, 4.0 * K * (2.0 * g.full + g.fresh));
+  k_merge_write<K, true><<<(unsigned)g.tiles, kDT, 0, c.st>>>(
+      ColsIn{}, 0, ColsIn{}, 0, splits, corank, pre, ColsOut{}, ColsOut{}, none, g.tiles, jobs, njobs);
   return cudaGetLastError();
 }
 
@@ -580,6 +725,32 @@ size_t diff_merge_workspace(uint64_t n_full, uint64_t n_fresh) {
   const uint64_t tiles = dm_tiles(n_full, n_fresh);
   return up256((tiles + 1) * 8) + up256(tiles * 4) + up256(tiles * 8) +
          up256((n_fresh ? n_fresh : 1) * 4) + scan_workspace(tiles) + 256;
+}
+
+void MergeGroup::add(MergeJob& j) {
+  const uint64_t t = dm_tiles(j.nF, j.nU);
+  j.tile0 = tiles;
+  j.split0 = splits;
+  j.u0 = fresh;
+  tiles += t;
+  splits += t + 1;
+  full += j.nF;
+  fresh += j.nU;
+}
+
+size_t merge_group_workspace(const MergeGroup& g) {
+  return up256(g.splits * 8) + up256(g.tiles * 4) + up256(g.tiles * 8) +
+         up256((g.fresh ? g.fresh : 1) * 4) + 256 + scan_workspace(g.tiles);
+}
+
+cudaError_t diff_merge_group(Ctx& c, uint32_t k, const MergeJob* jobs, uint32_t njobs,
+                             const MergeGroup& g, void* ws) {
+  switch (k) {
+    case 1: return run_group<1>(c, jobs, njobs, g, ws);
+    case 2: return run_group<2>(c, jobs, njobs, g, ws);
+    case 3: return run_group<3>(c, jobs, njobs, g, ws);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t diff_merge(Ctx& c, uint32_t k, ColsIn full, uint64_t n_full, ColsIn fresh,

@@ -864,6 +864,69 @@ struct cdl_engine {
     return CDL_OK;
   }
 
+  // The round's merges of several relations, those of one arity as one set of
+  // launches where there are a few of them and none is large enough to fill
+  // the GPU by itself.  (Not under a memory limit: all merged versions are
+  // allocated before the first old one is freed.)
+  static constexpr uint64_t kMergeGroupRows = 1 << 22;
+  static constexpr size_t kMergeGroupMin = 3;
+  cdl_status merge_all(std::vector<std::pair<uint32_t, DCols*>>& todo) {
+    for (uint32_t k = 1; k <= 3 && !opt.mem_limit; ++k) {
+      std::vector<std::pair<uint32_t, DCols*>> grp;
+      for (auto& t : todo) {
+        const Relation& R = *rels[t.first];
+        if (R.arity == k && !R.dsm.on && !R.host_full && R.full.n + t.second->n <= kMergeGroupRows)
+          grp.push_back(t);
+      }
+      if (grp.size() < kMergeGroupMin) continue;
+      std::vector<MergeJob> jobs;
+      std::vector<DCols> merged(grp.size()), delta(grp.size());
+      MergeGroup g;
+      for (size_t i = 0; i < grp.size(); ++i) {
+        const Relation& R = *rels[grp[i].first];
+        const DCols& U = *grp[i].second;
+        if (!alloc_cols(merged[i], k, R.full.n + U.n) || !alloc_cols(delta[i], k, U.n))
+          return fail(CDL_E_NOMEM, "merge buffers");
+        MergeJob j{};
+        j.F = R.full.in();
+        j.U = U.in();
+        j.D = delta[i].out();
+        j.M = merged[i].out();
+        j.nF = R.full.n;
+        j.nU = U.n;
+        j.nd = dslot(kSlotDelta + grp[i].first);
+        g.add(j);
+        jobs.push_back(j);
+      }
+      DBuf dj = alloc(sizeof(MergeJob) * jobs.size()), ws = alloc(merge_group_workspace(g));
+      if (!dj.p || !ws.p) return fail(CDL_E_NOMEM, "merge workspace");
+      cudaError_t e = cudaMemcpyAsync(dj.p, jobs.data(), sizeof(MergeJob) * jobs.size(),
+                                      cudaMemcpyHostToDevice, st);
+      if (e == cudaSuccess)
+        e = diff_merge_group(ctx, k, static_cast<const MergeJob*>(dj.p), (uint32_t)jobs.size(), g, ws.p);
+      if (e != cudaSuccess) return cuda_fail(e, "grouped merge");
+      for (size_t i = 0; i < grp.size(); ++i) {
+        Relation& R = *rels[grp[i].first];
+        merged[i].n = R.full.n;  // grows by |delta| once it is read back
+        R.full = std::move(merged[i]);
+        R.version[kFull]++;
+        R.delta_version = R.version[kFull];
+        R.delta = std::move(delta[i]);
+      }
+      todo.erase(std::remove_if(todo.begin(), todo.end(),
+                                [&](const std::pair<uint32_t, DCols*>& t) {
+                                  return std::find(grp.begin(), grp.end(), t) != grp.end();
+                                }),
+                 todo.end());
+    }
+    for (auto& t : todo) {
+      Relation& R = *rels[t.first];
+      cdl_status r = merge_into(R, *t.second, &R.delta, kSlotDelta + t.first);
+      if (r != CDL_OK) return r;
+    }
+    return CDL_OK;
+  }
+
   // ------------------------------------------- Algorithm 2 (option dedup)
   // Derived relations whose Full no rule variant reads after round 1 (every
   // rule that names them has no other derived body atom, so its semi-naive
@@ -3455,6 +3518,7 @@ struct cdl_engine {
       if (!opt.n_instances) status = sort_groups(group_bufs, sorted_rows, grouped);
       if (status != CDL_OK) break;
       std::vector<uint8_t> merged(nr, 0);
+      std::vector<std::pair<uint32_t, DCols*>> todo;  // relations and their sorted new rows
       for (uint32_t i = 0; i < nr; ++i) {
         Relation& R = *rels[i];
         if (!R.idb) continue;
@@ -3488,8 +3552,7 @@ struct cdl_engine {
           break;
         }
         if (grouped[i]) {  // sorted with its group: a segment of the group's rows
-          status = merge_into(R, sorted_rows[i], &R.delta, kSlotDelta + i);
-          if (status != CDL_OK) break;
+          todo.emplace_back(i, &sorted_rows[i]);
           merged[i] = 1;
           continue;
         }
@@ -3497,10 +3560,10 @@ struct cdl_engine {
         for (uint32_t k = 0; k < R.arity; ++k) bits[k] = bits_of(R.bound[k]);
         status = sort_cols(R.fresh, bits);
         if (status != CDL_OK) break;
-        status = merge_into(R, R.fresh, &R.delta, kSlotDelta + i);
-        if (status != CDL_OK) break;
+        todo.emplace_back(i, &R.fresh);
         merged[i] = 1;
       }
+      if (status == CDL_OK) status = merge_all(todo);
       if (status != CDL_OK) break;
       for (uint32_t i = 0; i < nr; ++i)  // a merge's delta size is read now
         if (merged[i] && !rels[i]->set_on) delta_known = false;

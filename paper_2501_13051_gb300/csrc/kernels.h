@@ -347,6 +347,25 @@ cudaError_t diff_merge(Ctx& c, uint32_t k, ColsIn full, uint64_t n_full, ColsIn 
                        uint64_t n_fresh, ColsOut delta, ColsOut merged, uint64_t* d_ndelta,
                        void* ws, const DevMerge* dm = nullptr);
 
+// Merges of several relations of one arity (1 to 3) as one set of launches.
+// A round of a program over hundreds of relations merges a dozen that change,
+// each far too small to fill the GPU: 85 us of four launches apiece.
+struct MergeJob {
+  ColsIn F, U;
+  ColsOut D, M;
+  uint64_t nF, nU;  // nF + nU > 0
+  uint64_t* nd;     // (device) receives |delta|
+  uint64_t tile0, split0, u0;  // set by MergeGroup::add
+};
+struct MergeGroup {
+  uint64_t tiles = 0, splits = 0, full = 0, fresh = 0;
+  void add(MergeJob& j);
+};
+size_t merge_group_workspace(const MergeGroup& g);
+// jobs: device copy of the jobs in the order of their add.
+cudaError_t diff_merge_group(Ctx& c, uint32_t k, const MergeJob* jobs, uint32_t njobs,
+                             const MergeGroup& g, void* ws);
+
 // Selection + projection of one atom: keeps rows with col == const, col ==
 // col and (on output refs) out != out; writes out tuples packed at
 // *d_cursor (atomic).  Refs use side 0 (input column) or 2 (constant).
