@@ -487,6 +487,16 @@ cudaError_t gather_segments(Ctx& c, uint32_t k, ColsIn a, ColsIn b, const uint64
 // Reserved-value check and column maxima of loaded data.
 cudaError_t check_values(Ctx& c, ColsIn in, uint32_t k, uint64_t n, uint32_t* d_max);
 
+// The same for many columns in one launch (jobs in device memory, the maxima
+// zeroed; most, total: the longest column's and all columns' rows).
+struct CheckJob {
+  const uint32_t* col;
+  uint64_t n;
+  uint32_t* max;
+};
+cudaError_t check_columns(Ctx& c, const CheckJob* jobs, uint32_t njobs, uint64_t most,
+                          uint64_t total);
+
 // ------------------------------------------------------------ estimator
 constexpr int kMlpIn = 16, kMlpHidden = 64;
 constexpr int kMlpParams = kMlpHidden * kMlpIn + kMlpHidden + kMlpHidden * kMlpHidden + kMlpHidden +

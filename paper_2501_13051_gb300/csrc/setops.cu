@@ -73,6 +73,28 @@ __global__ void k_check_values(ColsIn in, uint32_t k, uint64_t n, uint32_t* d_ma
   }
 }
 
+// The same for the columns of many loads at once: blockIdx.y is the column.
+__global__ void __launch_bounds__(256) k_check_columns(const CheckJob* __restrict__ jobs,
+                                                       uint32_t* err) {
+  const CheckJob j = jobs[blockIdx.y];
+  const uint64_t step = (uint64_t)gridDim.x * 256;
+  uint32_t m = 0;
+  bool bad = false;
+  for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < j.n; i += 4 * step) {
+    uint32_t v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = i + u * step < j.n ? __ldg(j.col + i + u * step) : 0u;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      bad |= v[u] == kEmpty;
+      m = max(m, v[u]);
+    }
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (bad && err) atomicOr(err, kErrValue);
+  if (lane_id() == 0 && m) atomicMax(j.max, m);
+}
+
 // Batched fixpoints: the delta of a relation whose column 0 is an instance
 // id is sorted by instance, so every run head marks an instance that derived
 // something in this round.
@@ -283,6 +305,19 @@ cudaError_t select_project(Ctx& c, const SelectSpec& s, ColsOut out, uint64_t* d
                                                reinterpret_cast<unsigned long long*>(d_cursor),
                                                out_cap,
                                                soft_overflow ? soft_overflow : c.d_err);
+  return cudaGetLastError();
+}
+
+cudaError_t check_columns(Ctx& c, const CheckJob* jobs, uint32_t njobs, uint64_t most,
+                          uint64_t total) {
+  if (njobs == 0 || most == 0) return cudaSuccess;
+  ProfScope p(c, kMisc, 4.0 * total);
+  uint64_t blocks = (most + 4095) / 4096;
+  if (blocks > 64) blocks = 64;
+  constexpr uint32_t kMost = 65535;  // of a grid's second dimension
+  for (uint32_t at = 0; at < njobs; at += kMost)
+    k_check_columns<<<dim3((unsigned)blocks, njobs - at < kMost ? njobs - at : kMost), 256, 0, c.st>>>(
+        jobs + at, c.d_err);
   return cudaGetLastError();
 }
 
