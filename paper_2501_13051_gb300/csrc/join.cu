@@ -355,38 +355,6 @@ __device__ __forceinline__ void set_tuples(const JoinSpec& j, const SetRefs& s, 
     if (!((live & ~out) >> q & 1u)) idx[q] = kNoTuple;
 }
 
-// Places for a block's outputs in `mask`, packed at *cursor with one claim:
-// output q goes to *pos + at[q].  wsum: THREADS / 32 + 2 words.  false (for
-// the whole block) where there are none.
-template <int THREADS, int N>
-__device__ __forceinline__ bool claim_places(uint32_t mask, unsigned long long* cursor,
-                                             uint32_t* wsum, uint32_t (&at)[N], uint64_t* pos) {
-  constexpr int W = THREADS / 32;
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, lt = (1u << lane) - 1u;
-  uint32_t n = 0;
-#pragma unroll
-  for (int q = 0; q < N; ++q) {
-    const uint32_t bal = __ballot_sync(0xffffffffu, (mask >> q) & 1u);
-    at[q] = n + __popc(bal & lt);
-    n += __popc(bal);
-  }
-  if (lane == 0) wsum[warp] = n;
-  __syncthreads();
-  unsigned long long* claim = reinterpret_cast<unsigned long long*>(wsum + W);
-  uint32_t before = 0, total = 0;
-#pragma unroll
-  for (int w = 0; w < W; ++w) {
-    const uint32_t c = wsum[w];
-    before += w < (int)warp ? c : 0u;
-    total += c;
-  }
-  if (total == 0) return false;
-  if (threadIdx.x == 0) *claim = atomicAdd(cursor, (unsigned long long)total);
-  __syncthreads();
-  *pos = *claim + before;
-  return true;
-}
-
 // New tuples (bit q of fresh) to the head's columns; those past cap are taken
 // out of the set again and true is returned to their threads.
 template <int THREADS, int N>

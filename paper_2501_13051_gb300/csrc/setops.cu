@@ -12,46 +12,60 @@ namespace {
 constexpr int kST = 256;
 constexpr int kSItems = 8;
 
-__device__ __forceinline__ uint32_t sel_ref(const SelectSpec& s, const Ref& r, uint64_t row) {
-  return r.side == 2 ? r.v : __ldg(s.in.c[r.v] + row);
-}
-
+// Eight rows per thread: their filters, then one claim of the output for the
+// block, then the columns one after the other, eight loads in flight.  (With
+// a scan and a claim for every 256 rows, one after another, the 270 copies of
+// an OWL-RL fixpoint took 10.4 us each; the fixpoint 37.2 -> 35.4 ms.)
 __global__ void __launch_bounds__(kST) k_select(const SelectSpec s, ColsOut out,
                                                 unsigned long long* cursor, uint64_t cap,
                                                 uint32_t* err) {
-  __shared__ uint32_t red[kST / 32 + 1];
-  __shared__ unsigned long long s_base;
-  const uint64_t base = (uint64_t)blockIdx.x * kST * kSItems;
-  for (int it = 0; it < kSItems; ++it) {
-    const uint64_t row = base + (uint64_t)it * kST + threadIdx.x;
-    bool keep = row < s.n;
-    uint32_t vals[kMaxK] = {0, 0, 0, 0};
-    if (keep) {
-      for (uint32_t q = 0; q < s.n_const; ++q)
-        keep &= __ldg(s.in.c[s.const_col[q]] + row) == s.const_val[q];
-      for (uint32_t q = 0; q < s.n_same; ++q)
-        keep &= __ldg(s.in.c[s.same[q][0]] + row) == __ldg(s.in.c[s.same[q][1]] + row);
-      for (uint32_t q = 0; q < s.n_neq; ++q)
-        keep &= sel_ref(s, s.neq[q][0], row) != sel_ref(s, s.neq[q][1], row);
+  __shared__ __align__(8) uint32_t red[kST / 32 + 2];
+  const uint64_t base = (uint64_t)blockIdx.x * kST * kSItems + threadIdx.x;
+  uint32_t live = 0;
 #pragma unroll
-      for (int k = 0; k < kMaxK; ++k)
-        if (k < (int)s.out_k) vals[k] = sel_ref(s, s.out[k], row);
-    }
-    uint32_t cnt;
-    const uint32_t local = block_exclusive_sum<kST, uint32_t>(keep ? 1u : 0u, red, &cnt);
-    if (threadIdx.x == 0) s_base = cnt ? atomicAdd(cursor, (unsigned long long)cnt) : 0ull;
-    __syncthreads();
-    const uint64_t pos = s_base + local;
-    __syncthreads();
-    if (keep) {
-      if (pos < cap) {
+  for (int i = 0; i < kSItems; ++i) live |= (base + (uint64_t)i * kST < s.n ? 1u : 0u) << i;
+  auto load = [&](const Ref& r, uint32_t (&v)[kSItems]) {
+    const uint32_t* p = r.side == 2 ? nullptr : s.in.c[r.v] + base;
 #pragma unroll
-        for (int k = 0; k < kMaxK; ++k)
-          if (k < (int)s.out_k) out.c[k][pos] = vals[k];
-      } else {
-        if (err) atomicOr(err, kErrCapacity);
-      }
+    for (int i = 0; i < kSItems; ++i) {
+      v[i] = r.v;
+      if (p && ((live >> i) & 1u)) v[i] = __ldg(p + (uint64_t)i * kST);
     }
+  };
+  auto filter = [&](const Ref& x, const Ref& y, bool equal) {
+    uint32_t a[kSItems], b[kSItems];
+    load(x, a);
+    load(y, b);
+#pragma unroll
+    for (int i = 0; i < kSItems; ++i)
+      if ((a[i] == b[i]) != equal) live &= ~(1u << i);
+  };
+#pragma unroll 1
+  for (uint32_t q = 0; q < s.n_const; ++q) filter(Ref{0, s.const_col[q]}, Ref{2, s.const_val[q]}, true);
+#pragma unroll 1
+  for (uint32_t q = 0; q < s.n_same; ++q) filter(Ref{0, s.same[q][0]}, Ref{0, s.same[q][1]}, true);
+#pragma unroll 1
+  for (uint32_t q = 0; q < s.n_neq; ++q) filter(s.neq[q][0], s.neq[q][1], false);
+  uint32_t at[kSItems];
+  uint64_t pos;
+  if (!claim_places<kST, kSItems>(live, cursor, red, at, &pos)) return;
+  const uint64_t room = cap > pos ? cap - pos : 0;
+  bool over = false;
+#pragma unroll
+  for (int i = 0; i < kSItems; ++i)
+    if (((live >> i) & 1u) && at[i] >= room) {
+      over = true;
+      live &= ~(1u << i);
+    }
+  if (over && err) atomicOr(err, kErrCapacity);
+#pragma unroll 1
+  for (uint32_t k = 0; k < s.out_k; ++k) {
+    uint32_t v[kSItems];
+    load(s.out[k], v);
+    uint32_t* o = out.c[k] + pos;
+#pragma unroll
+    for (int i = 0; i < kSItems; ++i)
+      if ((live >> i) & 1u) o[at[i]] = v[i];
   }
 }
 
