@@ -103,7 +103,8 @@ typedef struct {
                            per-instance iteration counts in cdl_stats */
   int32_t retire;       /* batched runs: 0 = default, the rows of an instance that reached
                            its fixpoint leave the merged relation until the end of the
-                           run; -1 = every instance stays in it every round */
+                           run; -1 = every instance stays in it every round (no rows
+                           leave, or need to, once Full is a hash set, see dense_bits) */
   int32_t autotune;     /* launch-parameter tuner (radix digit width and block size, hash
                            load factor): 0 off (the values above); 1 use what tune_cache
                            holds; 2 also time untried candidates (CUDA events) and write
@@ -124,7 +125,11 @@ typedef struct {
                            bits: join outputs set bits instead of being written, and the
                            bits read back in order are the sorted unique tuples (no radix
                            sort).  0 = default 28; -1 = never; values above 34 act as 34
-                           (a 2 GB bitmap).  Results never depend on it */
+                           (a 2 GB bitmap).  Where no rule variant reads such a relation's
+                           Full after round 1 the bitmap is Full itself; larger ones (to
+                           2^37 tuples) go over to that form when it pays, and in batched
+                           runs Full becomes a hash set of tuples.  -1 keeps sorted rows
+                           throughout.  Results never depend on it */
   int32_t dedup;        /* step (d) of derived relations whose Full no rule variant reads
                            after round 1 (every rule naming them has no other derived body
                            atom; batched runs excluded): 0 = default, the difference and

@@ -396,8 +396,9 @@ __device__ __forceinline__ bool set_store(const JoinSpec& j, const DenseSet& d, 
 // so the round needs no sort and no merge.  Bound by the random accesses to
 // the bitmap: a block's outputs are taken in one sweep, eight per thread,
 // all reads and then all atomics in flight.  Same generation on 200,000
-// nodes, where the bitmap is 8 GB: 1.6e9 outputs in 62 ms (2.6e10 per
-// second; the sorts, merges and writes it replaces took 231 ms of 267).
+// nodes, where the bitmap is 8 GB: 1.6e9 outputs in 62 ms when all of its
+// joins were written by this form (the sorts, merges and writes it replaced
+// took 231 ms of 267); k_join_set has since taken most of them over.
 enum Form : int { kRows = 0, kBits = 1, kSet = 2 };
 template <bool FILTER, int FORM, bool STAR>
 __global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5) k_join_write(const JoinSpec j, const uint64_t* __restrict__ off,
