@@ -378,7 +378,8 @@ struct Relation {
   bool set_single = false;  // a single-pass join of this round wrote sdelta
   bool set_redo = false;    // ... and ran out of room: its rules run again, exact
   DCols sdelta;          // the round's new tuples so far (dslot(kSlotDelta + i) of them)
-  uint64_t sdelta_ub = 0;
+  uint64_t sdelta_ub = 0;   // rows of it taken: counted, or what one-pass joins are expected to add
+  uint64_t set_outputs = 0; // outputs of the round's counted joins and copies into the set
   double merged_bytes = 0;  // row form: bytes its sorts and merges have moved
 };
 
@@ -566,7 +567,8 @@ struct cdl_engine {
     std::tuple<size_t, size_t, size_t> key;
     uint32_t head;
     uint64_t probe;
-    bool chunks;  // the kernel for long ranges was launched
+    bool chunks;   // the kernel for long ranges was launched
+    bool counted;  // its size was known (and is in set_outputs)
   };
   std::vector<SetStep> set_steps;
   bool delta_known = false;  // h_ctl holds the set relations' delta sizes
@@ -1095,15 +1097,19 @@ struct cdl_engine {
     return 0;
   }
 
-  // Room for the round's new tuples of a join with `extra` outputs (or
-  // set_redo where an earlier one-pass join already lacks room).
-  cdl_status ensure_sdelta(Relation& R, uint64_t extra) {
-    if (!R.set_free && R.sdelta_ub + extra > 0xFFFFFFFFull)
-      return fail(CDL_E_CAPACITY, "relation " + R.name + " would receive more than 2^32 new "
-                                  "tuples in one round");
-    if (R.set_single && R.sdelta_ub + extra > R.sdelta.cap) {
-      // the one-pass joins so far may have run out of room: their rows are
-      // all there only if not
+  // Room for the round's new tuples of a join with `extra` outputs, counted
+  // ones or what a one-pass join is expected to have (or set_redo where an
+  // earlier one-pass join already lacks room).
+  cdl_status ensure_sdelta(Relation& R, uint64_t extra, bool counted) {
+    if (counted) {
+      R.set_outputs += extra;
+      if (!R.set_free && R.set_outputs > 0xFFFFFFFFull) return too_many_new(R);
+    }
+    if (R.set_single && ((counted && !R.fset.keys) || R.sdelta_ub + extra > R.sdelta.cap)) {
+      // the one-pass joins so far may have added more than was expected of
+      // them, up to the buffer's end, or have run out of room: a counted
+      // join into a bitmap, which takes the room it is given for enough,
+      // starts behind what they really added, and only if that is all there
       cdl_status r = fetch(kSlotDelta + rel_id(R), 1);
       if (r != CDL_OK) return r;
       const uint64_t at = h_ctl[kSlotDelta + rel_id(R)];
@@ -1131,6 +1137,11 @@ struct cdl_engine {
     return CDL_OK;
   }
 
+  cdl_status too_many_new(const Relation& R) {
+    return fail(CDL_E_CAPACITY, "relation " + R.name + " would receive more than 2^32 new "
+                                "tuples in one round");
+  }
+
   // The rows written to fresh this round (copies, single-pass joins) join
   // the set as well.
   cdl_status set_fresh_rows() {
@@ -1140,7 +1151,7 @@ struct cdl_engine {
       const uint64_t nf = std::min<uint64_t>(h_ctl[kSlotCursor + i], R.fresh.cap);
       if (nf == 0) continue;
       // (the rows so far are counted and all there)
-      R.sdelta_ub = std::max(R.sdelta_ub, h_ctl[kSlotDelta + i]);
+      R.sdelta_ub = h_ctl[kSlotDelta + i];
       R.set_single = false;
       delta_known = false;
       if (R.fset.keys) {
@@ -1149,7 +1160,7 @@ struct cdl_engine {
         if (s == CDL_OK && !ok) s = fail(CDL_E_NOMEM, "full set");
         if (s != CDL_OK) return s;
       }
-      cdl_status r = ensure_sdelta(R, nf);
+      cdl_status r = ensure_sdelta(R, nf, true);
       if (r != CDL_OK) return r;
       cudaError_t e = set_insert(ctx, R.fset, R.fresh.in(), nf, R.sdelta.out(), dslot(kSlotDelta + i),
                                  R.sdelta.cap);
@@ -2237,7 +2248,7 @@ struct cdl_engine {
       }
       if (last && rels[rule.head.rel]->set_on) {  // Full is a set: new tuples go to delta
         Relation& H = *rels[rule.head.rel];
-        r = ensure_sdelta(H, total);
+        r = ensure_sdelta(H, total, true);
         if (r != CDL_OK || H.set_redo) return r;
         e = join_write(ctx, js, static_cast<const uint64_t*>(off.p), total, H.sdelta.out(), 0,
                        dslot(kSlotDelta + rule.head.rel), H.sdelta.cap, wsp.p, wws, nullptr, nullptr,
@@ -2317,7 +2328,7 @@ struct cdl_engine {
       if (!exact) return CDL_OK;
       return fail(CDL_E_CAPACITY, "too many joins into hash sets in one round");
     }
-    cdl_status r = ensure_sdelta(H, want);
+    cdl_status r = ensure_sdelta(H, want, exact != 0);
     if (r == CDL_E_NOMEM && !exact) {  // (nothing was changed but the bound)
       err.clear();
       H.sdelta_ub -= want;
@@ -2346,7 +2357,7 @@ struct cdl_engine {
                              H.sdelta.cap, dslot(slot), list, chunks);
     if (e != cudaSuccess) return cuda_fail(e, "one-pass join");
     H.set_single = true;
-    set_steps.push_back(SetStep{key, rule.head.rel, np, chunks});
+    set_steps.push_back(SetStep{key, rule.head.rel, np, chunks, exact != 0});
     ++joins;
     return CDL_OK;
   }
@@ -2423,7 +2434,7 @@ struct cdl_engine {
     uint64_t* cursor = nullptr;
     uint64_t cap = 0;
     if (H.set_on) {
-      r = ensure_sdelta(H, total);
+      r = ensure_sdelta(H, total, true);
       if (r != CDL_OK) return r;
       if (H.set_redo) {
         done = true;
@@ -2834,21 +2845,18 @@ struct cdl_engine {
   // One-pass joins after the round's read-back: their sizes, and the
   // relations that lacked room (to be redone).
   cdl_status set_results(std::vector<bool>& redo, bool& any) {
-    std::map<uint32_t, uint64_t> outputs;
     for (size_t i = 0; i < set_steps.size(); ++i) {
       const SetStep& t = set_steps[i];
       const uint64_t total = h_ctl[kSlotSetTotal + 2 * i], listed = h_ctl[kSlotSetTotal + 2 * i + 1];
       if ((total & kSetListFull) || (listed && !t.chunks)) redo[t.head] = any = true;
       set_seen[t.key] = SetSeen{t.probe, total & (kSetListFull - 1), listed != 0};
       prev_out[t.key] = total & (kSetListFull - 1);
-      outputs[t.head] += total & (kSetListFull - 1);
+      if (!t.counted) rels[t.head]->set_outputs += total & (kSetListFull - 1);
     }
     for (uint32_t i = 0; i < rels.size(); ++i) {
       Relation& R = *rels[i];
       if (!R.set_on) continue;
-      if (!R.set_free && outputs[i] > 0xFFFFFFFFull)
-        return fail(CDL_E_CAPACITY, "relation " + R.name + " would receive more than 2^32 new "
-                                    "tuples in one round");
+      if (!R.set_free && R.set_outputs > 0xFFFFFFFFull) return too_many_new(R);
       if (R.set_redo || (R.set_single && h_ctl[kSlotDelta + i] > R.sdelta.cap)) redo[i] = any = true;
     }
     return CDL_OK;
@@ -2874,7 +2882,7 @@ struct cdl_engine {
       r->fresh_ub = 0;
       r->fresh_overflow = false;
       r->dense_ub = 0;
-      r->sdelta_ub = 0;
+      r->sdelta_ub = r->set_outputs = 0;
       r->set_single = r->set_redo = false;
     }
     if (est_ready() && est_bio.p) {  // the round's predictions, with one wait
@@ -2941,6 +2949,7 @@ struct cdl_engine {
           Relation& S = *rels[i];
           const uint64_t at = std::min<uint64_t>(h_ctl[kSlotDelta + i], S.sdelta.cap);
           h_ctl[kSlotDelta + i] = S.sdelta_ub = at;
+          S.set_outputs = 0;  // its joins are counted anew
           S.set_single = S.set_redo = false;
           if (S.fset.keys) {  // without the slots of the tuples that found no room
             bool ok = false;
