@@ -1169,53 +1169,82 @@ struct cdl_engine {
     return CDL_OK;
   }
 
+  // Takes the tuples of a round that was not completed out of the sets.
+  cdl_status sets_undo_round() {
+    const size_t nr = rels.size();
+    cudaError_t e = cudaMemcpyAsync(h_ctl + kSlotDelta, dslot(kSlotDelta), 8 * nr,
+                                    cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    for (size_t i = 0; i < nr && e == cudaSuccess; ++i) {
+      Relation& R = *rels[i];
+      if (!R.set_on) continue;
+      if (R.sdelta.buf.p)
+        e = dense_remove(ctx, R.fset, R.sdelta.in(), std::min(h_ctl[kSlotDelta + i], R.sdelta.cap));
+      R.sdelta.clear();
+      R.sdelta_ub = 0;
+    }
+    return e == cudaSuccess ? CDL_OK : cuda_fail(e, "full set");
+  }
+
+  // Full's rows out of the set, in order: R has the row form then (without
+  // rows where memory is short).  count: the set may hold other than full.n
+  // tuples.
+  cdl_status set_to_rows(Relation& R, bool count) {
+    R.set_on = false;
+    if (R.full.buf.p) return CDL_OK;  // (round 1 keeps its rows)
+    uint64_t n = R.full.n;
+    R.full.n = 0;
+    DCols rows;
+    if (R.fset.keys) {
+      cdl_status r = hash_rows(R, n, rows);
+      if (r != CDL_OK) return r;
+      n = rows.n;
+    } else if (n || count) {
+      DBuf ws = alloc(dense_extract_workspace(R.fset.nbits));
+      for (;;) {
+        if (!alloc_cols(rows, R.arity, n) || !ws.p) return fail(CDL_E_NOMEM, "sorted rows");
+        cudaError_t e = dense_extract(ctx, R.fset, rows.out(), n, dslot(kSlotScratch), ws.p);
+        if (e == cudaSuccess && count) {
+          e = cudaMemcpyAsync(h_ctl + kSlotScratch, dslot(kSlotScratch), 8, cudaMemcpyDeviceToHost, st);
+          if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "sorted rows");
+        const uint64_t had = n;
+        if (count) n = h_ctl[kSlotScratch];
+        if (n <= had) break;
+        cudaMemsetAsync(dslot(kSlotErr), 0, 8, st);  // (the copy that did not fit)
+      }
+    }
+    rows.k = R.arity;
+    rows.n = n;
+    R.full = std::move(rows);
+    R.version[kFull]++;
+    return CDL_OK;
+  }
+
   // At the end of the run Full's rows come out of the set in order; a delta
-  // that a checkpoint may save is put in order too.  After a failed run the
-  // set also holds the stopped round's tuples so far.
+  // that a checkpoint may save is put in order too.  A failed run leaves the
+  // tuples of its completed rounds (or, where an error in captured rounds
+  // hides how many they were, of all tuples derived).
   cdl_status set_finish(bool failed) {
+    bool any = false;
+    for (auto& r : rels) any |= r->set_on;
+    if (!any) return CDL_OK;
+    if (failed) {
+      cudaMemsetAsync(dslot(kSlotErr), 0, 8, st);  // (reported already)
+      cdl_status r = sets_undo_round();
+      if (r != CDL_OK) return r;
+    }
+    cdl_status status = CDL_OK;
     for (auto& rp : rels) {
       Relation& R = *rp;
       if (!R.set_on) continue;
-      uint64_t n = R.full.n;
-      if (failed) n = std::min(R.fset.nbits, n + std::min(R.sdelta_ub, R.sdelta.cap));
       R.sdelta.clear();
-      DCols rows;
-      if (R.fset.keys) {
-        cdl_status r = hash_rows(R, n, rows);
-        R.set_on = false;
-        if (r != CDL_OK) {
-          R.full.n = 0;
-          return r;
-        }
-        R.full = std::move(rows);
-        R.version[kFull]++;
-        r = set_sorted_delta(R);
-        if (r != CDL_OK) return r;
-        continue;
-      }
-      DBuf ws = alloc(dense_extract_workspace(R.fset.nbits));
-      if (!alloc_cols(rows, R.arity, n) || !ws.p) {
-        R.set_on = false;  // (no rows to export)
-        R.full.n = 0;
-        return fail(CDL_E_NOMEM, "sorted rows");
-      }
-      if (n) {
-        cudaError_t e = dense_extract(ctx, R.fset, rows.out(), n, dslot(kSlotScratch), ws.p);
-        if (e == cudaSuccess && failed) {
-          e = cudaMemcpyAsync(h_ctl + kSlotScratch, dslot(kSlotScratch), 8, cudaMemcpyDeviceToHost, st);
-          if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-          n = std::min(n, h_ctl[kSlotScratch]);
-        }
-        if (e != cudaSuccess) return cuda_fail(e, "sorted rows");
-      }
-      rows.n = n;
-      R.full = std::move(rows);
-      R.version[kFull]++;
-      R.set_on = false;
-      cdl_status r = set_sorted_delta(R);
-      if (r != CDL_OK) return r;
+      cdl_status r = set_to_rows(R, failed);
+      if (r == CDL_OK) r = set_sorted_delta(R);
+      if (status == CDL_OK) status = r;
     }
-    return CDL_OK;
+    return status;
   }
 
   cdl_status set_sorted_delta(Relation& R) {
@@ -1227,24 +1256,30 @@ struct cdl_engine {
     return sort_cols(R.delta, bits);
   }
 
-  // The keys of a hash set (at most n) as sorted rows.
+  // The keys of a hash set (about n) as sorted rows.
   cdl_status hash_rows(Relation& R, uint64_t n, DCols& rows) {
     DCols keys;
-    if (!alloc_cols(keys, 2, n)) return fail(CDL_E_NOMEM, "sorted rows");
-    cudaError_t e = hash_keys(ctx, R.fset, keys.c[0], keys.c[1], n, dslot(kSlotScratch));
-    if (e != cudaSuccess) return cuda_fail(e, "sorted rows");
-    cdl_status r = fetch(kSlotScratch, 1);
-    if (r != CDL_OK) return r;
-    keys.n = h_ctl[kSlotScratch];
+    for (;;) {
+      if (!alloc_cols(keys, 2, n)) return fail(CDL_E_NOMEM, "sorted rows");
+      cudaError_t e = hash_keys(ctx, R.fset, keys.c[0], keys.c[1], n, dslot(kSlotScratch));
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(h_ctl + kSlotScratch, dslot(kSlotScratch), 8, cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      if (e != cudaSuccess) return cuda_fail(e, "sorted rows");
+      keys.n = h_ctl[kSlotScratch];
+      if (keys.n <= n) break;
+      n = keys.n;
+      cudaMemsetAsync(dslot(kSlotErr), 0, 8, st);  // (the copy that did not fit)
+    }
     const DenseSet d = R.fset;
     R.fset_buf.reset();
     const uint32_t t = bits_of(d.nbits - 1);
     const uint32_t bits[2] = {t > 32 ? t - 32 : 0, std::min<uint32_t>(t, 32)};
-    r = sort_cols(keys, bits);
+    cdl_status r = sort_cols(keys, bits);
     if (r != CDL_OK) return r;
     if (!alloc_cols(rows, R.arity, keys.n)) return fail(CDL_E_NOMEM, "sorted rows");
     rows.n = keys.n;
-    e = hash_unpack(ctx, d, keys.c[0], keys.c[1], keys.n, rows.out());
+    cudaError_t e = hash_unpack(ctx, d, keys.c[0], keys.c[1], keys.n, rows.out());
     return e == cudaSuccess ? CDL_OK : cuda_fail(e, "sorted rows");
   }
 
@@ -3538,12 +3573,8 @@ struct cdl_engine {
         R.delta.clear();
         R.delta.k = R.arity;
         R.version[kDelta]++;
-        if (R.set_on) {  // the new tuples are delta already
-          if (R.full.buf.p) set_drop_rows(R);
-          R.delta = std::move(R.sdelta);
-          R.sdelta = DCols{};
+        if (R.set_on) {  // the new tuples are sdelta already
           merged[i] = R.sdelta_ub > 0;
-          R.version[kFull]++;
           continue;
         }
         if (R.dset.words) {  // the dense form: the round's rows come out sorted and unique
@@ -3586,12 +3617,19 @@ struct cdl_engine {
         Relation& R = *rels[i];
         if (!R.idb) continue;
         const uint64_t nd = merged[i] ? h_ctl[kSlotDelta + i] : 0;
+        if (R.set_on) {
+          if (R.full.n + nd > 0xFFFFFFFFull) {
+            status = fail(CDL_E_CAPACITY, "relation " + R.name + " would exceed 2^32 tuples");
+            break;
+          }
+          if (R.full.buf.p) set_drop_rows(R);
+          R.delta = std::move(R.sdelta);
+          R.delta.k = R.arity;
+          R.sdelta = DCols{};
+          R.version[kFull]++;
+        }
         R.delta.n = nd;
         R.full.n += nd;
-        if (R.set_on && R.full.n > 0xFFFFFFFFull) {
-          status = fail(CDL_E_CAPACITY, "relation " + R.name + " would exceed 2^32 tuples");
-          break;
-        }
         if (merged[i] && !R.set_on)  // the sort's passes and the merge, about
           R.merged_bytes += 8.0 * R.arity * (double)R.full.n + 64.0 * (double)R.fresh.n;
         if (R.set_on) {
