@@ -128,8 +128,9 @@ typedef struct {
                            (a 2 GB bitmap).  Where no rule variant reads such a relation's
                            Full after round 1 the bitmap is Full itself; larger ones (to
                            2^37 tuples) go over to that form when it pays, and in batched
-                           runs Full becomes a hash set of tuples.  -1 keeps sorted rows
-                           throughout.  Results never depend on it */
+                           runs Full becomes a hash set of tuples; where memory runs short
+                           they go back to sorted rows.  -1 keeps sorted rows throughout.
+                           Results never depend on it */
   int32_t dedup;        /* step (d) of derived relations whose Full no rule variant reads
                            after round 1 (every rule naming them has no other derived body
                            atom; batched runs excluded): 0 = default, the difference and

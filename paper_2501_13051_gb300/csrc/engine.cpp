@@ -100,6 +100,12 @@ class Pool {
     by_size_.emplace(b.size, p);
   }
 
+  size_t unused() const {
+    size_t b = 0;
+    for (auto& f : by_size_) b += f.first;
+    return b;
+  }
+
   // Returns every chunk with nothing allocated in it to the allocator.
   void trim() {
     for (auto it = chunks_.begin(); it != chunks_.end();) {
@@ -377,6 +383,7 @@ struct Relation {
   DBuf fset_buf;
   bool set_single = false;  // a single-pass join of this round wrote sdelta
   bool set_redo = false;    // ... and ran out of room: its rules run again, exact
+  bool delta_unsorted = false;  // delta came from a set: its rows are in no order
   DCols sdelta;          // the round's new tuples so far (dslot(kSlotDelta + i) of them)
   uint64_t sdelta_ub = 0;   // rows of it taken: counted, or what one-pass joins are expected to add
   uint64_t set_outputs = 0; // outputs of the round's counted joins and copies into the set
@@ -525,6 +532,8 @@ struct cdl_engine {
   static constexpr uint64_t kHashRows = 1 << 18;
   bool hashed = false;  // batched run: the derived relations' Fulls are hash sets
   static constexpr double kSetSwitch = 0.2;
+  // less than this is not given back without a memory limit (give_back_room)
+  static constexpr size_t kRoomBytes = 64 << 20;
   // hub joins (hub_join): outputs in all, and per row of both sides, from
   // which they are tried (below, the second count and the other index are
   // not small beside the write); build rows that make a hub, where OR-ing
@@ -1015,17 +1024,27 @@ struct cdl_engine {
     size_t free_b = 0, total_b = 0;
     if (rows < kHashRows || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return CDL_OK;
     if (hash_slots((hash_room + 1) * rows) * 8 > free_b / 4) return CDL_OK;
+    bool room = true;
     for (auto& r : rels) {
-      if (!r->idb) continue;
+      if (!r->idb || !room) continue;
       tuple_space(*r, kHashBits, r->fset);
       r->fset.append = 1;
-      bool ok = false;
       // (a graph wants its room at once: moving the keys later costs as much
       // as inserting them)
-      const uint64_t room = opt.graph ? hash_room + 1 : 4;
-      cdl_status s = hash_reserve(*r, room * r->full.n + (1 << 16), false, ok);
-      if (s == CDL_OK && !ok) s = fail(CDL_E_NOMEM, "full set");
+      const uint64_t times = opt.graph ? hash_room + 1 : 4;
+      cdl_status s = hash_reserve(*r, times * r->full.n + (1 << 16), false, room);
       if (s != CDL_OK) return s;
+    }
+    if (!room) {  // not for all of them: rows throughout
+      for (auto& r : rels) {
+        r->hash_ok = false;
+        r->fset_buf.reset();
+        r->fset = DenseSet{};
+      }
+      return CDL_OK;
+    }
+    for (auto& r : rels) {
+      if (!r->idb) continue;
       cudaError_t e = dense_insert(ctx, r->fset, r->full.in(), r->full.n);
       if (e != cudaSuccess) return cuda_fail(e, "full set");
       r->set_on = true;
@@ -1186,6 +1205,86 @@ struct cdl_engine {
     return e == cudaSuccess ? CDL_OK : cuda_fail(e, "full set");
   }
 
+  // Where a buffer of new tuples, sized by a bound on them, holds far fewer
+  // (n) and another of its size would take a good part of the memory there
+  // still is, its rows move to one of their own size.
+  void give_back_room(DCols& d, uint64_t n) {
+    if (!d.buf.p || n > d.cap / 2) return;
+    const size_t waste = 4ull * d.k * (d.cap - n);
+    size_t room = 0, total = 0;
+    if (opt.mem_limit)
+      room = opt.mem_limit - std::min(opt.mem_limit, pool.held);
+    else if (waste < kRoomBytes || cudaMemGetInfo(&room, &total) != cudaSuccess)
+      return;
+    if (waste < (room + pool.unused()) / 4) return;
+    DCols own;
+    if (!alloc_cols(own, d.k, n)) return;
+    for (uint32_t k = 0; k < d.k && n; ++k)
+      if (cudaMemcpyAsync(own.c[k], d.c[k], 4 * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+        return;
+    own.n = d.n;
+    d = std::move(own);
+  }
+
+  bool sets_used() const {
+    for (auto& r : rels)
+      if (r->set_on) return true;
+    return false;
+  }
+
+  // Memory ran short in a round while relations were kept as sets: the
+  // round's tuples leave them, Full's rows come out, and the run goes on in
+  // the row form (a round's new tuples as a bitmap where the tuple space is
+  // within dense_bits), which needs no room for a join's outputs beside a
+  // delta that had such room itself, and no larger hash table beside a full
+  // one.  The round is then run again.
+  cdl_status sets_to_rows() {
+    cdl_status r = sets_undo_round();
+    if (r != CDL_OK) return r;
+    cache.clear();
+    prev_full.clear();
+    set_heavy_buf.reset();
+    set_heavy = HeavyList{};
+    hashed = false;
+    for (auto& rp : rels) {
+      Relation& R = *rp;
+      R.set_ok = R.hash_ok = false;
+      if (!R.set_on) continue;
+      if (!R.delta.n) {
+        R.delta.clear();
+        R.delta.k = R.arity;
+      } else if (R.delta.n <= R.delta.cap / 2) {
+        DCols own;
+        if (alloc_cols(own, R.arity, R.delta.n)) {
+          own.n = R.delta.n;
+          for (uint32_t k = 0; k < R.arity; ++k) {
+            cudaError_t e = cudaMemcpyAsync(own.c[k], R.delta.c[k], 4 * own.n, cudaMemcpyDeviceToDevice, st);
+            if (e != cudaSuccess) return cuda_fail(e, "delta");
+          }
+          R.delta = std::move(own);
+          R.version[kDelta]++;
+        }
+      }
+    }
+    for (auto& rp : rels) {
+      Relation& R = *rp;
+      if (!R.set_on) continue;
+      r = set_to_rows(R, false);
+      if (r != CDL_OK) return r;
+      if (R.set_free) {
+        cudaError_t e = cudaMemsetAsync(R.fset_buf.p, 0, R.fset_buf.bytes, st);
+        if (e != cudaSuccess) return cuda_fail(e, "dense set");
+        R.dset = R.fset;
+        R.dset.append = 0;
+        R.dset_buf = std::move(R.fset_buf);
+        R.set_free = false;
+      }
+      R.fset_buf.reset();
+      R.fset = DenseSet{};
+    }
+    return CDL_OK;
+  }
+
   // Full's rows out of the set, in order: R has the row form then (without
   // rows where memory is short).  count: the set may hold other than full.n
   // tuples.
@@ -1250,7 +1349,8 @@ struct cdl_engine {
   cdl_status set_sorted_delta(Relation& R) {
     R.fset_buf.reset();
     R.fset = DenseSet{};
-    if (!R.delta.n) return CDL_OK;
+    if (!R.delta.n || !R.delta_unsorted) return CDL_OK;
+    R.delta_unsorted = false;
     uint32_t bits[kMaxK];
     for (uint32_t k = 0; k < R.arity; ++k) bits[k] = bits_of(R.bound[k]);
     return sort_cols(R.delta, bits);
@@ -1494,8 +1594,7 @@ struct cdl_engine {
     ix->n = s.n;
     bool prefix = true;
     for (size_t i = 0; i < key.size(); ++i) prefix &= key[i] == i;
-    // (a delta of a relation kept as a set is in no order)
-    if (s.rel >= 0 && s.ver == kDelta && rels[s.rel]->set_on) prefix = false;
+    if (s.rel >= 0 && s.ver == kDelta && rels[s.rel]->delta_unsorted) prefix = false;
     if (prefix) {
       for (uint32_t c = 0; c < s.k; ++c) ix->cols[c] = s.c[c];
     } else {
@@ -2361,7 +2460,7 @@ struct cdl_engine {
     }
     if (set_steps.size() >= kSetSteps) {
       if (!exact) return CDL_OK;
-      return fail(CDL_E_CAPACITY, "too many joins into hash sets in one round");
+      return fail(CDL_E_NOMEM, "too many joins into hash sets in one round");
     }
     cdl_status r = ensure_sdelta(H, want, exact != 0);
     if (r == CDL_E_NOMEM && !exact) {  // (nothing was changed but the bound)
@@ -3009,7 +3108,7 @@ struct cdl_engine {
     if (s != CDL_OK) return s;
     for (size_t i = steps_before; i < set_steps.size(); ++i)
       if (h_ctl[kSlotSetTotal + 2 * i] & kSetListFull)
-        return fail(CDL_E_CAPACITY, "a hash set ran out of slots");
+        return fail(CDL_E_NOMEM, "a hash set ran out of slots");
     for (uint32_t i = 0; i < nr; ++i)
       if (redo[i] && h_ctl[kSlotCursor + i] > rels[i]->fresh.cap)
         return fail(CDL_E_CAPACITY, "an exact join overflowed its buffer");
@@ -3449,6 +3548,7 @@ struct cdl_engine {
       }
       R.delta = std::move(G.D[dside]);
       R.delta.n = cur[j].nD;
+      R.delta_unsorted = G.set;
       R.version[kFull]++;
       R.version[kDelta]++;
     }
@@ -3461,8 +3561,7 @@ struct cdl_engine {
     for (size_t i = 0; i < rels.size() && ctl.done == 2; ++i)  // (without the undone tuples' slots)
       if (rels[i]->set_on && rels[i]->fset.keys) {
         bool ok = false;
-        r = hash_reserve(*rels[i], rels[i]->full.n, true, ok);
-        if (r == CDL_OK && !ok) r = fail(CDL_E_NOMEM, "full set");
+        r = hash_reserve(*rels[i], rels[i]->full.n, true, ok);  // (!ok: they stay taken)
         if (r != CDL_OK) return r;
       }
     if (ctl.done == 2) {
@@ -3491,6 +3590,20 @@ struct cdl_engine {
     }
     for (size_t s = 0; s < grec.size(); ++s)
       gcap_i[s] = std::max<uint64_t>(8 * grec[s].seen_total, floor);
+  }
+
+  // The round's new tuples, up to the sorts and merges of the row form.
+  cdl_status new_tuples(uint64_t round, bool first_semi) {
+    recording = opt.graph && first_semi;  // the first semi-naive round is the plan
+    if (recording) {
+      grec.clear();
+      grec_bad = false;
+    }
+    cdl_status s = eval_round(round);
+    recording = false;
+    if (s == CDL_OK) s = extract_dense();
+    if (s == CDL_OK) s = set_fresh_rows();
+    return s;
   }
 
   cdl_status run(cdl_stats* stats) {
@@ -3552,12 +3665,14 @@ struct cdl_engine {
     g_rounds = g_builds = g_retirements = 0;
     for (uint64_t round = resume_rounds + 1; status == CDL_OK; ++round) {
       cur_round = round;
-      cudaError_t e = cudaSuccess;
-      recording = opt.graph && round == first_semi;  // the first semi-naive round is the plan
-      status = eval_round(round);
-      recording = false;
-      if (status == CDL_OK) status = extract_dense();
-      if (status == CDL_OK) status = set_fresh_rows();
+      const uint64_t joins0 = joins, stars0 = star_joins;
+      status = new_tuples(round, round == first_semi);
+      if (status == CDL_E_NOMEM && sets_used()) {
+        status = sets_to_rows();
+        joins = joins0;
+        star_joins = stars0;
+        if (status == CDL_OK) status = new_tuples(round, round == first_semi);
+      }
       if (status != CDL_OK) break;
       // relations of one arity with few new tuples each are sorted as one
       std::vector<DCols> group_bufs, sorted_rows(nr);
@@ -3572,8 +3687,10 @@ struct cdl_engine {
         R.fresh.n = h_ctl[kSlotCursor + i];
         R.delta.clear();
         R.delta.k = R.arity;
+        R.delta_unsorted = R.set_on;
         R.version[kDelta]++;
-        if (R.set_on) {  // the new tuples are sdelta already
+        if (R.set_on) {  // the new tuples are in sdelta already
+          if (delta_known) give_back_room(R.sdelta, h_ctl[kSlotDelta + i]);
           merged[i] = R.sdelta_ub > 0;
           continue;
         }
@@ -3623,6 +3740,7 @@ struct cdl_engine {
             break;
           }
           if (R.full.buf.p) set_drop_rows(R);
+          give_back_room(R.sdelta, nd);
           R.delta = std::move(R.sdelta);
           R.delta.k = R.arity;
           R.sdelta = DCols{};
