@@ -877,8 +877,9 @@ struct cdl_engine {
 
   // The round's merges of several relations, those of one arity as one set of
   // launches where there are a few of them and none is large enough to fill
-  // the GPU by itself.  (Not under a memory limit: all merged versions are
-  // allocated before the first old one is freed.)
+  // the GPU by itself.  (Not under a memory limit, and not where memory is
+  // short: all merged versions are allocated before the first old one is
+  // freed.)
   static constexpr uint64_t kMergeGroupRows = 1 << 22;
   static constexpr size_t kMergeGroupMin = 3;
   cdl_status merge_all(std::vector<std::pair<uint32_t, DCols*>>& todo) {
@@ -893,11 +894,11 @@ struct cdl_engine {
       std::vector<MergeJob> jobs;
       std::vector<DCols> merged(grp.size()), delta(grp.size());
       MergeGroup g;
-      for (size_t i = 0; i < grp.size(); ++i) {
+      bool room = true;
+      for (size_t i = 0; i < grp.size() && room; ++i) {
         const Relation& R = *rels[grp[i].first];
         const DCols& U = *grp[i].second;
-        if (!alloc_cols(merged[i], k, R.full.n + U.n) || !alloc_cols(delta[i], k, U.n))
-          return fail(CDL_E_NOMEM, "merge buffers");
+        room = alloc_cols(merged[i], k, R.full.n + U.n) && alloc_cols(delta[i], k, U.n);
         MergeJob j{};
         j.F = R.full.in();
         j.U = U.in();
@@ -910,7 +911,7 @@ struct cdl_engine {
         jobs.push_back(j);
       }
       DBuf dj = alloc(sizeof(MergeJob) * jobs.size()), ws = alloc(merge_group_workspace(g));
-      if (!dj.p || !ws.p) return fail(CDL_E_NOMEM, "merge workspace");
+      if (!room || !dj.p || !ws.p) continue;  // one by one, then
       cudaError_t e = cudaMemcpyAsync(dj.p, jobs.data(), sizeof(MergeJob) * jobs.size(),
                                       cudaMemcpyHostToDevice, st);
       if (e == cudaSuccess)
