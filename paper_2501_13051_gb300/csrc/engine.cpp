@@ -616,6 +616,7 @@ struct cdl_engine {
   std::vector<GRelRes> grel;
   std::vector<GStepRes> gstep;
   std::vector<uint64_t> gcap_u, gcap_i, gcap_f;  // capacities by relation / step
+  uint64_t gcap_heavy = kSetHeavyCap;             // chunks of long ranges a captured round may list
   DBuf gdev;
   // device-side retirement of a batched graph: RetireCtl, then the
   // relations' RetireRel, then live / conv flags and the per-instance arrays
@@ -3226,7 +3227,7 @@ struct cdl_engine {
         ok &= alloc_cols(G.D[side], R.arity, G.Ucap);
       }
       if (G.set) {
-        ok &= set_heavy_list(kSetHeavyCap);
+        ok &= set_heavy_list(gcap_heavy);
       } else {
         ok &= alloc_cols(G.fresh, R.arity, G.Ucap) && alloc_cols(G.alt, R.arity, G.Ucap);
         G.sort_ws = alloc(radix_workspace(G.Ucap, G.plan.bits, G.plan.threads));
@@ -3342,6 +3343,7 @@ struct cdl_engine {
       if (H && H->set) {
         js.dout = reinterpret_cast<const ColsOut*>(&g_next()[slot[g.head]].D);
         HeavyList list = set_heavy;
+        list.cap = std::min(list.cap, gcap_heavy);
         list.n = g_step(s, 1);  // (zero, as the round's end leaves it)
         e = join_set(ctx, js, rels[g.head]->fset, ColsOut{}, g_cursor(slot[g.head]), H->Ucap,
                      g_step(s, 0), list);
@@ -3529,6 +3531,14 @@ struct cdl_engine {
       r = graph_retire_collect();
       if (r != CDL_OK) return r;
     }
+    if (ctl.done == 2) {  // a list of long ranges that was too short grows to what was listed
+      std::vector<uint64_t> w(3 * gstep.size());
+      e = cudaMemcpy(w.data(), g_step(0, 0), 8 * w.size(), cudaMemcpyDeviceToHost);
+      if (e != cudaSuccess) return cuda_fail(e, "graph steps");
+      for (size_t s = 0; s < gstep.size(); ++s)
+        if (grec[s].last && rels[grec[s].head]->set_on && (w[3 * s] & kSetListFull))
+          gcap_heavy = std::max(gcap_heavy, 2 * w[3 * s + 1]);
+    }
     for (size_t j = 0; j < grel.size(); ++j) {
       GRelRes& G = grel[j];
       Relation& R = *rels[G.rel];
@@ -3585,6 +3595,7 @@ struct cdl_engine {
     // option graph >= 2: that many rows at least instead of 2^16 (small
     // values make later rounds outgrow the buffers, as tests want)
     const uint64_t floor = opt.graph >= 2 ? (uint64_t)opt.graph : (1u << 16);
+    gcap_heavy = opt.graph >= 2 ? (uint64_t)opt.graph : kSetHeavyCap;
     for (size_t i = 0; i < rels.size(); ++i) {
       if (!rels[i]->idb) continue;
       gcap_u[i] = std::max<uint64_t>({8 * seen[i], 8 * rels[i]->delta.n, floor});
