@@ -1659,15 +1659,15 @@ struct cdl_engine {
     // features read the exact count, the tuner times hash tables, and under
     // a memory limit the direct form, up to 32 bytes a row where the hash
     // form may need few slots, stays small.)
-    const uint64_t bound = 1ull << s.bits[key[0]];
     const bool counted = opt.estimator || tuner.mode;
-    if (!k1 && !counted && bound <= direct_keys(opt.mem_limit ? 0 : s.n)) {
-      ix->table = alloc(8 * bound);
-      if (ix->table.p) ix->range = (uint32_t)bound;
+    const uint32_t entries = k1 || counted ? 0u : direct_entries(s.bits[key[0]], s.n, opt.mem_limit != 0);
+    if (entries) {
+      ix->table = alloc(8ull * entries);
+      if (ix->table.p) ix->range = entries;
     }
     cudaError_t e = cudaSuccess;
     if (ix->range) {
-      ix->distinct = std::min(bound, s.n);
+      ix->distinct = std::min<uint64_t>(ix->range, s.n);
     } else if (!counted && !opt.mem_limit && s.n <= kUncountedRows) {
       ix->distinct = s.n;
     } else {

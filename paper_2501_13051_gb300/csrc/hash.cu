@@ -207,8 +207,6 @@ cudaError_t hash_build(Ctx& c, const uint32_t* k0, const uint32_t* k1, uint64_t 
   return cudaGetLastError();
 }
 
-uint64_t direct_keys(uint64_t n) { return 4 * n > 65536 ? 4 * n : 65536; }
-
 cudaError_t index_build(Ctx& c, const uint32_t* k0, uint64_t n, const KeyIndex& x) {
   if (!x.range) return hash_build(c, k0, nullptr, n, const_cast<Slot*>(x.table), x.slots);
   const unsigned grid = (unsigned)((n + kThreads - 1) / kThreads);

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "limits.h"
 
 namespace cdl {
 
@@ -84,13 +85,6 @@ uint64_t table_slots(uint64_t n_keys, double load);
 // keys: columns k0 (and k1 when non-null) sorted lexicographically, n rows.
 cudaError_t hash_build(Ctx& c, const uint32_t* k0, const uint32_t* k1, uint64_t n, Slot* table,
                        uint64_t slots);
-// Keys (one word) up to which the direct form of an index over n rows is
-// taken where their bound is known: its array is then cleared and read at no
-// more than 32 bytes per row (hash slots take 32 to 64 per distinct key), or
-// is small beside a launch.  It also spares the count of the keys and the
-// wait for it: points-to at 2^-7 15.6 -> 14.9 ms, a closure of 4,001 nodes
-// 5.26 -> 4.89 ms.
-uint64_t direct_keys(uint64_t n);
 // Fills x.table (8 * range bytes, or 16 * slots) from n sorted one-word
 // keys: the form x describes (a hash form through hash_build).  With x.last
 // the table has room for 16 * slots bytes whichever form the keys give; the
