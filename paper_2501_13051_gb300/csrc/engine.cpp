@@ -3214,9 +3214,8 @@ struct cdl_engine {
       // (Full as a bitmap: the joins append to delta; no rows of Full, no
       // sort, no merge)
       G.set = R.set_on;
-      uint64_t set_full = ~0ull;
+      const uint64_t set_full = graph_set_rows(R.full.n, G.set && R.fset.keys ? hash_room : 0);
       if (R.fset.keys && G.set) {  // room for the rows of many rounds, and what one may add
-        set_full = std::max<uint64_t>(hash_room * R.full.n, 1 << 16);
         bool fits = false;
         cdl_status hs = hash_reserve(R, set_full + G.Ucap / 8, false, fits);
         if (hs != CDL_OK) return hs;

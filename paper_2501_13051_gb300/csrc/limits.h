@@ -22,4 +22,14 @@ inline uint32_t direct_entries(uint32_t bits, uint64_t rows, bool limited) {
   return !limited && keys <= 4 * rows && keys <= kDirectKeysMax ? (uint32_t)keys : 0u;
 }
 
+// Rows that Full, kept as a set, may have at the end of a captured round: with
+// more the round leaves the graph and is run by the host, which stops at the
+// 2^32 tuples a relation may hold.  times: a hash set's table is for so many
+// times the rows there are (0: a bitmap, which has room for every tuple).
+inline uint64_t graph_set_rows(uint64_t rows, uint64_t times) {
+  constexpr uint64_t kMost = 0xFFFFFFFFull, kLeast = 1ull << 16;
+  if (times == 0 || rows > kMost / times) return kMost;
+  return times * rows > kLeast ? times * rows : kLeast;
+}
+
 }  // namespace cdl

@@ -36,3 +36,13 @@ def test_direct_entries(tmp_path):
         assert g < 1 << 32 and 8 * g <= max(32 * n, 512 << 10)
     # 2^32 keys do not fit the 32-bit number of entries: rows or not, the hash form
     assert [g for (b, n, lim), g in zip(cases, got) if b == 32] == [0] * 22
+
+
+def test_graph_set_rows(tmp_path):
+    cases = [(n, t) for t in (0, 1, 8) for n in (0, 1, 8192, 8193, 1 << 20, (1 << 29) - 1, 1 << 29, (1 << 29) + 1,
+                                                 1 << 31, (1 << 32) - 1)]
+    got = values(tmp_path, ["graph_set_rows(%dull, %d)" % c for c in cases])
+    most = (1 << 32) - 1
+    for (n, t), g in zip(cases, got):
+        assert g == (most if t == 0 else min(most, max(1 << 16, t * n))), (n, t)
+        assert g >= n  # (Full fits when the graph begins)
