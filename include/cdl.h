@@ -459,7 +459,10 @@ cdl_status cdl_join(const uint32_t* const* probe_cols, uint32_t probe_arity, uin
 /* The write of cdl_join alone, for a caller that sizes its output first: to
  * be called after a cdl_join with the same arguments and workspace that
  * returned CDL_E_CAPACITY, the workspace untouched since, with *n_out as
- * that call left it.  Nothing is indexed or counted again. */
+ * that call left it.  Nothing is indexed or counted again.  As often as
+ * wanted; a workspace that bears the mark of no such call, or of one with
+ * other sizes, key columns or workspace size, is CDL_E_INVALID and nothing
+ * is written (what else was written into it in between is not noticed). */
 cdl_status cdl_join_write(const uint32_t* const* probe_cols, uint32_t probe_arity,
                           uint64_t n_probe, uint32_t probe_key, const uint32_t* const* build_cols,
                           uint32_t build_arity, uint64_t n_build, uint32_t build_key,

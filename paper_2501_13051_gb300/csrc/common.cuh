@@ -24,7 +24,8 @@ enum : uint32_t {
   kErrTimeout = 1u,   // a bounded wait ran out
   kErrCapacity = 2u,  // an output cursor passed its capacity
   kErrValue = 4u,     // the reserved value was seen in input
-  kErrTable = 8u      // a hash table had no free slot
+  kErrTable = 8u,     // a hash table had no free slot
+  kErrState = 16u     // a write whose count was another one (join_open)
 };
 
 // 32-bit finaliser of MurmurHash3 (Austin Appleby, public domain): a

@@ -422,6 +422,8 @@ __global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5)
   __shared__ unsigned long long s_base;
   __shared__ SetRefs refs;
   if constexpr (FORM == kSet) stage_refs(j, dset, out, refs);
+  if constexpr (FORM == kRows)
+    if (j.gate && *j.gate == 0) return;
   const uint64_t n_probe = dev_size(j.dn, j.n_probe);
   const ColsIn probe = probe_cols(j);
   // a device-given join size past the capacity the launch was sized for:
@@ -1352,6 +1354,32 @@ cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, 
   else
     CDL_JOIN_SET(false, false);
 #undef CDL_JOIN_SET
+  return cudaGetLastError();
+}
+
+// A count's mark and its check (kernels.h): one thread.
+constexpr uint64_t kMarkTag = 0x6a6f696e636f756eull;
+__global__ void k_join_mark(uint64_t* head, JoinMark m) {
+  head[4] = kMarkTag;
+  head[5] = m.probe;
+  head[6] = m.build;
+  head[7] = m.form;
+}
+__global__ void k_join_open(uint64_t* head, JoinMark m, uint64_t total) {
+  const bool ok = head[1] == total && head[4] == kMarkTag && head[5] == m.probe &&
+                  head[6] == m.build && head[7] == m.form;
+  head[0] = ok ? 0 : kErrState;
+  head[2] = 0;
+  head[3] = ok;
+}
+
+cudaError_t join_mark(Ctx& c, uint64_t* head, const JoinMark& m) {
+  k_join_mark<<<1, 1, 0, c.st>>>(head, m);
+  return cudaGetLastError();
+}
+
+cudaError_t join_open(Ctx& c, uint64_t* head, const JoinMark& m, uint64_t total) {
+  k_join_open<<<1, 1, 0, c.st>>>(head, m, total);
   return cudaGetLastError();
 }
 

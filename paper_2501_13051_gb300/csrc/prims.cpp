@@ -43,6 +43,7 @@ cdl_status read_flags(uint64_t* head, cudaStream_t st, uint64_t* host, int n) {
     return CDL_E_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return CDL_E_CUDA;
   const uint32_t f = (uint32_t)host[0];
+  if (f & kErrState) return CDL_E_INVALID;
   if (f & kErrTimeout) return CDL_E_TIMEOUT;
   if (f & kErrCapacity) return CDL_E_CAPACITY;
   if (f & kErrTable) return CDL_E_CAPACITY;
@@ -124,7 +125,8 @@ cdl_status cdl_exclusive_scan(const uint32_t* in, uint64_t n, uint64_t* out, uin
 // cdl_join and cdl_join_write: checked arguments and the workspace's parts.
 struct JoinCall {
   JoinSpec j{};
-  uint64_t* head;  // error word, total, output cursor
+  uint64_t* head;  // error word, total, output cursor; gate and mark (join_open)
+  JoinMark mark;
   Slot* table;
   uint64_t* off;
   void* cws;
@@ -180,6 +182,9 @@ static cdl_status join_setup(const uint32_t* const* probe_cols, uint32_t probe_a
     // (from 2^22 rows the entries by key may outgrow L2: offsets instead)
     if (n_build >= 1ull << 22) j.ix.rows = (uint32_t)n_build;
   }
+  // what the offsets and the kept starts depend on
+  jc.mark = JoinMark{n_probe, n_build, (uint64_t)probe_key | (uint64_t)build_key << 8 |
+                                           (uint64_t)(j.starts != nullptr) << 16};
   return CDL_OK;
 }
 
@@ -234,7 +239,8 @@ cdl_status cdl_join(const uint32_t* const* probe_cols, uint32_t probe_arity, uin
   const uint64_t total = h[1];
   *n_out = total;
   if (total == 0) return CDL_OK;
-  if (out_cap < total) return CDL_E_CAPACITY;
+  if (out_cap < total)  // (the workspace is ready for cdl_join_write)
+    return join_mark(c, jc.head, jc.mark) == cudaSuccess ? CDL_E_CAPACITY : CDL_E_CUDA;
   return join_output(jc, out_cols, out_arity, out_cap, total, n_out, c);
 }
 
@@ -257,6 +263,8 @@ cdl_status cdl_join_write(const uint32_t* const* probe_cols, uint32_t probe_arit
   Ctx c;
   c.st = static_cast<cudaStream_t>(stream);
   c.d_err = reinterpret_cast<uint32_t*>(jc.head);
+  if (join_open(c, jc.head, jc.mark, total) != cudaSuccess) return CDL_E_CUDA;
+  jc.j.gate = jc.head + 3;
   return join_output(jc, out_cols, out_arity, out_cap, total, n_out, c);
 }
 
