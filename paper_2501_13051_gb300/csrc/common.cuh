@@ -288,9 +288,10 @@ __device__ __forceinline__ uint32_t set_column(const DenseSet& d, uint64_t idx, 
 
 // Adds the tuples idx[0..N) (kNoTuple: none) to Full's bitmap; bit q of the
 // result tells that this call set tuple q's bit, i.e. the tuple is new.  A
-// set bit never goes back, so one seen set by a plain read (of any age, from
-// L1 or L2) needs no atomic; the N reads, then the N atomics, are in flight
-// together.
+// bit seen set by a plain read (of any age, from L1 or L2) needs no atomic: a
+// set bit is cleared again only where a new tuple found no room (set_store),
+// and then the round's rules for the relation run again.  The N reads, then
+// the N atomics, are in flight together.
 template <int N>
 __device__ __forceinline__ uint32_t set_add(const DenseSet& d, const uint64_t (&idx)[N]) {
   uint32_t seen[N];
@@ -376,49 +377,27 @@ __device__ __forceinline__ void set_remove(const DenseSet& d, uint64_t idx) {
 }
 
 // Writes a block's new tuples (bit q of fresh: tuple idx[q] is new) packed at
-// *cursor: one claim per block, each warp's tuples of one q side by side.
-// wsum: THREADS / 32 + 2 words of shared memory (the last two hold the
-// claimed position).  Rows past cap are dropped; false tells the caller.
+// *cursor.  wsum as for claim_places.  Rows past cap are dropped; false tells
+// the caller.
 template <int THREADS, int N>
 __device__ __forceinline__ bool set_emit(const DenseSet& d, const uint64_t (&idx)[N],
-                                         uint32_t fresh, ColsOut out, uint64_t base,
-                                         unsigned long long* cursor, uint64_t cap,
-                                         uint32_t* wsum) {
-  constexpr int W = THREADS / 32;
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t lt = (1u << lane) - 1u;
-  uint32_t n = 0;
-#pragma unroll
-  for (int q = 0; q < N; ++q) n += __popc(__ballot_sync(0xffffffffu, (fresh >> q) & 1u));
-  if (lane == 0) wsum[warp] = n;
-  __syncthreads();
-  unsigned long long* at = reinterpret_cast<unsigned long long*>(wsum + W);
-  uint32_t before = 0, total = 0;
-#pragma unroll
-  for (int w = 0; w < W; ++w) {
-    const uint32_t c = wsum[w];
-    before += w < (int)warp ? c : 0u;
-    total += c;
-  }
-  if (total == 0) return true;  // uniform
-  if (threadIdx.x == 0) *at = atomicAdd(cursor, (unsigned long long)total);
-  __syncthreads();
-  uint64_t pos = base + *at + before;
+                                         uint32_t fresh, ColsOut out, unsigned long long* cursor,
+                                         uint64_t cap, uint32_t* wsum) {
+  uint32_t at[N];
+  uint64_t pos;
+  if (!claim_places<THREADS, N>(fresh, cursor, wsum, at, &pos)) return true;
   bool ok = true;
 #pragma unroll
   for (int q = 0; q < N; ++q) {
-    const uint32_t bal = __ballot_sync(0xffffffffu, (fresh >> q) & 1u);
-    if ((fresh >> q) & 1u) {
-      const uint64_t p = pos + __popc(bal & lt);
-      if (p < cap) {
+    if (!((fresh >> q) & 1u)) continue;
+    const uint64_t p = pos + at[q];
+    if (p < cap) {
 #pragma unroll
-        for (int k = 0; k < kMaxK; ++k)
-          if (k < (int)d.k) out.c[k][p] = set_column(d, idx[q], k);
-      } else {
-        ok = false;
-      }
+      for (int k = 0; k < kMaxK; ++k)
+        if (k < (int)d.k) out.c[k][p] = set_column(d, idx[q], k);
+    } else {
+      ok = false;
     }
-    pos += __popc(bal);
   }
   return ok;
 }

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kAT) k_set_insert(DenseSet d, ColsIn rows, uin
     else
       fresh = set_add<kAItems>(d, idx);
     if constexpr (EMIT) {
-      bad |= !set_emit<kAT, kAItems>(d, idx, fresh, out, 0, cursor, cap, red);
+      bad |= !set_emit<kAT, kAItems>(d, idx, fresh, out, cursor, cap, red);
       __syncthreads();  // the next tile reuses red
     }
     if (bad && err) atomicOr(err, kErrCapacity);

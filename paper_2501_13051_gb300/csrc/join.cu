@@ -66,24 +66,6 @@ __device__ __forceinline__ uint32_t lookup2(const JoinSpec& j, const ColsIn& pro
   return find_key(j.ix2, direct_range(j.ix2), __ldg(col_of(probe, j.qk0) + row), k1, start);
 }
 
-// Output count of probe row `row`: its range length, or for a star join the
-// product of its two range lengths (a product past 2^32 - 1 raises
-// kErrCapacity and counts 0: no relation holds that many rows).
-__device__ __forceinline__ uint32_t row_count(const JoinSpec& j, const ColsIn& probe,
-                                             uint32_t range, uint64_t row, uint32_t* err) {
-  uint32_t st;
-  const uint32_t c1 = lookup(j, probe, range, row, &st);
-  if (j.starts) j.starts[row] = st;
-  if (j.hub_min && c1 >= j.hub_min) return 0;  // hub_or's
-  if (!j.star || c1 == 0) return c1;
-  const uint64_t prod = (uint64_t)c1 * lookup2(j, probe, row, &st);
-  if (prod > 0xFFFFFFFFull) {
-    if (err) atomicOr(err, kErrCapacity);
-    return 0;
-  }
-  return (uint32_t)prod;
-}
-
 // The probe side of a launch: the spec's columns and row count, or (inside
 // a captured round) the ones device memory holds, the count clamped to the
 // capacity the spec's n_probe then gives.
@@ -193,11 +175,10 @@ __global__ void __launch_bounds__(kCT) k_join_count(const JoinSpec j, uint32_t* 
 }
 
 __global__ void __launch_bounds__(kCT) k_join_count_only(const JoinSpec j,
-                                                         uint32_t* __restrict__ counts,
-                                                         uint32_t* err) {
+                                                         uint32_t* __restrict__ counts) {
   const uint64_t row = (uint64_t)blockIdx.x * kCT + threadIdx.x;
-  if (row >= j.n_probe) return;
-  counts[row] = row_count(j, j.probe, direct_range(j.ix), row, err);
+  uint32_t start;
+  if (row < j.n_probe) counts[row] = lookup(j, j.probe, direct_range(j.ix), row, &start);
 }
 
 // Number of probe rows among the first d items of the merge of the row
@@ -674,8 +655,7 @@ __global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5)
 cudaError_t join_count_only(Ctx& c, const JoinSpec& j, uint32_t* counts) {
   if (j.n_probe == 0) return cudaSuccess;
   ProfScope p(c, kJoinCount, (j.pk1 == 0xFFu ? 4.0 : 8.0) * j.n_probe + 20.0 * j.n_probe);
-  k_join_count_only<<<(unsigned)((j.n_probe + kCT - 1) / kCT), kCT, 0, c.st>>>(j, counts,
-                                                                              c.d_err);
+  k_join_count_only<<<(unsigned)((j.n_probe + kCT - 1) / kCT), kCT, 0, c.st>>>(j, counts);
   return cudaGetLastError();
 }
 

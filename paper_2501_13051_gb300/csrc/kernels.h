@@ -393,7 +393,7 @@ cudaError_t select_project(Ctx& c, const SelectSpec& s, ColsOut out, uint64_t* d
                            uint64_t out_cap, uint32_t* soft_overflow = nullptr);
 
 // last_round[v] = round for every instance id v < n_instances present in the
-// sorted instance column inst (n rows).
+// instance column inst (n rows, in any order).
 // Inside a captured round (dinst non-null): column 0 of *dinst, the count
 // *dn (clamped to n) and round + *dround.
 cudaError_t mark_instances(Ctx& c, const uint32_t* inst, uint64_t n, uint32_t n_instances,

@@ -386,7 +386,7 @@ cdl_status cdl_sort_unique(const uint32_t* const* cols, uint32_t arity, uint64_t
 cdl_status cdl_mlp_forward(const float* params, const float* X, uint64_t n, float* out,
                            void* workspace, size_t* ws_bytes, void* stream) {
   if (!ws_bytes) return CDL_E_INVALID;
-  const size_t need = mlp_workspace(n);
+  const size_t need = mlp_workspace(n);  // (the call's contract; the kernel keeps nothing in it)
   if (!workspace) {
     *ws_bytes = need;
     return CDL_OK;

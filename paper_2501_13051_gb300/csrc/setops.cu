@@ -109,9 +109,11 @@ __global__ void __launch_bounds__(256) k_check_columns(const CheckJob* __restric
   if (lane_id() == 0 && m) atomicMax(j.max, m);
 }
 
-// Batched fixpoints: the delta of a relation whose column 0 is an instance
-// id is sorted by instance, so every run head marks an instance that derived
-// something in this round.
+// Batched fixpoints: every row of a delta whose column 0 is an instance id
+// marks its instance as one that derived something in this round; a row whose
+// neighbour before it has the same instance leaves the store to that one.
+// The rows may be in any order (a delta of sorted rows stores once per
+// instance, one that came from a hash set about once per row).
 __global__ void k_mark_instances(const uint32_t* __restrict__ inst, uint64_t n,
                                  uint32_t n_instances, uint64_t* __restrict__ last_round,
                                  uint64_t round, const ColsIn* dinst, const uint64_t* dn,
@@ -128,8 +130,8 @@ __global__ void k_mark_instances(const uint32_t* __restrict__ inst, uint64_t n,
   }
 }
 
-// bounds[i] = the first row whose instance id (column 0, sorted) is >= i,
-// for i in [0, n_instances].
+// bounds[i] = the first row whose instance id (column 0, sorted: Full's rows,
+// not a delta from a hash set) is >= i, for i in [0, n_instances].
 __global__ void k_instance_bounds(const uint32_t* __restrict__ inst, uint64_t n,
                                   uint32_t n_instances, uint64_t* __restrict__ bounds) {
   const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
