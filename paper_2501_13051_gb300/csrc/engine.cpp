@@ -532,8 +532,10 @@ struct cdl_engine {
   static constexpr uint64_t kHashRows = 1 << 18;
   bool hashed = false;  // batched run: the derived relations' Fulls are hash sets
   static constexpr double kSetSwitch = 0.2;
-  // less than this is not given back without a memory limit (give_back_room)
-  static constexpr size_t kRoomBytes = 64 << 20;
+  // less than this, a seventieth of the device's memory, is not given back
+  // without a memory limit (give_back_room): asking what is free takes longer
+  // than a small round
+  static constexpr size_t kRoomBytes = size_t(4) << 30;
   // hub joins (hub_join): outputs in all, and per row of both sides, from
   // which they are tried (below, the second count and the other index are
   // not small beside the write); build rows that make a hub, where OR-ing

@@ -826,8 +826,7 @@ __global__ void __launch_bounds__(kCT) k_hub_or(const JoinSpec j, const DenseSet
                 for (int c2 = 0; c2 < kMaxK; ++c2)
                   if (c2 < (int)d.k) out.c[c2][pos] = set_column(d, idx, c2);
               } else {
-                set_remove(d, idx);
-                atomicOr(err, kErrCapacity);
+                atomicOr(err, kErrCapacity);  // (cannot happen: the caller gives room for all)
               }
               ++pos;
             }
