@@ -25,7 +25,7 @@ enum : uint32_t {
   kErrCapacity = 2u,  // an output cursor passed its capacity
   kErrValue = 4u,     // the reserved value was seen in input
   kErrTable = 8u,     // a hash table had no free slot
-  kErrState = 16u     // a write whose count was another one (join_open)
+  kErrState = 16u     // a write whose count was another one (join_begin)
 };
 
 // 32-bit finaliser of MurmurHash3 (Austin Appleby, public domain): a

@@ -202,12 +202,41 @@ __device__ __forceinline__ uint64_t merge_split(const uint64_t* off, uint64_t n,
 // Inside a captured round an unfiltered join's output range is claimed here
 // too (thread 0): *d_base = *cursor, *cursor += the join's size, and a range
 // past cap raises *overflow.
+// A count's mark and its check (kernels.h).  The check costs the write no
+// launch and no wait of its own: the splits bear its result (kClosed), and
+// only a write that searches its splits itself has it from a launch before.
+constexpr uint64_t kMarkTag = 0x6a6f696e636f756eull, kClosed = ~0ull;
+__device__ __forceinline__ bool marked(const uint64_t* head, const JoinMark& m, uint64_t total) {
+  return head[1] == total && head[4] == kMarkTag && head[5] == m.probe && head[6] == m.build &&
+         head[7] == m.form;
+}
+__device__ __forceinline__ void open_write(uint64_t* head, bool open) {
+  head[0] = open ? 0 : kErrState;
+  head[2] = 0;
+  head[3] = open;
+}
+__global__ void k_join_begin(uint64_t* head, JoinMark m) {
+  head[0] = head[1] = head[2] = head[3] = 0;
+  head[4] = kMarkTag;
+  head[5] = m.probe;
+  head[6] = m.build;
+  head[7] = m.form;
+}
+__global__ void k_join_open(uint64_t* head, JoinMark m, uint64_t total) {
+  open_write(head, marked(head, m, total));
+}
+
 __global__ void k_write_splits(const uint64_t* __restrict__ off, uint64_t n, uint64_t total,
                                uint64_t* __restrict__ splits, uint64_t nblocks,
                                const uint64_t* dn, const uint64_t* dtotal,
                                unsigned long long* cursor, uint64_t* d_base, uint64_t cap,
-                               uint32_t* overflow) {
+                               uint32_t* overflow, uint64_t* head, JoinMark mark) {
   const uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  bool open = true;
+  if (head) {
+    open = marked(head, mark, total);
+    if (b == 0) open_write(head, open);
+  }
   if (d_base && b == 0) {
     const uint64_t b0 = *cursor, t = *dtotal;
     *d_base = b0;
@@ -221,7 +250,7 @@ __global__ void k_write_splits(const uint64_t* __restrict__ off, uint64_t n, uin
   }
   if (b > nblocks) return;
   const uint64_t d = b * kJTile < n + total ? b * kJTile : n + total;
-  splits[b] = merge_split(off, n, total, d);
+  splits[b] = open ? merge_split(off, n, total, d) : kClosed;
 }
 
 __device__ __forceinline__ uint32_t ref_value(const JoinSpec& j, const ColsIn& probe, const Ref& r,
@@ -403,8 +432,6 @@ __global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5)
   __shared__ unsigned long long s_base;
   __shared__ SetRefs refs;
   if constexpr (FORM == kSet) stage_refs(j, dset, out, refs);
-  if constexpr (FORM == kRows)
-    if (j.gate && *j.gate == 0) return;
   const uint64_t n_probe = dev_size(j.dn, j.n_probe);
   const ColsIn probe = probe_cols(j);
   // a device-given join size past the capacity the launch was sized for:
@@ -424,13 +451,16 @@ __global__ void __launch_bounds__(kJT, FORM == kBits ? 8 : FORM == kSet ? 4 : 5)
   if (splits) {
     if (threadIdx.x < 2) s_split[threadIdx.x] = splits[tile + threadIdx.x];
   } else {
-    if (threadIdx.x == 0) s_split[0] = merge_split(off, n_probe, total, d0);
+    if (threadIdx.x == 0)
+      s_split[0] = FORM == kRows && j.head && !j.head[3] ? kClosed : merge_split(off, n_probe, total, d0);
     if (threadIdx.x == 32) s_split[1] = merge_split(off, n_probe, total, d1);
   }
   // (a device-sized launch had its range claimed by the split kernel)
   if (!FILTER && FORM == kRows && !dbase && tile == 0 && threadIdx.x == 0)
     atomicAdd(cursor, (unsigned long long)total);
   __syncthreads();
+  if constexpr (FORM == kRows)
+    if (s_split[0] == kClosed) return;
   const uint64_t j0 = s_split[0], j1 = s_split[1];
   const uint64_t o0 = d0 - j0, o1 = d1 - j1;
   const uint64_t r_lo = j0 > 0 ? j0 - 1 : 0;
@@ -1336,29 +1366,8 @@ cudaError_t join_set(Ctx& c, const JoinSpec& j, const DenseSet& d, ColsOut out, 
   return cudaGetLastError();
 }
 
-// A count's mark and its check (kernels.h): one thread.
-constexpr uint64_t kMarkTag = 0x6a6f696e636f756eull;
-__global__ void k_join_mark(uint64_t* head, JoinMark m) {
-  head[4] = kMarkTag;
-  head[5] = m.probe;
-  head[6] = m.build;
-  head[7] = m.form;
-}
-__global__ void k_join_open(uint64_t* head, JoinMark m, uint64_t total) {
-  const bool ok = head[1] == total && head[4] == kMarkTag && head[5] == m.probe &&
-                  head[6] == m.build && head[7] == m.form;
-  head[0] = ok ? 0 : kErrState;
-  head[2] = 0;
-  head[3] = ok;
-}
-
-cudaError_t join_mark(Ctx& c, uint64_t* head, const JoinMark& m) {
-  k_join_mark<<<1, 1, 0, c.st>>>(head, m);
-  return cudaGetLastError();
-}
-
-cudaError_t join_open(Ctx& c, uint64_t* head, const JoinMark& m, uint64_t total) {
-  k_join_open<<<1, 1, 0, c.st>>>(head, m, total);
+cudaError_t join_begin(Ctx& c, uint64_t* head, const JoinMark& m) {
+  k_join_begin<<<1, 1, 0, c.st>>>(head, m);
   return cudaGetLastError();
 }
 
@@ -1381,7 +1390,9 @@ cudaError_t join_write(Ctx& c, const JoinSpec& j, const uint64_t* d_off, uint64_
     k_write_splits<<<(unsigned)((blocks + 1 + 255) / 256), 256, 0, c.st>>>(
         d_off, j.n_probe, total, splits, blocks, j.dn, d_total,
         reinterpret_cast<unsigned long long*>(d_cursor), d_base, out_cap,
-        d_soft_err ? d_soft_err : c.d_err);
+        d_soft_err ? d_soft_err : c.d_err, j.head, j.mark);
+  } else if (j.head) {
+    k_join_open<<<1, 1, 0, c.st>>>(j.head, j.mark, total);
   }
   // per probe row: two offsets, key, re-probed slot (a star join: both
   // keys and slots), its own head columns; per output: the gathered build

@@ -111,6 +111,9 @@ struct Ref {
   uint8_t side;  // 0 probe, 1 build, 2 constant, 3 second build side (star joins)
   uint32_t v;
 };
+struct JoinMark {
+  uint64_t probe, build, form;
+};
 struct JoinSpec {
   ColsIn probe;
   uint64_t n_probe;
@@ -143,7 +146,10 @@ struct JoinSpec {
   // rows matching a key of at least hub_min build rows count 0 outputs: they
   // are left to hub_or (0: no such keys)
   uint32_t hub_min;
-  const uint64_t* gate;  // (rows) when set: nothing is written where it holds 0
+  // (rows) when set, the write is another call's than the count's: it checks
+  // the count's mark (join_begin) before it writes
+  uint64_t* head;
+  JoinMark mark;
 };
 // Hub keys of an unfiltered join into a bitmap, where the build side gives
 // the last head column (the lowest bits of a tuple's position, hub_words
@@ -163,15 +169,13 @@ size_t hub_workspace(const JoinSpec& j, const HubPlan& h);
 cudaError_t hub_or(Ctx& c, const JoinSpec& j, const HubPlan& h, const DenseSet& d, ColsOut out,
                    uint64_t* d_cursor, uint64_t out_cap, void* ws);
 size_t join_count_workspace(uint64_t n_probe);
-// The count's mark in the caller's memory (head: error word, total, output
-// cursor, gate, mark), and its check before a write of its own call: the
-// error word and the cursor are cleared, and the gate opens only where the
-// mark and the total are these (else kErrState in the error word).
-struct JoinMark {
-  uint64_t probe, build, form;
-};
-cudaError_t join_mark(Ctx& c, uint64_t* head, const JoinMark& m);
-cudaError_t join_open(Ctx& c, uint64_t* head, const JoinMark& m, uint64_t total);
+// A count's mark in the caller's memory (head: error word, total, output
+// cursor, gate, mark): join_begin clears the other words and leaves the mark,
+// in place of a memset.  A write by another call than the count's (join_write
+// with j.head and j.mark) checks it: the error word and the cursor are
+// cleared, and rows are written only where the mark and the total are the
+// write's own (else kErrState in the error word).
+cudaError_t join_begin(Ctx& c, uint64_t* head, const JoinMark& m);
 // Pass 1 alone: counts[i] for every probe row.
 cudaError_t join_count_only(Ctx& c, const JoinSpec& j, uint32_t* counts);
 // Pass 1 + 2: counts and exclusive offsets of every probe row; total in *d_total.

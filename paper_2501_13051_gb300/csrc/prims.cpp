@@ -125,7 +125,7 @@ cdl_status cdl_exclusive_scan(const uint32_t* in, uint64_t n, uint64_t* out, uin
 // cdl_join and cdl_join_write: checked arguments and the workspace's parts.
 struct JoinCall {
   JoinSpec j{};
-  uint64_t* head;  // error word, total, output cursor; gate and mark (join_open)
+  uint64_t* head;  // error word, total, output cursor; gate and mark (join_begin)
   JoinMark mark;
   Slot* table;
   uint64_t* off;
@@ -229,7 +229,7 @@ cdl_status cdl_join(const uint32_t* const* probe_cols, uint32_t probe_arity, uin
   Ctx c;
   c.st = static_cast<cudaStream_t>(stream);
   c.d_err = reinterpret_cast<uint32_t*>(jc.head);
-  cudaError_t e = cudaMemsetAsync(jc.head, 0, kHead, c.st);
+  cudaError_t e = join_begin(c, jc.head, jc.mark);
   if (e == cudaSuccess) e = index_build(c, build_cols[build_key], n_build, jc.j.ix);
   if (e == cudaSuccess) e = join_count_scan(c, jc.j, jc.off, jc.head + 1, jc.cws);
   if (e != cudaSuccess) return CDL_E_CUDA;
@@ -239,8 +239,7 @@ cdl_status cdl_join(const uint32_t* const* probe_cols, uint32_t probe_arity, uin
   const uint64_t total = h[1];
   *n_out = total;
   if (total == 0) return CDL_OK;
-  if (out_cap < total)  // (the workspace is ready for cdl_join_write)
-    return join_mark(c, jc.head, jc.mark) == cudaSuccess ? CDL_E_CAPACITY : CDL_E_CUDA;
+  if (out_cap < total) return CDL_E_CAPACITY;  // (the workspace is ready for cdl_join_write)
   return join_output(jc, out_cols, out_arity, out_cap, total, n_out, c);
 }
 
@@ -263,8 +262,8 @@ cdl_status cdl_join_write(const uint32_t* const* probe_cols, uint32_t probe_arit
   Ctx c;
   c.st = static_cast<cudaStream_t>(stream);
   c.d_err = reinterpret_cast<uint32_t*>(jc.head);
-  if (join_open(c, jc.head, jc.mark, total) != cudaSuccess) return CDL_E_CUDA;
-  jc.j.gate = jc.head + 3;
+  jc.j.head = jc.head;
+  jc.j.mark = jc.mark;
   return join_output(jc, out_cols, out_arity, out_cap, total, n_out, c);
 }
 

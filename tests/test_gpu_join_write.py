@@ -23,11 +23,11 @@ def cdl():
 class Call:
     """One join's arguments; key = column 0 on both sides."""
 
-    def __init__(self, cdl, n_probe, n_build, neq=False, seed=0):
+    def __init__(self, cdl, n_probe, n_build, neq=False, seed=0, keys=None):
         import torch
         self.L, self.cdl, self.neq = cdl.lib(), cdl, neq
         rng = np.random.default_rng(seed)
-        keys = max(1, n_build // 2)
+        keys = keys or max(1, n_build // 2)
         self.probe = np.stack([rng.integers(0, keys, n_probe), rng.integers(0, 3, n_probe)])
         self.build = np.stack([np.sort(rng.integers(0, keys, n_build)), rng.integers(0, 3, n_build)])
         dev = lambda a: [torch.from_numpy(np.ascontiguousarray(c.astype(np.int32))).cuda() for c in a]
@@ -111,9 +111,11 @@ def refused(c, total, size=None):
 
 
 # (the workspace is a well-formed one of another call, or zeros: a library
-# without the check reads and writes within its buffers all the same)
-def test_write_without_its_query(cdl):
-    c = Call(cdl, 3000, 2000)
+# without the check reads and writes within its buffers all the same.  Of five
+# rows the workspace has no room for the write's splits.)
+@pytest.mark.parametrize("n", [(3000, 2000, None), (5, 400000, 2)])
+def test_write_without_its_query(cdl, n):
+    c = Call(cdl, n[0], n[1], keys=n[2])
     assert c.join(c.ws.data_ptr(), None, 0) == CAPACITY
     total = c.n.value
     assert total > 4
@@ -128,6 +130,7 @@ def test_write_without_its_query(cdl):
     outs = c.outs(total)
     c.n.value = total
     assert c.write(outs, total) == OK and c.n.value == total
+    assert int((outs[0] == -1).sum()) == 0
 
 
 def test_write_of_another_size(cdl):
