@@ -267,7 +267,7 @@ __device__ __forceinline__ uint32_t ref_value(const JoinSpec& j, const ColsIn& p
 // a thread's outputs is, so that its loads are in flight together.  (With the
 // columns unrolled as well -- eight outputs times eight columns times the
 // sides a value may come from -- half of all warp cycles waited for
-// instructions: 77 ms of same generation on 200,000 nodes; 47 so.)
+// instructions: same generation on 200,000 nodes took 98 ms, 68 so.)
 struct SetRefs {
   const uint32_t* p[kMaxK + 16];
   uint32_t side[kMaxK + 16], v[kMaxK + 16];
@@ -770,8 +770,9 @@ __global__ void __launch_bounds__(kCT) k_hub_render(const uint2* __restrict__ hu
 // walks the task's head rows (kHubU of them in flight), reading the four
 // words there and setting only what is missing.  A hub of d build rows costs
 // a probe row 2^b / 128 coalesced 16-byte reads (b the bits of the last head
-// column) instead of d scattered bit reads; bound by the reads of the head's
-// bitmap from L2.  Points-to at scale 2^-7: the joins on hubs took 137 ms
+// column) instead of d scattered bit reads; bound by the latency of those
+// reads (L2 hits 90 to 96 %, L2 9 to 14 % busy) and by the barriers between
+// tasks, at four blocks per SM.  Points-to at scale 2^-7: the joins on hubs took 137 ms
 // pair by pair, 6.8 ms here (the fixpoint 143 -> 15.4 ms); one word per
 // output inside the write kernel took 92 ms (row searches per word).
 constexpr int kHubU = 4;
@@ -1131,9 +1132,12 @@ cudaError_t join_direct(Ctx& c, const JoinSpec& j, ColsOut out, uint64_t* d_curs
 // and walks the outputs in windows of four per thread as k_join_write does.
 // Rows with more than kHeavyChunk outputs are listed and taken in chunks by
 // a second kernel, so that one hot key does not hold one block.
-// Bound by the random accesses to the bitmap.  Same generation on 200,000
-// nodes: 25 ms of counts and scans and 66 of writes become 47 ms; a round of a
-// small closure takes one launch and one wait (4,001 nodes, 46 rounds: 4.9 ->
+// Bound by the latency of its random reads, of entries and of the set (one
+// launch of 53M rows into a 2 GB bitmap: DRAM 8 %, L2 18 % busy; of 0.3M rows
+// into a hash set: DRAM 41 %, L2 23 %, 25 of 39 cycles an instruction waiting
+// for them).  Same generation on 200,000 nodes: 25 ms of counts and scans and
+// 66 of writes became 52 ms, all joins' writes together; a round of a small
+// closure takes one launch and one wait (4,001 nodes, 46 rounds: 4.9 ->
 // 2.3 ms).  Four rows and outputs a thread in 48 registers and five blocks per
 // SM: 57.1 ms for the run on 200,000 nodes (six blocks, 40 registers, 57.4;
 // eight rows in four blocks 62.7, in five blocks, spilling, 77.8).
