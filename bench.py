@@ -30,7 +30,8 @@ Also reported: an end-to-end figure through the C ABI with host buffers
 (input upload and export of every derived relation inside the timed
 region), the roofline of the dominant kernel (its algorithmic bytes / its
 CUDA-event time over the timed steps, against the measured HBM copy
-bandwidth), and the CPU oracle timed on a bounded sample of the same
+bandwidth; joins into a bitmap or a hash set are bound by the latency of
+random accesses, and their fraction counts useful bytes only), and the CPU oracle timed on a bounded sample of the same
 workload on the host cores.
 """
 from __future__ import annotations
@@ -570,7 +571,9 @@ def bench_gb300(args, rank, world, dist):
                           "form in host rounds (events cannot wrap launches inside a captured "
                           "graph)") if in_graph else
                          "CUDA events around every launch of the kernel in the last timed step",
-                "peak_source": peak_src}
+                "peak_source": peak_src,
+                "bytes": "algorithmic: useful bytes, not traffic (a join into a bitmap or hash set "
+                         "is bound by the latency of its random accesses)"}
     # step (d) as a whole: its algorithmic bytes (New and Full read, Full and
     # delta written) over the count pass (with its tile scan) and the write
     # pass, from the step with every class timed
