@@ -572,7 +572,7 @@ def bench_gb300(args, rank, world, dist):
                           "graph)") if in_graph else
                          "CUDA events around every launch of the kernel in the last timed step",
                 "peak_source": peak_src,
-                "bytes": "algorithmic: useful bytes, not traffic (a join into a bitmap or hash set "
+                "note": "algorithmic bytes: useful bytes, not traffic (a join into a bitmap or hash set "
                          "is bound by the latency of its random accesses)"}
     # step (d) as a whole: its algorithmic bytes (New and Full read, Full and
     # delta written) over the count pass (with its tile scan) and the write
