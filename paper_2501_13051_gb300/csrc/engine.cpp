@@ -1245,8 +1245,12 @@ struct cdl_engine {
   cdl_status sets_to_rows() {
     cdl_status r = sets_undo_round();
     if (r != CDL_OK) return r;
+    // every index too: they lie anywhere in the chunks.  The plan of captured
+    // rounds points to those of input relations, so an earlier one lapses (a
+    // round that records it records it again).
     cache.clear();
     prev_full.clear();
+    graph_ready = false;
     set_heavy_buf.reset();
     set_heavy = HeavyList{};
     hashed = false;
