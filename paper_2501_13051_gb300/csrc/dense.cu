@@ -142,6 +142,22 @@ __global__ void __launch_bounds__(kAT) k_hash_keys(DenseSet d, uint32_t* __restr
   }
 }
 
+// Keys as high and low words to 8-byte words, and back.
+__global__ void __launch_bounds__(256) k_hash_zip(const uint32_t* __restrict__ hi,
+                                                  const uint32_t* __restrict__ lo, uint64_t n,
+                                                  uint64_t* __restrict__ out) {
+  for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256)
+    out[i] = (uint64_t)hi[i] << 32 | lo[i];
+}
+__global__ void __launch_bounds__(256) k_hash_unzip(const uint64_t* __restrict__ in, uint64_t n,
+                                                    uint32_t* __restrict__ hi,
+                                                    uint32_t* __restrict__ lo) {
+  for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) {
+    hi[i] = (uint32_t)(in[i] >> 32);
+    lo[i] = (uint32_t)in[i];
+  }
+}
+
 __global__ void __launch_bounds__(256) k_hash_unpack(DenseSet d, const uint32_t* __restrict__ hi,
                                                      const uint32_t* __restrict__ lo, uint64_t n,
                                                      ColsOut out) {
@@ -294,6 +310,25 @@ cudaError_t hash_keys(Ctx& c, const DenseSet& d, uint32_t* hi, uint32_t* lo, uin
   if (blocks > 152 * 16) blocks = 152 * 16;
   k_hash_keys<<<(unsigned)blocks, kAT, 0, c.st>>>(
       d, hi, lo, cap, reinterpret_cast<unsigned long long*>(d_count), c.d_err);
+  return cudaGetLastError();
+}
+
+static unsigned zip_grid(uint64_t n) {
+  const uint64_t blocks = (n + 1023) / 1024;
+  return (unsigned)(blocks < 152 * 64 ? blocks : 152 * 64);
+}
+
+cudaError_t hash_zip(Ctx& c, const uint32_t* hi, const uint32_t* lo, uint64_t n, uint64_t* out) {
+  if (n == 0) return cudaSuccess;
+  ProfScope p(c, kDense, 16.0 * n);
+  k_hash_zip<<<zip_grid(n), 256, 0, c.st>>>(hi, lo, n, out);
+  return cudaGetLastError();
+}
+
+cudaError_t hash_unzip(Ctx& c, const uint64_t* in, uint64_t n, uint32_t* hi, uint32_t* lo) {
+  if (n == 0) return cudaSuccess;
+  ProfScope p(c, kDense, 16.0 * n);
+  k_hash_unzip<<<zip_grid(n), 256, 0, c.st>>>(in, n, hi, lo);
   return cudaGetLastError();
 }
 

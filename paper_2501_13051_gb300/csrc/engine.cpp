@@ -100,6 +100,17 @@ class Pool {
     by_size_.emplace(b.size, p);
   }
 
+  // A block's end past `bytes` goes back.
+  void shrink(void* vp, size_t bytes) {
+    bytes = bytes ? (bytes + 255) & ~size_t(255) : 256;
+    char* p = static_cast<char*>(vp);
+    auto it = used_.find(p);
+    if (it == used_.end() || it->second.size <= bytes) return;
+    used_[p + bytes] = Block{it->second.size - bytes, it->second.chunk};
+    used_[p].size = bytes;
+    put(p + bytes);
+  }
+
   size_t unused() const {
     size_t b = 0;
     for (auto& f : by_size_) b += f.first;
@@ -536,6 +547,7 @@ struct cdl_engine {
   // without a memory limit (give_back_room): asking what is free takes longer
   // than a small round
   static constexpr size_t kRoomBytes = size_t(4) << 30;
+  static constexpr uint64_t kSlabSlots = 1 << 20;  // of a table read at a time (hash_compact)
   // hub joins (hub_join): outputs in all, and per row of both sides, from
   // which they are tried (below, the second count and the other index are
   // not small beside the write); build rows that make a hub, where OR-ing
@@ -1337,6 +1349,9 @@ struct cdl_engine {
     bool any = false;
     for (auto& r : rels) any |= r->set_on;
     if (!any) return CDL_OK;
+    cache.clear();
+    set_heavy_buf.reset();
+    set_heavy = HeavyList{};
     if (failed) {
       cudaMemsetAsync(dslot(kSlotErr), 0, 8, st);  // (reported already)
       cdl_status r = sets_undo_round();
@@ -1364,11 +1379,45 @@ struct cdl_engine {
     return sort_cols(R.delta, bits);
   }
 
+  // A hash set's keys to the front of its table, whose end goes back: where
+  // there is no room for them beside it.  The table is read a slab at a time,
+  // and no more keys are written than slots have been read.
+  cdl_status hash_compact(Relation& R, uint64_t& n) {
+    const uint64_t slots = R.fset.kmask + 1, slab = std::min<uint64_t>(slots, kSlabSlots);
+    DCols part;
+    if (!alloc_cols(part, 2, slab)) return fail(CDL_E_NOMEM, "sorted rows");
+    n = 0;
+    for (uint64_t at = 0; at < slots; at += slab) {
+      DenseSet d = R.fset;
+      d.keys += at;
+      d.kmask = slab - 1;
+      cudaError_t e = hash_keys(ctx, d, part.c[0], part.c[1], slab, dslot(kSlotScratch));
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(h_ctl + kSlotScratch, dslot(kSlotScratch), 8, cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      if (e == cudaSuccess)
+        e = hash_zip(ctx, part.c[0], part.c[1], h_ctl[kSlotScratch],
+                     static_cast<uint64_t*>(R.fset_buf.p) + n);
+      if (e != cudaSuccess) return cuda_fail(e, "sorted rows");
+      n += h_ctl[kSlotScratch];
+    }
+    pool.shrink(R.fset_buf.p, 8 * n);
+    return CDL_OK;
+  }
+
   // The keys of a hash set (about n) as sorted rows.
   cdl_status hash_rows(Relation& R, uint64_t n, DCols& rows) {
     DCols keys;
     for (;;) {
-      if (!alloc_cols(keys, 2, n)) return fail(CDL_E_NOMEM, "sorted rows");
+      if (!alloc_cols(keys, 2, n)) {
+        cdl_status r = hash_compact(R, n);
+        if (r != CDL_OK) return r;
+        if (!alloc_cols(keys, 2, n)) return fail(CDL_E_NOMEM, "sorted rows");
+        keys.n = n;
+        cudaError_t e = hash_unzip(ctx, static_cast<const uint64_t*>(R.fset_buf.p), n, keys.c[0], keys.c[1]);
+        if (e != cudaSuccess) return cuda_fail(e, "sorted rows");
+        break;
+      }
       cudaError_t e = hash_keys(ctx, R.fset, keys.c[0], keys.c[1], n, dslot(kSlotScratch));
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(h_ctl + kSlotScratch, dslot(kSlotScratch), 8, cudaMemcpyDeviceToHost, st);

@@ -230,6 +230,9 @@ cudaError_t set_insert(Ctx& c, const DenseSet& d, ColsIn rows, uint64_t n, ColsO
 cudaError_t hash_move(Ctx& c, const DenseSet& d, const unsigned long long* old, uint64_t slots);
 cudaError_t hash_keys(Ctx& c, const DenseSet& d, uint32_t* hi, uint32_t* lo, uint64_t cap,
                       uint64_t* d_count);
+// Keys as two columns to 8-byte words, and back.
+cudaError_t hash_zip(Ctx& c, const uint32_t* hi, const uint32_t* lo, uint64_t n, uint64_t* out);
+cudaError_t hash_unzip(Ctx& c, const uint64_t* in, uint64_t n, uint32_t* hi, uint32_t* lo);
 cudaError_t hash_unpack(Ctx& c, const DenseSet& d, const uint32_t* hi, const uint32_t* lo,
                         uint64_t n, ColsOut out);
 // Takes n rows out of the set.

@@ -91,3 +91,36 @@ def test_batched(cdl, monkeypatch, budget, graph):
     want = run(cdl, prog, n_instances=40, dense_bits=-1)
     monkeypatch.setattr(cdl, "_TorchArena", arena(cdl, budget))
     same(run(cdl, prog, n_instances=40, graph=graph), want)
+
+
+# Captured rounds that are outgrown by a burst: the round the host then runs
+# may be the one that finds no memory for its sets, and the graph is captured
+# again with sorted rows.
+@pytest.mark.parametrize("graph", [True, 64])
+def test_back_to_rows_behind_captured_rounds(cdl, monkeypatch, graph):
+    from tests.test_gpu_hash_set import bursts, inst
+    prog = W.batched_program([], [])
+    prog.edb["tc_edge"] = np.concatenate([inst(0, bursts(60_000, 400_001)), inst(2, W.er_graph(3000, 3600, 2)),
+                                          inst(4, bursts(3, 70_000))])
+    prog.edb["sg_edge"] = np.concatenate([inst(1, W.random_forest(2500, 3)), inst(3, W.random_forest(700, 4))])
+    want = run(cdl, prog, n_instances=5, dense_bits=-1)
+    assert want[1].derived_tuples > 1 << 18
+
+    def at(budget, **opts):
+        with monkeypatch.context() as m:
+            m.setattr(cdl, "_TorchArena", arena(cdl, budget))
+            try:
+                return run(cdl, prog, n_instances=5, **opts)
+            except cdl.CdlError as ex:
+                assert ex.name == "CDL_E_NOMEM"
+
+    budget, ran = 200_000_000, 0
+    while budget < 2_000_000_000:
+        got = at(budget, graph=graph)
+        if got:
+            same(got, want)
+            ran += 1
+        else:  # no more than sorted rows take
+            assert not at(int(budget * 0.95), dense_bits=-1, graph=graph), budget
+        budget = int(budget * 1.1)
+    assert ran > 8
